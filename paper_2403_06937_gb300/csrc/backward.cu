@@ -216,31 +216,31 @@ struct OzBufs {
     OzMat U, Uc, B, A2;
     double* yr;
     double* yi;
-    long long* lo_r;
-    long long* lo_i;
+    void* scratch;
     int group;
 };
 
 size_t oz_backward_extra(int n) {
     const size_t N = (size_t)1 << n;
-    return 4 * oz_mat_bytes((int)N) + 4 * round256(N * N * sizeof(double)) + 256;
+    return 3 * oz_mat_bytes((int)N, true) + oz_mat_bytes((int)N, false) + oz_scratch_bytes((int)N) +
+           2 * round256(N * N * sizeof(double)) + 256;
 }
 
 // P <- U' P U'^dag with U' = U (or conj U for the adjoint step), emulated FP64
 tc_status step_oz(int N, OzBufs& z, bool adjoint, CM P, CM X, cudaStream_t s) {
     const OzMat& A = adjoint ? z.Uc : z.U;
     TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
-    TC_TRY(oz_product(0, A, z.B, OzOut{X.r, X.i, z.lo_r, z.lo_i}, z.group, s));       // X = U' P^H = U' P
+    TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));       // X = U' P^H = U' P
     TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s));
-    return oz_product(1, A, z.B, OzOut{P.r, P.i, z.lo_r, z.lo_i}, z.group, s);        // P' = U' X^H
+    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{P.r, P.i, z.scratch}, z.group, s);        // P' = U' X^H
 }
 
 // W += rho Lambda = rho Lambda^H (Lambda Hermitian), emulated FP64
 tc_status w_accumulate_oz(int N, OzBufs& z, CM rho, CM L, CM W, bool init, cudaStream_t s) {
     TC_TRY(oz_mat_load(z.A2, rho.r, rho.i, false, false, N, (size_t)N, s));
     TC_TRY(oz_mat_load(z.B, L.r, L.i, false, false, N, (size_t)N, s));
-    if (init) return oz_product(0, z.A2, z.B, OzOut{W.r, W.i, z.lo_r, z.lo_i}, z.group, s);
-    TC_TRY(oz_product(0, z.A2, z.B, OzOut{z.yr, z.yi, z.lo_r, z.lo_i}, z.group, s));
+    if (init) return oz_product(0, z.A2, z.B, L.r, L.i, N, (size_t)N, OzOut{W.r, W.i, z.scratch}, z.group, s);
+    TC_TRY(oz_product(0, z.A2, z.B, L.r, L.i, N, (size_t)N, OzOut{z.yr, z.yi, z.scratch}, z.group, s));
     const size_t NN = (size_t)N * N;
     axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, W.r, W.i, 1.0, z.yr, z.yi, W.r, W.i, NN);
     TC_LAUNCH_CHECK();
@@ -314,15 +314,14 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     const bool oz = precision == TC_FP64_OZAKI;
     OzBufs z{};
     if (oz) {
-        TC_TRY(oz_mat_init(z.U, ar, N));
-        TC_TRY(oz_mat_init(z.Uc, ar, N));
-        TC_TRY(oz_mat_init(z.B, ar, N));
-        TC_TRY(oz_mat_init(z.A2, ar, N));
+        TC_TRY(oz_mat_init(z.U, ar, N, true));
+        TC_TRY(oz_mat_init(z.Uc, ar, N, true));
+        TC_TRY(oz_mat_init(z.B, ar, N, false));
+        TC_TRY(oz_mat_init(z.A2, ar, N, true));
         z.yr = ar.take<double>(NN);
         z.yi = ar.take<double>(NN);
-        z.lo_r = ar.take<long long>(NN);
-        z.lo_i = ar.take<long long>(NN);
-        if (!z.lo_i) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
+        z.scratch = ar.take<uint8_t>(oz_scratch_bytes(N));
+        if (!z.scratch) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
         z.group = tune_lookup(n, TC_BF16X3).tc_group;
         TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));
         TC_TRY(oz_mat_load(z.Uc, static_cast<const double*>(U), nullptr, true, true, N, (size_t)N, s));

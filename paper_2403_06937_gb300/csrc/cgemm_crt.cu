@@ -1,0 +1,849 @@
+// cgemm_crt.cu -- FP64-accurate complex GEMM Y = A B^H on the BF16 tensor
+// cores in a residue number system (the second Ozaki scheme: Ozaki, Uchino
+// and Imamura 2025), for the step rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12) at
+// FP64 accuracy.
+//
+// Integers.  Row r of an operand is scaled by 2^ex[r] so that the 2-norm of
+// its rounded entries stays below 2^58.36.  An entry of A B^H is an inner
+// product of two such rows, so by Cauchy-Schwarz its real and imaginary part
+// stay below M / 2 = 2^116.77 and are fixed by their residues modulo the
+// fifteen p_s (crt_scheme.cuh).  A row whose weight sits in a few entries is
+// held to up to 58 bits of its largest entry, a flat row of K entries to
+// 58 - log2(K) / 2; FP64 holds 53.
+//
+// The diagonal of the left operand is not in the planes: the caller's U is
+// close to the identity, and Y = diag(U) B^H + V B^H with the first term in
+// FP64 leaves the integers the small part V only.
+//
+// Products.  For each p_s one BF16 product of the residue planes: A = the
+// rows of A_r and A_i (M = 128), B = the stack [B_r; B_i] (N = 256), two FP32
+// accumulators (512 TMEM columns).  A K chunk of 1024 is exact in FP32; the
+// epilogue reads it out, forms Y_r = A_r B_r^T + A_i B_i^T and Y_i = A_i B_r^T
+// - A_r B_i^T modulo p_s in FP32 (every intermediate an integer below 2^24)
+// and adds it to a packed pair of 16-bit sums in registers, which go out as
+// one byte each when all of K is done.  crt_combine_kernel turns the fifteen
+// bytes of an entry into FP64 (integer work up to one conversion) and adds the
+// diagonal term.
+//
+// Against the digit slices (cgemm_oz.cu: 28, 36 or 45 pair products, an int64
+// read-modify-write of the result after each): 15 products at every size, and
+// 15 bytes per result entry written once.
+//
+// Work unit: (modulus s, tile or tile pair), modulus outermost, so that the
+// units in flight share operand panels in L2; a persistent launch takes them
+// round-robin.  Roles of a CTA: warps 0-7 epilogue (warp w reads TMEM lanes
+// 32 (w % 4) .. + 31, columns 64 (w / 4) .. + 63 of the tile), warp 8 TMA,
+// warp 9 MMA.  Arrangement, barriers and bounded waits of the CTA pairs as
+// cgemm_oz_pair_kernel (cgemm_oz.cu).
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "cgemm_crt.cuh"
+#include "cgemm_dev.cuh"
+#include "cgemm_tc.cuh"
+#include "crt_scheme.cuh"
+
+namespace tc {
+namespace {
+
+using namespace sm100;
+using namespace cg;
+using crt::kModuli;
+
+__constant__ crt::Consts kC = crt::make_consts();
+
+constexpr int kEpiThreads = 256;
+constexpr int kThreads = kEpiThreads + 64;
+constexpr int kRB = 128;                     // bytes of K per operand row in a stage
+constexpr int kTile = 128 * kRB;             // one 128-row operand tile
+constexpr int kKPer = kRB / 2;               // BF16 K values per stage
+constexpr int kSteps = kRB / 32;             // MMA K steps per stage
+constexpr int kRing = 192 * 1024;
+constexpr int kSmem = kRing + 1024 /*align*/ + 512 /*barriers*/;
+constexpr int kChunkStages = crt::kChunk / kKPer;
+constexpr int kGroup = 6;                    // row pairs per raster group (a wave: ~12 row x 12 column tiles)
+constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN
+
+struct CrtLaunch {
+    int tiles;           // Np / 128
+    int kb_total;        // Np / kKPer stages per unit
+    int row0;            // first row pair (pairs) or row tile (single CTAs) of the band
+    int units_per;       // units per modulus
+    int units;           // units_per * kModuli
+    size_t Np;           // row stride of the byte planes
+    size_t band;         // rows of a byte plane
+    uint8_t* bytes;      // [kModuli][2][band][Np], rows from tile row row0 on
+    unsigned* status;
+};
+
+// unit -> (modulus, own row tile, column tile)
+template <bool PAIR, int MODE>
+__device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int rank, int& s, int& I, int& J) {
+    s = u / L.units_per;
+    const int t = u - s * L.units_per;
+    if (PAIR) {
+        if (L.row0 == 0 && L.units_per == pair_units(MODE, L.tiles)) {
+            pair_unit(MODE, L.tiles, kGroup, t, rank, I, J);
+        } else {   // a band of row pairs (even tile count)
+            const int lo = 2 * L.row0, hi = lo + (int)(L.band / 128);
+            if (MODE == 1) {
+                pair_tile_rows_range(1, L.tiles, kGroup, lo, hi, t, rank, I, J);
+            } else {
+                const int rows = (hi - lo) / 2;
+                I = lo + 2 * (t % rows) + rank;
+                J = t / rows;
+            }
+        }
+    } else {
+        if (MODE == 0) {
+            const int rows = (int)(L.band / 128);
+            I = L.row0 + t % rows;
+            J = t / rows;
+        } else {
+            int i, j;
+            tri_decode(t + L.row0 * (L.row0 + 1) / 2, i, j);
+            I = i;
+            J = j;
+        }
+    }
+}
+
+// Adds one K chunk of the tile, modulo p, to the packed sums acc[c]: the low
+// half holds Y_r, the high half Y_i of column 64 half + c (as one 32-bit sum
+// r + 65536 i).  At most 64 chunks of |r| <= p / 2 + 1 stay within 16 bits.
+__device__ __forceinline__ void add_chunk(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64]) {
+    constexpr float kMagic = 12582912.0f;   // 1.5 2^23: adding it rounds to an integer
+#pragma unroll
+    for (int c = 0; c < 64; c += 16) {
+        float d1r[16], d1i[16], d2r[16], d2i[16];
+        tmem_ld16(tl + c, d1r);            // A_r B_r^T
+        tmem_ld16(tl + 128 + c, d1i);      // A_r B_i^T
+        tmem_ld16(tl + 256 + c, d2r);      // A_i B_r^T
+        tmem_ld16(tl + 384 + c, d2i);      // A_i B_i^T
+        tmem_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            // the quotient may come from the rounded sum; the remainder is exact:
+            // |d1 - p q| <= |d2| + p < 2^24
+            const float qr = __fmaf_rn(__fadd_rn(d1r[q], d2i[q]), inv_p, kMagic) - kMagic;
+            const float qi = __fmaf_rn(__fsub_rn(d2r[q], d1i[q]), inv_p, kMagic) - kMagic;
+            const float yr = __fadd_rn(__fmaf_rn(-qr, p, d1r[q]), d2i[q]);
+            const float yi = __fsub_rn(__fmaf_rn(-qi, p, d2r[q]), d1i[q]);
+            const uint32_t br = __float_as_uint(__fadd_rn(yr, kMagic)), bi = __float_as_uint(__fadd_rn(yi, kMagic));
+            // both carry the magic's bits 0x4B400000; shifted by 16 they vanish modulo 2^32
+            acc[c + q] += br - 0x4B400000u + (bi << 16);
+        }
+    }
+}
+
+// sum of residues -> byte: balanced modulo p, plus 128
+__device__ __forceinline__ uint32_t to_byte(int v, float p, float inv_p) {
+    constexpr float kMagic = 12582912.0f;
+    const float f = __uint_as_float(0x4B400000u + (uint32_t)v) - kMagic;
+    const float q = __fmaf_rn(f, inv_p, kMagic) - kMagic;
+    const float r = __fmaf_rn(-q, p, f);
+    return (__float_as_uint(__fadd_rn(r, kMagic + 128.0f))) & 0xFFu;
+}
+
+template <bool PAIR, int MODE>
+__global__ void __launch_bounds__(kThreads, 1)
+    cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
+    constexpr int kOperandTiles = PAIR ? 3 : 4;   // own A_r, A_i rows; half the B stack, or all of it
+    constexpr int kStage = kOperandTiles * kTile;
+    constexpr int kStages = kRing / kStage;
+    constexpr uint32_t kIdesc = make_idesc(1u, PAIR ? 256u : 128u, 256u);
+
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
+    uint64_t* empty = full + kStages;
+    uint64_t* accum = empty + kStages;      // MMA -> epilogue, once per chunk
+    uint64_t* tmem_empty = accum + 1;       // epilogue -> MMA, once per chunk
+    uint64_t* drain = tmem_empty + 1;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t lim = kWaitLimitNs;
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
+    const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kStages; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        mbar_init(accum, 1);
+        mbar_init(tmem_empty, PAIR ? 2 : 1);
+        mbar_init(drain, 1);
+        *abort = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        if (PAIR) {
+            tmem_alloc_pair(saddr(tmem_slot), 512);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(saddr(tmem_slot), 512);
+            tmem_relinquish();
+        }
+    }
+    if (warp == 8 && lane == 0) {
+        prefetch_tmap(&tmA);
+        prefetch_tmap(&tmB);
+    }
+    __syncthreads();
+    if (PAIR) cluster_sync();   // both CTAs' barriers exist before either arrives on the other's
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t peer_abort = PAIR ? cluster_addr(saddr(const_cast<int*>(abort)), rank ^ 1u) : 0u;
+    const int chunks = (L.kb_total + kChunkStages - 1) / kChunkStages;
+
+    if (warp == 8) {
+        // ---------------------------------------------------------- producer
+        if (lane == 0) {
+            const uint32_t lead_full = PAIR ? cluster_addr(saddr(&full[0]), 0u) : saddr(&full[0]);
+            uint32_t it = 0;
+            bool ok = true;
+            for (int u = worker; u < L.units && ok; u += workers) {
+                int s, I, J;
+                unit_at<PAIR, MODE>(L, u, (int)rank, s, I, J);
+                for (int kb = 0; kb < L.kb_total; kb++, it++) {
+                    const int b = it % kStages;
+                    const uint32_t ph = (it / kStages) & 1u;
+                    if (!mbar_wait_bounded(&empty[b], ph ^ 1u, abort, lim, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* st = smem + b * kStage;
+                    const int kx = kb * kKPer;
+                    if (!PAIR) {
+                        mbar_arrive_expect_tx(&full[b], kStage);
+                        const uint32_t fb = saddr(&full[b]);
+                        tma_load_3d(saddr(st), &tmA, fb, kx, I * 128, s);
+                        tma_load_3d(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
+                        tma_load_3d(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, s);
+                        tma_load_3d(saddr(st + 3 * kTile), &tmB, fb, kx, J * 128, kModuli + s);
+                    } else if (rank == 0) {
+                        mbar_arrive_expect_tx(&full[b], 2 * kStage);   // both CTAs' bytes
+                        const uint32_t fb = saddr(&full[b]);
+                        tma_load_3d(saddr(st), &tmA, fb, kx, I * 128, s);
+                        tma_load_3d(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
+                        tma_load_3d(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, s);                  // B_r
+                    } else {
+                        const uint32_t fb = lead_full + 8u * (uint32_t)b;
+                        tma_load_3d_pair(saddr(st), &tmA, fb, kx, I * 128, s);
+                        tma_load_3d_pair(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
+                        tma_load_3d_pair(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, kModuli + s);   // B_i
+                    }
+                }
+            }
+            const uint32_t from = it > (uint32_t)kStages ? it - kStages : 0u;
+            if (!ok || *abort) {
+                *abort = 1;
+                if (PAIR) st_cluster_u32(peer_abort, 1u);
+                // the copies in flight land before the CTAs go away
+                if (rank == 0) {
+                    for (uint32_t k = from; k < it; k++)
+                        (void)mbar_wait_bounded(&full[k % kStages], (k / kStages) & 1u, nullptr, 10000000ull, 0);
+                } else {
+                    spin_ns(1000000ull);
+                }
+            } else {
+                // the last releases of this CTA's stages have arrived
+                for (uint32_t k = from; k < it; k++)
+                    (void)mbar_wait_bounded(&empty[k % kStages], (k / kStages) & 1u, abort, lim, 0);
+            }
+        }
+    } else if (warp == 9) {
+        if (lane == 0 && rank == 0) {
+            // ------------------------------------------------------ MMA issuer
+            const uint32_t peer_empty = PAIR ? cluster_addr(saddr(&empty[0]), 1u) : 0u;
+            const uint32_t peer_accum = PAIR ? cluster_addr(saddr(accum), 1u) : 0u;
+            uint32_t it = 0, pass = 0;
+            bool ok = true;
+            for (int u = worker; u < L.units && ok; u += workers) {
+                for (int c = 0; c < chunks && ok; c++, pass++) {
+                    if (pass > 0 && !mbar_wait_bounded_cluster(tmem_empty, (pass - 1) & 1u, abort, lim, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const int kb0 = c * kChunkStages;
+                    const int kb1 = kb0 + kChunkStages < L.kb_total ? kb0 + kChunkStages : L.kb_total;
+                    for (int kb = kb0; kb < kb1; kb++, it++) {
+                        const int b = it % kStages;
+                        const uint32_t ph = (it / kStages) & 1u;
+                        if (!mbar_wait_bounded_cluster(&full[b], ph, abort, lim, 0)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        uint8_t* st = smem + b * kStage;
+                        const uint64_t ar = desc_kmajor<kRB>(saddr(st));
+                        const uint64_t ai = desc_kmajor<kRB>(saddr(st + kTile));
+                        const uint64_t bd = desc_kmajor<kRB>(saddr(st + 2 * kTile));
+#pragma unroll
+                        for (int ks = 0; ks < kSteps; ks++) {
+                            const uint32_t acc = (kb > kb0 || ks > 0) ? 1u : 0u;
+                            const uint64_t off = 2u * (uint64_t)ks;   // 32 bytes of K further in each row
+                            if (PAIR) {
+                                umma_pair(tmem, ar + off, bd + off, kIdesc, acc);
+                                umma_pair(tmem + 256, ai + off, bd + off, kIdesc, acc);
+                            } else {
+                                umma<0>(tmem, ar + off, bd + off, kIdesc, acc);
+                                umma<0>(tmem + 256, ai + off, bd + off, kIdesc, acc);
+                            }
+                        }
+                        if (PAIR) {
+                            umma_commit_pair(saddr(&empty[b]));
+                            umma_commit_pair(peer_empty + 8u * (uint32_t)b);
+                        } else {
+                            umma_commit(saddr(&empty[b]));
+                        }
+                    }
+                    if (!ok) break;
+                    if (PAIR) {
+                        umma_commit_pair(saddr(accum));
+                        umma_commit_pair(peer_accum);
+                    } else {
+                        umma_commit(saddr(accum));
+                    }
+                }
+            }
+            // the MMAs complete before TMEM is freed
+            if (PAIR)
+                umma_commit_pair(saddr(drain));
+            else
+                umma_commit(saddr(drain));
+            (void)mbar_wait_bounded(drain, 0u, nullptr, lim, 0);
+            if (PAIR && *abort) st_cluster_u32(peer_abort, 1u);
+        }
+    } else {
+        // ---------------------------------------------------------- epilogue
+        const uint32_t lead_tmem_empty = PAIR ? cluster_addr(saddr(tmem_empty), 0u) : 0u;
+        const int half = warp >> 2;
+        const int row = (warp & 3) * 32 + lane;   // TMEM lane = row of the tile
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 64u * (uint32_t)half;
+        uint32_t pass = 0;
+        bool stop = false;
+        for (int u = worker; u < L.units && !stop; u += workers) {
+            int s, I, J;
+            unit_at<PAIR, MODE>(L, u, (int)rank, s, I, J);
+            const float p = (float)kC.p[s], inv_p = 1.0f / p;
+            // rows past an odd tile count, and the tile above the diagonal of a
+            // Hermitian product, are not written
+            const bool own = I < L.tiles && !(MODE == 1 && J > I);
+            uint32_t acc[64];
+#pragma unroll
+            for (int c = 0; c < 64; c++) acc[c] = 0u;
+            for (int c = 0; c < chunks; c++, pass++) {
+                const bool ok = mbar_wait_bounded_cluster(accum, pass & 1u, abort, lim, 32);
+                tc_fence_after();
+                // the epilogue warps leave together or not at all
+                uint32_t bad = (!ok || *abort) ? 1u : 0u, any;
+                asm volatile(
+                    "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+                    "bar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
+                    : "=r"(any)
+                    : "r"(bad)
+                    : "memory");
+                if (any) {
+                    if (threadIdx.x == 0) {
+                        *abort = 1;
+                        if (PAIR) st_cluster_u32(peer_abort, 1u);
+                    }
+                    stop = true;
+                    break;
+                }
+                add_chunk(tl, p, inv_p, acc);
+                tc_fence_before();
+                asm volatile("bar.sync 1, 256;" ::: "memory");   // every epilogue warp has read TMEM
+                if (threadIdx.x == 0) {
+                    if (rank == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");
+                    else
+                        mbar_arrive_cluster(lead_tmem_empty);
+                }
+            }
+            if (stop || !own) continue;
+            const size_t r0 = (size_t)I * 128 - (size_t)L.row0 * (PAIR ? 256 : 128) + row;   // row within the band
+            uint8_t* yr = L.bytes + ((size_t)(2 * s) * L.band + r0) * L.Np + (size_t)J * 128 + 64 * half;
+            uint8_t* yi = yr + L.band * L.Np;
+#pragma unroll
+            for (int c = 0; c < 64; c += 16) {
+                uint32_t wr[4], wi[4];
+#pragma unroll
+                for (int w = 0; w < 4; w++) {
+                    wr[w] = 0u;
+                    wi[w] = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const uint32_t v = acc[c + 4 * w + q];
+                        const int r = (int)(short)(v & 0xFFFFu);
+                        const int i = (int)(v - (uint32_t)r) >> 16;
+                        wr[w] |= to_byte(r, p, inv_p) << (8 * q);
+                        wi[w] |= to_byte(i, p, inv_p) << (8 * q);
+                    }
+                }
+                *reinterpret_cast<uint4*>(yr + c) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
+                *reinterpret_cast<uint4*>(yi + c) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
+            }
+        }
+        if (*abort && threadIdx.x == 0) atomicOr(L.status, kStatusTimeout);
+    }
+
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (PAIR) cluster_sync();   // neither CTA frees TMEM or leaves while the other may still use it
+    if (warp == 0) {
+        tc_fence_after();
+        if (PAIR)
+            tmem_dealloc_pair(tmem, 512);
+        else
+            tmem_dealloc(tmem, 512);
+    }
+}
+
+// ---------------------------------------------------------------- residues
+// Row scale and residue planes of one operand.  A row is handled by TPR
+// consecutive threads of a 128-thread block (8 columns a thread and step):
+// first the scale from the row's largest exponent and its 2-norm, then the
+// residues.  Bound by HBM for large matrices (16 B read, 60 B written per
+// entry; the second read of the row comes from L2); no FP64 instruction, since
+// one FP64 conversion per entry alone would take as long as a third of the
+// writes on this GPU.
+struct RowStat {
+    int e;       // largest biased exponent (0: all zero, 0x7FF: not finite)
+    float ss;    // sum of squares over 2^(2 (e - 1022))
+};
+__device__ __forceinline__ RowStat stat_join(RowStat a, RowStat b) {
+    RowStat r;
+    r.e = max(a.e, b.e);
+    const int da = max(a.e - r.e, -63), db = max(b.e - r.e, -63);
+    r.ss = a.ss * __uint_as_float((uint32_t)(127 + 2 * da) << 23) + b.ss * __uint_as_float((uint32_t)(127 + 2 * db) << 23);
+    return r;
+}
+__device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits) {
+    const uint32_t hi = (uint32_t)(bits >> 32) & 0x7FFFFFFFu;
+    if ((bits << 1) == 0) return;
+    const int e = max((int)(hi >> 20), 1);   // a subnormal counts as the normal number of the same significand bits
+    if (e > a.e) {   // rescale to the new exponent
+        const int d = max(a.e - e, -63);
+        a.ss *= __uint_as_float((uint32_t)(127 + 2 * d) << 23);
+        a.e = e;
+    }
+    const int d = e - a.e;
+    // |x| / 2^(a.e - 1022) from the top 24 significand bits
+    const float f = d < -60 ? 0.0f
+                            : __uint_as_float(((uint32_t)(126 + d) << 23) | ((hi & 0xFFFFFu) << 3) |
+                                              (uint32_t)((bits >> 29) & 7u));
+    a.ss = fmaf(f, f, a.ss);
+}
+
+template <bool INTERLEAVED, bool LEFT>
+__global__ void __launch_bounds__(128)
+    crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
+                       int tpr, uint64_t im_flip, __nv_bfloat16* __restrict__ planes, int* __restrict__ ex,
+                       double* __restrict__ diag) {
+    const int sub = threadIdx.x % tpr;                       // thread within the row
+    const int r = blockIdx.x * (128 / tpr) + threadIdx.x / tpr;
+    // 8 consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
+    auto load8 = [&](int c0, uint64_t (&xr)[8], uint64_t (&xi)[8]) {
+        if (INTERLEAVED) {
+            const ulonglong2* p = reinterpret_cast<const ulonglong2*>(re) + (size_t)r * ld + c0;
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                ulonglong2 v = make_ulonglong2(0, 0);
+                if (r < N && c0 + q < N) v = p[q];
+                xr[q] = v.x;
+                xi[q] = v.y;
+            }
+        } else {
+            const double* pr = re + (size_t)r * ld + c0;
+            const double* pi = im + (size_t)r * ld + c0;
+            if (r < N && c0 + 8 <= N) {   // ld even, planes 16-byte aligned (checked on the host)
+#pragma unroll
+                for (int q = 0; q < 8; q += 2) {
+                    const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pr + q);
+                    const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(pi + q);
+                    xr[q] = a.x;
+                    xr[q + 1] = a.y;
+                    xi[q] = b.x;
+                    xi[q + 1] = b.y;
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < 8; q++) {
+                    const bool in = r < N && c0 + q < N;
+                    xr[q] = in ? (uint64_t)__double_as_longlong(pr[q]) : 0;
+                    xi[q] = in ? (uint64_t)__double_as_longlong(pi[q]) : 0;
+                }
+            }
+        }
+        if (LEFT && r >= c0 && r < c0 + 8) {
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+                if (c0 + q == r) {
+                    xr[q] = 0;
+                    xi[q] = 0;
+                }
+        }
+    };
+    RowStat st{0, 0.0f};
+    for (int c0 = 8 * sub; c0 < Np; c0 += 8 * tpr) {
+        uint64_t xr[8], xi[8];
+        load8(c0, xr, xi);
+#pragma unroll
+        for (int q = 0; q < 8; q++) {
+            stat_add(st, xr[q]);
+            stat_add(st, xi[q]);
+        }
+    }
+    for (int o = min(tpr, 32) / 2; o > 0; o >>= 1) {
+        RowStat b;
+        b.e = __shfl_xor_sync(0xffffffffu, st.e, o);
+        b.ss = __shfl_xor_sync(0xffffffffu, st.ss, o);
+        st = stat_join(st, b);
+    }
+    if (tpr > 32) {   // one row per tpr / 32 warps
+        __shared__ RowStat part[4];
+        const int w = threadIdx.x >> 5;
+        if ((threadIdx.x & 31) == 0) part[w] = st;
+        __syncthreads();
+        const int w0 = (threadIdx.x / tpr) * (tpr / 32);
+        st = part[w0];
+        for (int k = 1; k < tpr / 32; k++) st = stat_join(st, part[w0 + k]);
+    }
+    // ex = the largest shift with 2-norm * 2^ex <= 2^58.35 (any for a row of zeros)
+    const bool finite = st.e < 0x7FF;
+    const int sh = st.e == 0 ? 0 : (int)floorf(58.35f - 0.5f * log2f(st.ss * 1.0001f)) - (st.e - 1022);
+    if (r < Np && sub == 0) {
+        ex[r] = finite ? sh : kNoScale;
+        if (LEFT) {
+            double dr = 0.0, di = 0.0;
+            if (r < N) {
+                dr = INTERLEAVED ? re[2 * ((size_t)r * ld + r)] : re[(size_t)r * ld + r];
+                di = INTERLEAVED ? re[2 * ((size_t)r * ld + r) + 1] : im[(size_t)r * ld + r];
+                if (im_flip) di = -di;
+            }
+            diag[r] = dr;
+            diag[Np + r] = di;
+        }
+    }
+    const size_t plane = (size_t)Np * Np;
+    for (int c0 = 8 * sub; c0 < Np; c0 += 8 * tpr) {
+        uint64_t xr[8], xi[8];
+        load8(c0, xr, xi);
+#pragma unroll
+        for (int part = 0; part < 2; part++) {
+            crt::Pieces pc[8];
+            uint32_t sign[4];
+#pragma unroll
+            for (int q = 0; q < 8; q++) {
+                const uint64_t b = part ? xi[q] ^ im_flip : xr[q];
+                pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0);
+                const uint32_t sg = (uint32_t)(b >> 63) << 15;
+                if (q & 1)
+                    sign[q / 2] |= sg << 16;
+                else
+                    sign[q / 2] = sg;
+            }
+            __nv_bfloat16* dst = planes + (size_t)(part * kModuli) * plane + (size_t)r * Np + c0;
+#pragma unroll
+            for (int s = 0; s < kModuli; s++) {
+                const int p = crt::modulus(s);
+                uint32_t w[4];
+#pragma unroll
+                for (int h = 0; h < 4; h++) {
+                    uint32_t b[2];
+#pragma unroll
+                    for (int k = 0; k < 2; k++) {
+                        const int v = LEFT ? crt::residue(pc[2 * h + k], p, kC.inv[s]) : crt::residue(pc[2 * h + k], p, 1);
+                        // exact conversion: |v| <= 127 through the 1.5 2^23 magic
+                        b[k] = __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)v) - 12582912.0f);
+                    }
+                    w[h] = __byte_perm(b[0], b[1], 0x7632) ^ sign[h];   // the top halves are the BF16 values
+                }
+                *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+            }
+        }
+    }
+}
+
+// ---------------------------------------------------------------- recombination
+__device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
+
+// mag 2^e in FP64, e of any size (one rounding unless the result is subnormal)
+__device__ __forceinline__ double scaled(uint64_t mag, bool neg, int e) {
+    double v = __ull2double_rn(mag);
+    if (mag) {
+        if (e >= -1000 && e <= 900) {
+            v *= pow2d(e);
+        } else {
+            const int e1 = max(min(e, 900), -1000), e2 = max(min(e - e1, 900), -1000);
+            v = v * pow2d(e1) * pow2d(e2);
+        }
+    }
+    return neg ? -v : v;
+}
+
+struct CrtCombine {
+    const uint8_t* bytes;    // [kModuli][2][band][Np]
+    size_t Np, band;
+    int row0;                // first matrix row of the band
+    int N;                   // valid rows and columns of B
+    size_t ldb;
+    const int* ea;
+    const int* eb;
+    const double* diag;      // [2][Np] or null
+    const double* br;
+    const double* bi;
+    double* yr;
+    double* yi;
+};
+
+// One 32 x 32 tile of Y per block of 256 threads, four consecutive columns a
+// thread.  MODE 1: tiles on and below the diagonal, each mirrored.  B's
+// entries of the diagonal term, and the mirrored half, are transposed through
+// shared memory so that every global access runs along rows.
+template <int MODE>
+__global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
+    __shared__ double sr[32][33], si[32][33];
+    const int i0 = p.row0 + 32 * (int)blockIdx.y, j0 = 32 * (int)blockIdx.x;
+    if (MODE == 1 && j0 > i0) return;
+    const int ti = threadIdx.x >> 3, tj = (threadIdx.x & 7) * 4;
+    // B[j0 + a][i0 + b] -> s[a][b]
+    if (p.diag) {
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            const int a = ti, b = tj + k;
+            const bool in = j0 + a < p.N && i0 + b < p.N;
+            const size_t o = (size_t)(j0 + a) * p.ldb + (size_t)(i0 + b);
+            sr[a][b] = in ? p.br[o] : 0.0;
+            si[a][b] = in ? p.bi[o] : 0.0;
+        }
+    }
+    const int i = i0 + ti, j = j0 + tj;
+    const size_t o = (size_t)(i - p.row0) * p.Np + j;
+    crt::Acc ar[4] = {}, ai[4] = {};
+#pragma unroll
+    for (int s = 0; s < kModuli; s++) {
+        const uint32_t wr = *reinterpret_cast<const uint32_t*>(p.bytes + (size_t)(2 * s) * p.band * p.Np + o);
+        const uint32_t wi = *reinterpret_cast<const uint32_t*>(p.bytes + (size_t)(2 * s + 1) * p.band * p.Np + o);
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            crt::acc_add(ar[k], (wr >> (8 * k)) & 0xFFu, kC.frac[s]);
+            crt::acc_add(ai[k], (wi >> (8 * k)) & 0xFFu, kC.frac[s]);
+        }
+    }
+    const int ea = p.ea[i];
+    double vr[4], vi[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int eb = p.eb[j + k];
+        if (ea == kNoScale || eb == kNoScale) {   // an infinity or a NaN in either row
+            vr[k] = vi[k] = __longlong_as_double(0x7FF8000000000000ll);
+            continue;
+        }
+        bool neg;
+        int e;
+        uint64_t mag = crt::acc_finish(ar[k], kC, neg, e);
+        vr[k] = scaled(mag, neg, e - ea - eb);
+        mag = crt::acc_finish(ai[k], kC, neg, e);
+        vi[k] = scaled(mag, neg, e - ea - eb);
+    }
+    if (p.diag) {
+        __syncthreads();
+        const double dr = p.diag[i], di = p.diag[p.Np + i];
+#pragma unroll
+        for (int k = 0; k < 4; k++) {   // A_ii conj(B_ji)
+            const double br = sr[tj + k][ti], bi = si[tj + k][ti];
+            vr[k] = fma(dr, br, fma(di, bi, vr[k]));
+            vi[k] = fma(di, br, fma(-dr, bi, vi[k]));
+        }
+    }
+    double* yr = p.yr + (size_t)i * p.Np + j;
+    double* yi = p.yi + (size_t)i * p.Np + j;
+    if (MODE == 0 || i0 > j0) {
+        *reinterpret_cast<double2*>(yr) = make_double2(vr[0], vr[1]);
+        *reinterpret_cast<double2*>(yr + 2) = make_double2(vr[2], vr[3]);
+        *reinterpret_cast<double2*>(yi) = make_double2(vi[0], vi[1]);
+        *reinterpret_cast<double2*>(yi + 2) = make_double2(vi[2], vi[3]);
+    }
+    if (MODE == 1) {
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 4; k++) {
+            sr[ti][tj + k] = vr[k];
+            si[ti][tj + k] = vi[k];
+        }
+        __syncthreads();
+        if (i0 > j0) {   // Y[j0 + ti][i0 + tj ..] = conj(Y[i0 + tj ..][j0 + ti])
+            double* mr = p.yr + (size_t)(j0 + ti) * p.Np + i0 + tj;
+            double* mi = p.yi + (size_t)(j0 + ti) * p.Np + i0 + tj;
+            *reinterpret_cast<double2*>(mr) = make_double2(sr[tj][ti], sr[tj + 1][ti]);
+            *reinterpret_cast<double2*>(mr + 2) = make_double2(sr[tj + 2][ti], sr[tj + 3][ti]);
+            *reinterpret_cast<double2*>(mi) = make_double2(-si[tj][ti], -si[tj + 1][ti]);
+            *reinterpret_cast<double2*>(mi + 2) = make_double2(-si[tj + 2][ti], -si[tj + 3][ti]);
+        } else {         // a diagonal tile: the lower half, its mirror, a real diagonal
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int c = tj + k;
+                yr[k] = c <= ti ? vr[k] : sr[c][ti];
+                yi[k] = c < ti ? vi[k] : (c == ti ? 0.0 : -si[c][ti]);
+            }
+        }
+    }
+}
+
+int sm_count() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+template <bool PAIR, int MODE>
+tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
+    auto k = cgemm_crt_kernel<PAIR, MODE>;
+    static bool attr_set[64] = {};
+    int dev = 0;
+    TC_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return fail(TC_ERR_UNSUPPORTED_DEVICE, "device index out of range");
+    if (!attr_set[dev]) {
+        TC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
+        attr_set[dev] = true;
+    }
+    const int workers = std::min(L.units, PAIR ? sm_count() / 2 : sm_count());
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(PAIR ? 2 * workers : workers));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = kSmem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    TC_CUDA(cudaLaunchKernelEx(&cfg, k, tmA, tmB, L));
+    TC_LAUNCH_CHECK();
+    return TC_OK;
+}
+
+// rows of a band: all of them up to 16384, else 4096 (bounds the byte scratch)
+int band_rows(int Np) { return Np <= 16384 ? Np : 4096; }
+
+}  // namespace
+
+size_t crt_mat_bytes(int Np, bool left) {
+    return round256((size_t)2 * kModuli * Np * Np * 2) + round256((size_t)Np * sizeof(int)) +
+           (left ? round256((size_t)2 * Np * sizeof(double)) : 0);
+}
+
+size_t crt_scratch_bytes(int Np) { return round256((size_t)2 * kModuli * band_rows(Np) * Np); }
+
+tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left) {
+    m.Np = Np;
+    m.left = left;
+    m.planes = ar.take<uint8_t>((size_t)2 * kModuli * Np * Np * 2);
+    m.ex = ar.take<int>((size_t)Np);
+    m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
+    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
+    return make_part_map_rows(&m.map, m.planes, Np, 2 * kModuli, TC_BF16X3, kRB);
+}
+
+tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
+    if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
+    view = base;
+    view.Np = Np;
+    return make_part_map_rows(&view.map, base.planes, Np, 2 * kModuli, TC_BF16X3, kRB);
+}
+
+tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
+                       size_t ld, cudaStream_t s) {
+    if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
+        (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
+        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
+    const int tpr = std::min(128, m.Np / 8);   // Np is a multiple of 128: 16, 32, 48, ... threads a row
+    // only powers of two divide the block evenly; ragged sizes take the next one below
+    int t = 16;
+    while (2 * t <= tpr) t *= 2;
+    const unsigned grid = (unsigned)((m.Np + 128 / t - 1) / (128 / t));
+    const uint64_t flip = conj ? 1ull << 63 : 0;
+    auto* out = static_cast<__nv_bfloat16*>(m.planes);
+    if (interleaved) {
+        if (m.left)
+            crt_residue_kernel<true, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+        else
+            crt_residue_kernel<true, false><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+    } else {
+        if (m.left)
+            crt_residue_kernel<false, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+        else
+            crt_residue_kernel<false, false><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+    }
+    TC_LAUNCH_CHECK();
+    return TC_OK;
+}
+
+tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
+                      size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s) {
+    const int Np = A.Np;
+    if (B.Np != Np || !A.left || B.left || Np < 128 || Np % 128 != 0 || Np > 65536)
+        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes or roles");
+    if (mode != 0 && mode != 1) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: mode");
+    const int T = Np / 128;
+    if (T < 2) pairs = false;
+    const int band = band_rows(Np);   // Np itself, or a divisor that is a multiple of 256
+    for (int row0 = 0; row0 < Np; row0 += band) {
+        CrtLaunch L{};
+        L.tiles = T;
+        L.kb_total = Np / kKPer;
+        L.row0 = pairs ? row0 / 256 : row0 / 128;
+        L.Np = (size_t)Np;
+        L.band = (size_t)band;
+        L.bytes = static_cast<uint8_t*>(out.scratch);
+        L.status = device_status_word();
+        const int t0 = row0 / 128, t1 = (row0 + band) / 128;
+        if (band == Np)
+            L.units_per = pairs ? (int)pair_units(mode, T) : (mode == 0 ? T * T : T * (T + 1) / 2);
+        else if (pairs)
+            L.units_per = mode == 0 ? T * (t1 - t0) / 2 : (int)pair_count(1, T, t0, t1);
+        else
+            L.units_per = mode == 0 ? T * (t1 - t0) : t1 * (t1 + 1) / 2 - t0 * (t0 + 1) / 2;
+        L.units = L.units_per * kModuli;
+        if (pairs)
+            TC_TRY((mode == 0 ? launch<true, 0>(A.map, B.map, L, s) : launch<true, 1>(A.map, B.map, L, s)));
+        else
+            TC_TRY((mode == 0 ? launch<false, 0>(A.map, B.map, L, s) : launch<false, 1>(A.map, B.map, L, s)));
+        CrtCombine c{};
+        c.bytes = L.bytes;
+        c.Np = (size_t)Np;
+        c.band = (size_t)band;
+        c.row0 = row0;
+        c.N = N;
+        c.ldb = ldb;
+        c.ea = A.ex;
+        c.eb = B.ex;
+        c.diag = A.diag;
+        c.br = br;
+        c.bi = bi;
+        c.yr = out.yr;
+        c.yi = out.yi;
+        const dim3 grid((unsigned)((mode == 0 ? Np : row0 + band) / 32), (unsigned)(band / 32));
+        if (mode == 0)
+            crt_combine_kernel<0><<<grid, 256, 0, s>>>(c);
+        else
+            crt_combine_kernel<1><<<grid, 256, 0, s>>>(c);
+        TC_LAUNCH_CHECK();
+    }
+    return TC_OK;
+}
+
+}  // namespace tc

@@ -1,0 +1,45 @@
+// cgemm_crt.cuh -- FP64-accurate complex GEMM Y = A B^H on the BF16 tensor
+// cores in a residue number system (see cgemm_crt.cu).
+#pragma once
+
+#include <cuda.h>
+
+#include "common.cuh"
+
+namespace tc {
+
+// One operand: 2 x 15 residue planes [Np][Np] in BF16 (re, then im), the
+// power-of-two scale of each row, and, for a left operand, its diagonal.
+struct CrtMat {
+    void* planes;
+    int* ex;          // row r holds round(x 2^ex[r])
+    double* diag;     // left operands: [2][Np], the diagonal kept in FP64 (planes hold zero there)
+    CUtensorMap map;
+    int Np;
+    bool left;
+};
+
+size_t crt_mat_bytes(int Np, bool left);
+tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left);
+// `view`: the buffers of `base` seen as an operand of the smaller padded size Np
+tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np);
+// Residues of the N x N matrix (row stride ld; zero-padded to Np).  interleaved:
+// re points to complex128; conj negates the imaginary part.
+tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
+                       size_t ld, cudaStream_t s);
+// Bytes of scratch of a product: one byte per residue of the result (of a band
+// of rows above Np = 16384).
+size_t crt_scratch_bytes(int Np);
+// Y = A B^H, FP64 planes of row stride Np.  mode 1: Y Hermitian, the
+// block-lower half computed and mirrored.  (br, bi): B's FP64 planes of row
+// stride ldb, valid for N rows and columns, for the diagonal term of A.
+// pairs: CTA pairs on the 2-SM MMA, else single CTAs (the same bits).
+struct CrtOut {
+    double* yr;
+    double* yi;
+    void* scratch;
+};
+tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
+                      size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s);
+
+}  // namespace tc

@@ -37,6 +37,7 @@
 #include "cgemm_dev.cuh"
 #include "cgemm_oz.cuh"
 #include "cgemm_tc.cuh"
+#include "crt_scheme.cuh"
 
 namespace tc {
 namespace {
@@ -709,8 +710,7 @@ tc_status launch_pair(const CUtensorMap& tmU, const CUtensorMap& tmP, const OzEp
 // Both arrangements give the same bits.
 std::atomic<int> g_oz_pairs{-1};
 
-// -1: not chosen yet (TC_OZ_BITS=6 in the environment: 6-bit digits at every
-// size; else the widest digits K allows)
+// -1: not read yet; 1: TC_OZ_BITS=6 in the environment (digit form)
 std::atomic<int> g_oz_narrow{-1};
 
 }  // namespace
@@ -725,16 +725,18 @@ bool oz_use_pairs(int tiles) {
     return v != 0 && tiles >= 2;
 }
 
-OzDigits oz_digits(int Np) {
+bool oz_modular() {
     int narrow = g_oz_narrow.load();
     if (narrow < 0) {
         const char* e = std::getenv("TC_OZ_BITS");
         narrow = e && std::atoi(e) == 6 ? 1 : 0;
         g_oz_narrow.store(narrow);
     }
-    if (!narrow && Np <= 1024) return OzDigits{8, 7, 28, 1024};
-    if (!narrow && Np <= 4096) return OzDigits{7, 8, 36, 4096};
-    return OzDigits{6, 9, 45, 16384};
+    return narrow == 0;
+}
+
+int oz_products() {
+    return oz_modular() ? crt::kModuli : kOzDigits.slices * (kOzDigits.slices + 1) / 2;
 }
 
 tc_status oz_slice(const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld, int Np,
@@ -773,7 +775,7 @@ tc_status cgemm_oz(int mode, const CUtensorMap& tmU, const CUtensorMap& tmP, con
                    const CUtensorMap& tmP_w, const OzEpi& ep, cudaStream_t s) {
     if (ep.Np < 128 || ep.Np % 128 != 0 || ep.tiles * 128 != ep.Np)
         return fail(TC_ERR_INVALID_ARG, "cgemm_oz: padded dimension must be a multiple of 128");
-    const OzDigits dg = oz_digits(ep.Np);
+    const OzDigits dg = kOzDigits;
     if (ep.bits != dg.bits || ep.slices != dg.slices)
         return fail(TC_ERR_INVALID_ARG, "cgemm_oz: digit width does not match the dimension");
     if (ep.Np > dg.kmax && ep.Np % dg.kmax != 0)
@@ -795,39 +797,50 @@ tc_status cgemm_oz(int mode, const CUtensorMap& tmU, const CUtensorMap& tmP, con
 }
 
 size_t oz_slice_bytes(int Np) {
-    return round256((size_t)2 * oz_digits(Np).slices * Np * Np * sizeof(__nv_bfloat16));
+    return round256((size_t)2 * kOzDigits.slices * Np * Np * sizeof(__nv_bfloat16));
 }
 
-size_t oz_mat_bytes(int Np) { return oz_slice_bytes(Np) + round256((size_t)Np * sizeof(int)); }
+size_t oz_mat_bytes(int Np, bool left) {
+    return oz_modular() ? crt_mat_bytes(Np, left) : oz_slice_bytes(Np) + round256((size_t)Np * sizeof(int));
+}
 
-tc_status oz_mat_init(OzMat& m, Arena& ar, int Np) {
+// residue form: the result's residue bytes; digit form: two int64 planes of the low levels
+size_t oz_scratch_bytes(int Np) {
+    return oz_modular() ? crt_scratch_bytes(Np) : 2 * round256((size_t)Np * Np * sizeof(long long));
+}
+
+tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left) {
     m.Np = Np;
-    m.dg = oz_digits(Np);
+    m.left = left;
+    if (oz_modular()) return crt_mat_init(m.crt, ar, Np, left);
     m.slices = ar.take<uint8_t>(oz_slice_bytes(Np));
     m.ex = ar.take<int>((size_t)Np);
     if (!m.ex) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
-    TC_TRY(make_part_map_rows(&m.map_w, m.slices, Np, 2 * m.dg.slices, TC_BF16X3, oz_pair_rows()));
-    return make_part_map(&m.map, m.slices, Np, 2 * m.dg.slices, TC_BF16X3);
+    TC_TRY(make_part_map_rows(&m.map_w, m.slices, Np, 2 * kOzDigits.slices, TC_BF16X3, oz_pair_rows()));
+    return make_part_map(&m.map, m.slices, Np, 2 * kOzDigits.slices, TC_BF16X3);
 }
 
 tc_status oz_mat_view(OzMat& view, const OzMat& base, int Np) {
-    if (Np > base.Np || oz_slice_bytes(Np) > oz_slice_bytes(base.Np))
-        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
+    if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
     view = base;
     view.Np = Np;
-    view.dg = oz_digits(Np);
-    TC_TRY(make_part_map_rows(&view.map_w, base.slices, Np, 2 * view.dg.slices, TC_BF16X3, oz_pair_rows()));
-    return make_part_map(&view.map, base.slices, Np, 2 * view.dg.slices, TC_BF16X3);
+    if (oz_modular()) return crt_mat_view(view.crt, base.crt, Np);
+    TC_TRY(make_part_map_rows(&view.map_w, base.slices, Np, 2 * kOzDigits.slices, TC_BF16X3, oz_pair_rows()));
+    return make_part_map(&view.map, base.slices, Np, 2 * kOzDigits.slices, TC_BF16X3);
 }
 
 tc_status oz_mat_load(OzMat& m, const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld,
                       cudaStream_t s) {
-    return oz_slice(re, im, interleaved, conj, N, ld, m.Np, m.dg, m.slices, m.ex, s);
+    if (oz_modular()) return crt_mat_load(m.crt, re, im, interleaved, conj, N, ld, s);
+    return oz_slice(re, im, interleaved, conj, N, ld, m.Np, kOzDigits, m.slices, m.ex, s);
 }
 
-tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const OzOut& out, int group, cudaStream_t s) {
-    if (A.Np != B.Np || A.dg.bits != B.dg.bits)
-        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
+tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br, const double* bi, int N, size_t ldb,
+                     const OzOut& out, int group, cudaStream_t s) {
+    if (A.Np != B.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
+    if (oz_modular())
+        return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch},
+                           oz_use_pairs(A.Np / 128), s);
     OzEpi ep{};
     ep.Np = A.Np;
     ep.tiles = A.Np / 128;
@@ -836,10 +849,10 @@ tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const OzOut& out,
     ep.eP = B.ex;
     ep.yr = out.yr;
     ep.yi = out.yi;
-    ep.lo_r = out.lo_r;
-    ep.lo_i = out.lo_i;
-    ep.bits = A.dg.bits;
-    ep.slices = A.dg.slices;
+    ep.lo_r = static_cast<long long*>(out.scratch);
+    ep.lo_i = ep.lo_r + round256((size_t)A.Np * A.Np * sizeof(long long)) / sizeof(long long);
+    ep.bits = kOzDigits.bits;
+    ep.slices = kOzDigits.slices;
     ep.status = device_status_word();
     TC_TRY(cgemm_oz(mode, A.map, B.map, A.map_w, B.map_w, ep, s));
     if (mode == 1) TC_TRY(oz_mirror(out.yr, out.yi, A.Np, s));

@@ -4,25 +4,25 @@
 
 #include <cuda.h>
 
+#include "cgemm_crt.cuh"
 #include "common.cuh"
 
 namespace tc {
 
-// Digit width of the slices for the inner dimension K of a product (the
-// padded size Np).  One pass sums K products of two digits of magnitude at
-// most 2^(bits - 1); K 2^(2 bits - 2) <= 2^24 keeps that FP32 sum exact, so
-// the smaller K is, the wider the digits and the fewer the slice pairs:
-//   K <= 1024:  8-bit digits, 7 slices (56 bits), 28 pairs
-//   K <= 4096:  7-bit digits, 8 slices (56 bits), 36 pairs
-//   otherwise:  6-bit digits, 9 slices (54 bits), 45 pairs; K in chunks of 16384
-// TC_OZ_BITS=6 in the environment keeps the 6-bit digits at every size.
+// The FP64-accurate products run in the residue form (cgemm_crt.cu): fifteen
+// BF16 products modulo coprime p_s.  TC_OZ_BITS=6 in the environment takes
+// the digit form (cgemm_oz.cu) instead: nine balanced 6-bit digits an entry
+// and the 45 digit products with t + u < 9, K in chunks of 16384
+// (K 2^(2 bits - 2) <= 2^24 keeps an FP32 sum of digit products exact).
+bool oz_modular();
+int oz_products();   // BF16 products per real product: 15 or 45
+
 struct OzDigits {
     int bits;     // digit width
     int slices;   // digits per entry
-    int pairs;    // slice pairs (t, u) with t + u < slices
     int kmax;     // K per exact pass, 2^(26 - 2 bits)
 };
-OzDigits oz_digits(int Np);
+constexpr OzDigits kOzDigits{6, 9, 16384};
 
 struct OzEpi {
     int Np;             // padded dimension, a multiple of 128
@@ -34,14 +34,14 @@ struct OzEpi {
     double* yi;
     long long* lo_r;    // int64 scratch planes [Np][Np] of the low levels
     long long* lo_i;
-    int bits;           // digit width and slices per entry (oz_digits(Np))
+    int bits;           // digit width and slices per entry
     int slices;
     unsigned* status;
     unsigned long long wait_ns;   // limit of every barrier wait (0 = 2 s)
 };
 
 // Slices [2 * S][Np][Np] (BF16 digits: re slices, then im slices; S digits of
-// `bits` bits, oz_digits(Np)) and row exponents ex[Np] of the N x N matrix
+// `bits` bits) and row exponents ex[Np] of the N x N matrix
 // (zero-padded to Np); conj negates the imaginary part.
 tc_status oz_slice(const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld, int Np,
                    const OzDigits& dg, void* slices, int* ex, cudaStream_t s);
@@ -61,40 +61,44 @@ tc_status oz_mirror(double* yr, double* yi, int Np, cudaStream_t s);
 // CTAs.  Both give the same bits.
 bool oz_use_pairs(int tiles);
 
-// One operand of the emulated product: its digit slices, row exponents and
-// TMA map (row r of the operand = row r of A, or row r of B in A B^H).
+// One operand of an emulated product A B^H (row r of the operand = row r of A
+// or of B): its residue planes or digit slices, row scales and TMA maps.
 struct OzMat {
-    void* slices;
+    CrtMat crt;          // residue form
+    void* slices;        // digit form
     int* ex;
     CUtensorMap map;     // 32-byte rows (single-CTA kernel)
     CUtensorMap map_w;   // oz_pair_rows() bytes per row (CTA-pair kernel)
     int Np;
-    OzDigits dg;   // oz_digits(Np)
+    bool left;           // A (else B)
 };
 struct OzOut {
     double* yr;        // FP64 planes of the result, row stride Np
     double* yi;
-    long long* lo_r;   // int64 scratch planes [Np][Np]
-    long long* lo_i;
+    void* scratch;     // oz_scratch_bytes(Np)
 };
-size_t oz_mat_bytes(int Np);
-tc_status oz_mat_init(OzMat& m, Arena& ar, int Np);
+size_t oz_mat_bytes(int Np, bool left);
+size_t oz_scratch_bytes(int Np);
+tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left);
 // `view` = `base`'s buffers seen as an operand of the smaller padded size Np
 tc_status oz_mat_view(OzMat& view, const OzMat& base, int Np);
 tc_status oz_mat_load(OzMat& m, const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld,
                       cudaStream_t s);
-// Y = A B^H at FP64 accuracy; mode 1 (Hermitian result): block-lower tiles and the mirror.
-tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const OzOut& out, int group, cudaStream_t s);
+// Y = A B^H at FP64 accuracy; mode 1 (Hermitian result): block-lower tiles and
+// the mirror.  (br, bi): the FP64 planes B was loaded from (N valid rows and
+// columns, row stride ldb), distinct from the result's.
+tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br, const double* bi, int N, size_t ldb,
+                     const OzOut& out, int group, cudaStream_t s);
 
-// The FP64-accurate step loop of one system (evolve_oz.cu): its slices,
-// FP64 planes of rho and X (stride Np = max(N, 128)) and int64 scratch, carved
-// from an arena; first() slices U and pads rho in, step(k) is one step
+// The FP64-accurate step loop of one system (evolve_oz.cu): its operands,
+// FP64 planes of rho and X (stride Np = max(N, 128)) and scratch, carved
+// from an arena; first() prepares U and pads rho in, step(k) is one step
 // (observable row k when obs is given), tail() writes rho back interleaved.
 struct OzSystem {
     int n = 0, N = 0, Np = 0, group = 8, renorm_every = 0;
     OzMat Us{}, Ps{};
     double *Rr = nullptr, *Ri = nullptr, *Xr = nullptr, *Xi = nullptr, *scratch = nullptr;
-    long long *Lr = nullptr, *Li = nullptr;
+    void* prod = nullptr;   // scratch of the products
     const Model* m = nullptr;
     double* obs = nullptr;
     tc_status carve(int n, Arena& ar);

@@ -1,0 +1,212 @@
+// crt_scheme.cuh -- the residue number system of the FP64-accurate products
+// (cgemm_crt.cu): fifteen pairwise coprime moduli p_s <= 255, their product
+// M = 2^117.77, and the constants that turn residues back into a number
+// (Chinese remainder theorem).  Plain C++ with host and device linkage, so
+// that host tests can run the very arithmetic of the kernels.
+//
+// Why 255 and 1024: balanced residues |r| <= 127 are exact in BF16 (8
+// significand bits), and 1024 products of two of them sum to at most
+// 1024 * 127^2 = 2^24 - 261120, so an FP32 accumulator holds a K chunk of
+// 1024 exactly.  Moduli up to 511 would also be exact in BF16 and save one
+// of the fifteen products, but cut the exact chunk to 256.
+#pragma once
+
+#include <stdint.h>
+
+#ifdef __CUDACC__
+#define TC_CRT_HD __host__ __device__ __forceinline__
+#else
+#define TC_CRT_HD inline
+#endif
+
+namespace tc {
+namespace crt {
+
+constexpr int kModuli = 15;
+constexpr int kChunk = 1024;      // K values whose sum is exact in FP32
+typedef unsigned __int128 u128;
+
+TC_CRT_HD constexpr int modulus(int s) {
+    constexpr int p[kModuli] = {255, 254, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
+    return p[s];
+}
+
+// M / p_s, M and the inverse of M / p_s modulo p_s
+constexpr u128 product_without(int s) {
+    u128 m = 1;
+    for (int t = 0; t < kModuli; t++)
+        if (t != s) m *= (u128)modulus(t);
+    return m;
+}
+constexpr u128 product_all() { return product_without(0) * (u128)modulus(0); }
+constexpr int inverse_of_rest(int s) {
+    const int p = modulus(s), a = (int)(product_without(s) % (u128)p);
+    for (int x = 1; x < p; x++)
+        if (a * x % p == 1) return x;
+    return 0;
+}
+// round(2^96 / p): the weight of residue s in the fraction x / M (limb 0 lowest)
+constexpr u128 fraction(int s) {
+    const u128 one = (u128)1 << 96;
+    const u128 p = (u128)modulus(s);
+    return (one + p / 2) / p;
+}
+// Residues are stored with 128 added (1 .. 255); this takes the 128s out again.
+constexpr u128 fraction_bias() {
+    u128 b = 0;
+    for (int s = 0; s < kModuli; s++) b += (u128)128 * fraction(s);
+    return b & (((u128)1 << 96) - 1);
+}
+constexpr int product_bits() {
+    int b = 0;
+    for (u128 m = product_all(); m; m >>= 1) b++;
+    return b;
+}
+
+struct Consts {
+    uint32_t frac[kModuli][3];   // fraction(s), limbs
+    uint32_t bias[3];            // fraction_bias(), limbs
+    uint64_t mtop;               // M / 2^(bits - 64): the top 64 bits of M
+    int mbits;                   // bits of M
+    int inv[kModuli];            // inverse_of_rest(s)
+    int p[kModuli];              // modulus(s)
+};
+constexpr Consts make_consts() {
+    Consts c{};
+    for (int s = 0; s < kModuli; s++) {
+        const u128 f = fraction(s);
+        for (int l = 0; l < 3; l++) c.frac[s][l] = (uint32_t)(f >> (32 * l));
+        c.inv[s] = inverse_of_rest(s);
+        c.p[s] = modulus(s);
+    }
+    for (int l = 0; l < 3; l++) c.bias[l] = (uint32_t)(fraction_bias() >> (32 * l));
+    c.mbits = product_bits();
+    c.mtop = (uint64_t)(product_all() >> (c.mbits - 64));
+    return c;
+}
+
+// ---------------------------------------------------------------- residues
+// A magnitude below 2^59 in three pieces of 20 bits; 2^20 and 2^40 mod p are
+// below 255, so lo + mid c1 + hi c2 < 2^29.
+struct Pieces {
+    uint32_t lo, mid, hi;
+};
+TC_CRT_HD Pieces split_pieces(uint64_t mag) {
+    Pieces q;
+    q.lo = (uint32_t)mag & 0xFFFFFu;
+    q.mid = (uint32_t)(mag >> 20) & 0xFFFFFu;
+    q.hi = (uint32_t)(mag >> 40);
+    return q;
+}
+TC_CRT_HD uint32_t mulhi_u32(uint32_t a, uint32_t b) {
+#ifdef __CUDA_ARCH__
+    return __umulhi(a, b);
+#else
+    return (uint32_t)(((uint64_t)a * b) >> 32);
+#endif
+}
+// t mod p, balanced (|r| <= p / 2), for t < 2^29: the quotient
+// floor((t + p/2) / p) from the 37-bit reciprocal ceil(2^37 / p), whose error
+// (t + p/2) / 2^37 < 1/256 of a unit never reaches the next integer.
+TC_CRT_HD int balanced_mod(uint32_t t, int p) {
+    const uint32_t m = (uint32_t)(((1ull << 37) + (uint64_t)p - 1) / (uint64_t)p);
+    const uint32_t q = mulhi_u32(t + (uint32_t)(p / 2), m) >> 5;
+    return (int)t - (int)q * p;
+}
+// Residue of the magnitude, times inv when it is not 1 (operands of the left
+// role carry the inverse of the remainder theorem).
+TC_CRT_HD int residue(const Pieces& x, int p, int inv) {
+    const uint32_t c1 = (uint32_t)((1u << 20) % (uint32_t)p);
+    const uint32_t c2 = (uint32_t)((1ull << 40) % (uint64_t)p);
+    int r = balanced_mod(x.lo + x.mid * c1 + x.hi * c2, p);
+    if (inv != 1) {
+        const uint32_t u = (uint32_t)(r < 0 ? r + p : r);
+        r = balanced_mod(u * (uint32_t)inv, p);
+    }
+    return r;
+}
+
+// FP64 bits -> sign and integer magnitude round(|x| 2^sh); |x| 2^sh < 2^59.
+// Integer work only (the FP64 pipe of this GPU is slow).
+TC_CRT_HD uint64_t to_magnitude(uint64_t bits, int sh) {
+    const int e = (int)((bits >> 52) & 0x7FFu);
+    uint64_t m = bits & 0xFFFFFFFFFFFFFull;
+    if (e) m |= 1ull << 52;
+    const int up = (e ? e : 1) - 1075 + sh;   // |x| 2^sh = m 2^up
+    if (up >= 0) return up > 10 ? 0 : m << up;   // up <= 6 for rows within their bound
+    const int dn = -up;
+    if (dn > 54) return 0;
+    return (m + (1ull << (dn - 1))) >> dn;
+}
+
+// ---------------------------------------------------------------- recombination
+// x / M modulo 1 as a signed 96-bit fraction from the fifteen stored bytes
+// (residue times inverse, plus 128) -> x 2^e in FP64 (e split in two factors
+// by the caller when it is out of range).  The fraction's error is below
+// 2^-86, so x is within 2^32 units of integers whose rows are held to 2^58
+// (|x| < M / 2 - 2^33).
+struct Acc {
+    uint64_t a0, a1, a2;
+};
+TC_CRT_HD void acc_add(Acc& a, uint32_t byte, const uint32_t (&f)[3]) {
+    a.a0 += (uint64_t)byte * f[0];
+    a.a1 += (uint64_t)byte * f[1];
+    a.a2 += (uint64_t)byte * f[2];
+}
+TC_CRT_HD int clz64(uint64_t v) {
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)v);
+#else
+    return v ? __builtin_clzll(v) : 64;
+#endif
+}
+TC_CRT_HD uint64_t mulhi_u64(uint64_t a, uint64_t b) {
+#ifdef __CUDA_ARCH__
+    return __umul64hi(a, b);
+#else
+    return (uint64_t)(((unsigned __int128)a * b) >> 64);
+#endif
+}
+// mag 2^exp2 (mag a 64-bit integer) with the sign returned through neg; mag = 0 for x = 0
+TC_CRT_HD uint64_t acc_finish(const Acc& a, const Consts& c, bool& neg, int& exp2) {
+    // carry-propagate to three 32-bit limbs modulo 2^96, minus the bias
+    uint64_t t = a.a0;
+    uint32_t l0 = (uint32_t)t;
+    t = (t >> 32) + a.a1;
+    uint32_t l1 = (uint32_t)t;
+    t = (t >> 32) + a.a2;
+    uint32_t l2 = (uint32_t)t;
+    int64_t d = (int64_t)l0 - c.bias[0];
+    l0 = (uint32_t)d;
+    d = (int64_t)l1 - c.bias[1] + (d >> 32);
+    l1 = (uint32_t)d;
+    d = (int64_t)l2 - c.bias[2] + (d >> 32);
+    l2 = (uint32_t)d;
+    neg = (l2 >> 31) != 0;
+    if (neg) {   // two's complement
+        uint64_t s = (uint64_t)(uint32_t)~l0 + 1;
+        l0 = (uint32_t)s;
+        s = (uint64_t)(uint32_t)~l1 + (s >> 32);
+        l1 = (uint32_t)s;
+        l2 = ~l2 + (uint32_t)(s >> 32);
+    }
+    const uint64_t hi = ((uint64_t)l2 << 32) | l1;
+    // the top 64 bits of the 96: |f| = top 2^(32 - lz), truncated
+    int lz = hi ? clz64(hi) : 64;
+    uint64_t top;
+    if (lz == 0) {
+        top = hi;
+    } else if (lz <= 32) {
+        top = (hi << lz) | ((uint64_t)l0 >> (32 - lz));
+    } else if (lz < 64) {
+        top = (hi << lz) | ((uint64_t)l0 << (lz - 32));
+    } else {
+        top = (uint64_t)l0 << 32;
+        // not normalised: below 2^-64 of M, well under the operands' own rounding
+    }
+    exp2 = 32 - lz - 96 + c.mbits;
+    return mulhi_u64(top, c.mtop);
+}
+
+}  // namespace crt
+}  // namespace tc

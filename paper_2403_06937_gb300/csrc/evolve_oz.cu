@@ -83,7 +83,8 @@ int padded_dim(int n) { return (1 << n) < 128 ? 128 : (1 << n); }
 
 size_t evolve_oz_bytes(int n) {
     const size_t Np = (size_t)padded_dim(n);
-    return 2 * oz_mat_bytes((int)Np) + 6 * round256(Np * Np * sizeof(double)) + observables_scratch_bytes(n) + 512;
+    return oz_mat_bytes((int)Np, true) + oz_mat_bytes((int)Np, false) + oz_scratch_bytes((int)Np) +
+           4 * round256(Np * Np * sizeof(double)) + observables_scratch_bytes(n) + 512;
 }
 
 tc_status OzSystem::carve(int n_, Arena& ar) {
@@ -91,14 +92,13 @@ tc_status OzSystem::carve(int n_, Arena& ar) {
     N = 1 << n;
     Np = padded_dim(n);
     const size_t NN = (size_t)Np * Np;
-    TC_TRY(oz_mat_init(Us, ar, Np));
-    TC_TRY(oz_mat_init(Ps, ar, Np));
+    TC_TRY(oz_mat_init(Us, ar, Np, true));
+    TC_TRY(oz_mat_init(Ps, ar, Np, false));
     Rr = ar.take<double>(NN);
     Ri = ar.take<double>(NN);
     Xr = ar.take<double>(NN);
     Xi = ar.take<double>(NN);
-    Lr = ar.take<long long>(NN);   // low-level integer sums of the products
-    Li = ar.take<long long>(NN);
+    prod = ar.take<uint8_t>(oz_scratch_bytes(Np));
     scratch = ar.take<double>(observables_scratch_bytes(n) / sizeof(double));
     if (!scratch) return fail(TC_ERR_WORKSPACE, "evolve: workspace too small");
     group = tune_lookup(n, TC_BF16X3).tc_group;
@@ -121,16 +121,16 @@ tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, d
 tc_status OzSystem::step(int k, cudaStream_t cs) {
     const size_t NN = (size_t)Np * Np;
     const double N3 = (double)N * N * N;
-    const OzOut X{Xr, Xi, Lr, Li}, R{Rr, Ri, Lr, Li};
+    const OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
     TC_TRY(oz_mat_load(Ps, Rr, Ri, false, false, N, (size_t)Np, cs));
     {
-        ProductTimer t(8.0 * N3 * Us.dg.pairs, cs);   // X = U rho^H
-        TC_TRY(oz_product(0, Us, Ps, X, group, cs));
+        ProductTimer t(8.0 * N3 * oz_products(), cs);   // X = U rho^H
+        TC_TRY(oz_product(0, Us, Ps, Rr, Ri, N, (size_t)Np, X, group, cs));
     }
     TC_TRY(oz_mat_load(Ps, Xr, Xi, false, false, N, (size_t)Np, cs));
     {
-        ProductTimer t(4.0 * N3 * Us.dg.pairs, cs);   // rho' = U X^H, Hermitian half + mirror
-        TC_TRY(oz_product(1, Us, Ps, R, group, cs));
+        ProductTimer t(4.0 * N3 * oz_products(), cs);   // rho' = U X^H, Hermitian half + mirror
+        TC_TRY(oz_product(1, Us, Ps, Xr, Xi, N, (size_t)Np, R, group, cs));
     }
     if (renorm_every > 0 && k % renorm_every == 0) {
         trace_pad_kernel<<<1, 1024, 0, cs>>>(Rr, N, Np, scratch);

@@ -679,9 +679,9 @@ size_t evolve_oz_bytes_blocks(int n) {
     const size_t PT = padded_total(L);
     const int NpMax = padded(L.N);
     size_t b = tables_bytes(n) + 2 * round256(PT * sizeof(double));
-    for (int k = 0; k <= n; k++) b += oz_mat_bytes(padded(L.dims[k]));   // U_k slices
-    b += oz_mat_bytes(NpMax);                                             // B operand slices
-    b += 4 * round256((size_t)NpMax * NpMax * sizeof(double));            // X planes, int64 scratch
+    for (int k = 0; k <= n; k++) b += oz_mat_bytes(padded(L.dims[k]), true);   // U_k slices
+    b += oz_mat_bytes(NpMax, false) + oz_scratch_bytes(NpMax);            // B operand, scratch of the products
+    b += 2 * round256((size_t)NpMax * NpMax * sizeof(double));            // X planes
     return b + obs_scratch_bytes(L) + 256;
 }
 
@@ -696,13 +696,12 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     double* Rr = ar.take<double>(PT);
     double* Ri = ar.take<double>(PT);
     std::vector<OzMat> Uk(n + 1);
-    for (int k = 0; k <= n; k++) TC_TRY(oz_mat_init(Uk[k], ar, padded(L.dims[k])));
+    for (int k = 0; k <= n; k++) TC_TRY(oz_mat_init(Uk[k], ar, padded(L.dims[k]), true));
     OzMat Bmax{};
-    TC_TRY(oz_mat_init(Bmax, ar, NpMax));
+    TC_TRY(oz_mat_init(Bmax, ar, NpMax, false));
     double* Xr = ar.take<double>(NN);
     double* Xi = ar.take<double>(NN);
-    long long* Lr = ar.take<long long>(NN);
-    long long* Li = ar.take<long long>(NN);
+    void* prod = ar.take<uint8_t>(oz_scratch_bytes(NpMax));
     double* scratch = ar.take<double>(obs_scratch_bytes(L) / sizeof(double));
     if (!scratch) return fail(TC_ERR_WORKSPACE, "lindblad evolve: workspace too small");
     // the B operand slices seen at each block's padded size (one map per block)
@@ -723,13 +722,13 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
             const double d3 = (double)d * d * d;
             TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs));
             {
-                ProductTimer pt(8.0 * d3 * Uk[k].dg.pairs, cs);   // X_k = U_k rho_k
-                TC_TRY(oz_product(0, Uk[k], Bk[k], OzOut{Xr, Xi, Lr, Li}, group, cs));
+                ProductTimer pt(8.0 * d3 * oz_products(), cs);   // X_k = U_k rho_k
+                TC_TRY(oz_product(0, Uk[k], Bk[k], rr, ri, d, (size_t)Np, OzOut{Xr, Xi, prod}, group, cs));
             }
             TC_TRY(oz_mat_load(Bk[k], Xr, Xi, false, false, d, (size_t)Np, cs));
             {
-                ProductTimer pt(4.0 * d3 * Uk[k].dg.pairs, cs);   // rho_k = U_k X_k^H, Hermitian
-                TC_TRY(oz_product(1, Uk[k], Bk[k], OzOut{rr, ri, Lr, Li}, group, cs));
+                ProductTimer pt(4.0 * d3 * oz_products(), cs);   // rho_k = U_k X_k^H, Hermitian
+                TC_TRY(oz_product(1, Uk[k], Bk[k], Xr, Xi, d, (size_t)Np, OzOut{rr, ri, prod}, group, cs));
             }
         }
         return TC_OK;
