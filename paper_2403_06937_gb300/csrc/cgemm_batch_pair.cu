@@ -38,7 +38,7 @@ namespace {
 using namespace sm100;
 using namespace cg;
 
-constexpr int kThreads = 192;
+constexpr int kThreads = 320;   // eight epilogue warps, TMA, MMA
 
 struct UnitRef {
     int b, I, J;
@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t tmem = *tmem_slot;
     const uint32_t peer_abort = cluster_addr(saddr(const_cast<int*>(abort)), rank ^ 1u);
 
-    if (warp == 4) {
+    if (warp == 8) {
         // ---------------------------------------------------------- producer (both CTAs)
         if (lane == 0) {
             const uint32_t lead_full = cluster_addr(saddr(&full[0]), 0u);
@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     (void)mbar_wait_bounded(&empty[k % STAGES], (k / STAGES) & 1u, abort, kWaitLimitNs, 0);
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         if (lane == 0 && rank == 0) {
             // ------------------------------------------------------ MMA issuer (even CTA)
             const uint32_t peer_empty = cluster_addr(saddr(&empty[0]), 1u);
@@ -227,17 +227,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     } else {
         // ---------------------------------------------------------- epilogue (both CTAs, own tile)
         const uint32_t lead_tmem_empty = cluster_addr(saddr(tmem_empty), 0u);
+        const int c0 = 64 * (warp >> 2);   // columns of this set of four warps
         int tl = 0, hint = 0;
         for (int u = cluster; u < nunits; u += clusters, tl++) {
             const UnitRef r = unit_at(sys, nsys, MODE, u, group, rank, hint);
             const BatchSys& d = sys[r.b];
             const bool ok = mbar_wait_bounded_cluster(accum, (uint32_t)tl & 1u, abort, kWaitLimitNs, 128);
             tc_fence_after();
-            // the four epilogue warps leave together or not at all (barrier 1 below)
+            // the eight epilogue warps leave together or not at all (barrier 1 below)
             uint32_t bad = (!ok || *abort) ? 1u : 0u, any;
             asm volatile(
                 "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-                "bar.red.or.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n}"
+                "bar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
                 : "=r"(any)
                 : "r"(bad)
                 : "memory");
@@ -251,12 +252,14 @@ __global__ void __launch_bounds__(kThreads, 1)
             // rows past an odd T, and the tile above the diagonal of the Hermitian product, are not written
             if (r.I < d.tiles && !(MODE == 1 && r.J > r.I)) {
                 if (MODE == 0)
-                    epilogue_tile<KIND, S, 0>(tmem, warp, lane, r.I, r.J, d.Np, d.Rr, d.Ri, d.Xparts, d.Xr, d.Xi);
+                    epilogue_tile<KIND, S, 0>(tmem, warp & 3, lane, r.I, r.J, d.Np, d.Rr, d.Ri, d.Xparts, d.Xr, d.Xi,
+                                              c0, c0 + 64);
                 else
-                    epilogue_tile<KIND, S, 1>(tmem, warp, lane, r.I, r.J, d.Np, d.Xr, d.Xi, d.Rparts, d.Rr, d.Ri);
+                    epilogue_tile<KIND, S, 1>(tmem, warp & 3, lane, r.I, r.J, d.Np, d.Xr, d.Xi, d.Rparts, d.Rr, d.Ri,
+                                              c0, c0 + 64);
             }
             tc_fence_before();
-            asm volatile("bar.sync 1, 128;" ::: "memory");   // all four epilogue warps have read TMEM
+            asm volatile("bar.sync 1, 256;" ::: "memory");   // all eight epilogue warps have read TMEM
             if (threadIdx.x == 0) {
                 if (rank == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");

@@ -70,6 +70,18 @@ __device__ __forceinline__ float tf32_rna(float x) {
 template <int KIND, int S>
 struct Parts {
     using T = typename std::conditional<KIND == 0, __nv_bfloat16, float>::type;
+    // the next part of what is left
+    __device__ static T take(float& rest) {
+        if constexpr (KIND == 0) {
+            const T p = __float2bfloat16_rn(rest);
+            rest = rest - __bfloat162float(p);
+            return p;
+        } else {
+            const T p = tf32_rna(rest);
+            rest = rest - p;
+            return p;
+        }
+    }
     __device__ static void split(float x, T (&p)[S]) {
         if constexpr (KIND == 0) {
             float r = x;
@@ -98,25 +110,55 @@ __device__ __forceinline__ void store16(T* dst, const T (&v)[16]) {
 }
 
 
-// Epilogue of tile (I, J): warps 0-3 read TMEM lanes 32w..32w+31 (row i of the
-// tile) and write Y[i][j] = conj(P[j][i]) + (V P^H)[i][j] as FP32 planes and
-// operand parts; MODE 1 keeps the block-lower part of a diagonal tile and
-// mirrors the conjugate transpose.  src_*: FP32 planes of P (row stride np_).
+// v[q] of lane l -> v[l] of lane q within each half-warp (q, l = 0..15): four
+// butterfly exchanges, eight shuffles each.
+__device__ __forceinline__ void transpose16(float (&v)[16], int l) {
+#pragma unroll
+    for (int s = 8; s > 0; s >>= 1) {
+        const bool up = (l & s) != 0;
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            if (q & s) continue;
+            const float x = __shfl_xor_sync(0xffffffffu, up ? v[q] : v[q | s], s);
+            if (up)
+                v[q] = x;
+            else
+                v[q | s] = x;
+        }
+    }
+}
+
+// Epilogue of the columns [c0, c1) of tile (I, J), by the four warps of the
+// lane quarters `quarter` = 0..3: each reads TMEM lanes 32 quarter .. + 31
+// (row i of the tile) and writes Y[i][j] = conj(P[j][i]) + (V P^H)[i][j] as
+// FP32 planes and operand parts; MODE 1 keeps the block-lower part of a
+// diagonal tile and mirrors the conjugate transpose.  src_*: FP32 planes of P
+// (row stride np_).
+//
+// A lane writes 16 consecutive entries of its row with vector stores, and the
+// mirror column by column with consecutive lanes on consecutive entries.  In
+// a diagonal tile the 16 x 16 blocks on the diagonal are made Hermitian in
+// registers (transpose16), so that they too go out as vector stores; written
+// entry by entry they were scattered stores of 2 and 4 bytes, 60-70 us for
+// the tile (n = 8: 104 us a launch; 40 us for the product without a mirror).
+// Two sets of four warps (the CTA-pair kernels) take 64 columns each: the
+// loads of the identity term are one dependent round trip per 16 columns.
 template <int KIND, int S, int MODE>
-__device__ __forceinline__ void epilogue_tile(uint32_t tmem, int warp, int lane, int I, int J, int np_,
+__device__ __forceinline__ void epilogue_tile(uint32_t tmem, int quarter, int lane, int I, int J, int np_,
                                               const float* __restrict__ src_r, const float* __restrict__ src_i,
-                                              void* parts_v, float* out_r, float* out_i) {
+                                              void* parts_v, float* out_r, float* out_i, int c0 = 0,
+                                              int c1 = 128) {
     using P = Parts<KIND, S>;
     using T = typename P::T;
-    const int row = warp * 32 + lane;                  // TMEM lane = row i of the tile
-    const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+    const int row = quarter * 32 + lane;                  // TMEM lane = row i of the tile
+    const uint32_t tl = tmem + ((uint32_t)(quarter * 32) << 16);
     const size_t Np = (size_t)np_;
     const size_t plane = Np * Np;
     const size_t gi = (size_t)I * 128 + row;
     T* parts = reinterpret_cast<T*>(parts_v);
     const bool diag = (MODE == 1) && (I == J);
 #pragma unroll 1
-    for (int c = 0; c < 128; c += 16) {
+    for (int c = c0; c < c1; c += 16) {
         float d1r[16], d1i[16], d2r[16], d2i[16];
         tmem_ld16(tl + c, d1r);            // U_r P_r^T
         tmem_ld16(tl + 128 + c, d1i);      // U_r P_i^T
@@ -132,45 +174,46 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem, int warp, int lane,
             yr[q] = (d1r[q] + d2i[q]) + src_r[t];
             yi[q] = (d2r[q] - d1i[q]) - src_i[t];
         }
-        if (MODE == 0 || !diag) {
-            // direct tile, full rows of 16: parts (and FP32 planes in mode 1)
-            T pr[S][16], pi[S][16];
+        if (MODE == 1 && diag && (c >> 5) == quarter) {
+            // rows c .. c + 15 hold the block on the diagonal: upper half from the
+            // lower one, real diagonal (the other half-warp keeps its values)
+            float tr[16], ti[16];
 #pragma unroll
-            for (int q = 0; q < 16; q++) {
-                T a[S], b[S];
-                P::split(yr[q], a);
-                P::split(yi[q], b);
+            for (int q = 0; q < 16; q++) { tr[q] = yr[q]; ti[q] = yi[q]; }
+            const int l = lane & 15;
+            transpose16(tr, l);
+            transpose16(ti, l);
+            if ((row & ~15) == c) {
 #pragma unroll
-                for (int s = 0; s < S; s++) { pr[s][q] = a[s]; pi[s][q] = b[s]; }
+                for (int q = 0; q < 16; q++) {
+                    yr[q] = q > l ? tr[q] : yr[q];
+                    yi[q] = q > l ? -ti[q] : (q == l ? 0.0f : yi[q]);
+                }
             }
-#pragma unroll
-            for (int s = 0; s < S; s++) {
-                store16(parts + (size_t)s * plane + gi * Np + gj0, pr[s]);
-                store16(parts + (size_t)(S + s) * plane + gi * Np + gj0, pi[s]);
-            }
+        }
+        if (MODE == 0 || !diag || row >= c) {
             store16(out_r + gi * Np + gj0, yr);
             store16(out_i + gi * Np + gj0, yi);
+            // part by part (fewer registers than all parts of both planes at once)
+#pragma unroll
+            for (int plane_i = 0; plane_i < 2; plane_i++) {
+                float rest[16];
+#pragma unroll
+                for (int q = 0; q < 16; q++) rest[q] = plane_i ? yi[q] : yr[q];
+#pragma unroll
+                for (int s = 0; s < S; s++) {
+                    T a[16];
+#pragma unroll
+                    for (int q = 0; q < 16; q++) a[q] = P::take(rest[q]);
+                    store16(parts + (size_t)(plane_i * S + s) * plane + gi * Np + gj0, a);
+                }
+            }
         }
-        if (MODE == 1) {
+        if (MODE == 1 && (!diag || row >= c + 16)) {
+            // mirror: rho'[j][i] = conj(rho'[i][j]); lanes write consecutive i
 #pragma unroll
             for (int q = 0; q < 16; q++) {
-                const int col = c + q;
                 const size_t gj = gj0 + q;
-                if (diag) {
-                    if (col > row) continue;
-                    float vr = yr[q], vi = (col == row) ? 0.0f : yi[q];
-                    T a[S], b[S];
-                    P::split(vr, a);
-                    P::split(vi, b);
-                    for (int s = 0; s < S; s++) {
-                        parts[(size_t)s * plane + gi * Np + gj] = a[s];
-                        parts[(size_t)(S + s) * plane + gi * Np + gj] = b[s];
-                    }
-                    out_r[gi * Np + gj] = vr;
-                    out_i[gi * Np + gj] = vi;
-                    if (col == row) continue;
-                }
-                // mirror: rho'[j][i] = conj(rho'[i][j]); lanes write consecutive i
                 T a[S], b[S];
                 P::split(yr[q], a);
                 P::split(-yi[q], b);

@@ -52,6 +52,7 @@ using namespace sm100;
 using namespace cg;
 
 constexpr int kThreads = 192;
+constexpr int kPairThreads = 320;   // CTA pairs: eight epilogue warps, TMA, MMA
 
 template <int KIND, int S, int STAGES, int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -224,7 +225,7 @@ tc_status launch(const CUtensorMap& tmU, const CUtensorMap& tmP, const CgemmEpi&
 // (split_pair_stages, cgemm_dev.cuh).
 
 template <int KIND, int S, int RB, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kPairThreads, 1)
     cgemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmP,
                          CgemmEpi ep) {
     constexpr int STAGES = split_pair_stages<S, RB>();
@@ -266,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         tmem_alloc_pair(saddr(tmem_slot), 512);
         tmem_relinquish_pair();
     }
-    if (warp == 4 && lane == 0) {
+    if (warp == 8 && lane == 0) {
         prefetch_tmap(&tmU);
         prefetch_tmap(&tmP);
     }
@@ -277,7 +278,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t peer_abort = cluster_addr(saddr(const_cast<int*>(abort)), rank ^ 1u);
     const int KB = ep.Np / kKPerStage;
 
-    if (warp == 4) {
+    if (warp == 8) {
         // ---------------------------------------------------------- producer (both CTAs)
         if (lane == 0) {
             const uint32_t lead_full = cluster_addr(saddr(&full[0]), 0u);
@@ -337,7 +338,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                     (void)mbar_wait_bounded(&empty[kb % STAGES], (uint32_t)(kb / STAGES) & 1u, abort, lim, 0);
             }
         }
-    } else if (warp == 5) {
+    } else if (warp == 9) {
         if (lane == 0 && rank == 0) {
             // ------------------------------------------------------ MMA issuer (even CTA)
             const uint32_t peer_empty = cluster_addr(saddr(&empty[0]), 1u);
@@ -376,7 +377,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool ok = mbar_wait_bounded_cluster(accum, 0u, abort, lim, 128);
         tc_fence_after();
         if (ok && !*abort && !(MODE == 1 && J > I))
-            cg::epilogue_tile<KIND, S, MODE>(tmem, warp, lane, I, J, ep.Np, ep.pr, ep.pi, ep.parts, ep.yr, ep.yi);
+            cg::epilogue_tile<KIND, S, MODE>(tmem, warp & 3, lane, I, J, ep.Np, ep.pr, ep.pi, ep.parts, ep.yr, ep.yi,
+                                             64 * (warp >> 2), 64 * (warp >> 2) + 64);
         if (!ok || *abort) {
             if (threadIdx.x == 0) {
                 atomicOr(ep.status, kStatusTimeout);
@@ -411,7 +413,7 @@ tc_status launch_pair(const CUtensorMap& tmU, const CUtensorMap& tmP, const Cgem
     const unsigned pairs = (unsigned)pair_count(MODE, ep.tiles, lo, hi);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * pairs);
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(kPairThreads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
