@@ -285,11 +285,11 @@ __global__ void obs_partial_kernel(BlockSet bs, Model m, int has_model, const in
     const int n = bs.n;
     const int stride = 2 * n + 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = lane; j < stride; j += 32) acc[warp][j] = 0.0;
-    __syncwarp();
     unsigned rows = 0;
     for (int k = 0; k <= n; k++) rows += (unsigned)bs.d[k];
     double pur = 0.0, epair = 0.0;
+    // one running sum per lane, as in the closed system's kernel (observables.cu)
+    double p_atom = 0.0, p_m = 0.0, mean = 0.0, trace = 0.0, ediag = 0.0;
     for (unsigned q = blockIdx.x * kObsWarps + warp; q < rows; q += gridDim.x * kObsWarps) {
         int k = 0;
         unsigned i = q;
@@ -324,14 +324,14 @@ __global__ void obs_partial_kernel(BlockSet bs, Model m, int has_model, const in
                              x3 = (double)re[row + c + 96];
                 const double y0 = (double)im[row + c], y1 = (double)im[row + c + 32], y2 = (double)im[row + c + 64],
                              y3 = (double)im[row + c + 96];
-                p0 += x0 * x0 + y0 * y0;
-                p1 += x1 * x1 + y1 * y1;
-                p2 += x2 * x2 + y2 * y2;
-                p3 += x3 * x3 + y3 * y3;
+                p0 = fma(x0, x0, fma(y0, y0, p0));
+                p1 = fma(x1, x1, fma(y1, y1, p1));
+                p2 = fma(x2, x2, fma(y2, y2, p2));
+                p3 = fma(x3, x3, fma(y3, y3, p3));
             }
             for (; c < d; c += 32) {
                 const double x = (double)re[row + c], y = (double)im[row + c];
-                p0 += x * x + y * y;
+                p0 = fma(x, x, fma(y, y, p0));
             }
         }
         pur += (p0 + p1) + (p2 + p3);
@@ -340,24 +340,25 @@ __global__ void obs_partial_kernel(BlockSet bs, Model m, int has_model, const in
             const unsigned c = (unsigned)pos[s ^ (1u << lane)];
             if (c < d) epair += h_pair(m, k, s, lane) * (double)re[row + c];
         }
-        if (lane == 0) {
-            const double v = (double)re[row + i];
-            const int pc = __popc(s), p = k - pc;
-            for (int a = 0; a < n; a++)
-                if ((s >> (n - 1 - a)) & 1u) acc[warp][a] += v;
-            acc[warp][n] += v * (double)p;
-            acc[warp][n + 1 + p] += v;
-            acc[warp][2 * n + 2] += v;
-            if (has_model) acc[warp][2 * n + 4] += h_diag(m, k, s) * v;
-        }
+        const double v = (double)re[row + i];
+        const int pc = __popc(s), p = k - pc;
+        if (lane < n && ((s >> (n - 1 - lane)) & 1u)) p_atom += v;
+        if (lane == p) p_m += v;
+        mean += v * (double)p;
+        trace += v;
+        if (has_model) ediag += h_diag(m, k, s) * v;
     }
     for (int o = 16; o > 0; o >>= 1) {
         pur += __shfl_xor_sync(0xffffffffu, pur, o);
         epair += __shfl_xor_sync(0xffffffffu, epair, o);
     }
+    if (lane < n) acc[warp][lane] = p_atom;
+    if (lane <= n) acc[warp][n + 1 + lane] = p_m;
     if (lane == 0) {
-        acc[warp][2 * n + 3] += pur;
-        acc[warp][2 * n + 4] += epair;
+        acc[warp][n] = mean;
+        acc[warp][2 * n + 2] = trace;
+        acc[warp][2 * n + 3] = pur;
+        acc[warp][2 * n + 4] = ediag + epair;
     }
     __syncthreads();
     for (int j = threadIdx.x; j < stride; j += blockDim.x) {
@@ -367,12 +368,15 @@ __global__ void obs_partial_kernel(BlockSet bs, Model m, int has_model, const in
     }
 }
 
-__global__ void obs_final_kernel(const double* __restrict__ partials, int blocks, int stride,
-                                 double* __restrict__ out) {
-    for (int j = threadIdx.x; j < stride; j += blockDim.x) {
+// as in observables.cu: one warp per column, a fixed order
+__global__ void __launch_bounds__(1024)
+    obs_final_kernel(const double* __restrict__ partials, int blocks, int stride, double* __restrict__ out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int j = warp; j < stride; j += 32) {
         double sum = 0.0;
-        for (int b = 0; b < blocks; b++) sum += partials[(size_t)b * stride + j];
-        out[j] = sum;
+        for (int b = lane; b < blocks; b += 32) sum += partials[(size_t)b * stride + j];
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_down_sync(0xffffffffu, sum, o);
+        if (lane == 0) out[j] = sum;
     }
 }
 
@@ -425,7 +429,7 @@ tc_status launch_block_observables(const Layout& L, const BlockSet& bs, const Mo
     const unsigned grid = obs_grid(L);
     obs_partial_kernel<T><<<grid, 32 * kObsWarps, 0, s>>>(bs, m, 1, t.order, t.pos, re, im, scratch);
     TC_LAUNCH_CHECK();
-    obs_final_kernel<<<1, 64, 0, s>>>(scratch, (int)grid, 2 * L.n + 5, out);
+    obs_final_kernel<<<1, 1024, 0, s>>>(scratch, (int)grid, 2 * L.n + 5, out);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }

@@ -8,8 +8,8 @@
 //
 // Deterministic two-pass reduction, no floating-point atomics: one warp per
 // row (lanes stride the row for the purity sum, lanes < n take the n energy
-// pairs of that row), warps fold in a fixed order into per-block partials,
-// and a single block sums the partials in block order.  The grid size is a
+// pairs and the n populations of that row), warps fold in a fixed order into
+// per-block partials, and a single block sums the partials in a fixed order.  The grid size is a
 // function of N only, so reruns are bitwise identical.
 #include <mutex>
 
@@ -49,10 +49,12 @@ __global__ void obs_partial_kernel(Rho<L> rho, Model m, int has_model, int n, do
     __shared__ double acc[kObsWarps][kMaxStride];
     const int stride = 2 * n + 5;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int j = lane; j < stride; j += 32) acc[warp][j] = 0.0;
-    __syncwarp();
     const unsigned N = 1u << n;
     double pur = 0.0, epair = 0.0;
+    // sums over this warp's rows of the diagonal entry, one per lane: P_(lane+1), P(m = lane), and in
+    // every lane <p>, the trace and the diagonal energy (a serial chain of shared-memory updates by
+    // one lane took longer than the row itself)
+    double p_atom = 0.0, p_m = 0.0, mean = 0.0, trace = 0.0, ediag = 0.0;
     for (unsigned r = blockIdx.x * kObsWarps + warp; r < N; r += gridDim.x * kObsWarps) {
         const size_t row = (size_t)r * rho.ld;
         // four independent loads per lane in flight, fixed summation order
@@ -86,14 +88,14 @@ __global__ void obs_partial_kernel(Rho<L> rho, Model m, int has_model, int n, do
                          x3 = rho.re(row + c + 96);
             const double y0 = rho.im(row + c), y1 = rho.im(row + c + 32), y2 = rho.im(row + c + 64),
                          y3 = rho.im(row + c + 96);
-            p0 += x0 * x0 + y0 * y0;
-            p1 += x1 * x1 + y1 * y1;
-            p2 += x2 * x2 + y2 * y2;
-            p3 += x3 * x3 + y3 * y3;
+            p0 = fma(x0, x0, fma(y0, y0, p0));   // two FP64 instructions an entry
+            p1 = fma(x1, x1, fma(y1, y1, p1));
+            p2 = fma(x2, x2, fma(y2, y2, p2));
+            p3 = fma(x3, x3, fma(y3, y3, p3));
         }
         for (; c < N; c += 32) {
             const double x = rho.re(row + c), y = rho.im(row + c);
-            p0 += x * x + y * y;
+            p0 = fma(x, x, fma(y, y, p0));
         }
         pur += (p0 + p1) + (p2 + p3);
         // energy pair of atom `lane` when that atom is excited in r
@@ -107,24 +109,25 @@ __global__ void obs_partial_kernel(Rho<L> rho, Model m, int has_model, int n, do
                 epair += h * (rho.re(row + sg) + rho.re((size_t)sg * rho.ld + r));
             }
         }
-        if (lane == 0) {
-            double d = rho.re(row + r);
-            int pc = __popc(r);
-            for (int i = 0; i < n; i++)
-                if ((r >> (n - 1 - i)) & 1u) acc[warp][i] += d;
-            acc[warp][n] += d * (double)(n - pc);
-            acc[warp][n + 1 + (n - pc)] += d;
-            acc[warp][2 * n + 2] += d;
-            if (has_model) acc[warp][2 * n + 4] += (m.omega_c * (double)(n - pc) + m.omega_a * (double)pc) * d;
-        }
+        const double d = rho.re(row + r);
+        const int pc = __popc(r);
+        if (lane < n && ((r >> (n - 1 - lane)) & 1u)) p_atom += d;
+        if (lane == n - pc) p_m += d;
+        mean += d * (double)(n - pc);
+        trace += d;
+        if (has_model) ediag += (m.omega_c * (double)(n - pc) + m.omega_a * (double)pc) * d;
     }
     for (int o = 16; o > 0; o >>= 1) {
         pur += __shfl_xor_sync(0xffffffffu, pur, o);
         epair += __shfl_xor_sync(0xffffffffu, epair, o);
     }
+    if (lane < n) acc[warp][lane] = p_atom;
+    if (lane <= n) acc[warp][n + 1 + lane] = p_m;
     if (lane == 0) {
-        acc[warp][2 * n + 3] += pur;
-        acc[warp][2 * n + 4] += epair;
+        acc[warp][n] = mean;
+        acc[warp][2 * n + 2] = trace;
+        acc[warp][2 * n + 3] = pur;
+        acc[warp][2 * n + 4] = ediag + epair;
     }
     __syncthreads();
     for (int j = threadIdx.x; j < stride; j += blockDim.x) {
@@ -134,11 +137,16 @@ __global__ void obs_partial_kernel(Rho<L> rho, Model m, int has_model, int n, do
     }
 }
 
-__global__ void obs_final_kernel(const double* partials, int blocks, int stride, double* out) {
-    for (int j = threadIdx.x; j < stride; j += blockDim.x) {
+// One warp per column of the partials: lanes stride the blocks, then a tree
+// in a fixed order.  (One thread per column, adding the blocks one after
+// another, waited for up to 1024 dependent loads: 57 us at n = 12.)
+__global__ void __launch_bounds__(1024) obs_final_kernel(const double* partials, int blocks, int stride, double* out) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int j = warp; j < stride; j += 32) {
         double s = 0.0;
-        for (int b = 0; b < blocks; b++) s += partials[(size_t)b * stride + j];
-        out[j] = s;
+        for (int b = lane; b < blocks; b += 32) s += partials[(size_t)b * stride + j];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (lane == 0) out[j] = s;
     }
 }
 
@@ -217,7 +225,7 @@ tc_status launch_observables(int layout, const void* a, const void* b, const Mod
             return fail(TC_ERR_INVALID_ARG, "observables: unknown layout");
     }
     TC_LAUNCH_CHECK();
-    obs_final_kernel<<<1, 64, 0, s>>>(scratch, (int)grid, 2 * n + 5, out);
+    obs_final_kernel<<<1, 1024, 0, s>>>(scratch, (int)grid, 2 * n + 5, out);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
