@@ -316,24 +316,25 @@ def _compulsory_bytes(prec, N):
     """Bytes one complex product Y = A B^H must move at least once: the A and B
     operand planes, and for the split forms the FP32 increment term read and
     the FP32 result plus its split planes written."""
-    if prec == "fp64":
+    if prec == "fp64" and not fp64_on_tensor_cores(N):
         return 3 * 16 * N * N
-    if prec == "ozaki":
-        # nine BF16 digit planes of U and of P read, the FP64 result written
-        return (2 * 2 * 9 * 2 + 16) * N * N
+    if prec in ("fp64", "ozaki"):
+        # BF16 residue (digit) planes of U and of P read, the FP64 result written
+        return (2 * 2 * (15 if oz_products() == 15 else 9) * 2 + 16) * N * N
     parts, pbytes = {"bf16x3": (3, 2), "tf32": (1, 4), "tf32x3": (2, 4)}[prec]
     planes = 2 * parts * pbytes
     return (3 * planes + 8 + 8) * N * N
 
 
-def oz_pairs(N):
-    """Digit-slice pairs per complex product of the FP64-emulated form: the
-    library takes 8-bit digits for inner dimension K <= 1024, 7-bit for
-    K <= 4096, else 6-bit (TC_OZ_BITS=6 forces 6-bit)."""
-    K = max(N, 128)
-    if os.environ.get("TC_OZ_BITS") == "6" or K > 4096:
-        return 45
-    return 28 if K <= 1024 else 36
+def oz_products():
+    """BF16 products per complex product of the FP64-accurate form: fifteen
+    residue products, or the 45 digit pairs under TC_OZ_BITS=6."""
+    return 45 if os.environ.get("TC_OZ_BITS") == "6" else 15
+
+
+def fp64_on_tensor_cores(N):
+    """TC_FP64 runs its products in the residue form for 7 <= n <= 14, on the DMMA elsewhere."""
+    return 1 << 7 <= N <= 1 << 14 and oz_products() == 15
 
 
 def _sample_entries(torch, rho, count=20000, top=48, seed=5):
@@ -511,7 +512,7 @@ def run_ours(a, cfg):
     peaks, peak_src = _measured_peaks()
 
     def peak_of(p, fp64_peak=None, tf32_peak=None):
-        if p == "fp64":
+        if p == "fp64" and not fp64_on_tensor_cores(N):
             return fp64_peak, "FP64: cuBLAS DGEMM 4096^3 measured live in this run (torch.matmul float64)"
         if p in ("tf32", "tf32x3"):
             if tf32_peak is not None:
@@ -546,7 +547,8 @@ def run_ours(a, cfg):
         "vs_baseline": None, "dtype": {"fp64": "f64", "bf16x3": "bf16", "tf32": "tf32", "tf32x3": "tf32", "ozaki": "bf16"}[prec],
         "data": "synthetic",
         "config": {"workload": cfg.description, "precision": prec, "dim": N,
-                   "products_per_complex_product": {"fp64": 1, "bf16x3": 6, "tf32": 1, "tf32x3": 3, "ozaki": oz_pairs(N)}[prec],
+                   "products_per_complex_product": {"fp64": oz_products() if fp64_on_tensor_cores(N) else 1, "bf16x3": 6,
+                                                    "tf32": 1, "tf32x3": 3, "ozaki": oz_products()}[prec],
                    "parallelism": "replicas" if world > 1 else "single GPU",
                    "l2": "inputs larger than L2 (U and rho are %d MiB each in complex128)" % (16 * N * N >> 20),
                    "setup_s": t_setup},
@@ -614,7 +616,7 @@ def run_ours(a, cfg):
                           "frac": ach / pk if pk else None, "peak_source": pk_note,
                           "error": {"vs_oracle": None, "drift": r2["drift"]}}
             if p2 == "ozaki":
-                others[p2]["digit_pairs"] = oz_pairs(1 << n)
+                others[p2]["bf16_products"] = oz_products()
         line["other_forms"] = others
         if "value" in others.get("fp64", {}):
             line["speedup_vs_fp64"] = (value / world) / others["fp64"]["value"]
@@ -784,7 +786,8 @@ def run_grad(a):
             "n_gpus": 1, "steps": cfg.steps, "warmup": 0, "ms_per_step": 1e3 * t / cfg.steps,
             "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": cfg.description,
-                       "products": "FP64 DMMA" if gprec == "fp64" else "FP64 emulated on the BF16 tensor cores"},
+                       "products": "FP64-accurate residue products on the BF16 tensor cores" if oz_products() == 15
+                       else ("FP64 DMMA" if gprec == "fp64" else "digit products on the BF16 tensor cores")},
             "loss": loss, "grad": grad.tolist(), "fp64_tflops": flops / t / 1e12}
     if not a.no_cpu:
         # the stated errors: against the oracle's forward-mode tangent (all 13 components) and

@@ -69,23 +69,29 @@ typedef enum tc_status {
 } tc_status;
 
 /* Arithmetic of the rho <- U rho U^dag products (the tensor-core path).
- *  TC_FP64   : FP64 DMMA (mma.sync .f64), rho stored in FP64.
+ *  TC_FP64   : products at FP64 accuracy, rho stored in FP64.  For
+ *              7 <= n <= 14 (gradient: 13) and a workspace of the size that
+ *              tc_workspace_size states they run as TC_FP64_OZAKI's residue
+ *              products; at other sizes, in a smaller workspace (down to the
+ *              six N x N FP64 planes of the DMMA form and its scratch) or
+ *              under TC_OZ_BITS=6, on the FP64 DMMA (mma.sync .f64).
  *  TC_BF16X3 : each FP32 operand split in three BF16 parts, six BF16 products
  *              accumulated in FP32 in tensor memory (tcgen05 kind::f16).
  *  TC_TF32   : one TF32 product, FP32 accumulate (tcgen05 kind::tf32).
  *  TC_TF32X3 : big/small TF32 split, three products (kind::tf32).
  *  TC_FP64_OZAKI : FP64-accurate products on the BF16 tensor cores: every
- *              operand row scaled by a power of two and written as S
- *              balanced base-2^b integer digits (exact in BF16): b = 6,
- *              S = 9 in general; b = 7, S = 8 for inner dimensions
- *              K <= 4096; b = 8, S = 7 for K <= 1024 (TC_OZ_BITS=6 in the
- *              environment keeps b = 6).  The S(S+1)/2 digit products with
- *              t + u < S (45 / 36 / 28) accumulate exactly in FP32 (sums
- *              stay below 2^24) and are scaled and summed in FP64.  Within
- *              2^-48 of the row and column scales per product term (worst
- *              case); rho stored in FP64.  tc_evolve, tc_evolve_host,
- *              tc_lindblad_evolve, tc_evolve_backward and tc_batch_evolve
- *              (there the systems run side by side on concurrent branches).
+ *              operand row is scaled by a power of two (its 2-norm just below
+ *              2^58.4), rounded to integers and reduced modulo fifteen
+ *              coprime p <= 255; one BF16 product per modulus, exact in FP32
+ *              over K chunks of 1024, and the remainder theorem give the
+ *              exact integer product.  The left operand's diagonal is kept
+ *              in FP64.  Within sqrt(2 K) 2^-56.3 of the product of the two
+ *              rows' 2-norms, plus the rounding of the result; a row with an
+ *              infinity or a NaN gives NaN in its row or column.  rho stored
+ *              in FP64.  TC_OZ_BITS=6 in the environment takes 45 products of
+ *              balanced 6-bit digits instead (within 2^-48 of the rows'
+ *              largest entries per term).  tc_evolve, tc_evolve_host,
+ *              tc_lindblad_evolve, tc_evolve_backward and tc_batch_evolve.
  * In the BF16/TF32 forms U is computed in FP64 and rho is stored in FP32
  * between steps. */
 typedef enum tc_precision {
@@ -355,9 +361,8 @@ TC_API tc_status tc_lindblad_evolve(const tc_params* params, double kappa, doubl
  * checkpoints stored every `ckpt_every` steps.
  *  rho0   : device, N*N c128 (Hermitian, read only).
  *  U      : device, N*N c128, e^{-iH dt} of the same params and dt.
- *  precision: TC_FP64 (DMMA products) or TC_FP64_OZAKI (the per-step
- *           products emulated at FP64 accuracy on the BF16 tensor cores;
- *           n >= 7).
+ *  precision: TC_FP64, or TC_FP64_OZAKI (n >= 7).  The products run on the
+ *           tensor cores (see tc_precision) or on the DMMA.
  *  O_diag : device, N doubles.
  *  grad   : host, n + 2 doubles, written when the call returns (this call
  *           synchronises `stream`).
@@ -446,9 +451,8 @@ TC_API size_t tc_batch_workspace_size(int count, const int* n, int precision);
  * (Eq. 6) as in tc_evolve.  The tensor-core forms run each product of a step
  * as ONE persistent launch over the tiles of all systems (systems in
  * decreasing size, static round-robin over the SMs; single CTAs or CTA
- * pairs, see tc_batch_autotune); TC_FP64 runs the systems' DMMA products one
- * after another; TC_FP64_OZAKI runs each system's step loop, with buffers of
- * its own, on one of eight concurrent branches of the graph (library-owned
+ * pairs, see tc_batch_autotune); TC_FP64 and TC_FP64_OZAKI run each system's
+ * step loop on one of eight concurrent branches of the graph (library-owned
  * streams, one such call at a time per device).  The step loop is captured
  * into one CUDA graph on a library-owned stream and launched once; the call
  * returns after the batch has finished.  Every system's result (rho, observables) is

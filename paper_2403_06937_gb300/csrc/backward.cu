@@ -1,6 +1,6 @@
 // backward.cu -- reverse-mode gradient of L = Tr(O rho_K) through the step
 // rho <- U rho U^dag (Sec. III.A, Eq. 6) and through U = e^{-iH dt}
-// (Eqs. 7-8), in FP64 on the DMMA GEMM.
+// (Eqs. 7-8), in FP64.
 //
 // With Lambda_K = O and Lambda_k = U^dag Lambda_{k+1} U (Hermitian),
 //     dL = sum_{k<K} 2 Re Tr(Lambda_{k+1} dU rho_k U^dag)
@@ -18,10 +18,13 @@
 // then s squarings D <- X D + D X, X <- X X (chain rule of X^2), and the
 // shift back: L(A, M) = e^{-i mu dt} L(A', M).
 //
-// precision TC_FP64_OZAKI runs the per-step products (the forward steps, the
-// adjoint steps and W += rho_k Lambda_k) as FP64-accurate products on the
-// BF16 tensor cores (cgemm_oz.cu); the few products of M and of the Frechet
-// derivative stay on the DMMA GEMM.
+// On the tensor cores (TC_FP64_OZAKI, and TC_FP64 for 7 <= n <= 13 given the
+// workspace that tc_workspace_size states) every product is an FP64-accurate
+// one of cgemm_crt.cu, Y = A B^H.  With B' = conj(S) for a symmetric S
+// (U, A', the T_k) that is A S; the Frechet recurrence is taken from the
+// right, F_k = (F_{k-1} A' + T_{k-1} E) / k, so that only E, once, needs an
+// explicit adjoint.  On the DMMA GEMM the recurrence alone took 1.7 s at
+// n = 11 (real products 16 ms, complex ones 64 ms; 0.5 ms here).
 #include <cmath>
 #include <vector>
 
@@ -103,6 +106,14 @@ __global__ void minus_i_kernel(double c, const double* pr, const double* pi, dou
         const double a = pr[e], b = pi[e];
         yr[e] = c * b;
         yi[e] = -c * a;
+    }
+}
+
+// T = -i B: planes (0, -B)
+__global__ void minus_i_kernel(const double* B, double* re, double* im, size_t n) {
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        re[e] = 0.0;
+        im[e] = -B[e];
     }
 }
 
@@ -210,12 +221,11 @@ tc_status minus_i_times(int N, const double* Bs, CM X, CM Y, CM Q, cudaStream_t 
     return TC_OK;
 }
 
-// Emulated-FP64 products: slices of U and conj(U) (A operands), of the
-// current B operand and of rho_k (A operand of the W product).
+// FP64-accurate products on the tensor cores: U and conj(U) as left operands,
+// one more left and one more right operand for whatever a product needs.
 struct OzBufs {
     OzMat U, Uc, B, A2;
-    double* yr;
-    double* yi;
+    CM Y;            // adjoint of a right operand that is not symmetric
     void* scratch;
     int group;
 };
@@ -226,36 +236,101 @@ size_t oz_backward_extra(int n) {
            2 * round256(N * N * sizeof(double)) + 256;
 }
 
-// P <- U' P U'^dag with U' = U (or conj U for the adjoint step), emulated FP64
-tc_status step_oz(int N, OzBufs& z, bool adjoint, CM P, CM X, cudaStream_t s) {
+// Q <- U' P U'^dag with U' = U (or conj U for the adjoint step); P Hermitian, Q may be P
+tc_status step_oz(int N, OzBufs& z, bool adjoint, CM P, CM Q, CM X, cudaStream_t s) {
     const OzMat& A = adjoint ? z.Uc : z.U;
     TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
-    TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));       // X = U' P^H = U' P
+    TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = U' P^H
     TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s));
-    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{P.r, P.i, z.scratch}, z.group, s);        // P' = U' X^H
+    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, z.scratch}, z.group, s);    // Q = U' X^H
 }
 
-// W += rho Lambda = rho Lambda^H (Lambda Hermitian), emulated FP64
-tc_status w_accumulate_oz(int N, OzBufs& z, CM rho, CM L, CM W, bool init, cudaStream_t s) {
-    TC_TRY(oz_mat_load(z.A2, rho.r, rho.i, false, false, N, (size_t)N, s));
-    TC_TRY(oz_mat_load(z.B, L.r, L.i, false, false, N, (size_t)N, s));
-    if (init) return oz_product(0, z.A2, z.B, L.r, L.i, N, (size_t)N, OzOut{W.r, W.i, z.scratch}, z.group, s);
-    TC_TRY(oz_product(0, z.A2, z.B, L.r, L.i, N, (size_t)N, OzOut{z.yr, z.yi, z.scratch}, z.group, s));
-    const size_t NN = (size_t)N * N;
-    axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, W.r, W.i, 1.0, z.yr, z.yi, W.r, W.i, NN);
+// out = A R^H (+ out): the left operand as it is, R's planes as they are or conjugated
+tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
+    if (A.r) TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s));   // else: as loaded last
+    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s));
+    OzOut o{out.r, out.i, z.scratch};
+    o.conj_b = conj_r;
+    if (add && !oz_modular()) {   // the digit form does not accumulate
+        o.yr = z.Y.r;
+        o.yi = z.Y.i;
+        TC_TRY(oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s));
+        const size_t NN = (size_t)N * N;
+        axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, out.r, out.i, 1.0, z.Y.r, z.Y.i, out.r, out.i, NN);
+        TC_LAUNCH_CHECK();
+        return TC_OK;
+    }
+    o.accumulate = add;
+    return oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s);
+}
+
+// conjugate transpose of planar R, one 32 x 32 tile per block of 32 x 8 threads (N a multiple of 32)
+__global__ void __launch_bounds__(256)
+    adjoint_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, double* __restrict__ outr,
+                   double* __restrict__ outi) {
+    __shared__ double tr[32][33], ti[32][33];
+    const size_t i0 = (size_t)blockIdx.y * 32, j0 = (size_t)blockIdx.x * 32;
+    for (int k = threadIdx.y; k < 32; k += 8) {
+        const size_t o = (j0 + k) * N + i0 + threadIdx.x;
+        tr[k][threadIdx.x] = re[o];
+        ti[k][threadIdx.x] = im[o];
+    }
+    __syncthreads();
+    for (int k = threadIdx.y; k < 32; k += 8) {
+        const size_t o = (i0 + k) * N + j0 + threadIdx.x;
+        outr[o] = tr[threadIdx.x][k];
+        outi[o] = -ti[threadIdx.x][k];
+    }
+}
+
+tc_status adjoint(int N, CM R, CM out, cudaStream_t s) {
+    adjoint_kernel<<<dim3((unsigned)(N / 32), (unsigned)(N / 32)), dim3(32, 8), 0, s>>>(R.r, R.i, N, out.r, out.i);
     TC_LAUNCH_CHECK();
     return TC_OK;
+}
+
+// (A', as a right operand) planes of conj(-i B) = i B: (0, B)
+__global__ void times_i_kernel(const double* B, double* re, double* im, size_t n) {
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        re[e] = 0.0;
+        im[e] = B[e];
+    }
+}
+
+// One term of the Frechet recurrence, elementwise: F = Fn / k, T = Tn / k, D += F, X += T
+__global__ void term_kernel(double inv, CM Fn, CM Tn, CM F, CM T, CM D, CM X, size_t n) {
+    for (size_t e = (size_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (size_t)gridDim.x * blockDim.x) {
+        const double fr = inv * Fn.r[e], fi = inv * Fn.i[e], tr = inv * Tn.r[e], ti = inv * Tn.i[e];
+        F.r[e] = fr;
+        F.i[e] = fi;
+        T.r[e] = tr;
+        T.i[e] = ti;
+        D.r[e] += fr;
+        D.i[e] += fi;
+        X.r[e] += tr;
+        X.i[e] += ti;
+    }
+}
+
+// TC_FP64 takes the tensor-core products from n = 7 to n = 13 (at n = 14 their
+// operands' 77 GB would come on top of 220 GB of checkpoints).
+bool backward_f64_on_tensor_cores(int n) { return f64_on_tensor_cores(n) && n <= 13; }
+
+size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
+    if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
+    const int nck = (steps + ckpt_every - 1) / ckpt_every;
+    const int c = ckpt_every < steps ? ckpt_every : steps;
+    // U, Lambda, X, W, seg0 + checkpoints + segment + Frechet (T, F, Tn, Fn, P, Q) + B + small
+    const size_t b = (size_t)(5 + nck + c + 6) * cm_bytes(n) + real_bytes(n) +
+                     round256((2 * ((size_t)1 << n) + 64) * 8) + 1024;
+    return precision == TC_FP64_OZAKI ? b + oz_backward_extra(n) : b;
 }
 
 }  // namespace
 
 size_t backward_bytes(int n, int steps, int ckpt_every, int precision) {
-    if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
-    if (precision == TC_FP64_OZAKI) return backward_bytes(n, steps, ckpt_every, TC_FP64) + oz_backward_extra(n);
-    const int nck = (steps + ckpt_every - 1) / ckpt_every;
-    const int c = ckpt_every < steps ? ckpt_every : steps;
-    // U, Lambda, X, W, seg0 + checkpoints + segment + Frechet (T, F, Tn, Fn, P, Q) + B + small
-    return (size_t)(5 + nck + c + 6) * cm_bytes(n) + real_bytes(n) + round256((2 * ((size_t)1 << n) + 64) * 8) + 1024;
+    return backward_least_bytes(n, steps, ckpt_every,
+                                precision == TC_FP64 && backward_f64_on_tensor_cores(n) ? TC_FP64_OZAKI : precision);
 }
 
 }  // namespace tc
@@ -279,7 +354,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     if (!rho0 || !U || !O_diag || !grad) return fail(TC_ERR_INVALID_ARG, "null pointer");
     if ((reinterpret_cast<uintptr_t>(rho0) | reinterpret_cast<uintptr_t>(U)) & 15u)
         return fail(TC_ERR_INVALID_ARG, "rho0 and U must be 16-byte aligned");
-    const size_t need = backward_bytes(n, steps, ckpt_every, precision);
+    const size_t need = backward_least_bytes(n, steps, ckpt_every, precision);
     if (!work) return fail(TC_ERR_WORKSPACE, "work is NULL (need %zu bytes)", need);
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(TC_ERR_WORKSPACE, "work is not 256-byte aligned");
     if (work_bytes < need) return fail(TC_ERR_WORKSPACE, "work has %zu bytes, need %zu", work_bytes, need);
@@ -311,29 +386,34 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     b.B = ar.take<double>(NN);
     b.small = ar.take<double>(2 * (size_t)N + 64);
     if (!b.small) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
-    const bool oz = precision == TC_FP64_OZAKI;
+    const bool oz = precision == TC_FP64_OZAKI || (backward_f64_on_tensor_cores(n) &&
+                                                   work_bytes >= backward_bytes(n, steps, ckpt_every, TC_FP64));
     OzBufs z{};
     if (oz) {
         TC_TRY(oz_mat_init(z.U, ar, N, true));
         TC_TRY(oz_mat_init(z.Uc, ar, N, true));
         TC_TRY(oz_mat_init(z.B, ar, N, false));
         TC_TRY(oz_mat_init(z.A2, ar, N, true));
-        z.yr = ar.take<double>(NN);
-        z.yi = ar.take<double>(NN);
+        z.Y = take_cm(ar, NN);
         z.scratch = ar.take<uint8_t>(oz_scratch_bytes(N));
         if (!z.scratch) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
         z.group = tune_lookup(n, TC_BF16X3).tc_group;
         TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));
         TC_TRY(oz_mat_load(z.Uc, static_cast<const double*>(U), nullptr, true, true, N, (size_t)N, s));
     }
-    auto fwd_step = [&](CM P) -> tc_status { return oz ? step_oz(N, z, false, P, b.X, s) : step(N, b.U, P, b.X, 0, s); };
+    // Q <- U P U^dag, Q may be P
+    auto fwd_step = [&](CM P, CM Q) -> tc_status {
+        if (oz) return step_oz(N, z, false, P, Q, b.X, s);
+        if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, s));
+        return step(N, b.U, Q, b.X, 0, s);
+    };
 
     // ---------------------------------------------------------------- forward
     TC_TRY(launch_split_c128(static_cast<const double*>(U), b.U.r, b.U.i, NN, s));
     TC_TRY(launch_split_c128(static_cast<const double*>(rho0), ck[0].r, ck[0].i, NN, s));
     TC_TRY(copy_cm(ck[0], b.seg0, NN, s));   // seg0 = running rho
     for (int k = 1; k <= steps; k++) {
-        TC_TRY(fwd_step(b.seg0));
+        TC_TRY(fwd_step(b.seg0, b.seg0));
         if (k < steps && k % ckpt_every == 0) TC_TRY(copy_cm(b.seg0, ck[k / ckpt_every], NN, s));
     }
     // loss from rho_K (in seg0)
@@ -350,14 +430,13 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         // recompute rho_{k0..k1-1} into seg[0..]
         TC_TRY(copy_cm(ck[j], seg[0], NN, s));
         for (int k = k0 + 1; k < k1; k++) {
-            TC_TRY(copy_cm(seg[k - 1 - k0], seg[k - k0], NN, s));
-            TC_TRY(fwd_step(seg[k - k0]));
+            TC_TRY(fwd_step(seg[k - 1 - k0], seg[k - k0]));
         }
         for (int k = k1 - 1; k >= k0; k--) {
             // Lambda_k = U^dag Lambda_{k+1} U  (the step with conj(U)); W += rho_k Lambda_k
             if (oz) {
-                TC_TRY(step_oz(N, z, true, b.L, b.X, s));
-                TC_TRY(w_accumulate_oz(N, z, seg[k - k0], b.L, b.W, !w_init, s));
+                TC_TRY(step_oz(N, z, true, b.L, b.L, b.X, s));
+                TC_TRY(mul_oz(N, z, seg[k - k0], b.L, false, b.W, w_init, s));   // Lambda Hermitian
             } else {
                 TC_TRY(step(N, b.U, b.L, b.X, 1, s));
                 TC_TRY(gemm_c(N, seg[k - k0], 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, s));
@@ -367,7 +446,10 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     }
     // M = W U^dag = W conj(U)  -> into L (free now)
     CM M = b.L;
-    TC_TRY(gemm_c(N, b.W, 0, b.U, 1, M, 1.0, 0.0, 0, s));
+    if (oz)
+        TC_TRY(mul_oz(N, z, b.W, b.U, false, M, false, s));   // W U^H, U symmetric
+    else
+        TC_TRY(gemm_c(N, b.W, 0, b.U, 1, M, 1.0, 0.0, 0, s));
 
     // ---------------------------------------------------------------- Frechet
     // plan from H's trace and norm (computed on the device, read back)
@@ -408,13 +490,28 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // T_1 = A' T_0 = -i B
     {
         // T1 = -i B: planes (0, -B)
-        identity_kernel<<<grid_for(NN), 256, 0, s>>>(b.Tn.r, b.Tn.i, N);
+        minus_i_kernel<<<grid_for(NN), 256, 0, s>>>(b.B, b.T.r, b.T.i, NN);
         TC_LAUNCH_CHECK();
-        TC_TRY(minus_i_times(N, b.B, b.Tn, b.T, b.Q, s));
         axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, Xs.r, Xs.i, 1.0, b.T.r, b.T.i, Xs.r, Xs.i, NN);
         TC_LAUNCH_CHECK();
     }
-    for (int k = 2; k <= mt; k++) {
+    const CM again{nullptr, nullptr};   // the left operand loaded last
+    const bool oz_frechet = oz && oz_modular();
+    if (oz_frechet) {
+        // Q = conj(A') (A' symmetric) and Y = E^H, the right operands of the recurrence
+        times_i_kernel<<<grid_for(NN), 256, 0, s>>>(b.B, b.Q.r, b.Q.i, NN);
+        TC_LAUNCH_CHECK();
+        TC_TRY(adjoint(N, b.P, z.Y, s));
+        for (int k = 2; k <= mt; k++) {
+            // F_k = (F_{k-1} A' + T_{k-1} E) / k ;  T_k = T_{k-1} A' / k
+            TC_TRY(mul_oz(N, z, b.F, b.Q, false, b.Fn, false, s));
+            TC_TRY(mul_oz(N, z, b.T, b.Q, false, b.Tn, false, s));
+            TC_TRY(mul_oz(N, z, again, z.Y, false, b.Fn, true, s));
+            term_kernel<<<grid_for(NN), 256, 0, s>>>(1.0 / k, b.Fn, b.Tn, b.F, b.T, D, Xs, NN);
+            TC_LAUNCH_CHECK();
+        }
+    }
+    for (int k = 2; k <= mt && !oz_frechet; k++) {
         // F_k = (A' F_{k-1} + E T_{k-1}) / k ;  T_k = A' T_{k-1} / k
         TC_TRY(minus_i_times(N, b.B, b.F, b.Fn, b.Q, s));                 // Fn = A' F
         TC_TRY(gemm_c(N, b.P, 0, b.T, 0, b.Fn, 1.0, 1.0, 0, s));          // Fn += E T
@@ -431,6 +528,15 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     }
     // squarings: D <- X D + D X ; X <- X X
     for (int q = 0; q < sq; q++) {
+        if (oz_frechet) {
+            TC_TRY(mul_oz(N, z, D, Xs, true, b.Fn, false, s));       // D X (X symmetric: X = conj(X)^H)
+            TC_TRY(mul_oz(N, z, Xs, Xs, true, b.Tn, false, s));      // X X
+            TC_TRY(adjoint(N, D, z.Y, s));
+            TC_TRY(mul_oz(N, z, again, z.Y, false, b.Fn, true, s));  // + X D
+            TC_TRY(copy_cm(b.Fn, D, NN, s));
+            TC_TRY(copy_cm(b.Tn, Xs, NN, s));
+            continue;
+        }
         TC_TRY(gemm_c(N, Xs, 0, D, 0, b.Fn, 1.0, 0.0, 0, s));
         TC_TRY(gemm_c(N, D, 0, Xs, 0, b.Fn, 1.0, 1.0, 0, s));
         TC_TRY(copy_cm(b.Fn, D, NN, s));

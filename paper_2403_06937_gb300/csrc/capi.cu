@@ -91,14 +91,17 @@ size_t expm_bytes(int n) {
     return 13 * mat_bytes(n, 8) + round256((2 * N + 4) * sizeof(double));
 }
 
-size_t evolve_f64_bytes(int n) {
-    return 6 * mat_bytes(n, 8) + observables_scratch_bytes(n) + 256 +
-           (((size_t)1 << n) <= (size_t)kSplitMaxDim ? gemm_f64_splitk_bytes() : 0);
-}
-
+// The least a call needs.  TC_FP64 runs its DMMA form in this much and the
+// tensor-core form in what tc_workspace_size states (wanted_evolve_bytes).
 size_t evolve_bytes(int n, int precision) {
     if (precision == TC_FP64_OZAKI) return evolve_oz_bytes(n);
     return precision == TC_FP64 ? evolve_f64_bytes(n) : evolve_lowp_bytes(n, precision);
+}
+
+size_t wanted_evolve_bytes(int n, int precision) {
+    const size_t least = evolve_bytes(n, precision);
+    if (precision != TC_FP64 || !f64_on_tensor_cores(n)) return least;
+    return least > evolve_oz_bytes(n) ? least : evolve_oz_bytes(n);
 }
 
 // device staging of tc_evolve_host: rho (c128) and the observable rows
@@ -364,12 +367,12 @@ TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ck
     size_t need = 0;
     auto upd = [&](size_t b) { if (b > need) need = b; };
     if (ops & TC_OP_EXPM) upd(expm_bytes(n));
-    if (ops & TC_OP_EVOLVE) upd(evolve_bytes(n, precision));
+    if (ops & TC_OP_EVOLVE) upd(wanted_evolve_bytes(n, precision));
     if (ops & TC_OP_OBSERVABLES) upd(observables_scratch_bytes(n));
     if (ops & TC_OP_EXPM_MODEL) upd(expm_model_bytes(n));
     if (ops & TC_OP_LINDBLAD) upd(lindblad_bytes(n, precision));
-    if (ops & TC_OP_EVOLVE_HOST) upd(evolve_bytes(n, precision) + evolve_host_extra(n, steps));
-    if (ops & TC_OP_EVOLVE_HOST_PINNED) upd(evolve_bytes(n, precision) + evolve_host_pinned_extra(n, steps, precision));
+    if (ops & TC_OP_EVOLVE_HOST) upd(wanted_evolve_bytes(n, precision) + evolve_host_extra(n, steps));
+    if (ops & TC_OP_EVOLVE_HOST_PINNED) upd(wanted_evolve_bytes(n, precision) + evolve_host_pinned_extra(n, steps, precision));
     if (ops & TC_OP_BACKWARD) upd(backward_bytes(n, steps, ckpt_every, precision));
     return need;
 }
@@ -441,6 +444,9 @@ TC_API tc_status tc_evolve(const void* U, void* rho, int n, int steps, int preci
     if (precision == TC_FP64_OZAKI)
         return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, renorm_every, mp, obs,
                          ar, s);
+    if (precision == TC_FP64 && f64_on_tensor_cores(n) && ar.size >= evolve_oz_bytes(n))
+        return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, renorm_every, mp, obs,
+                         ar, s);
     if (precision != TC_FP64)
         return evolve_lowp(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision,
                            renorm_every, mp, obs, ar, s);
@@ -487,8 +493,10 @@ TC_API tc_status tc_evolve_host(const void* U, void* rho_host, int n, int steps,
             TC_TRY(copy_by_sms(rho_dev, mapped, 16 * N * N, s));
         else
             TC_CUDA(cudaMemcpyAsync(rho_dev, rho_host, 16 * N * N, cudaMemcpyHostToDevice, s));
-        TC_TRY(precision == TC_FP64 ? evolve_f64(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s)
-                                    : evolve_oz(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));
+        if (precision == TC_FP64_OZAKI || (f64_on_tensor_cores(n) && ar.size - ar.used >= evolve_oz_bytes(n)))
+            TC_TRY(evolve_oz(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));
+        else
+            TC_TRY(evolve_f64(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));
         if (mapped)
             TC_TRY(copy_by_sms(const_cast<void*>(mapped), rho_dev, 16 * N * N, s));
         else

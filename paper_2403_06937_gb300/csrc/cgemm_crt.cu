@@ -38,6 +38,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "cgemm_crt.cuh"
 #include "cgemm_dev.cuh"
@@ -410,7 +411,8 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 // ---------------------------------------------------------------- residues
 // Row scale and residue planes of one operand.  A row is handled by TPR
-// consecutive threads of a 128-thread block (8 columns a thread and step):
+// consecutive threads of a 128-thread block (CPT columns a thread and step; 2
+// up to N = 512, where the threads would be too few to fill the SMs, else 8):
 // first the scale from the row's largest exponent and its 2-norm, then the
 // residues.  Bound by HBM for large matrices (16 B read, 60 B written per
 // entry; the second read of the row comes from L2); no FP64 instruction, since
@@ -444,19 +446,19 @@ __device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits) {
     a.ss = fmaf(f, f, a.ss);
 }
 
-template <bool INTERLEAVED, bool LEFT>
+template <bool INTERLEAVED, bool LEFT, int CPT>
 __global__ void __launch_bounds__(128)
     crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
                        int tpr, uint64_t im_flip, __nv_bfloat16* __restrict__ planes, int* __restrict__ ex,
                        double* __restrict__ diag) {
     const int sub = threadIdx.x % tpr;                       // thread within the row
     const int r = blockIdx.x * (128 / tpr) + threadIdx.x / tpr;
-    // 8 consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
-    auto load8 = [&](int c0, uint64_t (&xr)[8], uint64_t (&xi)[8]) {
+    // CPT consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
+    auto load = [&](int c0, uint64_t (&xr)[CPT], uint64_t (&xi)[CPT]) {
         if (INTERLEAVED) {
             const ulonglong2* p = reinterpret_cast<const ulonglong2*>(re) + (size_t)r * ld + c0;
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
+            for (int q = 0; q < CPT; q++) {
                 ulonglong2 v = make_ulonglong2(0, 0);
                 if (r < N && c0 + q < N) v = p[q];
                 xr[q] = v.x;
@@ -465,9 +467,9 @@ __global__ void __launch_bounds__(128)
         } else {
             const double* pr = re + (size_t)r * ld + c0;
             const double* pi = im + (size_t)r * ld + c0;
-            if (r < N && c0 + 8 <= N) {   // ld even, planes 16-byte aligned (checked on the host)
+            if (r < N && c0 + CPT <= N) {   // ld even, planes 16-byte aligned (checked on the host)
 #pragma unroll
-                for (int q = 0; q < 8; q += 2) {
+                for (int q = 0; q < CPT; q += 2) {
                     const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pr + q);
                     const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(pi + q);
                     xr[q] = a.x;
@@ -477,16 +479,16 @@ __global__ void __launch_bounds__(128)
                 }
             } else {
 #pragma unroll
-                for (int q = 0; q < 8; q++) {
+                for (int q = 0; q < CPT; q++) {
                     const bool in = r < N && c0 + q < N;
                     xr[q] = in ? (uint64_t)__double_as_longlong(pr[q]) : 0;
                     xi[q] = in ? (uint64_t)__double_as_longlong(pi[q]) : 0;
                 }
             }
         }
-        if (LEFT && r >= c0 && r < c0 + 8) {
+        if (LEFT && r >= c0 && r < c0 + CPT) {
 #pragma unroll
-            for (int q = 0; q < 8; q++)
+            for (int q = 0; q < CPT; q++)
                 if (c0 + q == r) {
                     xr[q] = 0;
                     xi[q] = 0;
@@ -494,11 +496,11 @@ __global__ void __launch_bounds__(128)
         }
     };
     RowStat st{0, 0.0f};
-    for (int c0 = 8 * sub; c0 < Np; c0 += 8 * tpr) {
-        uint64_t xr[8], xi[8];
-        load8(c0, xr, xi);
+    for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
+        uint64_t xr[CPT], xi[CPT];
+        load(c0, xr, xi);
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
+        for (int q = 0; q < CPT; q++) {
             stat_add(st, xr[q]);
             stat_add(st, xi[q]);
         }
@@ -535,15 +537,15 @@ __global__ void __launch_bounds__(128)
         }
     }
     const size_t plane = (size_t)Np * Np;
-    for (int c0 = 8 * sub; c0 < Np; c0 += 8 * tpr) {
-        uint64_t xr[8], xi[8];
-        load8(c0, xr, xi);
+    for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
+        uint64_t xr[CPT], xi[CPT];
+        load(c0, xr, xi);
 #pragma unroll
         for (int part = 0; part < 2; part++) {
-            crt::Pieces pc[8];
-            uint32_t sign[4];
+            crt::Pieces pc[CPT];
+            uint32_t sign[CPT / 2];
 #pragma unroll
-            for (int q = 0; q < 8; q++) {
+            for (int q = 0; q < CPT; q++) {
                 const uint64_t b = part ? xi[q] ^ im_flip : xr[q];
                 pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0);
                 const uint32_t sg = (uint32_t)(b >> 63) << 15;
@@ -556,9 +558,9 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
             for (int s = 0; s < kModuli; s++) {
                 const int p = crt::modulus(s);
-                uint32_t w[4];
+                uint32_t w[CPT / 2];
 #pragma unroll
-                for (int h = 0; h < 4; h++) {
+                for (int h = 0; h < CPT / 2; h++) {
                     uint32_t b[2];
 #pragma unroll
                     for (int k = 0; k < 2; k++) {
@@ -568,7 +570,10 @@ __global__ void __launch_bounds__(128)
                     }
                     w[h] = __byte_perm(b[0], b[1], 0x7632) ^ sign[h];   // the top halves are the BF16 values
                 }
-                *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+                if constexpr (CPT == 8)
+                    *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[0], w[1], w[2], w[3]);
+                else
+                    *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane) = w[0];
             }
         }
     }
@@ -577,16 +582,20 @@ __global__ void __launch_bounds__(128)
 // ---------------------------------------------------------------- recombination
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// mag 2^e in FP64, e of any size (one rounding unless the result is subnormal)
+// mag 2^e in FP64, e of any size.  Rounded to 53 bits and packed with integer
+// instructions (the FP64 pipe issues two instructions per clock and SM);
+// results outside the normal range take the slow way.
 __device__ __forceinline__ double scaled(uint64_t mag, bool neg, int e) {
+    const int lz = crt::clz64(mag);
+    const uint64_t m = mag << (lz & 63);
+    const uint64_t r = (m >> 11) + ((m >> 10) & 1);        // 53 bits, or 2^53 after a carry
+    const int be = e + 11 - lz + 1075;                     // biased exponent of r's leading bit
+    if (mag != 0 && be > 0 && be < 2046)
+        return __longlong_as_double((long long)(((uint64_t)(be - 1) << 52) + r) | (neg ? LLONG_MIN : 0));
     double v = __ull2double_rn(mag);
-    if (mag) {
-        if (e >= -1000 && e <= 900) {
-            v *= pow2d(e);
-        } else {
-            const int e1 = max(min(e, 900), -1000), e2 = max(min(e - e1, 900), -1000);
-            v = v * pow2d(e1) * pow2d(e2);
-        }
+    if (mag != 0) {
+        const int e1 = max(min(e, 900), -1000), e2 = max(min(e - e1, 900), -1000);
+        v = v * pow2d(e1) * pow2d(e2);
     }
     return neg ? -v : v;
 }
@@ -599,102 +608,131 @@ struct CrtCombine {
     size_t ldb;
     const int* ea;
     const int* eb;
-    const double* diag;      // [2][Np] or null
+    const double* diag;      // [2][Np]
     const double* br;
     const double* bi;
+    double bi_sign;          // -1 when B was loaded conjugated
+    int accumulate;          // MODE 0: add to Y
     double* yr;
     double* yi;
 };
 
-// One 32 x 32 tile of Y per block of 256 threads, four consecutive columns a
-// thread.  MODE 1: tiles on and below the diagonal, each mirrored.  B's
-// entries of the diagonal term, and the mirrored half, are transposed through
-// shared memory so that every global access runs along rows.
-template <int MODE>
+// One tile of 32 rows x 8 COLS columns of Y per block of 256 threads, COLS
+// consecutive columns a thread.  MODE 1: tiles that reach the diagonal or lie
+// below it, each mirrored.  B's entries of the diagonal term, and the mirrored
+// half, are transposed through shared memory so that every global access runs
+// along rows.  Bound by HBM for large matrices (30 B + 16 B read, 16 B
+// written per entry) beside 45 32 x 8-bit multiply-adds a number; at N <= 512
+// by latency, so there one column a thread (four times the threads).
+template <int MODE, int COLS>
 __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
-    __shared__ double sr[32][33], si[32][33];
-    const int i0 = p.row0 + 32 * (int)blockIdx.y, j0 = 32 * (int)blockIdx.x;
-    if (MODE == 1 && j0 > i0) return;
-    const int ti = threadIdx.x >> 3, tj = (threadIdx.x & 7) * 4;
-    // B[j0 + a][i0 + b] -> s[a][b]
-    if (p.diag) {
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            const int a = ti, b = tj + k;
-            const bool in = j0 + a < p.N && i0 + b < p.N;
-            const size_t o = (size_t)(j0 + a) * p.ldb + (size_t)(i0 + b);
-            sr[a][b] = in ? p.br[o] : 0.0;
-            si[a][b] = in ? p.bi[o] : 0.0;
-        }
-    }
+    constexpr int W = 8 * COLS;
+    __shared__ double sr[W][33], si[W][33];   // [column of the tile][row of the tile]
+    const int i0 = p.row0 + 32 * (int)blockIdx.y, j0 = W * (int)blockIdx.x;
+    if (MODE == 1 && j0 > i0 + 31) return;
+    const int ti = threadIdx.x >> 3, tj = (threadIdx.x & 7) * COLS;                      // along rows of Y
+    const int ta = threadIdx.x / (32 / COLS), tb = (threadIdx.x % (32 / COLS)) * COLS;   // along rows of B and the mirror
     const int i = i0 + ti, j = j0 + tj;
     const size_t o = (size_t)(i - p.row0) * p.Np + j;
-    crt::Acc ar[4] = {}, ai[4] = {};
+    uint32_t wr[kModuli], wi[kModuli];
 #pragma unroll
     for (int s = 0; s < kModuli; s++) {
-        const uint32_t wr = *reinterpret_cast<const uint32_t*>(p.bytes + (size_t)(2 * s) * p.band * p.Np + o);
-        const uint32_t wi = *reinterpret_cast<const uint32_t*>(p.bytes + (size_t)(2 * s + 1) * p.band * p.Np + o);
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            crt::acc_add(ar[k], (wr >> (8 * k)) & 0xFFu, kC.frac[s]);
-            crt::acc_add(ai[k], (wi >> (8 * k)) & 0xFFu, kC.frac[s]);
+        const uint8_t* a = p.bytes + (size_t)(2 * s) * p.band * p.Np + o;
+        if (COLS == 4) {
+            wr[s] = *reinterpret_cast<const uint32_t*>(a);
+            wi[s] = *reinterpret_cast<const uint32_t*>(a + p.band * p.Np);
+        } else {
+            wr[s] = a[0];
+            wi[s] = a[p.band * p.Np];
         }
     }
-    const int ea = p.ea[i];
-    double vr[4], vi[4];
+    // B[j0 + a][i0 + b] -> s[a][b]
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        const int eb = p.eb[j + k];
-        if (ea == kNoScale || eb == kNoScale) {   // an infinity or a NaN in either row
+    for (int k = 0; k < COLS; k++) {
+        const int b = tb + k;
+        const bool in = j0 + ta < p.N && i0 + b < p.N;
+        const size_t ob = (size_t)(j0 + ta) * p.ldb + (size_t)(i0 + b);
+        sr[ta][b] = in ? p.br[ob] : 0.0;
+        si[ta][b] = in ? p.bi_sign * p.bi[ob] : 0.0;
+    }
+    const int ea = p.ea[i];
+    int eb[COLS];
+#pragma unroll
+    for (int k = 0; k < COLS; k++) eb[k] = p.eb[j + k];
+    const double dr = p.diag[i], di = p.diag[p.Np + i];
+    double vr[COLS], vi[COLS];
+#pragma unroll
+    for (int k = 0; k < COLS; k++) {
+        crt::Acc ar = {}, ai = {};
+#pragma unroll
+        for (int s = 0; s < kModuli; s++) {
+            crt::acc_add(ar, (wr[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
+            crt::acc_add(ai, (wi[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
+        }
+        if (ea == kNoScale || eb[k] == kNoScale) {   // an infinity or a NaN in either row
             vr[k] = vi[k] = __longlong_as_double(0x7FF8000000000000ll);
             continue;
         }
         bool neg;
         int e;
-        uint64_t mag = crt::acc_finish(ar[k], kC, neg, e);
-        vr[k] = scaled(mag, neg, e - ea - eb);
-        mag = crt::acc_finish(ai[k], kC, neg, e);
-        vi[k] = scaled(mag, neg, e - ea - eb);
+        uint64_t mag = crt::acc_finish(ar, kC, neg, e);
+        vr[k] = scaled(mag, neg, e - ea - eb[k]);
+        mag = crt::acc_finish(ai, kC, neg, e);
+        vi[k] = scaled(mag, neg, e - ea - eb[k]);
     }
-    if (p.diag) {
-        __syncthreads();
-        const double dr = p.diag[i], di = p.diag[p.Np + i];
+    __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 4; k++) {   // A_ii conj(B_ji)
-            const double br = sr[tj + k][ti], bi = si[tj + k][ti];
-            vr[k] = fma(dr, br, fma(di, bi, vr[k]));
-            vi[k] = fma(di, br, fma(-dr, bi, vi[k]));
-        }
+    for (int k = 0; k < COLS; k++) {   // A_ii conj(B_ji)
+        const double br = sr[tj + k][ti], bi = si[tj + k][ti];
+        vr[k] = fma(dr, br, fma(di, bi, vr[k]));
+        vi[k] = fma(di, br, fma(-dr, bi, vi[k]));
     }
     double* yr = p.yr + (size_t)i * p.Np + j;
     double* yi = p.yi + (size_t)i * p.Np + j;
-    if (MODE == 0 || i0 > j0) {
-        *reinterpret_cast<double2*>(yr) = make_double2(vr[0], vr[1]);
-        *reinterpret_cast<double2*>(yr + 2) = make_double2(vr[2], vr[3]);
-        *reinterpret_cast<double2*>(yi) = make_double2(vi[0], vi[1]);
-        *reinterpret_cast<double2*>(yi + 2) = make_double2(vi[2], vi[3]);
+    if (MODE == 0 && p.accumulate) {
+#pragma unroll
+        for (int k = 0; k < COLS; k++) {
+            vr[k] += yr[k];
+            vi[k] += yi[k];
+        }
     }
-    if (MODE == 1) {
+    if (COLS == 4 && (MODE == 0 || j0 + W <= i0)) {
+#pragma unroll
+        for (int k = 0; k < COLS; k += 2) {
+            *reinterpret_cast<double2*>(yr + k) = make_double2(vr[k], vr[k + 1 < COLS ? k + 1 : k]);
+            *reinterpret_cast<double2*>(yi + k) = make_double2(vi[k], vi[k + 1 < COLS ? k + 1 : k]);
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < COLS; k++) {
+            if (MODE == 1 && j + k > i) continue;
+            yr[k] = vr[k];
+            yi[k] = MODE == 1 && j + k == i ? 0.0 : vi[k];
+        }
+    }
+    if (MODE == 1) {   // Y[j0 + a][i0 + b] = conj(Y[i0 + b][j0 + a]) above the diagonal
         __syncthreads();
 #pragma unroll
-        for (int k = 0; k < 4; k++) {
-            sr[ti][tj + k] = vr[k];
-            si[ti][tj + k] = vi[k];
+        for (int k = 0; k < COLS; k++) {
+            sr[tj + k][ti] = vr[k];
+            si[tj + k][ti] = vi[k];
         }
         __syncthreads();
-        if (i0 > j0) {   // Y[j0 + ti][i0 + tj ..] = conj(Y[i0 + tj ..][j0 + ti])
-            double* mr = p.yr + (size_t)(j0 + ti) * p.Np + i0 + tj;
-            double* mi = p.yi + (size_t)(j0 + ti) * p.Np + i0 + tj;
-            *reinterpret_cast<double2*>(mr) = make_double2(sr[tj][ti], sr[tj + 1][ti]);
-            *reinterpret_cast<double2*>(mr + 2) = make_double2(sr[tj + 2][ti], sr[tj + 3][ti]);
-            *reinterpret_cast<double2*>(mi) = make_double2(-si[tj][ti], -si[tj + 1][ti]);
-            *reinterpret_cast<double2*>(mi + 2) = make_double2(-si[tj + 2][ti], -si[tj + 3][ti]);
-        } else {         // a diagonal tile: the lower half, its mirror, a real diagonal
+        double* mr = p.yr + (size_t)(j0 + ta) * p.Np + i0 + tb;
+        double* mi = p.yi + (size_t)(j0 + ta) * p.Np + i0 + tb;
+        if (COLS == 4 && j0 + W <= i0) {
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                const int c = tj + k;
-                yr[k] = c <= ti ? vr[k] : sr[c][ti];
-                yi[k] = c < ti ? vi[k] : (c == ti ? 0.0 : -si[c][ti]);
+            for (int k = 0; k < COLS; k += 2) {
+                const int k1 = k + 1 < COLS ? k + 1 : k;
+                *reinterpret_cast<double2*>(mr + k) = make_double2(sr[ta][tb + k], sr[ta][tb + k1]);
+                *reinterpret_cast<double2*>(mi + k) = make_double2(-si[ta][tb + k], -si[ta][tb + k1]);
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < COLS; k++) {
+                if (j0 + ta >= i0 + tb + k) continue;
+                mr[k] = sr[ta][tb + k];
+                mi[k] = -si[ta][tb + k];
             }
         }
     }
@@ -770,24 +808,24 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
     if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
         (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
-    const int tpr = std::min(128, m.Np / 8);   // Np is a multiple of 128: 16, 32, 48, ... threads a row
-    // only powers of two divide the block evenly; ragged sizes take the next one below
-    int t = 16;
-    while (2 * t <= tpr) t *= 2;
-    const unsigned grid = (unsigned)((m.Np + 128 / t - 1) / (128 / t));
+    const int cpt = m.Np <= 512 ? 2 : 8;
+    int tpr = 16;   // threads a row: a power of two, at most 128 and Np / cpt
+    while (2 * tpr <= std::min(128, m.Np / cpt)) tpr *= 2;
+    const unsigned grid = (unsigned)((m.Np + 128 / tpr - 1) / (128 / tpr));
     const uint64_t flip = conj ? 1ull << 63 : 0;
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
-    if (interleaved) {
-        if (m.left)
-            crt_residue_kernel<true, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
-        else
-            crt_residue_kernel<true, false><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+#define TC_RES(I_, L_, C_) \
+    crt_residue_kernel<I_, L_, C_><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, out, m.ex, m.diag)
+    if (interleaved && m.left) {
+        if (cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 8);
+    } else if (interleaved) {
+        if (cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 8);
+    } else if (m.left) {
+        if (cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 8);
     } else {
-        if (m.left)
-            crt_residue_kernel<false, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
-        else
-            crt_residue_kernel<false, false><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, t, flip, out, m.ex, m.diag);
+        if (cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 8);
     }
+#undef TC_RES
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -836,11 +874,14 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
         c.bi = bi;
         c.yr = out.yr;
         c.yi = out.yi;
-        const dim3 grid((unsigned)((mode == 0 ? Np : row0 + band) / 32), (unsigned)(band / 32));
-        if (mode == 0)
-            crt_combine_kernel<0><<<grid, 256, 0, s>>>(c);
+        c.bi_sign = out.conj_b ? -1.0 : 1.0;
+        c.accumulate = out.accumulate ? 1 : 0;
+        const int cols = Np <= 512 ? 1 : 4;
+        const dim3 grid((unsigned)((mode == 0 ? Np : row0 + band) / (8 * cols)), (unsigned)(band / 32));
+        if (cols == 1)
+            mode == 0 ? crt_combine_kernel<0, 1><<<grid, 256, 0, s>>>(c) : crt_combine_kernel<1, 1><<<grid, 256, 0, s>>>(c);
         else
-            crt_combine_kernel<1><<<grid, 256, 0, s>>>(c);
+            mode == 0 ? crt_combine_kernel<0, 4><<<grid, 256, 0, s>>>(c) : crt_combine_kernel<1, 4><<<grid, 256, 0, s>>>(c);
         TC_LAUNCH_CHECK();
     }
     return TC_OK;

@@ -38,6 +38,8 @@ struct CrtOut {
     double* yr;
     double* yi;
     void* scratch;
+    bool accumulate;   // add to what yr, yi hold (mode 0)
+    bool conj_b;       // B was loaded with conj: (br, bi) are the planes before it
 };
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
                       size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s);

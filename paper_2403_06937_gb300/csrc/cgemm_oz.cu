@@ -839,8 +839,9 @@ tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br,
                      const OzOut& out, int group, cudaStream_t s) {
     if (A.Np != B.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
     if (oz_modular())
-        return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch},
+        return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch, out.accumulate, out.conj_b},
                            oz_use_pairs(A.Np / 128), s);
+    if (out.accumulate) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: the digit form does not accumulate");
     OzEpi ep{};
     ep.Np = A.Np;
     ep.tiles = A.Np / 128;

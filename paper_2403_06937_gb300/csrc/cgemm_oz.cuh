@@ -76,6 +76,8 @@ struct OzOut {
     double* yr;        // FP64 planes of the result, row stride Np
     double* yi;
     void* scratch;     // oz_scratch_bytes(Np)
+    bool accumulate = false;   // residue form only: add to what yr, yi hold (mode 0)
+    bool conj_b = false;       // B was loaded with conj: its planes (br, bi) hold the conjugate
 };
 size_t oz_mat_bytes(int Np, bool left);
 size_t oz_scratch_bytes(int Np);

@@ -1,4 +1,5 @@
-// evolve_f64.cu -- the plain FP64 form of the step loop: rho <- U rho U^dag
+// evolve_f64.cu -- the DMMA form of TC_FP64's step loop (n <= 6, n > 14, or a
+// workspace too small for the tensor-core form of evolve_oz.cu): rho <- U rho U^dag
 // (Sec. III.A, Eq. 6), evaluated as the two products of Eq. 12 on the DMMA
 // GEMM:  X = U rho (full), then rho' = X conj(U) (U complex symmetric, so
 // conj(U) = U^dag), of which only the block-lower triangle is computed and
@@ -9,6 +10,12 @@
 #include "timing.cuh"
 
 namespace tc {
+
+size_t evolve_f64_bytes(int n) {
+    const size_t N = (size_t)1 << n;
+    return 6 * round256(N * N * sizeof(double)) + observables_scratch_bytes(n) + 256 +
+           (N <= (size_t)kSplitMaxDim ? gemm_f64_splitk_bytes((int)N) : 0);
+}
 
 tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m,
                      double* obs, Arena& ar, cudaStream_t s) {
@@ -21,7 +28,7 @@ tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_
     double* Xr = ar.take<double>(NN);
     double* Xi = ar.take<double>(NN);
     double* scratch = ar.take<double>(observables_scratch_bytes(n) / sizeof(double));
-    double* partial = N <= kSplitMaxDim ? ar.take<double>(gemm_f64_splitk_bytes() / sizeof(double)) : nullptr;
+    double* partial = N <= kSplitMaxDim ? ar.take<double>(gemm_f64_splitk_bytes(N) / sizeof(double)) : nullptr;
     if (!scratch || (N <= kSplitMaxDim && !partial)) return fail(TC_ERR_WORKSPACE, "evolve: workspace too small");
     const int stride = TC_OBS_STRIDE(n);
 

@@ -1,13 +1,12 @@
 // evolve_oz.cu -- the FP64-accurate tensor-core form of the step loop
 // rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12): both products on the BF16
-// tensor cores from exact integer slices (cgemm_oz.cu), rho and X kept in
-// FP64 planes (row stride Np = max(N, 128), zero padding).
+// tensor cores (cgemm_crt.cu; cgemm_oz.cu under TC_OZ_BITS=6), rho and X kept
+// in FP64 planes (row stride Np = max(N, 128), zero padding).  It serves
+// TC_FP64_OZAKI at every size and TC_FP64 from n = 7 on (f64_on_tensor_cores).
 //
-// Per step: slice rho, X = U rho^H (all tiles), slice X, rho' = U X^H
-// (block-lower tiles, then the mirrored upper half), observables from the
-// FP64 planes; U is sliced once per call.  U enters as it is (no increment
-// form): the slice products are exact, so there is no accumulation bias to
-// scale down.
+// Per step: the operand form of rho, X = U rho^H (all tiles), that of X,
+// rho' = U X^H = U rho U^H (block-lower tiles, the upper half mirrored),
+// observables from the FP64 planes; U's is made once per call.
 #include "cgemm_oz.cuh"
 #include "cgemm_tc.cuh"
 #include "graph.cuh"
@@ -112,9 +111,10 @@ tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, d
     renorm_every = renorm_every_;
     const size_t NN = (size_t)Np * Np;
     TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs));
-    split_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(reinterpret_cast<const double2*>(rho), N, Np, Rr, Ri);
+    const double2* src = reinterpret_cast<const double2*>(rho);
+    split_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(src, N, Np, Rr, Ri);
     TC_LAUNCH_CHECK();
-    if (obs) TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs, scratch, cs, (size_t)Np));
+    if (obs) TC_TRY(launch_observables(kRhoInterleaved, rho, nullptr, m, n, obs, scratch, cs));
     return TC_OK;
 }
 
@@ -150,14 +150,28 @@ tc_status OzSystem::tail(double* rho, cudaStream_t cs) {
     return TC_OK;
 }
 
+// TC_FP64 takes the products of this file from n = 7 on: below, the padding to
+// 128 costs more than the DMMA product (n = 6: 64^3).  At n = 15 its operands
+// take 195 GB of workspace, which would not leave room for what a caller could
+// hold beside the DMMA form's 52 GB (n = 14: 50 GB, DMMA 26 GB).  Its error against 64
+// bits is no larger than the DMMA sums' (rows held to at least 51 bits of
+// their largest entry in a common scale, sums exact; the DMMA form rounds
+// each of N additions), its rate 4 times the DMMA form's at n = 8, 48 times at
+// n = 10, 92 times at n = 12.  TC_OZ_BITS=6 (the less accurate digit form) keeps
+// TC_FP64 on the DMMA.
+bool f64_on_tensor_cores(int n) { return n >= 7 && n <= 14 && oz_modular(); }
+
 tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m, double* obs,
                     Arena& ar, cudaStream_t s) {
     OzSystem z;
     TC_TRY(z.carve(n, ar));
+    if (steps == 0) {   // rho stays as it is
+        if (obs) TC_TRY(launch_observables(kRhoInterleaved, rho, nullptr, m, n, obs, z.scratch, s));
+        return TC_OK;
+    }
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(z.first(U, rho, m, obs, renorm_every, cs));
-        if (steps >= 1) TC_TRY(z.step(1, cs));
-        return TC_OK;
+        return z.step(1, cs);
     };
     auto rest = [&](cudaStream_t cs) -> tc_status {
         for (int k = 2; k <= steps; k++) TC_TRY(z.step(k, cs));

@@ -284,8 +284,8 @@ tc_status launch_bt(const GemmF64& g, cudaStream_t s) {
 
 int gemm_f64_default_tile(int N) { return N >= 4096 ? 64 : 32; }
 
-size_t gemm_f64_splitk_bytes() {
-    return round256(2 * (size_t)kMaxSplit * kSplitMaxDim * kSplitMaxDim * sizeof(double));
+size_t gemm_f64_splitk_bytes(int dim) {
+    return round256(2 * (size_t)kMaxSplit * dim * dim * sizeof(double));
 }
 
 tc_status gemm_f64(const GemmF64& g, cudaStream_t s) {

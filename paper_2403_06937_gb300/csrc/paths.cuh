@@ -30,13 +30,16 @@ tc_status expm_model_impl(const Model& m, double dt, const tc_expm_opts* opts, d
                           cudaStream_t s, int* used_degree, int* used_squarings);
 
 // FP64 step loop (DMMA products).
+size_t evolve_f64_bytes(int n);
 tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m,
                      double* obs, Arena& ar, cudaStream_t s);
 
-// FP64-accurate step loop on the BF16 tensor cores (exact integer slices).
+// FP64-accurate step loop on the BF16 tensor cores (exact integer products).
 size_t evolve_oz_bytes(int n);
 tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m, double* obs,
                     Arena& ar, cudaStream_t s);
+// True when TC_FP64 runs on those products for n atoms, given a workspace of their size.
+bool f64_on_tensor_cores(int n);
 
 // Low-precision step loop (tcgen05 products).
 size_t evolve_lowp_bytes(int n, int precision);
