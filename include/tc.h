@@ -195,8 +195,12 @@ TC_API tc_status tc_build_hamiltonian(const tc_params* params, double* H, void* 
  *  opts : NULL = automatic plan; {10, 0, 0} reproduces Eq. 10 (k_max = 10,
  *         no scaling, no shift).
  *  work : device, >= tc_workspace_size(n, TC_FP64, TC_OP_EXPM, 0, 0) bytes.
+ *         With the size that tc_workspace_size states the products run on the
+ *         tensor cores at FP64 accuracy for 8 <= n <= 14 (as TC_FP64, see
+ *         tc_precision); in 13 N^2 doubles and 2 N + 4 (plus padding to 256
+ *         bytes each) on the FP64 DMMA.
  *  The plan is made on the host from Tr H and ||H - mu I||_1, read back from
- *  the device: this call synchronises `stream` (twice with the shift).
+ *  the device: this call synchronises `stream` once.
  *  Errors: TC_ERR_INVALID_ARG (dt not finite or <= 0, bad opts),
  *          TC_ERR_WORKSPACE (short/misaligned work). */
 TC_API tc_status tc_expm(const double* H, int n, double dt, const tc_expm_opts* opts,

@@ -456,9 +456,8 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     double* Hs = b.B;   // build H into B, then shift and scale in place
     TC_TRY(launch_build_h(m, Hs, s));
     double trace = 0.0, norm1 = 0.0;
-    TC_TRY(matrix_trace_and_norm1(N, Hs, 0.0, &trace, &norm1, b.small + 8, s));
+    TC_TRY(matrix_trace_and_norm1(N, Hs, true, &trace, &norm1, b.small + 8, s));
     const double mu = trace / N;
-    TC_TRY(matrix_trace_and_norm1(N, Hs, mu, &trace, &norm1, b.small + 8, s));
     double bn = norm1 * dt;
     int sq = 0;
     while (bn > 0.5 && sq < 40) { bn *= 0.5; sq++; }

@@ -7,6 +7,7 @@
 #include <string>
 
 #include "kernels.cuh"
+#include "cgemm_oz.cuh"
 #include "cgemm_tc.cuh"
 #include "paths.cuh"
 
@@ -90,6 +91,17 @@ size_t expm_bytes(int n) {
     size_t N = (size_t)1 << n;
     return 13 * mat_bytes(n, 8) + round256((2 * N + 4) * sizeof(double));
 }
+
+// The polynomial's real products on the tensor cores: from n = 8 on, where the
+// 256 x 256 tiles begin (the call at n = 8: 0.20 ms, 0.43 ms on the DMMA; n = 9:
+// 0.24 / 1.29; n = 11: 1.55 / 62.9); up to n = 14, where their operands add
+// 20 GB to the 28 GB of scratch matrices.  TC_OZ_BITS=6 keeps the DMMA.
+bool expm_on_tensor_cores(int n) { return n >= 8 && n <= 14 && oz_modular(); }
+size_t expm_tensor_bytes(int n) {
+    const int N = 1 << n;
+    return crt_real_mat_bytes(N, true) + crt_real_mat_bytes(N, false) + crt_real_scratch_bytes(N);
+}
+size_t wanted_expm_bytes(int n) { return expm_bytes(n) + (expm_on_tensor_cores(n) ? expm_tensor_bytes(n) : 0); }
 
 // The least a call needs.  TC_FP64 runs its DMMA form in this much and the
 // tensor-core form in what tc_workspace_size states (wanted_evolve_bytes).
@@ -189,7 +201,22 @@ struct ExpmBufs {
     double* small;
 };
 
-tc_status gemm_real(int N, const double* A, const double* B, double* C, cudaStream_t s) {
+// C = A B of the real symmetric matrices of the polynomial.  On the tensor cores
+// (cgemm_crt.cu: A B^T, and B is symmetric) or on the DMMA GEMM.
+struct RealMul {
+    bool tensor = false;
+    CrtMat left{}, right{};
+    void* scratch = nullptr;
+    const double* loaded = nullptr;   // source of `left`, while it stays as it was
+};
+
+tc_status gemm_real(RealMul& rm, int N, const double* A, const double* B, double* C, cudaStream_t s) {
+    if (rm.tensor) {
+        if (rm.loaded != A) TC_TRY(crt_real_load(rm.left, A, s));
+        rm.loaded = A;
+        TC_TRY(crt_real_load(rm.right, B, s));
+        return crt_real_product(rm.left, rm.right, B, C, rm.scratch, s);
+    }
     GemmF64 g{};
     g.M = g.N = g.K = N;
     g.Ar = A; g.lda = N;
@@ -201,7 +228,7 @@ tc_status gemm_real(int N, const double* A, const double* B, double* C, cudaStre
 }
 
 // out = p(Y) = sum_{j<=d} a[j] Y^j with Y^1..Y^q in Y[1..q]; q >= 1.
-tc_status eval_poly(int N, const double* a, int d, int q, double* const* Y, double* out, double* tmp,
+tc_status eval_poly(RealMul& rm, int N, const double* a, int d, int q, double* const* Y, double* out, double* tmp,
                     cudaStream_t s) {
     if (d <= q) {
         const double* mats[4];
@@ -231,7 +258,7 @@ tc_status eval_poly(int N, const double* a, int d, int q, double* const* Y, doub
     }
     // ... then T = Y^q T + P_b for b = b-1 .. 0
     for (int k = b - 1; k >= 0; k--) {
-        TC_TRY(gemm_real(N, Y[q], out, tmp, s));
+        TC_TRY(gemm_real(rm, N, Y[q], out, tmp, s));
         const double* mats[4];
         double coef[4];
         int t = 0;
@@ -267,15 +294,20 @@ tc_status expm_impl(const double* H, int n, double dt, const tc_expm_opts* opts,
     b.CS = ar.take<double>((size_t)N * N);
     b.small = ar.take<double>(2 * (size_t)N + 4);
     if (!b.small) return fail(TC_ERR_WORKSPACE, "expm: workspace too small");
+    RealMul rm;
+    rm.tensor = expm_on_tensor_cores(n) && ar.size - ar.used >= expm_tensor_bytes(n);
+    if (rm.tensor) {
+        TC_TRY(crt_real_mat_init(rm.left, ar, N, true));
+        TC_TRY(crt_real_mat_init(rm.right, ar, N, false));
+        rm.scratch = ar.take<uint8_t>(crt_real_scratch_bytes(N));
+        if (!rm.scratch) return fail(TC_ERR_WORKSPACE, "expm: workspace too small");
+    }
 
     int shift = opts ? opts->shift : 1;
     double trace = 0.0, norm1 = 0.0, mu = 0.0;
-    TC_TRY(matrix_trace_and_norm1(N, H, 0.0, &trace, &norm1, b.small, s));
+    TC_TRY(matrix_trace_and_norm1(N, H, shift != 0, &trace, &norm1, b.small, s));
     if (!std::isfinite(trace) || !std::isfinite(norm1)) return fail(TC_ERR_NUMERIC, "expm: H is not finite");
-    if (shift) {
-        mu = trace / N;
-        TC_TRY(matrix_trace_and_norm1(N, H, mu, &trace, &norm1, b.small, s));
-    }
+    if (shift) mu = trace / N;
     Plan plan;
     if (opts && opts->taylor_degree > 0) {
         plan = cost_of_degree(opts->taylor_degree);
@@ -317,12 +349,12 @@ tc_status expm_impl(const double* H, int n, double dt, const tc_expm_opts* opts,
         double c1[1] = {1.0};
         TC_TRY(launch_lincomb(N, 0.0, 1, one, c1, b.S, s));
     } else {
-        TC_TRY(gemm_real(N, b.B, b.B, b.Y[1], s));
-        for (int j = 2; j <= q; j++) TC_TRY(gemm_real(N, b.Y[j - 1], b.Y[1], b.Y[j], s));
-        TC_TRY(eval_poly(N, cc, dc, q, b.Y, b.C, b.tmp, s));
+        TC_TRY(gemm_real(rm, N, b.B, b.B, b.Y[1], s));
+        for (int j = 2; j <= q; j++) TC_TRY(gemm_real(rm, N, b.Y[j - 1], b.Y[1], b.Y[j], s));
+        TC_TRY(eval_poly(rm, N, cc, dc, q, b.Y, b.C, b.tmp, s));
         if (ds >= 1) {
-            TC_TRY(eval_poly(N, sc, ds, q, b.Y, b.T, b.tmp, s));
-            TC_TRY(gemm_real(N, b.B, b.T, b.S, s));
+            TC_TRY(eval_poly(rm, N, sc, ds, q, b.Y, b.T, b.tmp, s));
+            TC_TRY(gemm_real(rm, N, b.B, b.T, b.S, s));
         } else {
             const double* one[1] = {b.B};
             double c1[1] = {1.0};
@@ -333,9 +365,10 @@ tc_status expm_impl(const double* H, int n, double dt, const tc_expm_opts* opts,
     double* C = b.C;
     double* S = b.S;
     for (int k = 0; k < sq; k++) {
-        TC_TRY(gemm_real(N, C, C, b.C2, s));
-        TC_TRY(gemm_real(N, S, S, b.S2, s));
-        TC_TRY(gemm_real(N, C, S, b.CS, s));
+        rm.loaded = nullptr;   // C and S are rewritten
+        TC_TRY(gemm_real(rm, N, C, C, b.C2, s));
+        TC_TRY(gemm_real(rm, N, S, S, b.S2, s));
+        TC_TRY(gemm_real(rm, N, C, S, b.CS, s));
         const double* m2[2] = {b.C2, b.S2};
         double c2[2] = {1.0, -1.0};
         TC_TRY(launch_lincomb(N, 0.0, 2, m2, c2, C, s));
@@ -366,7 +399,7 @@ TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ck
     if (n < 1 || n > kMaxAtoms) return 0;
     size_t need = 0;
     auto upd = [&](size_t b) { if (b > need) need = b; };
-    if (ops & TC_OP_EXPM) upd(expm_bytes(n));
+    if (ops & TC_OP_EXPM) upd(wanted_expm_bytes(n));
     if (ops & TC_OP_EVOLVE) upd(wanted_evolve_bytes(n, precision));
     if (ops & TC_OP_OBSERVABLES) upd(observables_scratch_bytes(n));
     if (ops & TC_OP_EXPM_MODEL) upd(expm_model_bytes(n));

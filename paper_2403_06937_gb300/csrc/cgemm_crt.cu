@@ -409,6 +409,265 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
 }
 
+// ---------------------------------------------------------------- real products
+// C = A B^T of real operands (the Taylor polynomials of tc_expm): one residue
+// plane an operand and modulus.  A CTA pair computes a 256 x 256 tile (its
+// CTAs 128 rows each, B's 256 rows split between them): one pair MMA a K step,
+// 256 TMEM columns, so the accumulator is double-buffered and a chunk's
+// epilogue runs beside the next chunk's MMAs.  Per MMA a CTA loads 8 KB
+// instead of the complex product's 6; the imaginary planes it does not have
+// would have doubled the MMAs.
+constexpr int kRealStage = 2 * kTile;
+constexpr int kRealStages = kRing / kRealStage;
+
+// Adds one K chunk, modulo p: acc[c] holds column c (low half) and c + 64.
+__device__ __forceinline__ void add_chunk_real(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64]) {
+    constexpr float kMagic = 12582912.0f;
+#pragma unroll
+    for (int c = 0; c < 64; c += 16) {
+        float lo[16], hi[16];
+        tmem_ld16(tl + c, lo);
+        tmem_ld16(tl + 64 + c, hi);
+        tmem_wait_ld();
+#pragma unroll
+        for (int q = 0; q < 16; q++) {
+            const float ql = __fmaf_rn(lo[q], inv_p, kMagic) - kMagic;
+            const float qh = __fmaf_rn(hi[q], inv_p, kMagic) - kMagic;
+            const float l = __fmaf_rn(-ql, p, lo[q]), h = __fmaf_rn(-qh, p, hi[q]);
+            const uint32_t bl = __float_as_uint(__fadd_rn(l, kMagic)), bh = __float_as_uint(__fadd_rn(h, kMagic));
+            acc[c + q] += bl - 0x4B400000u + (bh << 16);
+        }
+    }
+}
+
+__device__ __forceinline__ void real_unit(const CrtLaunch& L, int u, int& s, int& P, int& J) {
+    s = u / L.units_per;
+    const int t = u - s * L.units_per, side = L.tiles / 2;   // tiles of 256 a side
+    const int per_group = kGroup * side, g = t / per_group, in = t % per_group;
+    const int rows = min(kGroup, side - g * kGroup);
+    P = g * kGroup + in % rows;
+    J = in / rows;
+}
+
+__global__ void __launch_bounds__(kThreads, 1)
+    cgemm_crt_real_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
+    constexpr uint32_t kIdesc = make_idesc(1u, 256u, 256u);
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
+    uint64_t* empty = full + kRealStages;
+    uint64_t* accum = empty + kRealStages;   // [2] MMA -> epilogue, one per buffer
+    uint64_t* tmem_empty = accum + 2;        // [2] both epilogues -> MMA (even CTA, count 2)
+    uint64_t* drain = tmem_empty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint64_t lim = kWaitLimitNs;
+    const uint32_t rank = cluster_ctarank();
+    const int worker = (int)(blockIdx.x >> 1), workers = (int)(gridDim.x >> 1);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < kRealStages; s++) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; b++) {
+            mbar_init(&accum[b], 1);
+            mbar_init(&tmem_empty[b], 2);
+        }
+        mbar_init(drain, 1);
+        *abort = 0;
+        fence_mbar_init();
+    }
+    if (warp == 0) {
+        tmem_alloc_pair(saddr(tmem_slot), 512);
+        tmem_relinquish_pair();
+    }
+    if (warp == 8 && lane == 0) {
+        prefetch_tmap(&tmA);
+        prefetch_tmap(&tmB);
+    }
+    __syncthreads();
+    cluster_sync();   // both CTAs' barriers exist before either arrives on the other's
+    tc_fence_after();
+    const uint32_t tmem = *tmem_slot;
+    const uint32_t peer_abort = cluster_addr(saddr(const_cast<int*>(abort)), rank ^ 1u);
+    const int chunks = (L.kb_total + kChunkStages - 1) / kChunkStages;
+
+    if (warp == 8) {
+        // ---------------------------------------------------------- producer (both CTAs)
+        if (lane == 0) {
+            const uint32_t lead_full = cluster_addr(saddr(&full[0]), 0u);
+            uint32_t it = 0;
+            bool ok = true;
+            for (int u = worker; u < L.units && ok; u += workers) {
+                int s, P, J;
+                real_unit(L, u, s, P, J);
+                const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * 128;
+                for (int kb = 0; kb < L.kb_total; kb++, it++) {
+                    const int b = it % kRealStages;
+                    const uint32_t ph = (it / kRealStages) & 1u;
+                    if (!mbar_wait_bounded(&empty[b], ph ^ 1u, abort, lim, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    uint8_t* st = smem + b * kRealStage;
+                    const int kx = kb * kKPer;
+                    if (rank == 0) {
+                        mbar_arrive_expect_tx(&full[b], 2 * kRealStage);   // both CTAs' bytes
+                        tma_load_3d(saddr(st), &tmA, saddr(&full[b]), kx, ra, s);
+                        tma_load_3d(saddr(st + kTile), &tmB, saddr(&full[b]), kx, rb, s);
+                    } else {
+                        const uint32_t fb = lead_full + 8u * (uint32_t)b;
+                        tma_load_3d_pair(saddr(st), &tmA, fb, kx, ra, s);
+                        tma_load_3d_pair(saddr(st + kTile), &tmB, fb, kx, rb, s);
+                    }
+                }
+            }
+            const uint32_t from = it > (uint32_t)kRealStages ? it - kRealStages : 0u;
+            if (!ok || *abort) {
+                *abort = 1;
+                st_cluster_u32(peer_abort, 1u);
+                // the copies in flight land before the CTAs go away
+                if (rank == 0) {
+                    for (uint32_t k = from; k < it; k++)
+                        (void)mbar_wait_bounded(&full[k % kRealStages], (k / kRealStages) & 1u, nullptr, 10000000ull, 0);
+                } else {
+                    spin_ns(1000000ull);
+                }
+            } else {
+                // the last releases of this CTA's stages have arrived
+                for (uint32_t k = from; k < it; k++)
+                    (void)mbar_wait_bounded(&empty[k % kRealStages], (k / kRealStages) & 1u, abort, lim, 0);
+            }
+        }
+    } else if (warp == 9) {
+        if (lane == 0 && rank == 0) {
+            // ------------------------------------------------------ MMA issuer (even CTA)
+            const uint32_t peer_empty = cluster_addr(saddr(&empty[0]), 1u);
+            const uint32_t peer_accum = cluster_addr(saddr(&accum[0]), 1u);
+            uint32_t it = 0, pass = 0;
+            bool ok = true;
+            for (int u = worker; u < L.units && ok; u += workers) {
+                for (int c = 0; c < chunks && ok; c++, pass++) {
+                    const uint32_t buf = pass & 1u;
+                    if (pass >= 2 && !mbar_wait_bounded_cluster(&tmem_empty[buf], ((pass >> 1) - 1) & 1u, abort, lim, 0)) {
+                        ok = false;
+                        break;
+                    }
+                    tc_fence_after();
+                    const int kb0 = c * kChunkStages;
+                    const int kb1 = kb0 + kChunkStages < L.kb_total ? kb0 + kChunkStages : L.kb_total;
+                    for (int kb = kb0; kb < kb1; kb++, it++) {
+                        const int b = it % kRealStages;
+                        const uint32_t ph = (it / kRealStages) & 1u;
+                        if (!mbar_wait_bounded_cluster(&full[b], ph, abort, lim, 0)) {
+                            ok = false;
+                            break;
+                        }
+                        tc_fence_after();
+                        uint8_t* st = smem + b * kRealStage;
+                        const uint64_t ad = desc_kmajor<kRB>(saddr(st));
+                        const uint64_t bd = desc_kmajor<kRB>(saddr(st + kTile));
+#pragma unroll
+                        for (int ks = 0; ks < kSteps; ks++)   // 32 bytes of K further in each row
+                            umma_pair(tmem + 256u * buf, ad + 2u * (uint64_t)ks, bd + 2u * (uint64_t)ks, kIdesc,
+                                      (kb > kb0 || ks > 0) ? 1u : 0u);
+                        umma_commit_pair(saddr(&empty[b]));
+                        umma_commit_pair(peer_empty + 8u * (uint32_t)b);
+                    }
+                    if (!ok) break;
+                    umma_commit_pair(saddr(&accum[buf]));
+                    umma_commit_pair(peer_accum + 8u * buf);
+                }
+            }
+            // the MMAs complete before either CTA frees TMEM
+            umma_commit_pair(saddr(drain));
+            (void)mbar_wait_bounded(drain, 0u, nullptr, lim, 0);
+            if (*abort) st_cluster_u32(peer_abort, 1u);
+        }
+    } else {
+        // ---------------------------------------------------------- epilogue (both CTAs, own rows)
+        const uint32_t lead_tmem_empty = cluster_addr(saddr(&tmem_empty[0]), 0u);
+        const int half = warp >> 2;
+        const int row = (warp & 3) * 32 + lane;
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * (uint32_t)half;
+        uint32_t pass = 0;
+        bool stop = false;
+        for (int u = worker; u < L.units && !stop; u += workers) {
+            int s, P, J;
+            real_unit(L, u, s, P, J);
+            const float p = (float)kC.p[s], inv_p = 1.0f / p;
+            uint32_t acc[64];
+#pragma unroll
+            for (int c = 0; c < 64; c++) acc[c] = 0u;
+            for (int c = 0; c < chunks; c++, pass++) {
+                const uint32_t buf = pass & 1u;
+                const bool ok = mbar_wait_bounded_cluster(&accum[buf], (pass >> 1) & 1u, abort, lim, 32);
+                tc_fence_after();
+                // the epilogue warps leave together or not at all
+                uint32_t bad = (!ok || *abort) ? 1u : 0u, any;
+                asm volatile(
+                    "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+                    "bar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
+                    : "=r"(any)
+                    : "r"(bad)
+                    : "memory");
+                if (any) {
+                    if (threadIdx.x == 0) {
+                        *abort = 1;
+                        st_cluster_u32(peer_abort, 1u);
+                    }
+                    stop = true;
+                    break;
+                }
+                add_chunk_real(tl + 256u * buf, p, inv_p, acc);
+                tc_fence_before();
+                asm volatile("bar.sync 1, 256;" ::: "memory");   // every epilogue warp has read this buffer
+                if (threadIdx.x == 0) {
+                    if (rank == 0)
+                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&tmem_empty[buf])) : "memory");
+                    else
+                        mbar_arrive_cluster(lead_tmem_empty + 8u * buf);
+                }
+            }
+            if (stop) continue;
+            uint8_t* y = L.bytes + ((size_t)s * L.Np + (size_t)(2 * P + (int)rank) * 128 + row) * L.Np +
+                         (size_t)J * 256 + 128 * half;
+#pragma unroll
+            for (int c = 0; c < 64; c += 16) {
+                uint32_t wl[4], wh[4];
+#pragma unroll
+                for (int w = 0; w < 4; w++) {
+                    wl[w] = 0u;
+                    wh[w] = 0u;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const uint32_t v = acc[c + 4 * w + q];
+                        const int l = (int)(short)(v & 0xFFFFu);
+                        const int h = (int)(v - (uint32_t)l) >> 16;
+                        wl[w] |= to_byte(l, p, inv_p) << (8 * q);
+                        wh[w] |= to_byte(h, p, inv_p) << (8 * q);
+                    }
+                }
+                *reinterpret_cast<uint4*>(y + c) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
+                *reinterpret_cast<uint4*>(y + 64 + c) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
+            }
+        }
+        if (*abort && threadIdx.x == 0) atomicOr(L.status, kStatusTimeout);
+    }
+
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();   // neither CTA frees TMEM or leaves while the other may still use it
+    if (warp == 0) {
+        tc_fence_after();
+        tmem_dealloc_pair(tmem, 512);
+    }
+}
+
 // ---------------------------------------------------------------- residues
 // Row scale and residue planes of one operand.  A row is handled by TPR
 // consecutive threads of a 128-thread block (CPT columns a thread and step; 2
@@ -446,7 +705,7 @@ __device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits) {
     a.ss = fmaf(f, f, a.ss);
 }
 
-template <bool INTERLEAVED, bool LEFT, int CPT>
+template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false>
 __global__ void __launch_bounds__(128)
     crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
                        int tpr, uint64_t im_flip, __nv_bfloat16* __restrict__ planes, int* __restrict__ ex,
@@ -471,18 +730,20 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
                 for (int q = 0; q < CPT; q += 2) {
                     const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(pr + q);
-                    const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(pi + q);
                     xr[q] = a.x;
                     xr[q + 1] = a.y;
-                    xi[q] = b.x;
-                    xi[q + 1] = b.y;
+                    if (!REAL) {
+                        const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(pi + q);
+                        xi[q] = b.x;
+                        xi[q + 1] = b.y;
+                    }
                 }
             } else {
 #pragma unroll
                 for (int q = 0; q < CPT; q++) {
                     const bool in = r < N && c0 + q < N;
                     xr[q] = in ? (uint64_t)__double_as_longlong(pr[q]) : 0;
-                    xi[q] = in ? (uint64_t)__double_as_longlong(pi[q]) : 0;
+                    if (!REAL) xi[q] = in ? (uint64_t)__double_as_longlong(pi[q]) : 0;
                 }
             }
         }
@@ -502,7 +763,7 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
         for (int q = 0; q < CPT; q++) {
             stat_add(st, xr[q]);
-            stat_add(st, xi[q]);
+            if (!REAL) stat_add(st, xi[q]);
         }
     }
     for (int o = min(tpr, 32) / 2; o > 0; o >>= 1) {
@@ -529,7 +790,7 @@ __global__ void __launch_bounds__(128)
             double dr = 0.0, di = 0.0;
             if (r < N) {
                 dr = INTERLEAVED ? re[2 * ((size_t)r * ld + r)] : re[(size_t)r * ld + r];
-                di = INTERLEAVED ? re[2 * ((size_t)r * ld + r) + 1] : im[(size_t)r * ld + r];
+                di = INTERLEAVED ? re[2 * ((size_t)r * ld + r) + 1] : (REAL ? 0.0 : im[(size_t)r * ld + r]);
                 if (im_flip) di = -di;
             }
             diag[r] = dr;
@@ -541,12 +802,12 @@ __global__ void __launch_bounds__(128)
         uint64_t xr[CPT], xi[CPT];
         load(c0, xr, xi);
 #pragma unroll
-        for (int part = 0; part < 2; part++) {
+        for (int part = 0; part < (REAL ? 1 : 2); part++) {
             crt::Pieces pc[CPT];
             uint32_t sign[CPT / 2];
 #pragma unroll
             for (int q = 0; q < CPT; q++) {
-                const uint64_t b = part ? xi[q] ^ im_flip : xr[q];
+                const uint64_t b = !REAL && part ? xi[q] ^ im_flip : xr[q];
                 pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0);
                 const uint32_t sg = (uint32_t)(b >> 63) << 15;
                 if (q & 1)
@@ -738,6 +999,40 @@ __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
     }
 }
 
+// The same for a real product: 32 x 32 tiles, C[i][j] += A_ii B_ji on top.
+__global__ void __launch_bounds__(256) crt_combine_real_kernel(CrtCombine p) {
+    __shared__ double sr[32][33];   // [column of the tile][row of the tile]
+    const int i0 = 32 * (int)blockIdx.y, j0 = 32 * (int)blockIdx.x;
+    const int ti = threadIdx.x >> 3, tj = (threadIdx.x & 7) * 4;
+    const int i = i0 + ti, j = j0 + tj;
+    uint32_t w[kModuli];
+#pragma unroll
+    for (int s = 0; s < kModuli; s++)
+        w[s] = *reinterpret_cast<const uint32_t*>(p.bytes + ((size_t)s * p.Np + i) * p.Np + j);
+#pragma unroll
+    for (int k = 0; k < 4; k++) sr[ti][tj + k] = p.br[(size_t)(j0 + ti) * p.ldb + (size_t)(i0 + tj + k)];
+    const int ea = p.ea[i];
+    const double d = p.diag[i];
+    double v[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int eb = p.eb[j + k];
+        crt::Acc a = {};
+#pragma unroll
+        for (int s = 0; s < kModuli; s++) crt::acc_add(a, (w[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
+        bool neg;
+        int e;
+        const uint64_t mag = crt::acc_finish(a, kC, neg, e);
+        v[k] = ea == kNoScale || eb == kNoScale ? __longlong_as_double(0x7FF8000000000000ll) : scaled(mag, neg, e - ea - eb);
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < 4; k++) v[k] = fma(d, sr[tj + k][ti], v[k]);
+    double2* y = reinterpret_cast<double2*>(p.yr + (size_t)i * p.Np + j);
+    y[0] = make_double2(v[0], v[1]);
+    y[1] = make_double2(v[2], v[3]);
+}
+
 int sm_count() {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
@@ -745,9 +1040,10 @@ int sm_count() {
     return sms;
 }
 
-template <bool PAIR, int MODE>
+template <bool PAIR, int MODE, bool REAL = false>
 tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
-    auto k = cgemm_crt_kernel<PAIR, MODE>;
+    void (*k)(CUtensorMap, CUtensorMap, CrtLaunch) = cgemm_crt_kernel<PAIR, MODE>;
+    if constexpr (REAL) k = cgemm_crt_real_kernel;
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -884,6 +1180,64 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
             mode == 0 ? crt_combine_kernel<0, 4><<<grid, 256, 0, s>>>(c) : crt_combine_kernel<1, 4><<<grid, 256, 0, s>>>(c);
         TC_LAUNCH_CHECK();
     }
+    return TC_OK;
+}
+
+size_t crt_real_mat_bytes(int N, bool left) {
+    return round256((size_t)kModuli * N * N * 2) + round256((size_t)N * sizeof(int)) +
+           (left ? round256((size_t)2 * N * sizeof(double)) : 0);
+}
+
+size_t crt_real_scratch_bytes(int N) { return round256((size_t)kModuli * N * N); }
+
+tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) {
+    m.Np = N;
+    m.left = left;
+    m.planes = ar.take<uint8_t>((size_t)kModuli * N * N * 2);
+    m.ex = ar.take<int>((size_t)N);
+    m.diag = left ? ar.take<double>((size_t)2 * N) : nullptr;
+    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "real products: workspace too small");
+    return make_part_map_rows(&m.map, m.planes, N, kModuli, TC_BF16X3, kRB);
+}
+
+tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
+    if (reinterpret_cast<uintptr_t>(a) & 15u) return fail(TC_ERR_INVALID_ARG, "real products: operand misaligned");
+    const int N = m.Np, tpr = std::min(128, N / 8);   // N a power of two
+    const unsigned grid = (unsigned)(N / (128 / tpr));
+    auto* out = static_cast<__nv_bfloat16*>(m.planes);
+    if (m.left)
+        crt_residue_kernel<false, true, 8, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, m.diag);
+    else
+        crt_residue_kernel<false, false, 8, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, nullptr);
+    TC_LAUNCH_CHECK();
+    return TC_OK;
+}
+
+tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, double* c, void* scratch, cudaStream_t s) {
+    const int N = A.Np;
+    if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0)
+        return fail(TC_ERR_INVALID_ARG, "real products: operands of different sizes or roles");
+    CrtLaunch L{};
+    L.tiles = N / 128;
+    L.kb_total = N / kKPer;
+    L.Np = (size_t)N;
+    L.band = (size_t)N;
+    L.bytes = static_cast<uint8_t*>(scratch);
+    L.status = device_status_word();
+    L.units_per = (N / 256) * (N / 256);
+    L.units = L.units_per * kModuli;
+    TC_TRY((launch<true, 0, true>(A.map, B.map, L, s)));
+    CrtCombine p{};
+    p.bytes = L.bytes;
+    p.Np = (size_t)N;
+    p.ldb = (size_t)N;
+    p.ea = A.ex;
+    p.eb = B.ex;
+    p.diag = A.diag;
+    p.br = b;
+    p.yr = c;
+    crt_combine_real_kernel<<<dim3((unsigned)(N / 32), (unsigned)(N / 32)), 256, 0, s>>>(p);
+    TC_LAUNCH_CHECK();
     return TC_OK;
 }
 

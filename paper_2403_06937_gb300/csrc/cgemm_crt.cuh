@@ -44,4 +44,12 @@ struct CrtOut {
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
                       size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s);
 
+// Real operands (N x N, row stride N, N a power of two >= 256): fifteen planes
+// each; c = A B^T.  b: B's FP64 values (c must not overlap a or b).
+size_t crt_real_mat_bytes(int N, bool left);
+size_t crt_real_scratch_bytes(int N);
+tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left);
+tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s);
+tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, double* c, void* scratch, cudaStream_t s);
+
 }  // namespace tc

@@ -89,11 +89,27 @@ __global__ void expm_finish_kernel(const double* C, const double* S, double pr, 
     }
 }
 
-// per-row sum of |A_ij - mu delta_ij| (A symmetric: equals the column sum); one warp per row
-__global__ void row_abs_sum_kernel(const double* A, double mu, unsigned N, double* rows, double* diag) {
+// one block: trace[0] = sum of the diagonal in a fixed order
+__global__ void diag_sum_kernel(const double* A, unsigned N, double* trace) {
+    __shared__ double ssum[1024];
+    double sm = 0.0;
+    for (unsigned i = threadIdx.x; i < N; i += blockDim.x) sm += A[(size_t)i * N + i];
+    ssum[threadIdx.x] = sm;
+    __syncthreads();
+    for (unsigned w = blockDim.x / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) ssum[threadIdx.x] += ssum[threadIdx.x + w];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) trace[0] = ssum[0];
+}
+
+// per-row sum of |A_ij - mu delta_ij|, mu = trace[0] / N or 0 (A symmetric: equals the column sum); one
+// warp per row.  The shift is read on the device, so the host waits once for trace and norm together.
+__global__ void row_abs_sum_kernel(const double* A, const double* trace, int shift, unsigned N, double* rows) {
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const double mu = shift ? trace[0] / N : 0.0;
     for (unsigned r = warp; r < N; r += nwarps) {
         double acc = 0.0;
         const double* row = A + (size_t)r * N;
@@ -103,35 +119,22 @@ __global__ void row_abs_sum_kernel(const double* A, double mu, unsigned N, doubl
             acc += fabs(v);
         }
         for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) {
-            rows[r] = acc;
-            diag[r] = row[r];
-        }
+        if (lane == 0) rows[r] = acc;
     }
 }
 
-// one block: out[0] = max rows[], out[1] = sum diag[] in a fixed order
-__global__ void max_sum_kernel(const double* rows, const double* diag, unsigned N, double* out) {
-    __shared__ double smax[1024], ssum[1024];
-    double mx = 0.0, sm = 0.0;
-    for (unsigned i = threadIdx.x; i < N; i += blockDim.x) {
-        mx = fmax(mx, rows[i]);
-        sm += diag[i];
-    }
+// one block: out[0] = max rows[]
+__global__ void max_kernel(const double* rows, unsigned N, double* out) {
+    __shared__ double smax[1024];
+    double mx = 0.0;
+    for (unsigned i = threadIdx.x; i < N; i += blockDim.x) mx = fmax(mx, rows[i]);
     smax[threadIdx.x] = mx;
-    ssum[threadIdx.x] = sm;
     __syncthreads();
     for (unsigned w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) {
-            smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + w]);
-            ssum[threadIdx.x] += ssum[threadIdx.x + w];
-        }
+        if (threadIdx.x < w) smax[threadIdx.x] = fmax(smax[threadIdx.x], smax[threadIdx.x + w]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) {
-        out[0] = smax[0];
-        out[1] = ssum[0];
-    }
+    if (threadIdx.x == 0) out[0] = smax[0];
 }
 
 }  // namespace
@@ -212,14 +215,15 @@ tc_status launch_expm_finish(int N, const double* Cm, const double* Sm, double p
     return TC_OK;
 }
 
-tc_status matrix_trace_and_norm1(int N, const double* H, double mu_for_norm, double* trace,
-                                 double* norm1, double* scratch, cudaStream_t s) {
+tc_status matrix_trace_and_norm1(int N, const double* H, bool shift, double* trace, double* norm1, double* scratch,
+                                 cudaStream_t s) {
     double* rows = scratch;
-    double* diag = scratch + N;
-    double* out = scratch + 2 * (size_t)N;
-    row_abs_sum_kernel<<<grid_for((size_t)N * 32), 256, 0, s>>>(H, mu_for_norm, (unsigned)N, rows, diag);
+    double* out = scratch + 2 * (size_t)N;   // max, trace
+    diag_sum_kernel<<<1, 1024, 0, s>>>(H, (unsigned)N, out + 1);
     TC_LAUNCH_CHECK();
-    max_sum_kernel<<<1, 1024, 0, s>>>(rows, diag, (unsigned)N, out);
+    row_abs_sum_kernel<<<grid_for((size_t)N * 32), 256, 0, s>>>(H, out + 1, shift ? 1 : 0, (unsigned)N, rows);
+    TC_LAUNCH_CHECK();
+    max_kernel<<<1, 1024, 0, s>>>(rows, (unsigned)N, out);
     TC_LAUNCH_CHECK();
     double host[2];
     TC_CUDA(cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, s));

@@ -79,9 +79,10 @@ tc_status launch_expm_finish(int N, const double* Cm, const double* Sm, double p
                              double phase_im, double* U, cudaStream_t s);
 // B = (H - mu I) * dt  (real)
 tc_status launch_shift_scale(int N, const double* H, double mu, double dt, double* B, cudaStream_t s);
-// diag sum and max column abs sum of (H - mu I) on device -> host via stream sync
-tc_status matrix_trace_and_norm1(int N, const double* H, double mu_for_norm, double* trace,
-                                 double* norm1, double* scratch, cudaStream_t s);
+// trace = Tr H and norm1 = max column abs sum of H - mu I (mu = trace / N when
+// shift, else 0), read back with one stream synchronisation
+tc_status matrix_trace_and_norm1(int N, const double* H, bool shift, double* trace, double* norm1, double* scratch,
+                                 cudaStream_t s);
 
 // ---------------------------------------------------------------- observables
 // Deterministic observable row of a density matrix in one of three layouts.

@@ -138,3 +138,25 @@ def test_gradient_on_the_tensor_cores_with_squarings(tc, oracle):
                  ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
     ref = torch.tensor(list(ref), dtype=torch.float64)
     assert torch.max(torch.abs(grad - ref)).item() < 1e-11 * torch.max(torch.abs(ref)).item()
+
+
+@pytest.mark.parametrize("n,degree,squarings", [(8, 0, -1), (8, 6, 3), (9, 0, -1), (11, 12, 1)])
+def test_expm_on_the_tensor_cores_equals_the_dmma_form(tc, n, degree, squarings):
+    """One tile (n = 8), one and two K chunks; plans with and without squarings.  Every entry of the
+    polynomials is bounded by 1 (cos, sin of B), each product within 2 sqrt(K) 2^-58.35 of its rows'
+    norms (<= 1) plus roundings, the DMMA sums K 2^-53; at most 8 + 3 squarings products, doubled per
+    squaring."""
+    N = 1 << n
+    p = tc.Params(n, list(map(float, W.draw_couplings(n, 5) * 4)), 1.01, 1.0)
+    H = tc.build_hamiltonian(p)
+    a = tc.expm(H, n, 0.3, taylor_degree=degree, squarings=squarings)
+    b = torch.empty_like(a)
+    work = torch.empty(tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_EXPM) - 65536, dtype=torch.uint8, device="cuda")
+    opts = tc._abi.tc_expm_opts(degree, squarings, 1)
+    tc._abi.call("tc_expm", ctypes.c_void_p(H.data_ptr()), n, 0.3, ctypes.byref(opts), ctypes.c_void_p(b.data_ptr()),
+                 ctypes.c_void_p(work.data_ptr()), work.numel(),
+                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    one = 2 * np.sqrt(N) * 2.0 ** -58.35 + 4 * 2.0 ** -53 + N * 2.0 ** -53
+    assert torch.max(torch.abs(a - b)).item() < 2 ** max(squarings, 0) * (8 + 3 * max(squarings, 0)) * one
+    assert not torch.equal(a, b)
+    assert torch.equal(a, a.T)
