@@ -110,41 +110,125 @@ __device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int rank, int
     }
 }
 
-// Adds one K chunk of the tile, modulo p, to the packed sums acc[c]: the low
-// half holds Y_r, the high half Y_i of column 64 half + c (as one 32-bit sum
-// r + 65536 i).  At most 64 chunks of |r| <= p / 2 + 1 stay within 16 bits.
-__device__ __forceinline__ void add_chunk(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64]) {
-    constexpr float kMagic = 12582912.0f;   // 1.5 2^23: adding it rounds to an integer
+// Two FP32 numbers in one instruction (add, fma .f32x2).
+__device__ __forceinline__ uint64_t pack2(float a, float b) {
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, uint32_t& a, uint32_t& b) {
+    asm("mov.b64 {%0, %1}, %2;" : "=r"(a), "=r"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+    uint64_t r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// 32 lanes x 32 bits, eight consecutive columns a thread, in flight until
+// tmem_wait8 (whose operands keep every use behind the wait).
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait8(float (&a)[8], float (&b)[8]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(a[0]), "+f"(a[1]), "+f"(a[2]), "+f"(a[3]), "+f"(a[4]), "+f"(a[5]), "+f"(a[6]), "+f"(a[7]),
+                   "+f"(b[0]), "+f"(b[1]), "+f"(b[2]), "+f"(b[3]), "+f"(b[4]), "+f"(b[5]), "+f"(b[6]), "+f"(b[7])
+                 :
+                 : "memory");
+}
+
+constexpr float kMagic = 12582912.0f;   // 1.5 2^23: adding it rounds to an integer
+
+// y = (x + z) mod p for eight columns, as the bits of y + kMagic; sub: (x - z).
+// The quotient may come from the rounded sum; the remainder is exact:
+// |x - p q| <= |z| + p < 2^24.
+template <bool SUB>
+__device__ __forceinline__ void reduce8(const float (&x)[8], const float (&z)[8], uint64_t p2n, uint64_t inv2,
+                                        uint32_t (&out)[8]) {
+    const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic), one_n = pack2(-1.0f, -1.0f);
 #pragma unroll
-    for (int c = 0; c < 64; c += 16) {
-        float d1r[16], d1i[16], d2r[16], d2i[16];
-        tmem_ld16(tl + c, d1r);            // A_r B_r^T
-        tmem_ld16(tl + 128 + c, d1i);      // A_r B_i^T
-        tmem_ld16(tl + 256 + c, d2r);      // A_i B_r^T
-        tmem_ld16(tl + 384 + c, d2i);      // A_i B_i^T
-        tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < 16; q++) {
-            // the quotient may come from the rounded sum; the remainder is exact:
-            // |d1 - p q| <= |d2| + p < 2^24
-            const float qr = __fmaf_rn(__fadd_rn(d1r[q], d2i[q]), inv_p, kMagic) - kMagic;
-            const float qi = __fmaf_rn(__fsub_rn(d2r[q], d1i[q]), inv_p, kMagic) - kMagic;
-            const float yr = __fadd_rn(__fmaf_rn(-qr, p, d1r[q]), d2i[q]);
-            const float yi = __fsub_rn(__fmaf_rn(-qi, p, d2r[q]), d1i[q]);
-            const uint32_t br = __float_as_uint(__fadd_rn(yr, kMagic)), bi = __float_as_uint(__fadd_rn(yi, kMagic));
-            // both carry the magic's bits 0x4B400000; shifted by 16 they vanish modulo 2^32
-            acc[c + q] += br - 0x4B400000u + (bi << 16);
-        }
+    for (int q = 0; q < 8; q += 2) {
+        const uint64_t x2 = pack2(x[q], x[q + 1]), z2 = pack2(z[q], z[q + 1]);
+        const uint64_t s2 = SUB ? fma2(z2, one_n, x2) : add2(x2, z2);
+        const uint64_t q2 = add2(fma2(s2, inv2, m2), m2n);
+        const uint64_t t2 = fma2(q2, p2n, x2);
+        const uint64_t y2 = SUB ? fma2(z2, one_n, t2) : add2(t2, z2);
+        unpack2(add2(y2, m2), out[q], out[q + 1]);
     }
 }
 
-// sum of residues -> byte: balanced modulo p, plus 128
-__device__ __forceinline__ uint32_t to_byte(int v, float p, float inv_p) {
-    constexpr float kMagic = 12582912.0f;
+// Adds one K chunk of the tile, modulo p, to the packed sums acc[c]: the low
+// half holds Y_r, the high half Y_i of column c (as one 32-bit sum
+// r + 65536 i).  At most 64 chunks of |r| <= p / 2 + 1 stay within 16 bits.
+// The next eight columns are in flight while eight are reduced; `done` runs
+// once every load of the chunk has arrived (TMEM may be overwritten).
+// Bound by instruction issue: eight per complex entry (FP32 in pairs; one at a
+// time it was fourteen), two warps a scheduler.
+template <typename Done>
+__device__ __forceinline__ void add_chunk(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64], Done done) {
+    const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
+    float d1r[2][8], d1i[2][8], d2r[2][8], d2i[2][8];
+    auto load = [&](int c, int b) {
+        tmem_ld8(tl + c, d1r[b]);            // A_r B_r^T
+        tmem_ld8(tl + 128 + c, d1i[b]);      // A_r B_i^T
+        tmem_ld8(tl + 256 + c, d2r[b]);      // A_i B_r^T
+        tmem_ld8(tl + 384 + c, d2i[b]);      // A_i B_i^T
+    };
+    load(0, 0);
+#pragma unroll
+    for (int c = 0; c < 64; c += 8) {
+        const int b = (c >> 3) & 1;
+        tmem_wait8(d1r[b], d1i[b]);
+        tmem_wait8(d2r[b], d2i[b]);
+        if (c + 8 < 64)
+            load(c + 8, b ^ 1);
+        else
+            done();
+        uint32_t yr[8], yi[8];
+        reduce8<false>(d1r[b], d2i[b], p2n, inv2, yr);
+        reduce8<true>(d2r[b], d1i[b], p2n, inv2, yi);
+#pragma unroll
+        for (int q = 0; q < 8; q++)   // both carry the magic's bits 0x4B400000; shifted by 16 they vanish modulo 2^32
+            acc[c + q] += yr[q] - 0x4B400000u + (yi[q] << 16);
+    }
+}
+
+// sum of residues -> byte: times the inverse of M / p, balanced modulo p, plus 128
+__device__ __forceinline__ uint32_t to_byte(int v, float p, float inv_p, float inv) {
     const float f = __uint_as_float(0x4B400000u + (uint32_t)v) - kMagic;
-    const float q = __fmaf_rn(f, inv_p, kMagic) - kMagic;
-    const float r = __fmaf_rn(-q, p, f);
-    return (__float_as_uint(__fadd_rn(r, kMagic + 128.0f))) & 0xFFu;
+    return __float_as_uint(__fadd_rn(crt::times_inverse(f, inv, p, inv_p), kMagic + 128.0f)) & 0xFFu;
+}
+
+// Epilogue warps' wait for a chunk; false when the launch gives up (all lanes alike).
+template <bool PAIR>
+__device__ __forceinline__ bool chunk_ready(uint64_t* accum, uint32_t parity, volatile int* abort, uint64_t lim,
+                                            uint32_t peer_abort) {
+    const bool ok = mbar_wait_bounded_cluster(accum, parity, abort, lim, 0);
+    tc_fence_after();
+    if (!__any_sync(0xffffffffu, !ok || *abort)) return true;
+    *abort = 1;
+    if (PAIR) st_cluster_u32(peer_abort, 1u);
+    return false;
+}
+
+// One arrival a warp on tmem_empty of the MMA issuer's CTA, its loads complete.
+__device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_tmem_empty, uint32_t rank, int lane) {
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+        if (rank == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");
+        else
+            mbar_arrive_cluster(lead_tmem_empty);
+    }
 }
 
 template <bool PAIR, int MODE>
@@ -177,7 +261,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_init(&empty[s], 1);
         }
         mbar_init(accum, 1);
-        mbar_init(tmem_empty, PAIR ? 2 : 1);
+        mbar_init(tmem_empty, PAIR ? 16 : 8);   // one arrival per epilogue warp
         mbar_init(drain, 1);
         *abort = 0;
         fence_mbar_init();
@@ -333,7 +417,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = worker; u < L.units && !stop; u += workers) {
             int s, I, J;
             unit_at<PAIR, MODE>(L, u, (int)rank, s, I, J);
-            const float p = (float)kC.p[s], inv_p = 1.0f / p;
+            const float p = (float)kC.p[s], inv_p = 1.0f / p, inv = (float)kC.inv[s];
             // rows past an odd tile count, and the tile above the diagonal of a
             // Hermitian product, are not written
             const bool own = I < L.tiles && !(MODE == 1 && J > I);
@@ -341,33 +425,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
             for (int c = 0; c < 64; c++) acc[c] = 0u;
             for (int c = 0; c < chunks; c++, pass++) {
-                const bool ok = mbar_wait_bounded_cluster(accum, pass & 1u, abort, lim, 32);
-                tc_fence_after();
-                // the epilogue warps leave together or not at all
-                uint32_t bad = (!ok || *abort) ? 1u : 0u, any;
-                asm volatile(
-                    "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-                    "bar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
-                    : "=r"(any)
-                    : "r"(bad)
-                    : "memory");
-                if (any) {
-                    if (threadIdx.x == 0) {
-                        *abort = 1;
-                        if (PAIR) st_cluster_u32(peer_abort, 1u);
-                    }
+                if (!chunk_ready<PAIR>(accum, pass & 1u, abort, lim, peer_abort)) {
                     stop = true;
                     break;
                 }
-                add_chunk(tl, p, inv_p, acc);
-                tc_fence_before();
-                asm volatile("bar.sync 1, 256;" ::: "memory");   // every epilogue warp has read TMEM
-                if (threadIdx.x == 0) {
-                    if (rank == 0)
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");
-                    else
-                        mbar_arrive_cluster(lead_tmem_empty);
-                }
+                add_chunk(tl, p, inv_p, acc, [&]() { chunk_read(tmem_empty, lead_tmem_empty, rank, lane); });
             }
             if (stop || !own) continue;
             const size_t r0 = (size_t)I * 128 - (size_t)L.row0 * (PAIR ? 256 : 128) + row;   // row within the band
@@ -385,15 +447,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t v = acc[c + 4 * w + q];
                         const int r = (int)(short)(v & 0xFFFFu);
                         const int i = (int)(v - (uint32_t)r) >> 16;
-                        wr[w] |= to_byte(r, p, inv_p) << (8 * q);
-                        wi[w] |= to_byte(i, p, inv_p) << (8 * q);
+                        wr[w] |= to_byte(r, p, inv_p, inv) << (8 * q);
+                        wi[w] |= to_byte(i, p, inv_p, inv) << (8 * q);
                     }
                 }
                 *reinterpret_cast<uint4*>(yr + c) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
                 *reinterpret_cast<uint4*>(yi + c) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
             }
         }
-        if (*abort && threadIdx.x == 0) atomicOr(L.status, kStatusTimeout);
+        if (stop && lane == 0) atomicOr(L.status, kStatusTimeout);
     }
 
     __syncwarp();
@@ -421,22 +483,36 @@ constexpr int kRealStage = 2 * kTile;
 constexpr int kRealStages = kRing / kRealStage;
 
 // Adds one K chunk, modulo p: acc[c] holds column c (low half) and c + 64.
-__device__ __forceinline__ void add_chunk_real(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64]) {
-    constexpr float kMagic = 12582912.0f;
+template <typename Done>
+__device__ __forceinline__ void add_chunk_real(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64], Done done) {
+    const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
+    const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic);
+    auto reduce = [&](const float (&x)[8], uint32_t (&out)[8]) {
 #pragma unroll
-    for (int c = 0; c < 64; c += 16) {
-        float lo[16], hi[16];
-        tmem_ld16(tl + c, lo);
-        tmem_ld16(tl + 64 + c, hi);
-        tmem_wait_ld();
-#pragma unroll
-        for (int q = 0; q < 16; q++) {
-            const float ql = __fmaf_rn(lo[q], inv_p, kMagic) - kMagic;
-            const float qh = __fmaf_rn(hi[q], inv_p, kMagic) - kMagic;
-            const float l = __fmaf_rn(-ql, p, lo[q]), h = __fmaf_rn(-qh, p, hi[q]);
-            const uint32_t bl = __float_as_uint(__fadd_rn(l, kMagic)), bh = __float_as_uint(__fadd_rn(h, kMagic));
-            acc[c + q] += bl - 0x4B400000u + (bh << 16);
+        for (int q = 0; q < 8; q += 2) {
+            const uint64_t x2 = pack2(x[q], x[q + 1]);
+            const uint64_t q2 = add2(fma2(x2, inv2, m2), m2n);
+            unpack2(add2(fma2(q2, p2n, x2), m2), out[q], out[q + 1]);
         }
+    };
+    float lo[2][8], hi[2][8];
+    tmem_ld8(tl, lo[0]);
+    tmem_ld8(tl + 64, hi[0]);
+#pragma unroll
+    for (int c = 0; c < 64; c += 8) {
+        const int b = (c >> 3) & 1;
+        tmem_wait8(lo[b], hi[b]);
+        if (c + 8 < 64) {
+            tmem_ld8(tl + c + 8, lo[b ^ 1]);
+            tmem_ld8(tl + 64 + c + 8, hi[b ^ 1]);
+        } else {
+            done();
+        }
+        uint32_t l[8], h[8];
+        reduce(lo[b], l);
+        reduce(hi[b], h);
+#pragma unroll
+        for (int q = 0; q < 8; q++) acc[c + q] += l[q] - 0x4B400000u + (h[q] << 16);
     }
 }
 
@@ -474,7 +550,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         for (int b = 0; b < 2; b++) {
             mbar_init(&accum[b], 1);
-            mbar_init(&tmem_empty[b], 2);
+            mbar_init(&tmem_empty[b], 16);   // one arrival per epilogue warp of both CTAs
         }
         mbar_init(drain, 1);
         *abort = 0;
@@ -598,39 +674,18 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = worker; u < L.units && !stop; u += workers) {
             int s, P, J;
             real_unit(L, u, s, P, J);
-            const float p = (float)kC.p[s], inv_p = 1.0f / p;
+            const float p = (float)kC.p[s], inv_p = 1.0f / p, inv = (float)kC.inv[s];
             uint32_t acc[64];
 #pragma unroll
             for (int c = 0; c < 64; c++) acc[c] = 0u;
             for (int c = 0; c < chunks; c++, pass++) {
                 const uint32_t buf = pass & 1u;
-                const bool ok = mbar_wait_bounded_cluster(&accum[buf], (pass >> 1) & 1u, abort, lim, 32);
-                tc_fence_after();
-                // the epilogue warps leave together or not at all
-                uint32_t bad = (!ok || *abort) ? 1u : 0u, any;
-                asm volatile(
-                    "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\t"
-                    "bar.red.or.pred q, 1, 256, p;\n\tselp.u32 %0, 1, 0, q;\n}"
-                    : "=r"(any)
-                    : "r"(bad)
-                    : "memory");
-                if (any) {
-                    if (threadIdx.x == 0) {
-                        *abort = 1;
-                        st_cluster_u32(peer_abort, 1u);
-                    }
+                if (!chunk_ready<true>(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
                     stop = true;
                     break;
                 }
-                add_chunk_real(tl + 256u * buf, p, inv_p, acc);
-                tc_fence_before();
-                asm volatile("bar.sync 1, 256;" ::: "memory");   // every epilogue warp has read this buffer
-                if (threadIdx.x == 0) {
-                    if (rank == 0)
-                        asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(&tmem_empty[buf])) : "memory");
-                    else
-                        mbar_arrive_cluster(lead_tmem_empty + 8u * buf);
-                }
+                add_chunk_real(tl + 256u * buf, p, inv_p, acc,
+                               [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
             }
             if (stop) continue;
             uint8_t* y = L.bytes + ((size_t)s * L.Np + (size_t)(2 * P + (int)rank) * 128 + row) * L.Np +
@@ -647,15 +702,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t v = acc[c + 4 * w + q];
                         const int l = (int)(short)(v & 0xFFFFu);
                         const int h = (int)(v - (uint32_t)l) >> 16;
-                        wl[w] |= to_byte(l, p, inv_p) << (8 * q);
-                        wh[w] |= to_byte(h, p, inv_p) << (8 * q);
+                        wl[w] |= to_byte(l, p, inv_p, inv) << (8 * q);
+                        wh[w] |= to_byte(h, p, inv_p, inv) << (8 * q);
                     }
                 }
                 *reinterpret_cast<uint4*>(y + c) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
                 *reinterpret_cast<uint4*>(y + 64 + c) = make_uint4(wh[0], wh[1], wh[2], wh[3]);
             }
         }
-        if (*abort && threadIdx.x == 0) atomicOr(L.status, kStatusTimeout);
+        if (stop && lane == 0) atomicOr(L.status, kStatusTimeout);
     }
 
     __syncwarp();
@@ -804,16 +859,10 @@ __global__ void __launch_bounds__(128)
 #pragma unroll
         for (int part = 0; part < (REAL ? 1 : 2); part++) {
             crt::Pieces pc[CPT];
-            uint32_t sign[CPT / 2];
 #pragma unroll
             for (int q = 0; q < CPT; q++) {
                 const uint64_t b = !REAL && part ? xi[q] ^ im_flip : xr[q];
-                pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0);
-                const uint32_t sg = (uint32_t)(b >> 63) << 15;
-                if (q & 1)
-                    sign[q / 2] |= sg << 16;
-                else
-                    sign[q / 2] = sg;
+                pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
             }
             __nv_bfloat16* dst = planes + (size_t)(part * kModuli) * plane + (size_t)r * Np + c0;
 #pragma unroll
@@ -822,14 +871,9 @@ __global__ void __launch_bounds__(128)
                 uint32_t w[CPT / 2];
 #pragma unroll
                 for (int h = 0; h < CPT / 2; h++) {
-                    uint32_t b[2];
-#pragma unroll
-                    for (int k = 0; k < 2; k++) {
-                        const int v = LEFT ? crt::residue(pc[2 * h + k], p, kC.inv[s]) : crt::residue(pc[2 * h + k], p, 1);
-                        // exact conversion: |v| <= 127 through the 1.5 2^23 magic
-                        b[k] = __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)v) - 12582912.0f);
-                    }
-                    w[h] = __byte_perm(b[0], b[1], 0x7632) ^ sign[h];   // the top halves are the BF16 values
+                    // integers up to 127 are exact in BF16: the top halves of their FP32 bits
+                    w[h] = __byte_perm(__float_as_uint(crt::residue(pc[2 * h], p)),
+                                       __float_as_uint(crt::residue(pc[2 * h + 1], p)), 0x7632);
                 }
                 if constexpr (CPT == 8)
                     *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[0], w[1], w[2], w[3]);

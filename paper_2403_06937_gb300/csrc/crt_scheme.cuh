@@ -86,44 +86,59 @@ constexpr Consts make_consts() {
 }
 
 // ---------------------------------------------------------------- residues
-// A magnitude below 2^59 in three pieces of 20 bits; 2^20 and 2^40 mod p are
-// below 255, so lo + mid c1 + hi c2 < 2^29.
+// An integer below 2^59 in four pieces (20, 13, 13 and 13 bits) with its sign,
+// as FP32 numbers.  With the balanced remainders c_k (|c_k| <= 127) of 2^20,
+// 2^33 and 2^46, t = lo + a c_1 + b c_2 + c c_3 is an integer below 2^22, so
+// FP32 holds every step exactly, and so is t - q p.  The quotient
+// q = round(t / p) comes from the rounded reciprocal: its error t / p 2^-24 is
+// below half a unit in p, so the remainder is the balanced one, |r| <= 127.
+// (FP32 multiply-adds: twice the rate of integer ones here, and a third of
+// their number.)
 struct Pieces {
-    uint32_t lo, mid, hi;
+    float lo, a, b, c;
 };
-TC_CRT_HD Pieces split_pieces(uint64_t mag) {
-    Pieces q;
-    q.lo = (uint32_t)mag & 0xFFFFFu;
-    q.mid = (uint32_t)(mag >> 20) & 0xFFFFFu;
-    q.hi = (uint32_t)(mag >> 40);
-    return q;
-}
-TC_CRT_HD uint32_t mulhi_u32(uint32_t a, uint32_t b) {
+TC_CRT_HD float bits_to_float(uint32_t v) {
 #ifdef __CUDA_ARCH__
-    return __umulhi(a, b);
+    return __uint_as_float(v);
 #else
-    return (uint32_t)(((uint64_t)a * b) >> 32);
+    float f;
+    __builtin_memcpy(&f, &v, 4);
+    return f;
 #endif
 }
-// t mod p, balanced (|r| <= p / 2), for t < 2^29: the quotient
-// floor((t + p/2) / p) from the 37-bit reciprocal ceil(2^37 / p), whose error
-// (t + p/2) / 2^37 < 1/256 of a unit never reaches the next integer.
-TC_CRT_HD int balanced_mod(uint32_t t, int p) {
-    const uint32_t m = (uint32_t)(((1ull << 37) + (uint64_t)p - 1) / (uint64_t)p);
-    const uint32_t q = mulhi_u32(t + (uint32_t)(p / 2), m) >> 5;
-    return (int)t - (int)q * p;
+TC_CRT_HD float fma_f32(float a, float b, float c) {
+#ifdef __CUDA_ARCH__
+    return __fmaf_rn(a, b, c);
+#else
+    return __builtin_fmaf(a, b, c);
+#endif
 }
-// Residue of the magnitude, times inv when it is not 1 (operands of the left
-// role carry the inverse of the remainder theorem).
-TC_CRT_HD int residue(const Pieces& x, int p, int inv) {
-    const uint32_t c1 = (uint32_t)((1u << 20) % (uint32_t)p);
-    const uint32_t c2 = (uint32_t)((1ull << 40) % (uint64_t)p);
-    int r = balanced_mod(x.lo + x.mid * c1 + x.hi * c2, p);
-    if (inv != 1) {
-        const uint32_t u = (uint32_t)(r < 0 ? r + p : r);
-        r = balanced_mod(u * (uint32_t)inv, p);
-    }
-    return r;
+TC_CRT_HD Pieces split_pieces(uint64_t mag, bool neg) {
+    // v < 2^23 as FP32: 2^23 + v has v in its low bits; the sign rides along
+    const uint32_t base = neg ? 0xCB000000u : 0x4B000000u;
+    const float off = neg ? 8388608.0f : -8388608.0f;
+    Pieces q;
+    q.lo = bits_to_float(base | ((uint32_t)mag & 0xFFFFFu)) + off;
+    q.a = bits_to_float(base | ((uint32_t)(mag >> 20) & 0x1FFFu)) + off;
+    q.b = bits_to_float(base | ((uint32_t)(mag >> 33) & 0x1FFFu)) + off;
+    q.c = bits_to_float(base | (uint32_t)(mag >> 46)) + off;
+    return q;
+}
+TC_CRT_HD constexpr int balanced_pow2(int e, int p) {   // 2^e mod p, |.| <= p / 2
+    const int r = (int)((1ull << e) % (uint64_t)p);
+    return 2 * r > p ? r - p : r;
+}
+TC_CRT_HD float residue(const Pieces& x, int p) {
+    const float t = fma_f32(x.c, (float)balanced_pow2(46, p),
+                            fma_f32(x.b, (float)balanced_pow2(33, p), fma_f32(x.a, (float)balanced_pow2(20, p), x.lo)));
+    const float q = fma_f32(t, 1.0f / (float)p, 12582912.0f) - 12582912.0f;   // 1.5 2^23: rounds to an integer
+    return fma_f32(-q, (float)p, t);
+}
+// An integer below 2^24 / 254 (sum of residues) times inv, balanced modulo p
+TC_CRT_HD float times_inverse(float v, float inv, float p, float inv_p) {
+    const float f = v * inv;   // exact: below 2^24
+    const float q = fma_f32(f, inv_p, 12582912.0f) - 12582912.0f;
+    return fma_f32(-q, p, f);
 }
 
 // FP64 bits -> sign and integer magnitude round(|x| 2^sh); |x| 2^sh < 2^59.
@@ -141,7 +156,7 @@ TC_CRT_HD uint64_t to_magnitude(uint64_t bits, int sh) {
 
 // ---------------------------------------------------------------- recombination
 // x / M modulo 1 as a signed 96-bit fraction from the fifteen stored bytes
-// (residue times inverse, plus 128) -> x 2^e in FP64 (e split in two factors
+// (residue times the inverse of M / p, plus 128) -> x 2^e in FP64 (e split in two factors
 // by the caller when it is out of range).  The fraction's error is below
 // 2^-86, so x is within 2^32 units of integers whose rows are held to 2^58
 // (|x| < M / 2 - 2^33).

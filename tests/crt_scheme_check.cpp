@@ -32,35 +32,42 @@ int main() {
             if (x != 1) return fail("coprime", a, b);
         }
     }
-    // balanced_mod over its whole range: every boundary of a quotient, and random values
-    for (int s = 0; s < kModuli; s++) {
-        const int p = modulus(s);
-        auto check = [&](uint32_t t) {
-            const int r = balanced_mod(t, p);
-            return r >= -p / 2 && r <= p / 2 && ((long)t - r) % p == 0;
-        };
-        for (uint32_t q = 0; q < (1u << 29) / (uint32_t)p; q += 1 + (q > 4096 && q < (1u << 29) / (uint32_t)p - 4096 ? 61 : 0))
-            for (int d = -1; d <= 1; d++) {
-                const uint32_t t = q * (uint32_t)p + (uint32_t)(p / 2 + d);
-                if (t < (1u << 29) && !check(t)) return fail("balanced_mod", s, t);
-            }
-        for (int k = 0; k < 200000; k++) {
-            const uint32_t t = (uint32_t)(rng() & ((1u << 29) - 1));
-            if (!check(t)) return fail("balanced_mod", s, t);
+    // residues of integers up to 2^59 - 1: random sizes, both signs, the ends, and the neighbours of
+    // every kind of tie (odd multiples of p / 2 in the low piece, large pieces above)
+    auto check = [&](uint64_t m, bool neg) {
+        for (int s = 0; s < kModuli; s++) {
+            const int p = modulus(s);
+            const float f = residue(split_pieces(m, neg), p);
+            const int r = (int)f;
+            const i128 d = (neg ? -(i128)m : (i128)m) - r;
+            if ((float)r != f || std::abs(r) > p / 2 || d % p != 0) return s;
         }
-    }
-    // residues of magnitudes up to 2^59 - 1, plain and times the inverse
-    for (int k = 0; k < 100000; k++) {
+        return -1;
+    };
+    for (int k = 0; k < 1000000; k++) {
         uint64_t m = rng() >> (5 + rng() % 59);
         if (k == 0) m = (1ull << 59) - 1;
         if (k == 1) m = 0;
-        for (int s = 0; s < kModuli; s++) {
-            const int p = modulus(s);
-            for (int inv : {1, C.inv[s]}) {
-                const int r = residue(split_pieces(m), p, inv);
-                const i128 d = (i128)m * inv - r;
-                if (std::abs(r) > p / 2 || d % p != 0) return fail("residue", s, m);
-            }
+        if (k % 3 == 0) {   // a tie's neighbour: m = q p + p / 2 + {-1, 0, 1, 2}
+            const uint64_t p = (uint64_t)modulus((int)(rng() % kModuli));
+            m = m / p * p + p / 2 + rng() % 4 - 1;
+            if (m >> 59) m = 1;
+        }
+        const int s = check(m, (rng() & 1) != 0);
+        if (s >= 0) return fail("residue", s, m);
+    }
+    for (uint64_t m = 0; m < 70000; m++) {
+        const int s = check(m, (m & 1) != 0);
+        if (s >= 0) return fail("residue", s, m);
+    }
+    // sums of up to 64 chunks' residues times the inverse
+    for (int s = 0; s < kModuli; s++) {
+        const int p = modulus(s);
+        for (int v = -8300; v <= 8300; v++) {
+            const float f = times_inverse((float)v, (float)C.inv[s], (float)p, 1.0f / (float)p);
+            const int r = (int)f;
+            if ((float)r != f || std::abs(r) > p / 2 || ((long)v * C.inv[s] - r) % p != 0)
+                return fail("times_inverse", s, (unsigned long long)(v + 8300));
         }
     }
     // FP64 bits to integers: normal, subnormal, zero, both directions of the shift

@@ -151,7 +151,9 @@ def test_expm_on_the_tensor_cores_equals_the_dmma_form(tc, n, degree, squarings)
     H = tc.build_hamiltonian(p)
     a = tc.expm(H, n, 0.3, taylor_degree=degree, squarings=squarings)
     b = torch.empty_like(a)
-    work = torch.empty(tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_EXPM) - 65536, dtype=torch.uint8, device="cuda")
+    # one scratch matrix and a bit less than the tensor-core form needs
+    work = torch.empty(tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_EXPM) - 8 * N * N - 65536, dtype=torch.uint8,
+                       device="cuda")
     opts = tc._abi.tc_expm_opts(degree, squarings, 1)
     tc._abi.call("tc_expm", ctypes.c_void_p(H.data_ptr()), n, 0.3, ctypes.byref(opts), ctypes.c_void_p(b.data_ptr()),
                  ctypes.c_void_p(work.data_ptr()), work.numel(),
