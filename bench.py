@@ -320,21 +320,22 @@ def _compulsory_bytes(prec, N):
         return 3 * 16 * N * N
     if prec in ("fp64", "ozaki"):
         # BF16 residue (digit) planes of U and of P read, the FP64 result written
-        return (2 * 2 * (15 if oz_products() == 15 else 9) * 2 + 16) * N * N
+        return (2 * 2 * (16 if oz_products() == 8 else 9) * 2 + 16) * N * N
     parts, pbytes = {"bf16x3": (3, 2), "tf32": (1, 4), "tf32x3": (2, 4)}[prec]
     planes = 2 * parts * pbytes
     return (3 * planes + 8 + 8) * N * N
 
 
 def oz_products():
-    """BF16 products per complex product of the FP64-accurate form: fifteen
-    residue products, or the 45 digit pairs under TC_OZ_BITS=6."""
-    return 45 if os.environ.get("TC_OZ_BITS") == "6" else 15
+    """BF16 products per real product of the FP64-accurate form: 8 (a complex
+    product takes 32 real residue products, 2 for each of 16 moduli, where the
+    plain one takes 4), or the 45 digit pairs under TC_OZ_BITS=6."""
+    return 45 if os.environ.get("TC_OZ_BITS") == "6" else 8
 
 
 def fp64_on_tensor_cores(N):
     """TC_FP64 runs its products in the residue form for 7 <= n <= 14, on the DMMA elsewhere."""
-    return 1 << 7 <= N <= 1 << 14 and oz_products() == 15
+    return 1 << 7 <= N <= 1 << 14 and oz_products() == 8
 
 
 def _sample_entries(torch, rho, count=20000, top=48, seed=5):
@@ -786,7 +787,7 @@ def run_grad(a):
             "n_gpus": 1, "steps": cfg.steps, "warmup": 0, "ms_per_step": 1e3 * t / cfg.steps,
             "higher_is_better": False, "scaling": "weak", "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": cfg.description,
-                       "products": "FP64-accurate residue products on the BF16 tensor cores" if oz_products() == 15
+                       "products": "FP64-accurate residue products on the BF16 tensor cores" if oz_products() == 8
                        else ("FP64 DMMA" if gprec == "fp64" else "digit products on the BF16 tensor cores")},
             "loss": loss, "grad": grad.tolist(), "fp64_tflops": flops / t / 1e12}
     if not a.no_cpu:

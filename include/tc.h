@@ -81,9 +81,10 @@ typedef enum tc_status {
  *  TC_TF32X3 : big/small TF32 split, three products (kind::tf32).
  *  TC_FP64_OZAKI : FP64-accurate products on the BF16 tensor cores: every
  *              operand row is scaled by a power of two (its 2-norm just below
- *              2^58.4), rounded to integers and reduced modulo fifteen
- *              coprime p <= 255; one BF16 product per modulus, exact in FP32
- *              over K chunks of 1024, and the remainder theorem give the
+ *              2^58.3), rounded to integers and reduced modulo sixteen
+ *              coprime p <= 241 that have a square root of -1, so that a
+ *              complex product is two real BF16 products per modulus, exact
+ *              in FP32 over K chunks of 1024; the remainder theorem gives the
  *              exact integer product.  The left operand's diagonal is kept
  *              in FP64.  Within sqrt(2 K) 2^-56.3 of the product of the two
  *              rows' 2-norms, plus the rounding of the result; a row with an

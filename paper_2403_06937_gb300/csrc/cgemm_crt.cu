@@ -1,13 +1,14 @@
 // cgemm_crt.cu -- FP64-accurate complex GEMM Y = A B^H on the BF16 tensor
 // cores in a residue number system (the second Ozaki scheme: Ozaki, Uchino
-// and Imamura 2025), for the step rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12) at
+// and Imamura 2025; the complex product split in two as in number-theoretic
+// transforms), for the step rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12) at
 // FP64 accuracy.
 //
 // Integers.  Row r of an operand is scaled by 2^ex[r] so that the 2-norm of
-// its rounded entries stays below 2^58.36.  An entry of A B^H is an inner
+// its rounded entries stays below 2^58.32.  An entry of A B^H is an inner
 // product of two such rows, so by Cauchy-Schwarz its real and imaginary part
-// stay below M / 2 = 2^116.77 and are fixed by their residues modulo the
-// fifteen p_s (crt_scheme.cuh).  A row whose weight sits in a few entries is
+// stay below M / 2 = 2^116.69 and are fixed by their residues modulo the
+// sixteen p_s (crt_scheme.cuh).  A row whose weight sits in a few entries is
 // held to up to 58 bits of its largest entry, a flat row of K entries to
 // 58 - log2(K) / 2; FP64 holds 53.
 //
@@ -15,26 +16,33 @@
 // close to the identity, and Y = diag(U) B^H + V B^H with the first term in
 // FP64 leaves the integers the small part V only.
 //
-// Products.  For each p_s one BF16 product of the residue planes: A = the
-// rows of A_r and A_i (M = 128), B = the stack [B_r; B_i] (N = 256), two FP32
-// accumulators (512 TMEM columns).  A K chunk of 1024 is exact in FP32; the
-// epilogue reads it out, forms Y_r = A_r B_r^T + A_i B_i^T and Y_i = A_i B_r^T
-// - A_r B_i^T modulo p_s in FP32 (every intermediate an integer below 2^24)
-// and adds it to a packed pair of 16-bit sums in registers, which go out as
-// one byte each when all of K is done.  crt_combine_kernel turns the fifteen
-// bytes of an entry into FP64 (integer work up to one conversion) and adds the
-// diagonal term.
+// Products.  Modulo p_s a complex number is the pair a_r + iota a_i,
+// a_r - iota a_i (iota^2 = -1), and the pairs multiply componentwise, so each
+// modulus takes two real BF16 products: plane 0 of A with plane 0 of B, plane
+// 1 with plane 1 (B's pair is swapped for the conjugate).  32 real products of
+// N^3 multiply-adds in all; the digit slices (cgemm_oz.cu) take 180 (and 112
+// to 144 with the wider digits that small K allowed).
 //
-// Against the digit slices (cgemm_oz.cu: 28, 36 or 45 pair products, an int64
-// read-modify-write of the result after each): 15 products at every size, and
-// 15 bytes per result entry written once.
+// GEMM.  A CTA pair computes a 256 x 256 tile of one plane pair (its CTAs 128
+// rows each, B's 256 rows split between them; rows and columns past the end
+// read zeros and are not written): one M = 256, N = 256 pair MMA a K step into
+// 256 TMEM columns.  A K chunk of 1024 is exact in FP32; the epilogue reads it
+// out modulo p_s, in FP32 where every intermediate is an integer below 2^24,
+// and adds it to packed 16-bit sums in registers, which go out as one byte
+// each when all of K is done.  The accumulator is double-buffered (512
+// columns), so a chunk's epilogue runs beside the next chunk's MMAs; what
+// bounds the kernel is the operand traffic of 64 bytes per clock and SM (a
+// first version with the four products of a complex 128 x 128 tile a CTA, 512
+// columns and no overlap, had 47 and ran the tensor pipe 80 % busy at n = 12).
 //
-// Work unit: (modulus s, tile or tile pair), modulus outermost, so that the
-// units in flight share operand panels in L2; a persistent launch takes them
-// round-robin.  Roles of a CTA: warps 0-7 epilogue (warp w reads TMEM lanes
-// 32 (w % 4) .. + 31, columns 64 (w / 4) .. + 63 of the tile), warp 8 TMA,
-// warp 9 MMA.  Arrangement, barriers and bounded waits of the CTA pairs as
-// cgemm_oz_pair_kernel (cgemm_oz.cu).
+// Work unit: (plane, tile), plane outermost, so that the units in flight share
+// operand panels in L2; a persistent launch takes them round-robin.  Roles of
+// a CTA: warps 0-7 epilogue (warp w reads TMEM lanes 32 (w % 4) .. + 31,
+// columns 128 (w / 4) .. + 127 of the tile), warp 8 TMA, warp 9 MMA.  Barriers
+// and bounded waits of the CTA pairs as cgemm_oz_pair_kernel (cgemm_oz.cu).
+//
+// crt_combine_kernel turns the bytes of an entry into FP64 (integer work up to
+// the diagonal term's multiply-adds).
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -61,52 +69,37 @@ constexpr int kTile = 128 * kRB;             // one 128-row operand tile
 constexpr int kKPer = kRB / 2;               // BF16 K values per stage
 constexpr int kSteps = kRB / 32;             // MMA K steps per stage
 constexpr int kRing = 192 * 1024;
+constexpr int kStage = 2 * kTile;            // own 128 rows of A and of B
+constexpr int kStages = kRing / kStage;      // 6
 constexpr int kSmem = kRing + 1024 /*align*/ + 512 /*barriers*/;
 constexpr int kChunkStages = crt::kChunk / kKPer;
-constexpr int kGroup = 6;                    // row pairs per raster group (a wave: ~12 row x 12 column tiles)
+constexpr int kGroup = 8;                    // 256-row tiles per raster group (a wave: ~8 x 9 tiles)
 constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN
 
 struct CrtLaunch {
     int tiles;           // Np / 128
     int kb_total;        // Np / kKPer stages per unit
-    int row0;            // first row pair (pairs) or row tile (single CTAs) of the band
-    int units_per;       // units per modulus
-    int units;           // units_per * kModuli
+    int lo, hi;          // rows of 256-tiles: the band [lo, hi)
+    int units_per;       // units per plane
+    int units;           // units_per * planes
     size_t Np;           // row stride of the byte planes
     size_t band;         // rows of a byte plane
-    uint8_t* bytes;      // [kModuli][2][band][Np], rows from tile row row0 on
+    uint8_t* bytes;      // [planes][band][Np], rows from 256 lo on
     unsigned* status;
 };
 
-// unit -> (modulus, own row tile, column tile)
-template <bool PAIR, int MODE>
-__device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int rank, int& s, int& I, int& J) {
-    s = u / L.units_per;
-    const int t = u - s * L.units_per;
-    if (PAIR) {
-        if (L.row0 == 0 && L.units_per == pair_units(MODE, L.tiles)) {
-            pair_unit(MODE, L.tiles, kGroup, t, rank, I, J);
-        } else {   // a band of row pairs (even tile count)
-            const int lo = 2 * L.row0, hi = lo + (int)(L.band / 128);
-            if (MODE == 1) {
-                pair_tile_rows_range(1, L.tiles, kGroup, lo, hi, t, rank, I, J);
-            } else {
-                const int rows = (hi - lo) / 2;
-                I = lo + 2 * (t % rows) + rank;
-                J = t / rows;
-            }
-        }
-    } else {
-        if (MODE == 0) {
-            const int rows = (int)(L.band / 128);
-            I = L.row0 + t % rows;
-            J = t / rows;
-        } else {
-            int i, j;
-            tri_decode(t + L.row0 * (L.row0 + 1) / 2, i, j);
-            I = i;
-            J = j;
-        }
+// unit -> (plane, row tile, column tile), in tiles of 256
+template <int MODE>
+__device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int& z, int& P, int& J) {
+    z = u / L.units_per;
+    const int t = u - z * L.units_per, side = (L.tiles + 1) / 2;
+    if (MODE == 1) {
+        tile_of_range(1, side, kGroup, L.lo, L.hi, t, P, J);
+    } else {   // groups of kGroup row tiles, column by column
+        const int per_group = kGroup * side, g = t / per_group, in = t - g * per_group;
+        const int rows = tile_min(kGroup, L.hi - L.lo - g * kGroup);
+        P = L.lo + g * kGroup + in % rows;
+        J = in / rows;
     }
 }
 
@@ -147,344 +140,13 @@ __device__ __forceinline__ void tmem_wait8(float (&a)[8], float (&b)[8]) {
 
 constexpr float kMagic = 12582912.0f;   // 1.5 2^23: adding it rounds to an integer
 
-// y = (x + z) mod p for eight columns, as the bits of y + kMagic; sub: (x - z).
-// The quotient may come from the rounded sum; the remainder is exact:
-// |x - p q| <= |z| + p < 2^24.
-template <bool SUB>
-__device__ __forceinline__ void reduce8(const float (&x)[8], const float (&z)[8], uint64_t p2n, uint64_t inv2,
-                                        uint32_t (&out)[8]) {
-    const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic), one_n = pack2(-1.0f, -1.0f);
-#pragma unroll
-    for (int q = 0; q < 8; q += 2) {
-        const uint64_t x2 = pack2(x[q], x[q + 1]), z2 = pack2(z[q], z[q + 1]);
-        const uint64_t s2 = SUB ? fma2(z2, one_n, x2) : add2(x2, z2);
-        const uint64_t q2 = add2(fma2(s2, inv2, m2), m2n);
-        const uint64_t t2 = fma2(q2, p2n, x2);
-        const uint64_t y2 = SUB ? fma2(z2, one_n, t2) : add2(t2, z2);
-        unpack2(add2(y2, m2), out[q], out[q + 1]);
-    }
-}
-
-// Adds one K chunk of the tile, modulo p, to the packed sums acc[c]: the low
-// half holds Y_r, the high half Y_i of column c (as one 32-bit sum
-// r + 65536 i).  At most 64 chunks of |r| <= p / 2 + 1 stay within 16 bits.
-// The next eight columns are in flight while eight are reduced; `done` runs
-// once every load of the chunk has arrived (TMEM may be overwritten).
-// Bound by instruction issue: eight per complex entry (FP32 in pairs; one at a
-// time it was fourteen), two warps a scheduler.
+// Adds one K chunk, modulo p, to the packed sums: acc[c] holds column c (low
+// half) and c + 64 (as one 32-bit sum l + 65536 h).  At most 64 chunks of
+// |r| <= p / 2 + 1 stay within 16 bits.  The next eight columns are in flight
+// while eight are reduced; `done` runs once every load of the chunk has
+// arrived (TMEM may be overwritten).
 template <typename Done>
 __device__ __forceinline__ void add_chunk(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64], Done done) {
-    const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
-    float d1r[2][8], d1i[2][8], d2r[2][8], d2i[2][8];
-    auto load = [&](int c, int b) {
-        tmem_ld8(tl + c, d1r[b]);            // A_r B_r^T
-        tmem_ld8(tl + 128 + c, d1i[b]);      // A_r B_i^T
-        tmem_ld8(tl + 256 + c, d2r[b]);      // A_i B_r^T
-        tmem_ld8(tl + 384 + c, d2i[b]);      // A_i B_i^T
-    };
-    load(0, 0);
-#pragma unroll
-    for (int c = 0; c < 64; c += 8) {
-        const int b = (c >> 3) & 1;
-        tmem_wait8(d1r[b], d1i[b]);
-        tmem_wait8(d2r[b], d2i[b]);
-        if (c + 8 < 64)
-            load(c + 8, b ^ 1);
-        else
-            done();
-        uint32_t yr[8], yi[8];
-        reduce8<false>(d1r[b], d2i[b], p2n, inv2, yr);
-        reduce8<true>(d2r[b], d1i[b], p2n, inv2, yi);
-#pragma unroll
-        for (int q = 0; q < 8; q++)   // both carry the magic's bits 0x4B400000; shifted by 16 they vanish modulo 2^32
-            acc[c + q] += yr[q] - 0x4B400000u + (yi[q] << 16);
-    }
-}
-
-// sum of residues -> byte: times the inverse of M / p, balanced modulo p, plus 128
-__device__ __forceinline__ uint32_t to_byte(int v, float p, float inv_p, float inv) {
-    const float f = __uint_as_float(0x4B400000u + (uint32_t)v) - kMagic;
-    return __float_as_uint(__fadd_rn(crt::times_inverse(f, inv, p, inv_p), kMagic + 128.0f)) & 0xFFu;
-}
-
-// Epilogue warps' wait for a chunk; false when the launch gives up (all lanes alike).
-template <bool PAIR>
-__device__ __forceinline__ bool chunk_ready(uint64_t* accum, uint32_t parity, volatile int* abort, uint64_t lim,
-                                            uint32_t peer_abort) {
-    const bool ok = mbar_wait_bounded_cluster(accum, parity, abort, lim, 0);
-    tc_fence_after();
-    if (!__any_sync(0xffffffffu, !ok || *abort)) return true;
-    *abort = 1;
-    if (PAIR) st_cluster_u32(peer_abort, 1u);
-    return false;
-}
-
-// One arrival a warp on tmem_empty of the MMA issuer's CTA, its loads complete.
-__device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_tmem_empty, uint32_t rank, int lane) {
-    tc_fence_before();
-    __syncwarp();
-    if (lane == 0) {
-        if (rank == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");
-        else
-            mbar_arrive_cluster(lead_tmem_empty);
-    }
-}
-
-template <bool PAIR, int MODE>
-__global__ void __launch_bounds__(kThreads, 1)
-    cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
-    constexpr int kOperandTiles = PAIR ? 3 : 4;   // own A_r, A_i rows; half the B stack, or all of it
-    constexpr int kStage = kOperandTiles * kTile;
-    constexpr int kStages = kRing / kStage;
-    constexpr uint32_t kIdesc = make_idesc(1u, PAIR ? 256u : 128u, 256u);
-
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
-    uint64_t* empty = full + kStages;
-    uint64_t* accum = empty + kStages;      // MMA -> epilogue, once per chunk
-    uint64_t* tmem_empty = accum + 1;       // epilogue -> MMA, once per chunk
-    uint64_t* drain = tmem_empty + 1;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-    volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const uint64_t lim = kWaitLimitNs;
-    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;
-    const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
-    const int workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
-
-    if (threadIdx.x == 0) {
-        for (int s = 0; s < kStages; s++) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], 1);
-        }
-        mbar_init(accum, 1);
-        mbar_init(tmem_empty, PAIR ? 16 : 8);   // one arrival per epilogue warp
-        mbar_init(drain, 1);
-        *abort = 0;
-        fence_mbar_init();
-    }
-    if (warp == 0) {
-        if (PAIR) {
-            tmem_alloc_pair(saddr(tmem_slot), 512);
-            tmem_relinquish_pair();
-        } else {
-            tmem_alloc(saddr(tmem_slot), 512);
-            tmem_relinquish();
-        }
-    }
-    if (warp == 8 && lane == 0) {
-        prefetch_tmap(&tmA);
-        prefetch_tmap(&tmB);
-    }
-    __syncthreads();
-    if (PAIR) cluster_sync();   // both CTAs' barriers exist before either arrives on the other's
-    tc_fence_after();
-    const uint32_t tmem = *tmem_slot;
-    const uint32_t peer_abort = PAIR ? cluster_addr(saddr(const_cast<int*>(abort)), rank ^ 1u) : 0u;
-    const int chunks = (L.kb_total + kChunkStages - 1) / kChunkStages;
-
-    if (warp == 8) {
-        // ---------------------------------------------------------- producer
-        if (lane == 0) {
-            const uint32_t lead_full = PAIR ? cluster_addr(saddr(&full[0]), 0u) : saddr(&full[0]);
-            uint32_t it = 0;
-            bool ok = true;
-            for (int u = worker; u < L.units && ok; u += workers) {
-                int s, I, J;
-                unit_at<PAIR, MODE>(L, u, (int)rank, s, I, J);
-                for (int kb = 0; kb < L.kb_total; kb++, it++) {
-                    const int b = it % kStages;
-                    const uint32_t ph = (it / kStages) & 1u;
-                    if (!mbar_wait_bounded(&empty[b], ph ^ 1u, abort, lim, 0)) {
-                        ok = false;
-                        break;
-                    }
-                    uint8_t* st = smem + b * kStage;
-                    const int kx = kb * kKPer;
-                    if (!PAIR) {
-                        mbar_arrive_expect_tx(&full[b], kStage);
-                        const uint32_t fb = saddr(&full[b]);
-                        tma_load_3d(saddr(st), &tmA, fb, kx, I * 128, s);
-                        tma_load_3d(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
-                        tma_load_3d(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, s);
-                        tma_load_3d(saddr(st + 3 * kTile), &tmB, fb, kx, J * 128, kModuli + s);
-                    } else if (rank == 0) {
-                        mbar_arrive_expect_tx(&full[b], 2 * kStage);   // both CTAs' bytes
-                        const uint32_t fb = saddr(&full[b]);
-                        tma_load_3d(saddr(st), &tmA, fb, kx, I * 128, s);
-                        tma_load_3d(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
-                        tma_load_3d(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, s);                  // B_r
-                    } else {
-                        const uint32_t fb = lead_full + 8u * (uint32_t)b;
-                        tma_load_3d_pair(saddr(st), &tmA, fb, kx, I * 128, s);
-                        tma_load_3d_pair(saddr(st + kTile), &tmA, fb, kx, I * 128, kModuli + s);
-                        tma_load_3d_pair(saddr(st + 2 * kTile), &tmB, fb, kx, J * 128, kModuli + s);   // B_i
-                    }
-                }
-            }
-            const uint32_t from = it > (uint32_t)kStages ? it - kStages : 0u;
-            if (!ok || *abort) {
-                *abort = 1;
-                if (PAIR) st_cluster_u32(peer_abort, 1u);
-                // the copies in flight land before the CTAs go away
-                if (rank == 0) {
-                    for (uint32_t k = from; k < it; k++)
-                        (void)mbar_wait_bounded(&full[k % kStages], (k / kStages) & 1u, nullptr, 10000000ull, 0);
-                } else {
-                    spin_ns(1000000ull);
-                }
-            } else {
-                // the last releases of this CTA's stages have arrived
-                for (uint32_t k = from; k < it; k++)
-                    (void)mbar_wait_bounded(&empty[k % kStages], (k / kStages) & 1u, abort, lim, 0);
-            }
-        }
-    } else if (warp == 9) {
-        if (lane == 0 && rank == 0) {
-            // ------------------------------------------------------ MMA issuer
-            const uint32_t peer_empty = PAIR ? cluster_addr(saddr(&empty[0]), 1u) : 0u;
-            const uint32_t peer_accum = PAIR ? cluster_addr(saddr(accum), 1u) : 0u;
-            uint32_t it = 0, pass = 0;
-            bool ok = true;
-            for (int u = worker; u < L.units && ok; u += workers) {
-                for (int c = 0; c < chunks && ok; c++, pass++) {
-                    if (pass > 0 && !mbar_wait_bounded_cluster(tmem_empty, (pass - 1) & 1u, abort, lim, 0)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const int kb0 = c * kChunkStages;
-                    const int kb1 = kb0 + kChunkStages < L.kb_total ? kb0 + kChunkStages : L.kb_total;
-                    for (int kb = kb0; kb < kb1; kb++, it++) {
-                        const int b = it % kStages;
-                        const uint32_t ph = (it / kStages) & 1u;
-                        if (!mbar_wait_bounded_cluster(&full[b], ph, abort, lim, 0)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        uint8_t* st = smem + b * kStage;
-                        const uint64_t ar = desc_kmajor<kRB>(saddr(st));
-                        const uint64_t ai = desc_kmajor<kRB>(saddr(st + kTile));
-                        const uint64_t bd = desc_kmajor<kRB>(saddr(st + 2 * kTile));
-#pragma unroll
-                        for (int ks = 0; ks < kSteps; ks++) {
-                            const uint32_t acc = (kb > kb0 || ks > 0) ? 1u : 0u;
-                            const uint64_t off = 2u * (uint64_t)ks;   // 32 bytes of K further in each row
-                            if (PAIR) {
-                                umma_pair(tmem, ar + off, bd + off, kIdesc, acc);
-                                umma_pair(tmem + 256, ai + off, bd + off, kIdesc, acc);
-                            } else {
-                                umma<0>(tmem, ar + off, bd + off, kIdesc, acc);
-                                umma<0>(tmem + 256, ai + off, bd + off, kIdesc, acc);
-                            }
-                        }
-                        if (PAIR) {
-                            umma_commit_pair(saddr(&empty[b]));
-                            umma_commit_pair(peer_empty + 8u * (uint32_t)b);
-                        } else {
-                            umma_commit(saddr(&empty[b]));
-                        }
-                    }
-                    if (!ok) break;
-                    if (PAIR) {
-                        umma_commit_pair(saddr(accum));
-                        umma_commit_pair(peer_accum);
-                    } else {
-                        umma_commit(saddr(accum));
-                    }
-                }
-            }
-            // the MMAs complete before TMEM is freed
-            if (PAIR)
-                umma_commit_pair(saddr(drain));
-            else
-                umma_commit(saddr(drain));
-            (void)mbar_wait_bounded(drain, 0u, nullptr, lim, 0);
-            if (PAIR && *abort) st_cluster_u32(peer_abort, 1u);
-        }
-    } else {
-        // ---------------------------------------------------------- epilogue
-        const uint32_t lead_tmem_empty = PAIR ? cluster_addr(saddr(tmem_empty), 0u) : 0u;
-        const int half = warp >> 2;
-        const int row = (warp & 3) * 32 + lane;   // TMEM lane = row of the tile
-        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 64u * (uint32_t)half;
-        uint32_t pass = 0;
-        bool stop = false;
-        for (int u = worker; u < L.units && !stop; u += workers) {
-            int s, I, J;
-            unit_at<PAIR, MODE>(L, u, (int)rank, s, I, J);
-            const float p = (float)kC.p[s], inv_p = 1.0f / p, inv = (float)kC.inv[s];
-            // rows past an odd tile count, and the tile above the diagonal of a
-            // Hermitian product, are not written
-            const bool own = I < L.tiles && !(MODE == 1 && J > I);
-            uint32_t acc[64];
-#pragma unroll
-            for (int c = 0; c < 64; c++) acc[c] = 0u;
-            for (int c = 0; c < chunks; c++, pass++) {
-                if (!chunk_ready<PAIR>(accum, pass & 1u, abort, lim, peer_abort)) {
-                    stop = true;
-                    break;
-                }
-                add_chunk(tl, p, inv_p, acc, [&]() { chunk_read(tmem_empty, lead_tmem_empty, rank, lane); });
-            }
-            if (stop || !own) continue;
-            const size_t r0 = (size_t)I * 128 - (size_t)L.row0 * (PAIR ? 256 : 128) + row;   // row within the band
-            uint8_t* yr = L.bytes + ((size_t)(2 * s) * L.band + r0) * L.Np + (size_t)J * 128 + 64 * half;
-            uint8_t* yi = yr + L.band * L.Np;
-#pragma unroll
-            for (int c = 0; c < 64; c += 16) {
-                uint32_t wr[4], wi[4];
-#pragma unroll
-                for (int w = 0; w < 4; w++) {
-                    wr[w] = 0u;
-                    wi[w] = 0u;
-#pragma unroll
-                    for (int q = 0; q < 4; q++) {
-                        const uint32_t v = acc[c + 4 * w + q];
-                        const int r = (int)(short)(v & 0xFFFFu);
-                        const int i = (int)(v - (uint32_t)r) >> 16;
-                        wr[w] |= to_byte(r, p, inv_p, inv) << (8 * q);
-                        wi[w] |= to_byte(i, p, inv_p, inv) << (8 * q);
-                    }
-                }
-                *reinterpret_cast<uint4*>(yr + c) = make_uint4(wr[0], wr[1], wr[2], wr[3]);
-                *reinterpret_cast<uint4*>(yi + c) = make_uint4(wi[0], wi[1], wi[2], wi[3]);
-            }
-        }
-        if (stop && lane == 0) atomicOr(L.status, kStatusTimeout);
-    }
-
-    __syncwarp();
-    tc_fence_before();
-    __syncthreads();
-    if (PAIR) cluster_sync();   // neither CTA frees TMEM or leaves while the other may still use it
-    if (warp == 0) {
-        tc_fence_after();
-        if (PAIR)
-            tmem_dealloc_pair(tmem, 512);
-        else
-            tmem_dealloc(tmem, 512);
-    }
-}
-
-// ---------------------------------------------------------------- real products
-// C = A B^T of real operands (the Taylor polynomials of tc_expm): one residue
-// plane an operand and modulus.  A CTA pair computes a 256 x 256 tile (its
-// CTAs 128 rows each, B's 256 rows split between them): one pair MMA a K step,
-// 256 TMEM columns, so the accumulator is double-buffered and a chunk's
-// epilogue runs beside the next chunk's MMAs.  Per MMA a CTA loads 8 KB
-// instead of the complex product's 6; the imaginary planes it does not have
-// would have doubled the MMAs.
-constexpr int kRealStage = 2 * kTile;
-constexpr int kRealStages = kRing / kRealStage;
-
-// Adds one K chunk, modulo p: acc[c] holds column c (low half) and c + 64.
-template <typename Done>
-__device__ __forceinline__ void add_chunk_real(uint32_t tl, float p, float inv_p, uint32_t (&acc)[64], Done done) {
     const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
     const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic);
     auto reduce = [&](const float (&x)[8], uint32_t (&out)[8]) {
@@ -512,27 +174,50 @@ __device__ __forceinline__ void add_chunk_real(uint32_t tl, float p, float inv_p
         reduce(lo[b], l);
         reduce(hi[b], h);
 #pragma unroll
-        for (int q = 0; q < 8; q++) acc[c + q] += l[q] - 0x4B400000u + (h[q] << 16);
+        for (int q = 0; q < 8; q++)   // both carry the magic's bits 0x4B400000; shifted by 16 they vanish modulo 2^32
+            acc[c + q] += l[q] - 0x4B400000u + (h[q] << 16);
     }
 }
 
-__device__ __forceinline__ void real_unit(const CrtLaunch& L, int u, int& s, int& P, int& J) {
-    s = u / L.units_per;
-    const int t = u - s * L.units_per, side = L.tiles / 2;   // tiles of 256 a side
-    const int per_group = kGroup * side, g = t / per_group, in = t % per_group;
-    const int rows = min(kGroup, side - g * kGroup);
-    P = g * kGroup + in % rows;
-    J = in / rows;
+// sum of residues -> byte: balanced modulo p, plus 128
+__device__ __forceinline__ uint32_t to_byte(int v, float p, float inv_p) {
+    const float f = __uint_as_float(0x4B400000u + (uint32_t)v) - kMagic;
+    const float q = __fmaf_rn(f, inv_p, kMagic) - kMagic;
+    return __float_as_uint(__fadd_rn(__fmaf_rn(-q, p, f), kMagic + 128.0f)) & 0xFFu;
 }
 
+// Epilogue warps' wait for a chunk; false when the launch gives up (all lanes alike).
+__device__ __forceinline__ bool chunk_ready(uint64_t* accum, uint32_t parity, volatile int* abort, uint64_t lim,
+                                            uint32_t peer_abort) {
+    const bool ok = mbar_wait_bounded_cluster(accum, parity, abort, lim, 0);
+    tc_fence_after();
+    if (!__any_sync(0xffffffffu, !ok || *abort)) return true;
+    *abort = 1;
+    st_cluster_u32(peer_abort, 1u);
+    return false;
+}
+
+// One arrival a warp on tmem_empty of the MMA issuer's CTA, its loads complete.
+__device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_tmem_empty, uint32_t rank, int lane) {
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) {
+        if (rank == 0)
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(saddr(tmem_empty)) : "memory");
+        else
+            mbar_arrive_cluster(lead_tmem_empty);
+    }
+}
+
+template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
-    cgemm_crt_real_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
+    cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
     constexpr uint32_t kIdesc = make_idesc(1u, 256u, 256u);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
-    uint64_t* empty = full + kRealStages;
-    uint64_t* accum = empty + kRealStages;   // [2] MMA -> epilogue, one per buffer
+    uint64_t* empty = full + kStages;
+    uint64_t* accum = empty + kStages;   // [2] MMA -> epilogue, one per buffer
     uint64_t* tmem_empty = accum + 2;        // [2] both epilogues -> MMA (even CTA, count 2)
     uint64_t* drain = tmem_empty + 2;
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
@@ -544,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int worker = (int)(blockIdx.x >> 1), workers = (int)(gridDim.x >> 1);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < kRealStages; s++) {
+        for (int s = 0; s < kStages; s++) {
             mbar_init(&full[s], 1);
             mbar_init(&empty[s], 1);
         }
@@ -578,44 +263,44 @@ __global__ void __launch_bounds__(kThreads, 1)
             uint32_t it = 0;
             bool ok = true;
             for (int u = worker; u < L.units && ok; u += workers) {
-                int s, P, J;
-                real_unit(L, u, s, P, J);
+                int z, P, J;
+                unit_at<MODE>(L, u, z, P, J);
                 const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * 128;
                 for (int kb = 0; kb < L.kb_total; kb++, it++) {
-                    const int b = it % kRealStages;
-                    const uint32_t ph = (it / kRealStages) & 1u;
+                    const int b = it % kStages;
+                    const uint32_t ph = (it / kStages) & 1u;
                     if (!mbar_wait_bounded(&empty[b], ph ^ 1u, abort, lim, 0)) {
                         ok = false;
                         break;
                     }
-                    uint8_t* st = smem + b * kRealStage;
+                    uint8_t* st = smem + b * kStage;
                     const int kx = kb * kKPer;
                     if (rank == 0) {
-                        mbar_arrive_expect_tx(&full[b], 2 * kRealStage);   // both CTAs' bytes
-                        tma_load_3d(saddr(st), &tmA, saddr(&full[b]), kx, ra, s);
-                        tma_load_3d(saddr(st + kTile), &tmB, saddr(&full[b]), kx, rb, s);
+                        mbar_arrive_expect_tx(&full[b], 2 * kStage);   // both CTAs' bytes
+                        tma_load_3d(saddr(st), &tmA, saddr(&full[b]), kx, ra, z);
+                        tma_load_3d(saddr(st + kTile), &tmB, saddr(&full[b]), kx, rb, z);
                     } else {
                         const uint32_t fb = lead_full + 8u * (uint32_t)b;
-                        tma_load_3d_pair(saddr(st), &tmA, fb, kx, ra, s);
-                        tma_load_3d_pair(saddr(st + kTile), &tmB, fb, kx, rb, s);
+                        tma_load_3d_pair(saddr(st), &tmA, fb, kx, ra, z);
+                        tma_load_3d_pair(saddr(st + kTile), &tmB, fb, kx, rb, z);
                     }
                 }
             }
-            const uint32_t from = it > (uint32_t)kRealStages ? it - kRealStages : 0u;
+            const uint32_t from = it > (uint32_t)kStages ? it - kStages : 0u;
             if (!ok || *abort) {
                 *abort = 1;
                 st_cluster_u32(peer_abort, 1u);
                 // the copies in flight land before the CTAs go away
                 if (rank == 0) {
                     for (uint32_t k = from; k < it; k++)
-                        (void)mbar_wait_bounded(&full[k % kRealStages], (k / kRealStages) & 1u, nullptr, 10000000ull, 0);
+                        (void)mbar_wait_bounded(&full[k % kStages], (k / kStages) & 1u, nullptr, 10000000ull, 0);
                 } else {
                     spin_ns(1000000ull);
                 }
             } else {
                 // the last releases of this CTA's stages have arrived
                 for (uint32_t k = from; k < it; k++)
-                    (void)mbar_wait_bounded(&empty[k % kRealStages], (k / kRealStages) & 1u, abort, lim, 0);
+                    (void)mbar_wait_bounded(&empty[k % kStages], (k / kStages) & 1u, abort, lim, 0);
             }
         }
     } else if (warp == 9) {
@@ -636,14 +321,14 @@ __global__ void __launch_bounds__(kThreads, 1)
                     const int kb0 = c * kChunkStages;
                     const int kb1 = kb0 + kChunkStages < L.kb_total ? kb0 + kChunkStages : L.kb_total;
                     for (int kb = kb0; kb < kb1; kb++, it++) {
-                        const int b = it % kRealStages;
-                        const uint32_t ph = (it / kRealStages) & 1u;
+                        const int b = it % kStages;
+                        const uint32_t ph = (it / kStages) & 1u;
                         if (!mbar_wait_bounded_cluster(&full[b], ph, abort, lim, 0)) {
                             ok = false;
                             break;
                         }
                         tc_fence_after();
-                        uint8_t* st = smem + b * kRealStage;
+                        uint8_t* st = smem + b * kStage;
                         const uint64_t ad = desc_kmajor<kRB>(saddr(st));
                         const uint64_t bd = desc_kmajor<kRB>(saddr(st + kTile));
 #pragma unroll
@@ -672,23 +357,25 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t pass = 0;
         bool stop = false;
         for (int u = worker; u < L.units && !stop; u += workers) {
-            int s, P, J;
-            real_unit(L, u, s, P, J);
-            const float p = (float)kC.p[s], inv_p = 1.0f / p, inv = (float)kC.inv[s];
+            int z, P, J;
+            unit_at<MODE>(L, u, z, P, J);
+            const float p = (float)kC.p[z % kModuli], inv_p = 1.0f / p;
+            // rows and columns past the end (an odd number of 128-tiles) are not written
+            const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
             uint32_t acc[64];
 #pragma unroll
             for (int c = 0; c < 64; c++) acc[c] = 0u;
             for (int c = 0; c < chunks; c++, pass++) {
                 const uint32_t buf = pass & 1u;
-                if (!chunk_ready<true>(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
+                if (!chunk_ready(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
                     stop = true;
                     break;
                 }
-                add_chunk_real(tl + 256u * buf, p, inv_p, acc,
+                add_chunk(tl + 256u * buf, p, inv_p, acc,
                                [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
             }
-            if (stop) continue;
-            uint8_t* y = L.bytes + ((size_t)s * L.Np + (size_t)(2 * P + (int)rank) * 128 + row) * L.Np +
+            if (stop || !own) continue;
+            uint8_t* y = L.bytes + ((size_t)z * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
                          (size_t)J * 256 + 128 * half;
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
@@ -702,8 +389,8 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint32_t v = acc[c + 4 * w + q];
                         const int l = (int)(short)(v & 0xFFFFu);
                         const int h = (int)(v - (uint32_t)l) >> 16;
-                        wl[w] |= to_byte(l, p, inv_p, inv) << (8 * q);
-                        wh[w] |= to_byte(h, p, inv_p, inv) << (8 * q);
+                        wl[w] |= to_byte(l, p, inv_p) << (8 * q);
+                        wh[w] |= to_byte(h, p, inv_p) << (8 * q);
                     }
                 }
                 *reinterpret_cast<uint4*>(y + c) = make_uint4(wl[0], wl[1], wl[2], wl[3]);
@@ -811,6 +498,12 @@ __global__ void __launch_bounds__(128)
                 }
         }
     };
+    auto put = [](__nv_bfloat16* d, const uint32_t (&w)[CPT / 2]) {
+        if constexpr (CPT == 8)
+            *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+        else
+            *reinterpret_cast<uint32_t*>(d) = w[0];
+    };
     RowStat st{0, 0.0f};
     for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
         uint64_t xr[CPT], xi[CPT];
@@ -836,9 +529,9 @@ __global__ void __launch_bounds__(128)
         st = part[w0];
         for (int k = 1; k < tpr / 32; k++) st = stat_join(st, part[w0 + k]);
     }
-    // ex = the largest shift with 2-norm * 2^ex <= 2^58.35 (any for a row of zeros)
+    // ex = the largest shift with 2-norm * 2^ex <= 2^58.32 (any for a row of zeros)
     const bool finite = st.e < 0x7FF;
-    const int sh = st.e == 0 ? 0 : (int)floorf(58.35f - 0.5f * log2f(st.ss * 1.0001f)) - (st.e - 1022);
+    const int sh = st.e == 0 ? 0 : (int)floorf(crt::kNormBits - 0.5f * log2f(st.ss * 1.0001f)) - (st.e - 1022);
     if (r < Np && sub == 0) {
         ex[r] = finite ? sh : kNoScale;
         if (LEFT) {
@@ -856,30 +549,36 @@ __global__ void __launch_bounds__(128)
     for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
         uint64_t xr[CPT], xi[CPT];
         load(c0, xr, xi);
+        crt::Pieces pr[CPT], pi[CPT];
 #pragma unroll
-        for (int part = 0; part < (REAL ? 1 : 2); part++) {
-            crt::Pieces pc[CPT];
-#pragma unroll
-            for (int q = 0; q < CPT; q++) {
-                const uint64_t b = !REAL && part ? xi[q] ^ im_flip : xr[q];
-                pc[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
+        for (int q = 0; q < CPT; q++) {
+            pr[q] = crt::split_pieces(finite ? crt::to_magnitude(xr[q], sh) : 0, (xr[q] >> 63) != 0);
+            if (!REAL) {
+                const uint64_t b = xi[q] ^ im_flip;
+                pi[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
             }
-            __nv_bfloat16* dst = planes + (size_t)(part * kModuli) * plane + (size_t)r * Np + c0;
+        }
+        __nv_bfloat16* dst = planes + (size_t)r * Np + c0;
 #pragma unroll
-            for (int s = 0; s < kModuli; s++) {
-                const int p = crt::modulus(s);
-                uint32_t w[CPT / 2];
+        for (int s = 0; s < kModuli; s++) {
+            // integers up to 127 are exact in BF16: the top halves of their FP32 bits
+            uint32_t w0[CPT / 2], w1[CPT / 2];
 #pragma unroll
-                for (int h = 0; h < CPT / 2; h++) {
-                    // integers up to 127 are exact in BF16: the top halves of their FP32 bits
-                    w[h] = __byte_perm(__float_as_uint(crt::residue(pc[2 * h], p)),
-                                       __float_as_uint(crt::residue(pc[2 * h + 1], p)), 0x7632);
+            for (int h = 0; h < CPT / 2; h++) {
+                float u[2], v[2];
+#pragma unroll
+                for (int k = 0; k < 2; k++) {
+                    if (REAL)
+                        u[k] = crt::residue(pr[2 * h + k], crt::modulus(s));
+                    else
+                        crt::residue_pair(pr[2 * h + k], pi[2 * h + k], s, u[k], v[k]);
                 }
-                if constexpr (CPT == 8)
-                    *reinterpret_cast<uint4*>(dst + (size_t)s * plane) = make_uint4(w[0], w[1], w[2], w[3]);
-                else
-                    *reinterpret_cast<uint32_t*>(dst + (size_t)s * plane) = w[0];
+                w0[h] = __byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x7632);
+                if (!REAL) w1[h] = __byte_perm(__float_as_uint(v[0]), __float_as_uint(v[1]), 0x7632);
             }
+            // plane s: re + iota im of a left operand, its conjugate re - iota im of a right one
+            put(dst + (size_t)(REAL || LEFT ? s : kModuli + s) * plane, w0);
+            if (!REAL) put(dst + (size_t)(LEFT ? kModuli + s : s) * plane, w1);
         }
     }
 }
@@ -906,7 +605,7 @@ __device__ __forceinline__ double scaled(uint64_t mag, bool neg, int e) {
 }
 
 struct CrtCombine {
-    const uint8_t* bytes;    // [kModuli][2][band][Np]
+    const uint8_t* bytes;    // [planes][band][Np]
     size_t Np, band;
     int row0;                // first matrix row of the band
     int N;                   // valid rows and columns of B
@@ -926,8 +625,8 @@ struct CrtCombine {
 // consecutive columns a thread.  MODE 1: tiles that reach the diagonal or lie
 // below it, each mirrored.  B's entries of the diagonal term, and the mirrored
 // half, are transposed through shared memory so that every global access runs
-// along rows.  Bound by HBM for large matrices (30 B + 16 B read, 16 B
-// written per entry) beside 45 32 x 8-bit multiply-adds a number; at N <= 512
+// along rows.  Bound by HBM for large matrices (32 B + 16 B read, 16 B
+// written per entry) beside 48 32-bit multiply-adds a number; at N <= 512
 // by latency, so there one column a thread (four times the threads).
 template <int MODE, int COLS>
 __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
@@ -939,16 +638,17 @@ __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
     const int ta = threadIdx.x / (32 / COLS), tb = (threadIdx.x % (32 / COLS)) * COLS;   // along rows of B and the mirror
     const int i = i0 + ti, j = j0 + tj;
     const size_t o = (size_t)(i - p.row0) * p.Np + j;
-    uint32_t wr[kModuli], wi[kModuli];
+    uint32_t wu[kModuli], wv[kModuli];
 #pragma unroll
     for (int s = 0; s < kModuli; s++) {
-        const uint8_t* a = p.bytes + (size_t)(2 * s) * p.band * p.Np + o;
+        const uint8_t* a = p.bytes + (size_t)s * p.band * p.Np + o;
+        const uint8_t* b = a + (size_t)kModuli * p.band * p.Np;
         if (COLS == 4) {
-            wr[s] = *reinterpret_cast<const uint32_t*>(a);
-            wi[s] = *reinterpret_cast<const uint32_t*>(a + p.band * p.Np);
+            wu[s] = *reinterpret_cast<const uint32_t*>(a);
+            wv[s] = *reinterpret_cast<const uint32_t*>(b);
         } else {
-            wr[s] = a[0];
-            wi[s] = a[p.band * p.Np];
+            wu[s] = a[0];
+            wv[s] = b[0];
         }
     }
     // B[j0 + a][i0 + b] -> s[a][b]
@@ -971,8 +671,9 @@ __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
         crt::Acc ar = {}, ai = {};
 #pragma unroll
         for (int s = 0; s < kModuli; s++) {
-            crt::acc_add(ar, (wr[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
-            crt::acc_add(ai, (wi[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
+            const uint32_t u = (wu[s] >> (8 * k)) & 0xFFu, v = (wv[s] >> (8 * k)) & 0xFFu;
+            crt::acc_add(ar, u + v, kC.re[s]);
+            crt::acc_add(ai, u + 256u - v, kC.im[s]);
         }
         if (ea == kNoScale || eb[k] == kNoScale) {   // an infinity or a NaN in either row
             vr[k] = vi[k] = __longlong_as_double(0x7FF8000000000000ll);
@@ -980,9 +681,9 @@ __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
         }
         bool neg;
         int e;
-        uint64_t mag = crt::acc_finish(ar, kC, neg, e);
+        uint64_t mag = crt::acc_finish(ar, kC.re_bias, kC, neg, e);
         vr[k] = scaled(mag, neg, e - ea - eb[k]);
-        mag = crt::acc_finish(ai, kC, neg, e);
+        mag = crt::acc_finish(ai, kC.im_bias, kC, neg, e);
         vi[k] = scaled(mag, neg, e - ea - eb[k]);
     }
     __syncthreads();
@@ -1063,10 +764,10 @@ __global__ void __launch_bounds__(256) crt_combine_real_kernel(CrtCombine p) {
         const int eb = p.eb[j + k];
         crt::Acc a = {};
 #pragma unroll
-        for (int s = 0; s < kModuli; s++) crt::acc_add(a, (w[s] >> (8 * k)) & 0xFFu, kC.frac[s]);
+        for (int s = 0; s < kModuli; s++) crt::acc_add(a, (w[s] >> (8 * k)) & 0xFFu, kC.real[s]);
         bool neg;
         int e;
-        const uint64_t mag = crt::acc_finish(a, kC, neg, e);
+        const uint64_t mag = crt::acc_finish(a, kC.real_bias, kC, neg, e);
         v[k] = ea == kNoScale || eb == kNoScale ? __longlong_as_double(0x7FF8000000000000ll) : scaled(mag, neg, e - ea - eb);
     }
     __syncthreads();
@@ -1084,10 +785,9 @@ int sm_count() {
     return sms;
 }
 
-template <bool PAIR, int MODE, bool REAL = false>
+template <int MODE>
 tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
-    void (*k)(CUtensorMap, CUtensorMap, CrtLaunch) = cgemm_crt_kernel<PAIR, MODE>;
-    if constexpr (REAL) k = cgemm_crt_real_kernel;
+    auto k = cgemm_crt_kernel<MODE>;
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -1096,15 +796,15 @@ tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch
         TC_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem));
         attr_set[dev] = true;
     }
-    const int workers = std::min(L.units, PAIR ? sm_count() / 2 : sm_count());
+    const int workers = std::min(L.units, sm_count() / 2);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(PAIR ? 2 * workers : workers));
+    cfg.gridDim = dim3((unsigned)(2 * workers));
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = kSmem;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = PAIR ? 2 : 1;
+    attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -1117,30 +817,52 @@ tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch
 // rows of a band: all of them up to 16384, else 4096 (bounds the byte scratch)
 int band_rows(int Np) { return Np <= 16384 ? Np : 4096; }
 
+size_t plane_bytes(int Np, int planes) { return round256((size_t)planes * Np * Np * 2); }
+
+tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
+    m.Np = Np;
+    m.left = left;
+    m.count = planes;
+    m.planes = ar.take<uint8_t>((size_t)planes * Np * Np * 2);
+    m.ex = ar.take<int>((size_t)Np);
+    m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
+    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
+    return make_part_map_rows(&m.map, m.planes, Np, planes, TC_BF16X3, kRB);
+}
+
+// The residue products of one band of rows (all of them: lo = 0, hi = side).
+tc_status gemm(int mode, const CrtMat& A, const CrtMat& B, int lo, int hi, void* scratch, cudaStream_t s) {
+    CrtLaunch L{};
+    L.tiles = A.Np / 128;
+    const int side = (L.tiles + 1) / 2;
+    L.kb_total = A.Np / kKPer;
+    L.lo = lo;
+    L.hi = hi;
+    L.Np = (size_t)A.Np;
+    L.band = hi == side ? (size_t)A.Np - 256 * (size_t)lo : 256 * (size_t)(hi - lo);
+    L.bytes = static_cast<uint8_t*>(scratch);
+    L.status = device_status_word();
+    L.units_per = mode == 0 ? side * (hi - lo) : hi * (hi + 1) / 2 - lo * (lo + 1) / 2;
+    L.units = L.units_per * A.count;
+    return mode == 0 ? launch<0>(A.map, B.map, L, s) : launch<1>(A.map, B.map, L, s);
+}
+
 }  // namespace
 
 size_t crt_mat_bytes(int Np, bool left) {
-    return round256((size_t)2 * kModuli * Np * Np * 2) + round256((size_t)Np * sizeof(int)) +
+    return plane_bytes(Np, 2 * kModuli) + round256((size_t)Np * sizeof(int)) +
            (left ? round256((size_t)2 * Np * sizeof(double)) : 0);
 }
 
 size_t crt_scratch_bytes(int Np) { return round256((size_t)2 * kModuli * band_rows(Np) * Np); }
 
-tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left) {
-    m.Np = Np;
-    m.left = left;
-    m.planes = ar.take<uint8_t>((size_t)2 * kModuli * Np * Np * 2);
-    m.ex = ar.take<int>((size_t)Np);
-    m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
-    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
-    return make_part_map_rows(&m.map, m.planes, Np, 2 * kModuli, TC_BF16X3, kRB);
-}
+tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left) { return mat_init(m, ar, Np, left, 2 * kModuli); }
 
 tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
     if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
     view = base;
     view.Np = Np;
-    return make_part_map_rows(&view.map, base.planes, Np, 2 * kModuli, TC_BF16X3, kRB);
+    return make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
 }
 
 tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
@@ -1171,37 +893,16 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
 }
 
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
-                      size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s) {
+                      size_t ldb, const CrtOut& out, cudaStream_t s) {
     const int Np = A.Np;
     if (B.Np != Np || !A.left || B.left || Np < 128 || Np % 128 != 0 || Np > 65536)
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes or roles");
     if (mode != 0 && mode != 1) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: mode");
-    const int T = Np / 128;
-    if (T < 2) pairs = false;
-    const int band = band_rows(Np);   // Np itself, or a divisor that is a multiple of 256
+    const int band = band_rows(Np);   // Np itself, or a divisor that is a multiple of 256 kGroup
     for (int row0 = 0; row0 < Np; row0 += band) {
-        CrtLaunch L{};
-        L.tiles = T;
-        L.kb_total = Np / kKPer;
-        L.row0 = pairs ? row0 / 256 : row0 / 128;
-        L.Np = (size_t)Np;
-        L.band = (size_t)band;
-        L.bytes = static_cast<uint8_t*>(out.scratch);
-        L.status = device_status_word();
-        const int t0 = row0 / 128, t1 = (row0 + band) / 128;
-        if (band == Np)
-            L.units_per = pairs ? (int)pair_units(mode, T) : (mode == 0 ? T * T : T * (T + 1) / 2);
-        else if (pairs)
-            L.units_per = mode == 0 ? T * (t1 - t0) / 2 : (int)pair_count(1, T, t0, t1);
-        else
-            L.units_per = mode == 0 ? T * (t1 - t0) : t1 * (t1 + 1) / 2 - t0 * (t0 + 1) / 2;
-        L.units = L.units_per * kModuli;
-        if (pairs)
-            TC_TRY((mode == 0 ? launch<true, 0>(A.map, B.map, L, s) : launch<true, 1>(A.map, B.map, L, s)));
-        else
-            TC_TRY((mode == 0 ? launch<false, 0>(A.map, B.map, L, s) : launch<false, 1>(A.map, B.map, L, s)));
+        TC_TRY(gemm(mode, A, B, row0 / 256, (row0 + band + 255) / 256, out.scratch, s));
         CrtCombine c{};
-        c.bytes = L.bytes;
+        c.bytes = static_cast<const uint8_t*>(out.scratch);
         c.Np = (size_t)Np;
         c.band = (size_t)band;
         c.row0 = row0;
@@ -1228,21 +929,13 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
 }
 
 size_t crt_real_mat_bytes(int N, bool left) {
-    return round256((size_t)kModuli * N * N * 2) + round256((size_t)N * sizeof(int)) +
+    return plane_bytes(N, kModuli) + round256((size_t)N * sizeof(int)) +
            (left ? round256((size_t)2 * N * sizeof(double)) : 0);
 }
 
 size_t crt_real_scratch_bytes(int N) { return round256((size_t)kModuli * N * N); }
 
-tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) {
-    m.Np = N;
-    m.left = left;
-    m.planes = ar.take<uint8_t>((size_t)kModuli * N * N * 2);
-    m.ex = ar.take<int>((size_t)N);
-    m.diag = left ? ar.take<double>((size_t)2 * N) : nullptr;
-    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "real products: workspace too small");
-    return make_part_map_rows(&m.map, m.planes, N, kModuli, TC_BF16X3, kRB);
-}
+tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) { return mat_init(m, ar, N, left, kModuli); }
 
 tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
     if (reinterpret_cast<uintptr_t>(a) & 15u) return fail(TC_ERR_INVALID_ARG, "real products: operand misaligned");
@@ -1259,20 +952,11 @@ tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
 
 tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, double* c, void* scratch, cudaStream_t s) {
     const int N = A.Np;
-    if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0)
+    if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0 || N > 16384)
         return fail(TC_ERR_INVALID_ARG, "real products: operands of different sizes or roles");
-    CrtLaunch L{};
-    L.tiles = N / 128;
-    L.kb_total = N / kKPer;
-    L.Np = (size_t)N;
-    L.band = (size_t)N;
-    L.bytes = static_cast<uint8_t*>(scratch);
-    L.status = device_status_word();
-    L.units_per = (N / 256) * (N / 256);
-    L.units = L.units_per * kModuli;
-    TC_TRY((launch<true, 0, true>(A.map, B.map, L, s)));
+    TC_TRY(gemm(0, A, B, 0, N / 256, scratch, s));
     CrtCombine p{};
-    p.bytes = L.bytes;
+    p.bytes = static_cast<const uint8_t*>(scratch);
     p.Np = (size_t)N;
     p.ldb = (size_t)N;
     p.ea = A.ex;

@@ -8,14 +8,17 @@
 
 namespace tc {
 
-// One operand: 2 x 15 residue planes [Np][Np] in BF16 (re, then im), the
-// power-of-two scale of each row, and, for a left operand, its diagonal.
+// One operand: residue planes [Np][Np] in BF16 (2 x 16: re + iota im and
+// re - iota im, in that order for a left operand, the other way round for a
+// right one; a real operand has 16), the power-of-two scale of each row, and,
+// for a left operand, its diagonal.
 struct CrtMat {
     void* planes;
     int* ex;          // row r holds round(x 2^ex[r])
     double* diag;     // left operands: [2][Np], the diagonal kept in FP64 (planes hold zero there)
     CUtensorMap map;
     int Np;
+    int count;        // planes
     bool left;
 };
 
@@ -33,7 +36,6 @@ size_t crt_scratch_bytes(int Np);
 // Y = A B^H, FP64 planes of row stride Np.  mode 1: Y Hermitian, the
 // block-lower half computed and mirrored.  (br, bi): B's FP64 planes of row
 // stride ldb, valid for N rows and columns, for the diagonal term of A.
-// pairs: CTA pairs on the 2-SM MMA, else single CTAs (the same bits).
 struct CrtOut {
     double* yr;
     double* yi;
@@ -42,9 +44,9 @@ struct CrtOut {
     bool conj_b;       // B was loaded with conj: (br, bi) are the planes before it
 };
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
-                      size_t ldb, const CrtOut& out, bool pairs, cudaStream_t s);
+                      size_t ldb, const CrtOut& out, cudaStream_t s);
 
-// Real operands (N x N, row stride N, N a power of two >= 256): fifteen planes
+// Real operands (N x N, row stride N, N a power of two >= 256): sixteen planes
 // each; c = A B^T.  b: B's FP64 values (c must not overlap a or b).
 size_t crt_real_mat_bytes(int N, bool left);
 size_t crt_real_scratch_bytes(int N);

@@ -736,7 +736,7 @@ bool oz_modular() {
 }
 
 int oz_products() {
-    return oz_modular() ? crt::kModuli : kOzDigits.slices * (kOzDigits.slices + 1) / 2;
+    return oz_modular() ? crt::kModuli / 2 : kOzDigits.slices * (kOzDigits.slices + 1) / 2;
 }
 
 tc_status oz_slice(const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld, int Np,
@@ -840,7 +840,7 @@ tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br,
     if (A.Np != B.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
     if (oz_modular())
         return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch, out.accumulate, out.conj_b},
-                           oz_use_pairs(A.Np / 128), s);
+                           s);
     if (out.accumulate) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: the digit form does not accumulate");
     OzEpi ep{};
     ep.Np = A.Np;

@@ -9,13 +9,13 @@
 
 namespace tc {
 
-// The FP64-accurate products run in the residue form (cgemm_crt.cu): fifteen
-// BF16 products modulo coprime p_s.  TC_OZ_BITS=6 in the environment takes
+// The FP64-accurate products run in the residue form (cgemm_crt.cu): two real
+// BF16 products for each of sixteen coprime p_s.  TC_OZ_BITS=6 in the environment takes
 // the digit form (cgemm_oz.cu) instead: nine balanced 6-bit digits an entry
 // and the 45 digit products with t + u < 9, K in chunks of 16384
 // (K 2^(2 bits - 2) <= 2^24 keeps an FP32 sum of digit products exact).
 bool oz_modular();
-int oz_products();   // BF16 products per real product: 15 or 45
+int oz_products();   // BF16 products per real product: 8 (32 real ones for a complex product) or 45
 
 struct OzDigits {
     int bits;     // digit width

@@ -1,14 +1,19 @@
 // crt_scheme.cuh -- the residue number system of the FP64-accurate products
-// (cgemm_crt.cu): fifteen pairwise coprime moduli p_s <= 255, their product
-// M = 2^117.77, and the constants that turn residues back into a number
-// (Chinese remainder theorem).  Plain C++ with host and device linkage, so
-// that host tests can run the very arithmetic of the kernels.
+// (cgemm_crt.cu): sixteen pairwise coprime odd moduli p_s <= 241, their
+// product M = 2^117.69, and the constants that turn residues back into a
+// number (Chinese remainder theorem).  Plain C++ with host and device linkage,
+// so that host tests can run the very arithmetic of the kernels.
 //
-// Why 255 and 1024: balanced residues |r| <= 127 are exact in BF16 (8
-// significand bits), and 1024 products of two of them sum to at most
-// 1024 * 127^2 = 2^24 - 261120, so an FP32 accumulator holds a K chunk of
-// 1024 exactly.  Moduli up to 511 would also be exact in BF16 and save one
-// of the fifteen products, but cut the exact chunk to 256.
+// Every prime factor of a modulus is 1 modulo 4, so -1 has a square root iota
+// modulo p_s.  Then a_r + i a_i -> (a_r + iota a_i, a_r - iota a_i) maps
+// Gaussian integers modulo p_s to two independent residues, and a complex
+// product is TWO real products instead of four (as in number-theoretic
+// transforms): 32 real products in all, against 60 with the fifteen largest
+// moduli of any kind.
+//
+// Why at most 255 and 1024: balanced residues |r| <= 120 are exact in BF16 (8
+// significand bits), and 1024 products of two of them sum to less than 2^24,
+// so an FP32 accumulator holds a K chunk of 1024 exactly.
 #pragma once
 
 #include <stdint.h>
@@ -22,16 +27,22 @@
 namespace tc {
 namespace crt {
 
-constexpr int kModuli = 15;
+constexpr int kModuli = 16;
 constexpr int kChunk = 1024;      // K values whose sum is exact in FP32
+constexpr float kNormBits = 58.32f;   // rows' 2-norms stay below 2^58.32, so |entries of A B^H| < M / 2 = 2^116.69
 typedef unsigned __int128 u128;
 
 TC_CRT_HD constexpr int modulus(int s) {
-    constexpr int p[kModuli] = {255, 254, 253, 251, 247, 241, 239, 233, 229, 227, 223, 217, 211, 199, 197};
+    constexpr int p[kModuli] = {241, 233, 229, 221, 205, 197, 193, 181, 173, 157, 149, 137, 113, 109, 101, 97};
     return p[s];
 }
+// iota^2 = -1 modulo p_s, |iota| <= p_s / 2
+TC_CRT_HD constexpr int iota(int s) {
+    constexpr int x[kModuli] = {64, 89, 107, 21, 32, 14, 81, 19, 80, 28, 44, 37, 15, 33, 10, 22};
+    return x[s];
+}
 
-// M / p_s, M and the inverse of M / p_s modulo p_s
+// M / p_s, M and inverses modulo p_s
 constexpr u128 product_without(int s) {
     u128 m = 1;
     for (int t = 0; t < kModuli; t++)
@@ -39,23 +50,16 @@ constexpr u128 product_without(int s) {
     return m;
 }
 constexpr u128 product_all() { return product_without(0) * (u128)modulus(0); }
-constexpr int inverse_of_rest(int s) {
-    const int p = modulus(s), a = (int)(product_without(s) % (u128)p);
+constexpr int inverse(int a, int p) {
+    a %= p;
     for (int x = 1; x < p; x++)
         if (a * x % p == 1) return x;
     return 0;
 }
-// round(2^96 / p): the weight of residue s in the fraction x / M (limb 0 lowest)
-constexpr u128 fraction(int s) {
-    const u128 one = (u128)1 << 96;
-    const u128 p = (u128)modulus(s);
-    return (one + p / 2) / p;
-}
-// Residues are stored with 128 added (1 .. 255); this takes the 128s out again.
-constexpr u128 fraction_bias() {
-    u128 b = 0;
-    for (int s = 0; s < kModuli; s++) b += (u128)128 * fraction(s);
-    return b & (((u128)1 << 96) - 1);
+constexpr int inverse_of_rest(int s) { return inverse((int)(product_without(s) % (u128)modulus(s)), modulus(s)); }
+// round(2^96 (k mod p) / p): the weight of a residue in the fraction x / M
+constexpr u128 fraction(int k, int p) {
+    return ((((u128)1 << 96) * (u128)(k % p)) + (u128)(p / 2)) / (u128)p;
 }
 constexpr int product_bits() {
     int b = 0;
@@ -63,23 +67,41 @@ constexpr int product_bits() {
     return b;
 }
 
+// With y_u, y_v the residues of the two real products, Re = (y_u + y_v) / 2
+// and Im = (y_u - y_v) / (2 iota) modulo p: the halves and 1 / iota go into
+// the weights together with the inverse of M / p.  Residues are stored with
+// 128 added; re and im take 256 of their sum and (shifted to be positive)
+// difference out again, real 128.
 struct Consts {
-    uint32_t frac[kModuli][3];   // fraction(s), limbs
-    uint32_t bias[3];            // fraction_bias(), limbs
+    uint32_t re[kModuli][3];     // limbs, lowest first
+    uint32_t im[kModuli][3];
+    uint32_t real[kModuli][3];
+    uint32_t re_bias[3], im_bias[3], real_bias[3];
     uint64_t mtop;               // M / 2^(bits - 64): the top 64 bits of M
     int mbits;                   // bits of M
-    int inv[kModuli];            // inverse_of_rest(s)
     int p[kModuli];              // modulus(s)
 };
 constexpr Consts make_consts() {
     Consts c{};
+    u128 br = 0, bi = 0, b1 = 0;
     for (int s = 0; s < kModuli; s++) {
-        const u128 f = fraction(s);
-        for (int l = 0; l < 3; l++) c.frac[s][l] = (uint32_t)(f >> (32 * l));
-        c.inv[s] = inverse_of_rest(s);
-        c.p[s] = modulus(s);
+        const int p = modulus(s), w = inverse_of_rest(s), half = inverse(2, p);
+        const u128 fr = fraction(w * half % p, p), fi = fraction(w * half % p * inverse(iota(s), p), p), f1 = fraction(w, p);
+        for (int l = 0; l < 3; l++) {
+            c.re[s][l] = (uint32_t)(fr >> (32 * l));
+            c.im[s][l] = (uint32_t)(fi >> (32 * l));
+            c.real[s][l] = (uint32_t)(f1 >> (32 * l));
+        }
+        br += 256 * fr;
+        bi += 256 * fi;
+        b1 += 128 * f1;
+        c.p[s] = p;
     }
-    for (int l = 0; l < 3; l++) c.bias[l] = (uint32_t)(fraction_bias() >> (32 * l));
+    for (int l = 0; l < 3; l++) {
+        c.re_bias[l] = (uint32_t)(br >> (32 * l));
+        c.im_bias[l] = (uint32_t)(bi >> (32 * l));
+        c.real_bias[l] = (uint32_t)(b1 >> (32 * l));
+    }
     c.mbits = product_bits();
     c.mtop = (uint64_t)(product_all() >> (c.mbits - 64));
     return c;
@@ -87,11 +109,11 @@ constexpr Consts make_consts() {
 
 // ---------------------------------------------------------------- residues
 // An integer below 2^59 in four pieces (20, 13, 13 and 13 bits) with its sign,
-// as FP32 numbers.  With the balanced remainders c_k (|c_k| <= 127) of 2^20,
+// as FP32 numbers.  With the balanced remainders c_k (|c_k| <= 120) of 2^20,
 // 2^33 and 2^46, t = lo + a c_1 + b c_2 + c c_3 is an integer below 2^22, so
 // FP32 holds every step exactly, and so is t - q p.  The quotient
 // q = round(t / p) comes from the rounded reciprocal: its error t / p 2^-24 is
-// below half a unit in p, so the remainder is the balanced one, |r| <= 127.
+// below half a unit in p, so the remainder is the balanced one, |r| <= p / 2.
 // (FP32 multiply-adds: twice the rate of integer ones here, and a third of
 // their number.)
 struct Pieces {
@@ -128,17 +150,23 @@ TC_CRT_HD constexpr int balanced_pow2(int e, int p) {   // 2^e mod p, |.| <= p /
     const int r = (int)((1ull << e) % (uint64_t)p);
     return 2 * r > p ? r - p : r;
 }
-TC_CRT_HD float residue(const Pieces& x, int p) {
-    const float t = fma_f32(x.c, (float)balanced_pow2(46, p),
-                            fma_f32(x.b, (float)balanced_pow2(33, p), fma_f32(x.a, (float)balanced_pow2(20, p), x.lo)));
+// an integer below 2^22 + 2^14 congruent to x
+TC_CRT_HD float congruent(const Pieces& x, int p) {
+    return fma_f32(x.c, (float)balanced_pow2(46, p),
+                   fma_f32(x.b, (float)balanced_pow2(33, p), fma_f32(x.a, (float)balanced_pow2(20, p), x.lo)));
+}
+// its balanced residue
+TC_CRT_HD float balanced(float t, int p) {
     const float q = fma_f32(t, 1.0f / (float)p, 12582912.0f) - 12582912.0f;   // 1.5 2^23: rounds to an integer
     return fma_f32(-q, (float)p, t);
 }
-// An integer below 2^24 / 254 (sum of residues) times inv, balanced modulo p
-TC_CRT_HD float times_inverse(float v, float inv, float p, float inv_p) {
-    const float f = v * inv;   // exact: below 2^24
-    const float q = fma_f32(f, inv_p, 12582912.0f) - 12582912.0f;
-    return fma_f32(-q, p, f);
+TC_CRT_HD float residue(const Pieces& x, int p) { return balanced(congruent(x, p), p); }
+// re + iota im and re - iota im
+TC_CRT_HD void residue_pair(const Pieces& re, const Pieces& im, int s, float& plus, float& minus) {
+    const int p = modulus(s);
+    const float t = congruent(re, p), r = residue(im, p);
+    plus = balanced(fma_f32(r, (float)iota(s), t), p);
+    minus = balanced(fma_f32(r, (float)-iota(s), t), p);
 }
 
 // FP64 bits -> sign and integer magnitude round(|x| 2^sh); |x| 2^sh < 2^59.
@@ -155,18 +183,16 @@ TC_CRT_HD uint64_t to_magnitude(uint64_t bits, int sh) {
 }
 
 // ---------------------------------------------------------------- recombination
-// x / M modulo 1 as a signed 96-bit fraction from the fifteen stored bytes
-// (residue times the inverse of M / p, plus 128) -> x 2^e in FP64 (e split in two factors
-// by the caller when it is out of range).  The fraction's error is below
-// 2^-86, so x is within 2^32 units of integers whose rows are held to 2^58
-// (|x| < M / 2 - 2^33).
+// x / M modulo 1 as a signed 96-bit fraction -> mag 2^exp2.  The fraction's
+// error is below 2^-83, so x is within 2^35 units of integers whose rows are
+// held to 2^58 (|x| < M / 2 - 2^36).
 struct Acc {
     uint64_t a0, a1, a2;
 };
-TC_CRT_HD void acc_add(Acc& a, uint32_t byte, const uint32_t (&f)[3]) {
-    a.a0 += (uint64_t)byte * f[0];
-    a.a1 += (uint64_t)byte * f[1];
-    a.a2 += (uint64_t)byte * f[2];
+TC_CRT_HD void acc_add(Acc& a, uint32_t k, const uint32_t (&f)[3]) {
+    a.a0 += (uint64_t)k * f[0];
+    a.a1 += (uint64_t)k * f[1];
+    a.a2 += (uint64_t)k * f[2];
 }
 TC_CRT_HD int clz64(uint64_t v) {
 #ifdef __CUDA_ARCH__
@@ -183,7 +209,7 @@ TC_CRT_HD uint64_t mulhi_u64(uint64_t a, uint64_t b) {
 #endif
 }
 // mag 2^exp2 (mag a 64-bit integer) with the sign returned through neg; mag = 0 for x = 0
-TC_CRT_HD uint64_t acc_finish(const Acc& a, const Consts& c, bool& neg, int& exp2) {
+TC_CRT_HD uint64_t acc_finish(const Acc& a, const uint32_t (&bias)[3], const Consts& c, bool& neg, int& exp2) {
     // carry-propagate to three 32-bit limbs modulo 2^96, minus the bias
     uint64_t t = a.a0;
     uint32_t l0 = (uint32_t)t;
@@ -191,11 +217,11 @@ TC_CRT_HD uint64_t acc_finish(const Acc& a, const Consts& c, bool& neg, int& exp
     uint32_t l1 = (uint32_t)t;
     t = (t >> 32) + a.a2;
     uint32_t l2 = (uint32_t)t;
-    int64_t d = (int64_t)l0 - c.bias[0];
+    int64_t d = (int64_t)l0 - bias[0];
     l0 = (uint32_t)d;
-    d = (int64_t)l1 - c.bias[1] + (d >> 32);
+    d = (int64_t)l1 - bias[1] + (d >> 32);
     l1 = (uint32_t)d;
-    d = (int64_t)l2 - c.bias[2] + (d >> 32);
+    d = (int64_t)l2 - bias[2] + (d >> 32);
     l2 = (uint32_t)d;
     neg = (l2 >> 31) != 0;
     if (neg) {   // two's complement

@@ -23,15 +23,17 @@ static double value(uint64_t mag, bool neg, int e) { return (neg ? -1.0 : 1.0) *
 
 int main() {
     std::mt19937_64 rng(7);
-    // moduli: coprime, balanced residues exact in BF16, a K chunk exact in FP32
+    // moduli: coprime, balanced residues exact in BF16, a K chunk exact in FP32, iota a root of -1
     for (int a = 0; a < kModuli; a++) {
         if (modulus(a) / 2 > 127 || (long)kChunk * (modulus(a) / 2) * (modulus(a) / 2) >= (1l << 24)) return fail("chunk", a, 0);
+        if ((iota(a) * iota(a) + 1) % modulus(a) || std::abs(iota(a)) > modulus(a) / 2) return fail("iota", a, 0);
         for (int b = 0; b < a; b++) {
             int x = modulus(a), y = modulus(b);
             while (y) { int t = x % y; x = y; y = t; }
             if (x != 1) return fail("coprime", a, b);
         }
     }
+    if (2 * kNormBits >= std::log2((double)product_all()) - 1) return fail("range", -1, 0);
     // residues of integers up to 2^59 - 1: random sizes, both signs, the ends, and the neighbours of
     // every kind of tie (odd multiples of p / 2 in the low piece, large pieces above)
     auto check = [&](uint64_t m, bool neg) {
@@ -60,14 +62,19 @@ int main() {
         const int s = check(m, (m & 1) != 0);
         if (s >= 0) return fail("residue", s, m);
     }
-    // sums of up to 64 chunks' residues times the inverse
-    for (int s = 0; s < kModuli; s++) {
-        const int p = modulus(s);
-        for (int v = -8300; v <= 8300; v++) {
-            const float f = times_inverse((float)v, (float)C.inv[s], (float)p, 1.0f / (float)p);
-            const int r = (int)f;
-            if ((float)r != f || std::abs(r) > p / 2 || ((long)v * C.inv[s] - r) % p != 0)
-                return fail("times_inverse", s, (unsigned long long)(v + 8300));
+    // pairs: re +- iota im
+    for (int k = 0; k < 300000; k++) {
+        const uint64_t x = rng() >> (5 + rng() % 59), y = rng() >> (5 + rng() % 59);
+        const bool nx = rng() & 1, ny = rng() & 1;
+        for (int s = 0; s < kModuli; s++) {
+            const int p = modulus(s);
+            float u, v;
+            residue_pair(split_pieces(x, nx), split_pieces(y, ny), s, u, v);
+            const i128 X = nx ? -(i128)x : (i128)x, Y = ny ? -(i128)y : (i128)y;
+            const int iu = (int)u, iv = (int)v;
+            if ((float)iu != u || (float)iv != v || std::abs(iu) > p / 2 || std::abs(iv) > p / 2 ||
+                (X + iota(s) * Y - iu) % p || (X - iota(s) * Y - iv) % p)
+                return fail("residue_pair", s, x);
         }
     }
     // FP64 bits to integers: normal, subnormal, zero, both directions of the shift
@@ -84,32 +91,46 @@ int main() {
         if ((long double)got != want) return fail("to_magnitude", -1, bits);
     }
     // recombination: random sizes, small values, both ends of its range, which stops short of M / 2 by
-    // the fraction's own error of 2^32 units (nearer than that it may wrap; the operands' rows keep
-    // |x| below 2^116.73, M / 2 is 2^116.77)
-    const i128 M = (i128)product_all(), half = M / 2 - ((i128)1 << 33);
-    for (int k = 0; k < 300000; k++) {
+    // the fraction's own error of 2^35 units (nearer than that it may wrap; the operands' rows keep
+    // |x| below 2^116.64, M / 2 is 2^116.69)
+    const i128 M = (i128)product_all(), half = M / 2 - ((i128)1 << 36);
+    auto draw = [&](int k) {
         i128 x = (i128)(((u128)rng() << 64) | rng()) % half;
         x >>= (int)(rng() % 118);
         if (k == 0) x = half - 1;
         if (k == 1) x = 0;
         if (k == 2) x = 1;
-        if (k & 1) x = -x;
-        Acc a{};
+        return (rng() & 1) ? -x : x;
+    };
+    auto bal = [](i128 x, int p) {
+        int r = (int)(x % p);
+        if (r > p / 2) r -= p;
+        if (r < -(p / 2)) r += p;
+        return r;
+    };
+    // 2^35 units of the fraction's 96 bits, one rounding to FP64 and the 64-bit multiply
+    auto near = [](double got, i128 x) {
+        return std::fabs(got - (double)x) <= std::ldexp(1.0, 35) + std::fabs((double)x) * std::ldexp(1.0, -52);
+    };
+    for (int k = 0; k < 300000; k++) {
+        const i128 x = draw(k % 1000), y = draw((k + 1) % 1000);
+        Acc ar{}, ai{}, a1{};
         for (int s = 0; s < kModuli; s++) {
             const int p = modulus(s);
-            int r = (int)(x % p);                       // as an accumulated product with a left operand times inv
-            r = (int)(((long)r * C.inv[s]) % p);
-            if (r > p / 2) r -= p;
-            if (r < -(p / 2)) r += p;
-            acc_add(a, (uint32_t)(r + 128), C.frac[s]);
+            const int rx = bal(x, p), ry = bal(y, p);
+            const uint32_t bu = (uint32_t)(bal(rx + (i128)iota(s) * ry, p) + 128), bv = (uint32_t)(bal(rx - (i128)iota(s) * ry, p) + 128);
+            acc_add(ar, bu + bv, C.re[s]);
+            acc_add(ai, bu + 256 - bv, C.im[s]);
+            acc_add(a1, (uint32_t)(rx + 128), C.real[s]);
         }
         bool neg;
         int e;
-        const uint64_t mag = acc_finish(a, C, neg, e);
-        const double got = value(mag, neg, e);
-        // 2^32 units of the fraction's 96 bits, one rounding to FP64 and the 64-bit multiply
-        const double tol = std::ldexp(1.0, 32) + std::fabs((double)x) * std::ldexp(1.0, -52);
-        if (!(std::fabs(got - (double)x) <= tol)) return fail("recombination", -1, (unsigned long long)k);
+        uint64_t mag = acc_finish(ar, C.re_bias, C, neg, e);
+        if (!near(value(mag, neg, e), x)) return fail("recombination (re)", -1, (unsigned long long)k);
+        mag = acc_finish(ai, C.im_bias, C, neg, e);
+        if (!near(value(mag, neg, e), y)) return fail("recombination (im)", -1, (unsigned long long)k);
+        mag = acc_finish(a1, C.real_bias, C, neg, e);
+        if (!near(value(mag, neg, e), x)) return fail("recombination (real)", -1, (unsigned long long)k);
     }
     std::printf("ok\n");
     return 0;

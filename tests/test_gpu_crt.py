@@ -2,8 +2,8 @@
 
 The DMMA form is reached by a workspace below what tc_workspace_size states.
 Tolerance of one product, relative to the 2-norms of the two rows: each row
-is rounded to half a unit of 2^-57.35 of its norm per entry, 2 K entries, so
-2 sqrt(2 K) 2^-58.35 (Cauchy-Schwarz), plus 4 roundings of 2^-53 and, for the
+is rounded to half a unit of 2^-57.32 of its norm per entry, 2 K entries, so
+2 sqrt(2 K) 2^-58.32 (Cauchy-Schwarz), plus 4 roundings of 2^-53 and, for the
 DMMA sums, K 2^-52 (2 K additions in sequence of two products each).  A step
 is two products with rows of U of norm 1 (unitary), and every entry's error
 stays below that of the whole by the rows' norms.
@@ -30,7 +30,7 @@ def tc():
 
 def _bound(n, steps, scale=1.0):
     K = 1 << n
-    return steps * 2 * scale * (2 * np.sqrt(2 * K) * 2.0 ** -58.35 + 4 * 2.0 ** -53 + K * 2.0 ** -52)
+    return steps * 2 * scale * (2 * np.sqrt(2 * K) * 2.0 ** -58.32 + 4 * 2.0 ** -53 + K * 2.0 ** -52)
 
 
 def _setup(tc, n, dt=0.1, seed=0):
@@ -143,7 +143,7 @@ def test_gradient_on_the_tensor_cores_with_squarings(tc, oracle):
 @pytest.mark.parametrize("n,degree,squarings", [(8, 0, -1), (8, 6, 3), (9, 0, -1), (11, 12, 1)])
 def test_expm_on_the_tensor_cores_equals_the_dmma_form(tc, n, degree, squarings):
     """One tile (n = 8), one and two K chunks; plans with and without squarings.  Every entry of the
-    polynomials is bounded by 1 (cos, sin of B), each product within 2 sqrt(K) 2^-58.35 of its rows'
+    polynomials is bounded by 1 (cos, sin of B), each product within 2 sqrt(K) 2^-58.32 of its rows'
     norms (<= 1) plus roundings, the DMMA sums K 2^-53; at most 8 + 3 squarings products, doubled per
     squaring."""
     N = 1 << n
@@ -158,7 +158,7 @@ def test_expm_on_the_tensor_cores_equals_the_dmma_form(tc, n, degree, squarings)
     tc._abi.call("tc_expm", ctypes.c_void_p(H.data_ptr()), n, 0.3, ctypes.byref(opts), ctypes.c_void_p(b.data_ptr()),
                  ctypes.c_void_p(work.data_ptr()), work.numel(),
                  ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
-    one = 2 * np.sqrt(N) * 2.0 ** -58.35 + 4 * 2.0 ** -53 + N * 2.0 ** -53
+    one = 2 * np.sqrt(N) * 2.0 ** -58.32 + 4 * 2.0 ** -53 + N * 2.0 ** -53
     assert torch.max(torch.abs(a - b)).item() < 2 ** max(squarings, 0) * (8 + 3 * max(squarings, 0)) * one
     assert not torch.equal(a, b)
     assert torch.equal(a, a.T)
