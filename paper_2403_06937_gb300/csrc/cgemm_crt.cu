@@ -447,6 +447,38 @@ __device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits) {
     a.ss = fmaf(f, f, a.ss);
 }
 
+// crt::Pieces of two numbers, and crt::residue and crt::residue_pair on them,
+// step by step the same operations two at a time (the kernel is bound by
+// instruction issue: 77 % with one number an instruction).
+struct Pieces2 {
+    uint64_t lo, a, b, c;
+};
+__device__ __forceinline__ Pieces2 pieces2(const crt::Pieces& x, const crt::Pieces& y) {
+    return Pieces2{pack2(x.lo, y.lo), pack2(x.a, y.a), pack2(x.b, y.b), pack2(x.c, y.c)};
+}
+__device__ __forceinline__ uint64_t both(float v) { return pack2(v, v); }
+__device__ __forceinline__ uint64_t congruent2(const Pieces2& x, int p) {
+    return fma2(x.c, both((float)crt::balanced_pow2(46, p)),
+                fma2(x.b, both((float)crt::balanced_pow2(33, p)), fma2(x.a, both((float)crt::balanced_pow2(20, p)), x.lo)));
+}
+__device__ __forceinline__ uint64_t balanced2(uint64_t t, int p) {
+    const uint64_t q = add2(fma2(t, both(1.0f / (float)p), both(kMagic)), both(-kMagic));
+    return fma2(q, both(-(float)p), t);
+}
+__device__ __forceinline__ void residue_pair2(const Pieces2& re, const Pieces2& im, int s, uint64_t& plus,
+                                              uint64_t& minus) {
+    const int p = crt::modulus(s);
+    const uint64_t t = congruent2(re, p), r = balanced2(congruent2(im, p), p);
+    plus = balanced2(fma2(r, both((float)crt::iota(s)), t), p);
+    minus = balanced2(fma2(r, both((float)-crt::iota(s)), t), p);
+}
+// integers up to 127 are exact in BF16: the top halves of their FP32 bits
+__device__ __forceinline__ uint32_t bf16_pair(uint64_t v) {
+    uint32_t a, b;
+    unpack2(v, a, b);
+    return __byte_perm(a, b, 0x7632);
+}
+
 template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false>
 __global__ void __launch_bounds__(128)
     crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
@@ -499,8 +531,8 @@ __global__ void __launch_bounds__(128)
         }
     };
     auto put = [](__nv_bfloat16* d, const uint32_t (&w)[CPT / 2]) {
-        if constexpr (CPT == 8)
-            *reinterpret_cast<uint4*>(d) = make_uint4(w[0], w[1], w[2], w[3]);
+        if constexpr (CPT == 4)
+            *reinterpret_cast<uint2*>(d) = make_uint2(w[0], w[1]);
         else
             *reinterpret_cast<uint32_t*>(d) = w[0];
     };
@@ -549,32 +581,28 @@ __global__ void __launch_bounds__(128)
     for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
         uint64_t xr[CPT], xi[CPT];
         load(c0, xr, xi);
-        crt::Pieces pr[CPT], pi[CPT];
+        Pieces2 pr[CPT / 2], pi[CPT / 2];
+        auto pieces = [&](uint64_t b) {
+            return crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
+        };
 #pragma unroll
-        for (int q = 0; q < CPT; q++) {
-            pr[q] = crt::split_pieces(finite ? crt::to_magnitude(xr[q], sh) : 0, (xr[q] >> 63) != 0);
-            if (!REAL) {
-                const uint64_t b = xi[q] ^ im_flip;
-                pi[q] = crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
-            }
+        for (int h = 0; h < CPT / 2; h++) {
+            pr[h] = pieces2(pieces(xr[2 * h]), pieces(xr[2 * h + 1]));
+            if (!REAL) pi[h] = pieces2(pieces(xi[2 * h] ^ im_flip), pieces(xi[2 * h + 1] ^ im_flip));
         }
         __nv_bfloat16* dst = planes + (size_t)r * Np + c0;
 #pragma unroll
         for (int s = 0; s < kModuli; s++) {
-            // integers up to 127 are exact in BF16: the top halves of their FP32 bits
             uint32_t w0[CPT / 2], w1[CPT / 2];
 #pragma unroll
             for (int h = 0; h < CPT / 2; h++) {
-                float u[2], v[2];
-#pragma unroll
-                for (int k = 0; k < 2; k++) {
-                    if (REAL)
-                        u[k] = crt::residue(pr[2 * h + k], crt::modulus(s));
-                    else
-                        crt::residue_pair(pr[2 * h + k], pi[2 * h + k], s, u[k], v[k]);
-                }
-                w0[h] = __byte_perm(__float_as_uint(u[0]), __float_as_uint(u[1]), 0x7632);
-                if (!REAL) w1[h] = __byte_perm(__float_as_uint(v[0]), __float_as_uint(v[1]), 0x7632);
+                uint64_t u, v = 0;
+                if (REAL)
+                    u = balanced2(congruent2(pr[h], crt::modulus(s)), crt::modulus(s));
+                else
+                    residue_pair2(pr[h], pi[h], s, u, v);
+                w0[h] = bf16_pair(u);
+                w1[h] = bf16_pair(v);
             }
             // plane s: re + iota im of a left operand, its conjugate re - iota im of a right one
             put(dst + (size_t)(REAL || LEFT ? s : kModuli + s) * plane, w0);
@@ -586,12 +614,13 @@ __global__ void __launch_bounds__(128)
 // ---------------------------------------------------------------- recombination
 __device__ __forceinline__ double pow2d(int e) { return __longlong_as_double((long long)(e + 1023) << 52); }
 
-// mag 2^e in FP64, e of any size.  Rounded to 53 bits and packed with integer
-// instructions (the FP64 pipe issues two instructions per clock and SM);
-// results outside the normal range take the slow way.
+// mag 2^e in FP64 (mag 0 or with its top bit at 63 or 62), e of any size.
+// Rounded to 53 bits and packed with integer instructions (the FP64 pipe
+// issues two instructions per clock and SM); results outside the normal range
+// take the slow way.
 __device__ __forceinline__ double scaled(uint64_t mag, bool neg, int e) {
-    const int lz = crt::clz64(mag);
-    const uint64_t m = mag << (lz & 63);
+    const int lz = (int)(~mag >> 63);
+    const uint64_t m = mag << lz;
     const uint64_t r = (m >> 11) + ((m >> 10) & 1);        // 53 bits, or 2^53 after a carry
     const int be = e + 11 - lz + 1075;                     // biased exponent of r's leading bit
     if (mag != 0 && be > 0 && be < 2046)
@@ -615,7 +644,7 @@ struct CrtCombine {
     const double* diag;      // [2][Np]
     const double* br;
     const double* bi;
-    double bi_sign;          // -1 when B was loaded conjugated
+    long long bi_flip;       // the sign bit when B was loaded conjugated
     int accumulate;          // MODE 0: add to Y
     double* yr;
     double* yi;
@@ -629,7 +658,7 @@ struct CrtCombine {
 // written per entry) beside 48 32-bit multiply-adds a number; at N <= 512
 // by latency, so there one column a thread (four times the threads).
 template <int MODE, int COLS>
-__global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
+__global__ void __launch_bounds__(256, 4) crt_combine_kernel(CrtCombine p) {
     constexpr int W = 8 * COLS;
     __shared__ double sr[W][33], si[W][33];   // [column of the tile][row of the tile]
     const int i0 = p.row0 + 32 * (int)blockIdx.y, j0 = W * (int)blockIdx.x;
@@ -658,7 +687,7 @@ __global__ void __launch_bounds__(256) crt_combine_kernel(CrtCombine p) {
         const bool in = j0 + ta < p.N && i0 + b < p.N;
         const size_t ob = (size_t)(j0 + ta) * p.ldb + (size_t)(i0 + b);
         sr[ta][b] = in ? p.br[ob] : 0.0;
-        si[ta][b] = in ? p.bi_sign * p.bi[ob] : 0.0;
+        si[ta][b] = in ? __longlong_as_double(__double_as_longlong(p.bi[ob]) ^ p.bi_flip) : 0.0;
     }
     const int ea = p.ea[i];
     int eb[COLS];
@@ -870,7 +899,7 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
     if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
         (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
-    const int cpt = m.Np <= 512 ? 2 : 8;
+    const int cpt = m.Np <= 512 ? 2 : 4;
     int tpr = 16;   // threads a row: a power of two, at most 128 and Np / cpt
     while (2 * tpr <= std::min(128, m.Np / cpt)) tpr *= 2;
     const unsigned grid = (unsigned)((m.Np + 128 / tpr - 1) / (128 / tpr));
@@ -879,13 +908,13 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
 #define TC_RES(I_, L_, C_) \
     crt_residue_kernel<I_, L_, C_><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, out, m.ex, m.diag)
     if (interleaved && m.left) {
-        if (cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 8);
+        if (cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
     } else if (interleaved) {
-        if (cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 8);
+        if (cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 4);
     } else if (m.left) {
-        if (cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 8);
+        if (cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 4);
     } else {
-        if (cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 8);
+        if (cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 4);
     }
 #undef TC_RES
     TC_LAUNCH_CHECK();
@@ -915,7 +944,7 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
         c.bi = bi;
         c.yr = out.yr;
         c.yi = out.yi;
-        c.bi_sign = out.conj_b ? -1.0 : 1.0;
+        c.bi_flip = out.conj_b ? LLONG_MIN : 0;
         c.accumulate = out.accumulate ? 1 : 0;
         const int cols = Np <= 512 ? 1 : 4;
         const dim3 grid((unsigned)((mode == 0 ? Np : row0 + band) / (8 * cols)), (unsigned)(band / 32));
@@ -939,13 +968,13 @@ tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) { return mat
 
 tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
     if (reinterpret_cast<uintptr_t>(a) & 15u) return fail(TC_ERR_INVALID_ARG, "real products: operand misaligned");
-    const int N = m.Np, tpr = std::min(128, N / 8);   // N a power of two
+    const int N = m.Np, tpr = std::min(128, N / 4);   // N a power of two
     const unsigned grid = (unsigned)(N / (128 / tpr));
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
     if (m.left)
-        crt_residue_kernel<false, true, 8, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, m.diag);
+        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, m.diag);
     else
-        crt_residue_kernel<false, false, 8, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, nullptr);
+        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, nullptr);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }

@@ -57,9 +57,12 @@ constexpr int inverse(int a, int p) {
     return 0;
 }
 constexpr int inverse_of_rest(int s) { return inverse((int)(product_without(s) % (u128)modulus(s)), modulus(s)); }
-// round(2^96 (k mod p) / p): the weight of a residue in the fraction x / M
+// round(2^80 (k mod p) / p): the weight of a residue in the fraction x / M
 constexpr u128 fraction(int k, int p) {
-    return ((((u128)1 << 96) * (u128)(k % p)) + (u128)(p / 2)) / (u128)p;
+    return ((((u128)1 << 80) * (u128)(k % p)) + (u128)(p / 2)) / (u128)p;
+}
+constexpr uint32_t limb(u128 f, int l) {   // 16, 32 and 32 bits, lowest first
+    return l == 0 ? (uint32_t)f & 0xFFFFu : (uint32_t)(f >> (l == 1 ? 16 : 48));
 }
 constexpr int product_bits() {
     int b = 0;
@@ -88,9 +91,9 @@ constexpr Consts make_consts() {
         const int p = modulus(s), w = inverse_of_rest(s), half = inverse(2, p);
         const u128 fr = fraction(w * half % p, p), fi = fraction(w * half % p * inverse(iota(s), p), p), f1 = fraction(w, p);
         for (int l = 0; l < 3; l++) {
-            c.re[s][l] = (uint32_t)(fr >> (32 * l));
-            c.im[s][l] = (uint32_t)(fi >> (32 * l));
-            c.real[s][l] = (uint32_t)(f1 >> (32 * l));
+            c.re[s][l] = limb(fr, l);
+            c.im[s][l] = limb(fi, l);
+            c.real[s][l] = limb(f1, l);
         }
         br += 256 * fr;
         bi += 256 * fi;
@@ -98,9 +101,10 @@ constexpr Consts make_consts() {
         c.p[s] = p;
     }
     for (int l = 0; l < 3; l++) {
-        c.re_bias[l] = (uint32_t)(br >> (32 * l));
-        c.im_bias[l] = (uint32_t)(bi >> (32 * l));
-        c.real_bias[l] = (uint32_t)(b1 >> (32 * l));
+        // (the low limb at the top of its word, as acc_finish holds it)
+        c.re_bias[l] = limb(br, l) << (l == 0 ? 16 : 0);
+        c.im_bias[l] = limb(bi, l) << (l == 0 ? 16 : 0);
+        c.real_bias[l] = limb(b1, l) << (l == 0 ? 16 : 0);
     }
     c.mbits = product_bits();
     c.mtop = (uint64_t)(product_all() >> (c.mbits - 64));
@@ -183,14 +187,16 @@ TC_CRT_HD uint64_t to_magnitude(uint64_t bits, int sh) {
 }
 
 // ---------------------------------------------------------------- recombination
-// x / M modulo 1 as a signed 96-bit fraction -> mag 2^exp2.  The fraction's
-// error is below 2^-83, so x is within 2^35 units of integers whose rows are
-// held to 2^58 (|x| < M / 2 - 2^36).
+// x / M modulo 1 as a signed 80-bit fraction (limbs of 16, 32 and 32 bits) ->
+// mag 2^exp2.  The fraction's error is below 2^-67, so x is within 2^51 units
+// of integers whose rows are held to 2^58: 2^-65 of the product of the rows'
+// norms, below the rounding of the rows (|x| < M / 2 - 2^52).
 struct Acc {
-    uint64_t a0, a1, a2;
+    uint32_t a0;
+    uint64_t a1, a2;
 };
-TC_CRT_HD void acc_add(Acc& a, uint32_t k, const uint32_t (&f)[3]) {
-    a.a0 += (uint64_t)k * f[0];
+TC_CRT_HD void acc_add(Acc& a, uint32_t k, const uint32_t (&f)[3]) {   // k < 2^9, at most sixteen times
+    a.a0 += k * f[0];
     a.a1 += (uint64_t)k * f[1];
     a.a2 += (uint64_t)k * f[2];
 }
@@ -208,44 +214,35 @@ TC_CRT_HD uint64_t mulhi_u64(uint64_t a, uint64_t b) {
     return (uint64_t)(((unsigned __int128)a * b) >> 64);
 #endif
 }
-// mag 2^exp2 (mag a 64-bit integer) with the sign returned through neg; mag = 0 for x = 0
+// mag 2^exp2 with the sign returned through neg: mag has its top bit at 63 or
+// 62, or is 0
 TC_CRT_HD uint64_t acc_finish(const Acc& a, const uint32_t (&bias)[3], const Consts& c, bool& neg, int& exp2) {
-    // carry-propagate to three 32-bit limbs modulo 2^96, minus the bias
-    uint64_t t = a.a0;
-    uint32_t l0 = (uint32_t)t;
-    t = (t >> 32) + a.a1;
+    // carry-propagate modulo 2^80; the low limb goes to the top of its word
+    uint64_t t = (uint64_t)(a.a0 >> 16) + a.a1;
+    uint32_t l0 = a.a0 << 16;
     uint32_t l1 = (uint32_t)t;
-    t = (t >> 32) + a.a2;
-    uint32_t l2 = (uint32_t)t;
-    int64_t d = (int64_t)l0 - bias[0];
-    l0 = (uint32_t)d;
-    d = (int64_t)l1 - bias[1] + (d >> 32);
-    l1 = (uint32_t)d;
-    d = (int64_t)l2 - bias[2] + (d >> 32);
-    l2 = (uint32_t)d;
-    neg = (l2 >> 31) != 0;
+    uint32_t l2 = (uint32_t)((t >> 32) + a.a2);
+    // minus the bias
+    const uint64_t v = (((uint64_t)l2 << 32) | l1) - (((uint64_t)bias[2] << 32) | bias[1]) - (l0 < bias[0] ? 1 : 0);
+    l0 -= bias[0];
+    neg = (int64_t)v < 0;
+    uint64_t hi = v;
     if (neg) {   // two's complement
-        uint64_t s = (uint64_t)(uint32_t)~l0 + 1;
-        l0 = (uint32_t)s;
-        s = (uint64_t)(uint32_t)~l1 + (s >> 32);
-        l1 = (uint32_t)s;
-        l2 = ~l2 + (uint32_t)(s >> 32);
+        hi = ~v + (l0 == 0 ? 1 : 0);
+        l0 = 0u - l0;
     }
-    const uint64_t hi = ((uint64_t)l2 << 32) | l1;
-    // the top 64 bits of the 96: |f| = top 2^(32 - lz), truncated
-    int lz = hi ? clz64(hi) : 64;
+    // the top 64 bits: |f| = top 2^(16 - lz) in units of 2^-80, truncated
+    const int lz = hi ? clz64(hi) : 64;
     uint64_t top;
-    if (lz == 0) {
+    if (lz == 0)
         top = hi;
-    } else if (lz <= 32) {
+    else if (lz <= 32)
         top = (hi << lz) | ((uint64_t)l0 >> (32 - lz));
-    } else if (lz < 64) {
+    else if (lz < 64)
         top = (hi << lz) | ((uint64_t)l0 << (lz - 32));
-    } else {
-        top = (uint64_t)l0 << 32;
-        // not normalised: below 2^-64 of M, well under the operands' own rounding
-    }
-    exp2 = 32 - lz - 96 + c.mbits;
+    else
+        top = 0;   // below 2^-64 of M, where the fraction's own error begins
+    exp2 = 16 - lz - 80 + c.mbits;
     return mulhi_u64(top, c.mtop);
 }
 

@@ -91,9 +91,9 @@ int main() {
         if ((long double)got != want) return fail("to_magnitude", -1, bits);
     }
     // recombination: random sizes, small values, both ends of its range, which stops short of M / 2 by
-    // the fraction's own error of 2^35 units (nearer than that it may wrap; the operands' rows keep
+    // the fraction's own error of 2^51 units (nearer than that it may wrap; the operands' rows keep
     // |x| below 2^116.64, M / 2 is 2^116.69)
-    const i128 M = (i128)product_all(), half = M / 2 - ((i128)1 << 36);
+    const i128 M = (i128)product_all(), half = M / 2 - ((i128)1 << 52);
     auto draw = [&](int k) {
         i128 x = (i128)(((u128)rng() << 64) | rng()) % half;
         x >>= (int)(rng() % 118);
@@ -108,9 +108,11 @@ int main() {
         if (r < -(p / 2)) r += p;
         return r;
     };
-    // 2^35 units of the fraction's 96 bits, one rounding to FP64 and the 64-bit multiply
+    // 2^51 units of the fraction (2^54 where it has fewer than 64 bits left), one rounding to FP64 and
+    // the 64-bit multiply
     auto near = [](double got, i128 x) {
-        return std::fabs(got - (double)x) <= std::ldexp(1.0, 35) + std::fabs((double)x) * std::ldexp(1.0, -52);
+        return std::fabs(got - (double)x) <= std::ldexp(1.0, 51) + (std::fabs((double)x) < std::ldexp(1.0, 56) ? std::ldexp(1.0, 54) : 0) +
+                   std::fabs((double)x) * std::ldexp(1.0, -52);
     };
     for (int k = 0; k < 300000; k++) {
         const i128 x = draw(k % 1000), y = draw((k + 1) % 1000);
