@@ -220,25 +220,27 @@ TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, 
         plan.group = tuned.tc_group;
         plan.rb = plan.shape == kShapePairWide ? cgemm_pair_rows(precision) : 32;
     }
-    auto observe = [&](int k, int row) -> tc_status {
+    auto observe = [&](int k, int row, cudaStream_t os) -> tc_status {
         const int b = order[k];
         if (!obs || !obs[b]) return TC_OK;
         const int stride = TC_OBS_STRIDE(n[b]);
         const Model* mp = params ? &models[b] : nullptr;
         return launch_observables(kRhoPlanarF32, lb[k].Rr, lb[k].Ri, mp, n[b], obs[b] + (size_t)row * stride,
-                                  lb[k].scratch, s, (size_t)lb[k].Np);
+                                  lb[k].scratch, os, (size_t)lb[k].Np);
     };
-    // one step of every system, enqueued on s
+    // one step of every system, enqueued on s; the rows (two small launches a system) are read beside
+    // the next step's first product when `side` is a branch of s
     unsigned* status = device_status_word();
-    auto one_step = [&](int step) -> tc_status {
+    auto one_step = [&](int step, SideBranch& side) -> tc_status {
         TC_TRY(cgemm_batch(precision, 0, sys_dev, count, plan, status, s));
+        TC_TRY(side.wait());   // the states are overwritten from here on
         TC_TRY(cgemm_batch(precision, 1, sys_dev, count, plan, status, s));
         if (renorm_every > 0 && step % renorm_every == 0)
             for (int k = 0; k < count; k++) TC_TRY(lowp_renorm(precision, lb[k], s));
-        for (int k = 0; k < count; k++) TC_TRY(observe(k, step));
-        return TC_OK;
+        TC_TRY(side.begin());
+        for (int k = 0; k < count; k++) TC_TRY(observe(k, step, side.stream()));
+        return side.end();
     };
-
 
     auto first = [&](cudaStream_t cs) -> tc_status {
         s = cs;
@@ -255,14 +257,18 @@ TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, 
         TC_CUDA(cudaMemcpyAsync(sys_dev, host.data(), sizeof(BatchSys) * count, cudaMemcpyHostToDevice, s));
         TC_CUDA(cudaStreamSynchronize(s));   // host copy of the descriptors may go
 
-        for (int k = 0; k < count; k++) TC_TRY(observe(k, 0));
-        if (steps > 0) TC_TRY(one_step(1));
-        return TC_OK;
+        for (int k = 0; k < count; k++) TC_TRY(observe(k, 0, s));
+        SideBranch side(s);
+        if (steps > 0) TC_TRY(one_step(1, side));
+        return side.wait();
     };
     auto rest = [&](cudaStream_t cs) -> tc_status {
         s = cs;
-        for (int k = 2; k <= steps; k++) TC_TRY(one_step(k));
-        return TC_OK;
+        SideBranch side(s);
+        tc_status st = TC_OK;
+        for (int k = 2; k <= steps && st == TC_OK; k++) st = one_step(k, side);
+        const tc_status joined = side.wait();
+        return st == TC_OK ? joined : st;
     };
     auto tail = [&](cudaStream_t cs) -> tc_status {
         s = cs;

@@ -6,6 +6,7 @@
 
 #include "cgemm_crt.cuh"
 #include "common.cuh"
+#include "graph.cuh"
 
 namespace tc {
 
@@ -106,7 +107,8 @@ struct OzSystem {
     tc_status carve(int n, Arena& ar);
     tc_status first(const double* U, const double* rho, const Model* m, double* obs, int renorm_every,
                     cudaStream_t cs);
-    tc_status step(int k, cudaStream_t cs);
+    // the row is read beside the next step's first product when `side` is a branch of cs
+    tc_status step(int k, cudaStream_t cs, SideBranch& side);
     tc_status tail(double* rho, cudaStream_t cs);
 };
 

@@ -453,30 +453,39 @@ tc_status evolve_lowp(const double* U, double* rho, int n, int steps, int precis
     const double N3 = (double)b.N * b.N * b.N;
     const double prod = (double)cgemm_products(precision);
 
-    auto one_step = [&](int k, cudaStream_t cs) -> tc_status {
+    // the observable row is read beside the next step's first product when `side` is a branch of cs
+    auto one_step = [&](int k, cudaStream_t cs, SideBranch& side) -> tc_status {
         {
             ProductTimer t(8.0 * N3 * prod, cs);
             TC_TRY(cgemm_tc(precision, 0, tmU, tmR, e1, cs, tune.tc_stages, &sp.wU, &sp.wR));
         }
+        TC_TRY(side.wait());   // rho is overwritten from here on
         {
             ProductTimer t(4.0 * N3 * prod, cs);
             TC_TRY(cgemm_tc(precision, 1, tmU, tmX, e2, cs, tune.tc_stages, &sp.wU, &sp.wX));
         }
         if (renorm_every > 0 && k % renorm_every == 0) TC_TRY(lowp_renorm(precision, b, cs));
-        if (obs)
-            TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs + (size_t)k * stride, b.scratch, cs,
-                                      (size_t)b.Np));
+        if (obs) {
+            TC_TRY(side.begin());
+            TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs + (size_t)k * stride, b.scratch,
+                                      side.stream(), (size_t)b.Np));
+            TC_TRY(side.end());
+        }
         return TC_OK;
     };
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(lowp_prep(precision, U, rho, b, cs));
         if (obs) TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs, b.scratch, cs, (size_t)b.Np));
-        if (steps >= 1) TC_TRY(one_step(1, cs));
-        return TC_OK;
+        SideBranch side(cs);
+        if (steps >= 1) TC_TRY(one_step(1, cs, side));
+        return side.wait();
     };
     auto rest = [&](cudaStream_t cs) -> tc_status {
-        for (int k = 2; k <= steps; k++) TC_TRY(one_step(k, cs));
-        return TC_OK;
+        SideBranch side(cs);
+        tc_status st = TC_OK;
+        for (int k = 2; k <= steps && st == TC_OK; k++) st = one_step(k, cs, side);
+        const tc_status joined = side.wait();
+        return st == TC_OK ? joined : st;
     };
     auto tail = [&](cudaStream_t cs) -> tc_status { return lowp_finish(b, rho, cs); };
     return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());

@@ -118,7 +118,7 @@ tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, d
     return TC_OK;
 }
 
-tc_status OzSystem::step(int k, cudaStream_t cs) {
+tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side) {
     const size_t NN = (size_t)Np * Np;
     const double N3 = (double)N * N * N;
     const OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
@@ -128,6 +128,7 @@ tc_status OzSystem::step(int k, cudaStream_t cs) {
         TC_TRY(oz_product(0, Us, Ps, Rr, Ri, N, (size_t)Np, X, group, cs));
     }
     TC_TRY(oz_mat_load(Ps, Xr, Xi, false, false, N, (size_t)Np, cs));
+    TC_TRY(side.wait());   // rho is overwritten from here on
     {
         ProductTimer t(4.0 * N3 * oz_products(), cs);   // rho' = U X^H, Hermitian half + mirror
         TC_TRY(oz_product(1, Us, Ps, Xr, Xi, N, (size_t)Np, R, group, cs));
@@ -138,9 +139,12 @@ tc_status OzSystem::step(int k, cudaStream_t cs) {
         scale_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(Rr, Ri, Np, scratch, device_status_word());
         TC_LAUNCH_CHECK();
     }
-    if (obs)
-        TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs + (size_t)k * TC_OBS_STRIDE(n), scratch, cs,
-                                  (size_t)Np));
+    if (obs) {
+        TC_TRY(side.begin());
+        TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs + (size_t)k * TC_OBS_STRIDE(n), scratch,
+                                  side.stream(), (size_t)Np));
+        TC_TRY(side.end());
+    }
     return TC_OK;
 }
 
@@ -171,11 +175,16 @@ tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_e
     }
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(z.first(U, rho, m, obs, renorm_every, cs));
-        return z.step(1, cs);
+        SideBranch side(cs);
+        TC_TRY(z.step(1, cs, side));
+        return side.wait();
     };
     auto rest = [&](cudaStream_t cs) -> tc_status {
-        for (int k = 2; k <= steps; k++) TC_TRY(z.step(k, cs));
-        return TC_OK;
+        SideBranch side(cs);
+        tc_status st = TC_OK;
+        for (int k = 2; k <= steps && st == TC_OK; k++) st = z.step(k, cs, side);
+        const tc_status joined = side.wait();
+        return st == TC_OK ? joined : st;
     };
     auto tail = [&](cudaStream_t cs) -> tc_status { return z.tail(rho, cs); };
     return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());

@@ -8,6 +8,8 @@ namespace {
 struct GraphStream {
     cudaStream_t s = nullptr;
     cudaEvent_t before = nullptr, after = nullptr;
+    cudaStream_t side = nullptr;                     // SideBranch's stream and events
+    cudaEvent_t fork = nullptr, join = nullptr;
 };
 std::mutex g_mu;
 GraphStream g_gs[64];
@@ -22,6 +24,9 @@ tc_status graph_stream(GraphStream** out) {
         TC_CUDA(cudaStreamCreateWithFlags(&g.s, cudaStreamNonBlocking));
         TC_CUDA(cudaEventCreateWithFlags(&g.before, cudaEventDisableTiming));
         TC_CUDA(cudaEventCreateWithFlags(&g.after, cudaEventDisableTiming));
+        TC_CUDA(cudaStreamCreateWithFlags(&g.side, cudaStreamNonBlocking));
+        TC_CUDA(cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming));
+        TC_CUDA(cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming));
     }
     *out = &g;
     return TC_OK;
@@ -72,6 +77,40 @@ tc_status run_captured(cudaStream_t user, const std::function<tc_status(cudaStre
     cudaEventRecord(gs->after, s);
     cudaStreamWaitEvent(user, gs->after, 0);
     return st;
+}
+
+SideBranch::SideBranch(cudaStream_t main) : main_(main) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return;
+    std::lock_guard<std::mutex> lk(g_mu);
+    const GraphStream& g = g_gs[dev];
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (!g.join || main != g.s || cudaStreamIsCapturing(main, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusActive)
+        return;
+    side_ = g.side;
+    fork_ = g.fork;
+    join_ = g.join;
+}
+
+tc_status SideBranch::begin() {
+    if (!side_) return TC_OK;
+    TC_CUDA(cudaEventRecord(fork_, main_));
+    TC_CUDA(cudaStreamWaitEvent(side_, fork_, 0));
+    pending_ = true;
+    return TC_OK;
+}
+
+tc_status SideBranch::end() {
+    if (!side_) return TC_OK;
+    TC_CUDA(cudaEventRecord(join_, side_));
+    return TC_OK;
+}
+
+tc_status SideBranch::wait() {
+    if (!pending_) return TC_OK;
+    TC_CUDA(cudaStreamWaitEvent(main_, join_, 0));
+    pending_ = false;
+    return TC_OK;
 }
 
 }  // namespace tc

@@ -16,4 +16,26 @@ tc_status run_captured(cudaStream_t user, const std::function<tc_status(cudaStre
                        const std::function<tc_status(cudaStream_t)>& rest,
                        const std::function<tc_status(cudaStream_t)>& tail, bool capture);
 
+// A branch beside the main sequence of a step loop, for work that only reads
+// what the main sequence leaves alone for a while (the observable row of a
+// step beside the next step's first product: at n = 8 two of a step's eight
+// launches, 12 of 50 us).  While `main` is the library stream being captured
+// by run_captured, begin() forks the branch's stream from it, end() marks the
+// branch's end and wait() joins it; otherwise stream() is `main` itself and
+// nothing is forked.  Every begin() needs its end() and wait() before the
+// capture ends.
+class SideBranch {
+  public:
+    explicit SideBranch(cudaStream_t main);
+    cudaStream_t stream() const { return side_ ? side_ : main_; }
+    tc_status begin();
+    tc_status end();
+    tc_status wait();
+
+  private:
+    cudaStream_t main_, side_ = nullptr;
+    cudaEvent_t fork_ = nullptr, join_ = nullptr;
+    bool pending_ = false;
+};
+
 }  // namespace tc
