@@ -224,18 +224,24 @@ tc_status launch(const CUtensorMap& tmU, const CUtensorMap& tmP, const CgemmEpi&
 // TMA swizzle): a stage is 3 S tiles of 128 RB bytes and RB / 32 MMA K steps
 // (split_pair_stages, cgemm_dev.cuh).
 
-template <int KIND, int S, int RB, int MODE>
+// NC: columns of a complex tile, 128, or 64 for launches whose tiles would
+// leave half of the SMs idle (n <= 10): twice the CTAs with half the MMA time
+// and half the epilogue each (an N = 128 MMA re-reads its A operand for half
+// the work, which with the TMA writes takes all of the shared memory's
+// bandwidth, so larger launches keep 128).
+template <int KIND, int S, int RB, int MODE, int NC>
 __global__ void __launch_bounds__(kPairThreads, 1)
     cgemm_tc_pair_kernel(const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmP,
                          CgemmEpi ep) {
-    constexpr int STAGES = split_pair_stages<S, RB>();
+    constexpr int STAGES = split_pair_stages<S, RB, NC>();
     static_assert(STAGES >= 2, "ring too small for this row width");
-    constexpr int kTile = 128 * RB;          // one 128-row operand tile
-    constexpr int kStage = 3 * S * kTile;    // own U_r, U_i parts + own half of each B part
+    constexpr int kTile = 128 * RB;          // one 128-row operand tile of U
+    constexpr int kBTile = NC * RB;          // own half of a B part
+    constexpr int kStage = split_pair_stage_bytes<S, RB, NC>();   // own U_r, U_i parts + own half of each B part
     constexpr int kElem = KIND == 0 ? 2 : 4;
     constexpr int kKPerStage = RB / kElem;
     constexpr int kSteps = RB / 32;          // MMA K steps per stage
-    constexpr uint32_t kIdesc = make_idesc(KIND == 0 ? 1u : 2u, 256u, 256u);
+    constexpr uint32_t kIdesc = make_idesc(KIND == 0 ? 1u : 2u, 256u, 2u * NC);
 
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -251,7 +257,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     const uint32_t rank = cluster_ctarank();
     int I, J;
     pair_tile_rows_range(MODE, ep.tiles, ep.group > 1 ? ep.group / 2 : 1, ep.hi > 0 ? ep.lo : 0,
-                         ep.hi > 0 ? ep.hi : ep.tiles, (int)(blockIdx.x >> 1), (int)rank, I, J);
+                         ep.hi > 0 ? ep.hi : ep.tiles, (int)(blockIdx.x >> 1) / (128 / NC), (int)rank, I, J);
+    const bool above = MODE == 1 && J > I;                                   // not written
+    if (NC != 128) J = J * (128 / NC) + (int)(blockIdx.x >> 1) % (128 / NC);   // in tiles of NC columns
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; s++) {
@@ -305,7 +313,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                             tma_load_3d(saddr(st + (part * S + a) * kTile), &tmU, fb, kx, I * 128, part * S + a);
 #pragma unroll
                     for (int b = 0; b < S; b++)   // P_r part b
-                        tma_load_3d(saddr(st + (2 * S + b) * kTile), &tmP, fb, kx, J * 128, b);
+                        tma_load_3d(saddr(st + 2 * S * kTile + b * kBTile), &tmP, fb, kx, J * NC, b);
                 } else {
                     const uint32_t fb = lead_full + 8u * (uint32_t)s;
 #pragma unroll
@@ -316,7 +324,7 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                                              part * S + a);
 #pragma unroll
                     for (int b = 0; b < S; b++)   // P_i part b
-                        tma_load_3d_pair(saddr(st + (2 * S + b) * kTile), &tmP, fb, kx, J * 128, S + b);
+                        tma_load_3d_pair(saddr(st + 2 * S * kTile + b * kBTile), &tmP, fb, kx, J * NC, S + b);
                 }
             }
             const int from = issued - STAGES > 0 ? issued - STAGES : 0;
@@ -353,12 +361,12 @@ __global__ void __launch_bounds__(kPairThreads, 1)
                     const uint64_t off = 2u * (uint64_t)ks;   // 32 bytes of K further in each row
 #pragma unroll
                     for (int p = 0; p < Pairs<S>::n; p++) {
-                        const uint64_t bd = desc_kmajor<RB>(saddr(st + (2 * S + Pairs<S>::b(p)) * kTile)) + off;
+                        const uint64_t bd = desc_kmajor<RB>(saddr(st + 2 * S * kTile + Pairs<S>::b(p) * kBTile)) + off;
 #pragma unroll
                         for (int part = 0; part < 2; part++) {
                             const uint64_t ad =
                                 desc_kmajor<RB>(saddr(st + (part * S + Pairs<S>::a(p)) * kTile)) + off;
-                            umma_pair(tmem + part * 256, ad, bd, kIdesc, (kb > 0 || ks > 0 || p > 0) ? 1u : 0u);
+                            umma_pair(tmem + part * 2 * NC, ad, bd, kIdesc, (kb > 0 || ks > 0 || p > 0) ? 1u : 0u);
                         }
                     }
                 }
@@ -376,9 +384,9 @@ __global__ void __launch_bounds__(kPairThreads, 1)
         // ---------------------------------------------------------- epilogue (both CTAs, own tile)
         const bool ok = mbar_wait_bounded_cluster(accum, 0u, abort, lim, 128);
         tc_fence_after();
-        if (ok && !*abort && !(MODE == 1 && J > I))
-            cg::epilogue_tile<KIND, S, MODE>(tmem, warp & 3, lane, I, J, ep.Np, ep.pr, ep.pi, ep.parts, ep.yr, ep.yi,
-                                             64 * (warp >> 2), 64 * (warp >> 2) + 64);
+        if (ok && !*abort && !above)
+            cg::epilogue_tile<KIND, S, MODE, NC>(tmem, warp & 3, lane, I, J, ep.Np, ep.pr, ep.pi, ep.parts, ep.yr,
+                                                 ep.yi, NC / 2 * (warp >> 2), NC / 2 * (warp >> 2) + NC / 2);
         if (!ok || *abort) {
             if (threadIdx.x == 0) {
                 atomicOr(ep.status, kStatusTimeout);
@@ -397,10 +405,10 @@ __global__ void __launch_bounds__(kPairThreads, 1)
     }
 }
 
-template <int KIND, int S, int RB, int MODE>
+template <int KIND, int S, int RB, int MODE, int NC = 128>
 tc_status launch_pair(const CUtensorMap& tmU, const CUtensorMap& tmP, const CgemmEpi& ep, cudaStream_t s) {
-    auto k = cgemm_tc_pair_kernel<KIND, S, RB, MODE>;
-    constexpr int smem = split_pair_smem<S, RB>();
+    auto k = cgemm_tc_pair_kernel<KIND, S, RB, MODE, NC>;
+    constexpr int smem = split_pair_smem<S, RB, NC>();
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -410,7 +418,7 @@ tc_status launch_pair(const CUtensorMap& tmU, const CUtensorMap& tmP, const Cgem
         attr_set[dev] = true;
     }
     const int lo = ep.hi > 0 ? ep.lo : 0, hi = ep.hi > 0 ? ep.hi : ep.tiles;
-    const unsigned pairs = (unsigned)pair_count(MODE, ep.tiles, lo, hi);
+    const unsigned pairs = (unsigned)pair_count(MODE, ep.tiles, lo, hi) * (128 / NC);
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3(2 * pairs);
     cfg.blockDim = dim3(kPairThreads);
@@ -435,6 +443,15 @@ std::atomic<unsigned long long> g_inject_wait{0};
 // -1: not read yet; else TC_GEMM_PAIRS from the environment (0: kShapeAuto
 // resolves to single CTAs; anything else, or unset: to CTA pairs)
 std::atomic<int> g_pairs{-1};
+}  // namespace
+
+namespace {
+int sm_count() {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
 }  // namespace
 
 int cgemm_resolve_shape(int shape) {
@@ -477,7 +494,8 @@ int cgemm_pair_rows(int precision) {
 }
 
 tc_status cgemm_tc(int precision, int mode, const CUtensorMap& tmU, const CUtensorMap& tmP, const CgemmEpi& ep_in,
-                   cudaStream_t s, int stages, const CUtensorMap* tmU_w, const CUtensorMap* tmP_w) {
+                   cudaStream_t s, int stages, const CUtensorMap* tmU_w, const CUtensorMap* tmP_w,
+                   const CUtensorMap* tmP_n) {
     CgemmEpi ep = ep_in;
     if (g_inject_count.load() > 0 && g_inject_count.fetch_sub(1) > 0) {
         ep.withhold = 1;
@@ -508,6 +526,18 @@ tc_status cgemm_tc(int precision, int mode, const CUtensorMap& tmU, const CUtens
         const CUtensorMap& u = wide ? *tmU_w : tmU;
         const CUtensorMap& p = wide ? *tmP_w : tmP;
         const int rb = wide ? cgemm_pair_rows(precision) : 32;
+        // columns in tiles of 64 while those fit one wave (76 pairs on 152 SMs): n <= 10.  Split-BF16, the two
+        // products of a step: n = 8 37 + 49 -> 22 + 24 us, n = 10 76 + 88 -> 46 + 47 us
+        const bool whole = ep.hi <= 0;
+        if (wide && tmP_n && whole && 2 * pair_count(mode, ep.tiles, 0, ep.tiles) <= sm_count() / 2) {
+#define TC_NARROW(K, S_, RB_)                                              \
+    if (rb == RB_) return mode == 0 ? launch_pair<K, S_, RB_, 0, 64>(u, *tmP_n, ep, s) \
+                                    : launch_pair<K, S_, RB_, 1, 64>(u, *tmP_n, ep, s)
+            if (precision == TC_BF16X3) TC_NARROW(0, 3, 64);
+            if (precision == TC_TF32) TC_NARROW(1, 1, 128);
+            if (precision == TC_TF32X3) TC_NARROW(1, 2, 64);
+#undef TC_NARROW
+        }
 #define TC_PAIR(K, S_, RB_) \
     return mode == 0 ? launch_pair<K, S_, RB_, 0>(u, p, ep, s) : launch_pair<K, S_, RB_, 1>(u, p, ep, s)
         switch (precision) {

@@ -401,6 +401,7 @@ namespace {
 struct StepPlan {
     CUtensorMap tmU, tmR, tmX;
     CUtensorMap wU, wR, wX;   // cgemm_pair_rows()-byte rows, for the CTA-pair kernel
+    CUtensorMap nR, nX;       // the same in boxes of 64 rows, for its narrow column tiles
     CgemmEpi e1;   // X = rho^H + V rho^H
     CgemmEpi e2;   // rho' = X^H + V X^H
     TuneChoice tune;
@@ -414,6 +415,8 @@ tc_status plan_step(int n, int precision, const LowpBufs& b, StepPlan& p) {
     TC_TRY(make_part_map_rows(&p.wU, b.Uparts, b.Np, 2 * b.S, precision, rows));
     TC_TRY(make_part_map_rows(&p.wR, b.Rparts, b.Np, 2 * b.S, precision, rows));
     TC_TRY(make_part_map_rows(&p.wX, b.Xparts, b.Np, 2 * b.S, precision, rows));
+    TC_TRY(make_part_map_rows(&p.nR, b.Rparts, b.Np, 2 * b.S, precision, rows, 64));
+    TC_TRY(make_part_map_rows(&p.nX, b.Xparts, b.Np, 2 * b.S, precision, rows, 64));
     p.tune = tune_lookup(n, precision);
     p.e1 = CgemmEpi{};
     p.e1.Np = b.Np;
@@ -457,12 +460,12 @@ tc_status evolve_lowp(const double* U, double* rho, int n, int steps, int precis
     auto one_step = [&](int k, cudaStream_t cs, SideBranch& side) -> tc_status {
         {
             ProductTimer t(8.0 * N3 * prod, cs);
-            TC_TRY(cgemm_tc(precision, 0, tmU, tmR, e1, cs, tune.tc_stages, &sp.wU, &sp.wR));
+            TC_TRY(cgemm_tc(precision, 0, tmU, tmR, e1, cs, tune.tc_stages, &sp.wU, &sp.wR, &sp.nR));
         }
         TC_TRY(side.wait());   // rho is overwritten from here on
         {
             ProductTimer t(4.0 * N3 * prod, cs);
-            TC_TRY(cgemm_tc(precision, 1, tmU, tmX, e2, cs, tune.tc_stages, &sp.wU, &sp.wX));
+            TC_TRY(cgemm_tc(precision, 1, tmU, tmX, e2, cs, tune.tc_stages, &sp.wU, &sp.wX, &sp.nX));
         }
         if (renorm_every > 0 && k % renorm_every == 0) TC_TRY(lowp_renorm(precision, b, cs));
         if (obs) {
@@ -651,7 +654,7 @@ tc_status evolve_lowp_host_blocks(const double* U, double* rho_host, double* rho
         e.hi = (c + 1) * T / C;
         {
             ProductTimer t(tile_flops * (double)T * (e.hi - e.lo), s);
-            TC_TRY(cgemm_tc(precision, 0, sp.tmU, sp.tmR, e, s, sp.tune.tc_stages, &sp.wU, &sp.wR));
+            TC_TRY(cgemm_tc(precision, 0, sp.tmU, sp.tmR, e, s, sp.tune.tc_stages, &sp.wU, &sp.wR, &sp.nR));
         }
         mark("x", c, s);
     }
@@ -690,13 +693,13 @@ tc_status evolve_lowp_host_blocks(const double* U, double* rho_host, double* rho
     for (int k = 1; k <= steps; k++) {
         if (k > 1) {
             ProductTimer t(tile_flops * (double)T * T, s);
-            TC_TRY(cgemm_tc(precision, 0, sp.tmU, sp.tmR, sp.e1, s, sp.tune.tc_stages, &sp.wU, &sp.wR));
+            TC_TRY(cgemm_tc(precision, 0, sp.tmU, sp.tmR, sp.e1, s, sp.tune.tc_stages, &sp.wU, &sp.wR, &sp.nR));
         }
         const bool renorm = renorm_every > 0 && k % renorm_every == 0;
         if (k < steps || renorm) {
             {
                 ProductTimer t(tile_flops * 0.5 * T * (T + 1.0), s);
-                TC_TRY(cgemm_tc(precision, 1, sp.tmU, sp.tmX, sp.e2, s, sp.tune.tc_stages, &sp.wU, &sp.wX));
+                TC_TRY(cgemm_tc(precision, 1, sp.tmU, sp.tmX, sp.e2, s, sp.tune.tc_stages, &sp.wU, &sp.wX, &sp.nX));
             }
             if (renorm) TC_TRY(lowp_renorm(precision, b, s));
             if (obs) TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs + (size_t)k * stride, b.scratch,
@@ -716,7 +719,7 @@ tc_status evolve_lowp_host_blocks(const double* U, double* rho_host, double* rho
             {
                 // the block-lower tiles of rows [lo, hi)
                 ProductTimer t(tile_flops * 0.5 * ((double)e.hi * (e.hi + 1) - (double)e.lo * (e.lo + 1)), s);
-                TC_TRY(cgemm_tc(precision, 1, sp.tmU, sp.tmX, e, s, sp.tune.tc_stages, &sp.wU, &sp.wX));
+                TC_TRY(cgemm_tc(precision, 1, sp.tmU, sp.tmX, e, s, sp.tune.tc_stages, &sp.wU, &sp.wX, &sp.nX));
             }
             mark("y", c, s);
             TC_TRY(out_rows(c));

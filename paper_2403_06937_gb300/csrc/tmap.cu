@@ -41,7 +41,8 @@ tc_status make_part_map(CUtensorMap* map, const void* base, int Np, int planes, 
     return make_part_map_rows(map, base, Np, planes, precision, 32);
 }
 
-tc_status make_part_map_rows(CUtensorMap* map, const void* base, int Np, int planes, int precision, int row_bytes) {
+tc_status make_part_map_rows(CUtensorMap* map, const void* base, int Np, int planes, int precision, int row_bytes,
+                             int box_rows) {
     if (row_bytes != 32 && row_bytes != 64 && row_bytes != 128)
         return fail(TC_ERR_INVALID_ARG, "tensor map: rows of 32, 64 or 128 bytes");
     PFN_cuTensorMapEncodeTiled_v12000 enc;
@@ -51,7 +52,7 @@ tc_status make_part_map_rows(CUtensorMap* map, const void* base, int Np, int pla
         return fail(TC_ERR_INVALID_ARG, "operand planes must be 16-byte aligned with 16-byte row pitch");
     cuuint64_t dims[3] = {(cuuint64_t)Np, (cuuint64_t)Np, (cuuint64_t)planes};
     cuuint64_t strides[2] = {(cuuint64_t)Np * E, (cuuint64_t)Np * (cuuint64_t)Np * E};
-    cuuint32_t box[3] = {(cuuint32_t)(row_bytes / E), 128u, 1u};
+    cuuint32_t box[3] = {(cuuint32_t)(row_bytes / E), (cuuint32_t)box_rows, 1u};
     cuuint32_t estr[3] = {1u, 1u, 1u};
     CUtensorMapDataType dt = E == 2 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32;
     CUresult r = enc(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,

@@ -380,6 +380,9 @@ TC_API tc_status tc_autotune(int n, int precision, void* work, size_t work_bytes
         TC_TRY(make_part_map_rows(&wU, b.Uparts, b.Np, 2 * b.S, precision, rows));
         TC_TRY(make_part_map_rows(&wR, b.Rparts, b.Np, 2 * b.S, precision, rows));
         TC_TRY(make_part_map_rows(&wX, b.Xparts, b.Np, 2 * b.S, precision, rows));
+        CUtensorMap nR, nX;       // its narrow column tiles (small launches)
+        TC_TRY(make_part_map_rows(&nR, b.Rparts, b.Np, 2 * b.S, precision, rows, 64));
+        TC_TRY(make_part_map_rows(&nX, b.Xparts, b.Np, 2 * b.S, precision, rows, 64));
         CgemmEpi e{};   // X = rho^H + V rho^H
         e.Np = b.Np;
         e.tiles = b.Np / 128;
@@ -414,8 +417,8 @@ TC_API tc_status tc_autotune(int n, int precision, void* work, size_t work_bytes
         auto step = [&](const Cand& cd) {
             e.group = e2.group = cd.group;
             e.shape = e2.shape = cd.shape;
-            tc_status st = cgemm_tc(precision, 0, tmU, tmR, e, s, cd.stages, &wU, &wR);
-            return st == TC_OK ? cgemm_tc(precision, 1, tmU, tmX, e2, s, cd.stages, &wU, &wX) : st;
+            tc_status st = cgemm_tc(precision, 0, tmU, tmR, e, s, cd.stages, &wU, &wR, &nR);
+            return st == TC_OK ? cgemm_tc(precision, 1, tmU, tmX, e2, s, cd.stages, &wU, &wX, &nX) : st;
         };
         std::vector<double> score;
         TC_TRY(score_configs(s, (int)cands.size(), [&](int i) { return step(cands[i]); }, score));
