@@ -18,7 +18,7 @@ struct BatchSys {   // aligned as CUtensorMap (at least 64 bytes)
     CUtensorMap tmX_w;
     float* Rr;
     float* Ri;
-    void* Rparts;
+    void* Rparts;        // nullptr: the Hermitian product writes no parts
     float* Xr;
     float* Xi;
     void* Xparts;

@@ -177,7 +177,7 @@ __device__ __forceinline__ void store_rows(__nv_bfloat16* base, size_t pitch, in
 // column tile J (NC = 128 or 64 columns), by the four warps of the lane
 // quarters `quarter` = 0..3: each reads TMEM lanes 32 quarter .. + 31
 // (row i of the tile) and writes Y[i][j] = conj(P[j][i]) + (V P^H)[i][j] as
-// FP32 planes and operand parts; MODE 1 keeps the block-lower part of a
+// FP32 planes and operand parts (MODE 1 with parts_v == nullptr: planes only); MODE 1 keeps the block-lower part of a
 // diagonal tile and mirrors the conjugate transpose.  src_*: FP32 planes of P
 // (row stride np_).
 //
@@ -246,6 +246,7 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem, int quarter, int la
         // part by part (fewer registers than all parts of both planes at once)
 #pragma unroll
         for (int im = 0; im < 2; im++) {
+            if (MODE == 1 && !parts) break;
             float rest[16];
 #pragma unroll
             for (int q = 0; q < 16; q++) rest[q] = im ? yi[q] : yr[q];
@@ -262,13 +263,15 @@ __device__ __forceinline__ void epilogue_tile(uint32_t tmem, int quarter, int la
 #pragma unroll
             for (int q = 0; q < 16; q++) {
                 const size_t gj = gj0 + q;
-                T a[S], b[S];
-                P::split(yr[q], a);
-                P::split(-yi[q], b);
+                if (parts) {
+                    T a[S], b[S];
+                    P::split(yr[q], a);
+                    P::split(-yi[q], b);
 #pragma unroll
-                for (int s = 0; s < S; s++) {
-                    parts[(size_t)s * plane + gj * Np + gi] = a[s];
-                    parts[(size_t)(S + s) * plane + gj * Np + gi] = b[s];
+                    for (int s = 0; s < S; s++) {
+                        parts[(size_t)s * plane + gj * Np + gi] = a[s];
+                        parts[(size_t)(S + s) * plane + gj * Np + gi] = b[s];
+                    }
                 }
                 out_r[gj * Np + gi] = yr[q];
                 out_i[gj * Np + gi] = -yi[q];

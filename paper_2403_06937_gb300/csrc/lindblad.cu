@@ -306,7 +306,8 @@ __global__ void obs_partial_kernel(BlockSet bs, Model m, int has_model, const in
             // FP32 planes: the squares of each group of four entries summed in FP32
             // (fused multiply-adds), the group sums carried in FP64 (GB300 issues FP64
             // at a small fraction of its FP32 rate)
-            for (; c + 96 < d; c += 128) {
+#pragma unroll 4
+            for (; c + 96 < d; c += 128) {   // the loads of four groups in flight
                 const float x0 = re[row + c], x1 = re[row + c + 32], x2 = re[row + c + 64], x3 = re[row + c + 96];
                 const float y0 = im[row + c], y1 = im[row + c + 32], y2 = im[row + c + 64], y3 = im[row + c + 96];
                 const float q01 = fmaf(y1, y1, fmaf(x1, x1, fmaf(y0, y0, x0 * x0)));
@@ -576,7 +577,7 @@ tc_status evolve_lowp_t(const Layout& L, const Model& m, int precision, double k
         TC_TRY(batch_plan_add(plan, h, precision, Np, up.p[k], rp.p[k], xp.p[k]));
         h.Rr = Rr + bs.off[k];
         h.Ri = Ri + bs.off[k];
-        h.Rparts = rp.p[k];
+        h.Rparts = damp ? nullptr : rp.p[k];   // with damping the first half step rebuilds rho's parts
         h.Xr = Xr + bs.off[k];
         h.Xi = Xi + bs.off[k];
         h.Xparts = xp.p[k];
@@ -594,9 +595,14 @@ tc_status evolve_lowp_t(const Layout& L, const Model& m, int precision, double k
             ProductTimer pt(flops * prod * (4.0 / 12.0), cs);   // rho_k = X_k U_k^dag, Hermitian halves
             TC_TRY(cgemm_batch(precision, 1, sys_dev, n + 1, plan, status, cs));
         }
-        if (damp) TC_TRY((launch_damping<float, KIND, S>(L, bs, kappa, 0.5 * dt, t, Rr, Ri, rp, cs)));
-        if (renorm_every > 0 && k % renorm_every == 0)
-            TC_TRY((launch_block_renorm<float, KIND, S>(L, bs, Rr, Ri, rp, scratch, cs)));
+        // what follows is the next step's first half damping or the end: no operand parts from here on
+        if (damp) TC_TRY((launch_damping<float, KIND, 0>(L, bs, kappa, 0.5 * dt, t, Rr, Ri, PartsSet{}, cs)));
+        if (renorm_every > 0 && k % renorm_every == 0) {
+            if (damp)
+                TC_TRY((launch_block_renorm<float, KIND, 0>(L, bs, Rr, Ri, PartsSet{}, scratch, cs)));
+            else
+                TC_TRY((launch_block_renorm<float, KIND, S>(L, bs, Rr, Ri, rp, scratch, cs)));
+        }
         if (obs) TC_TRY(launch_block_observables<float>(L, bs, m, t, Rr, Ri, obs + (size_t)k * stride, scratch, cs));
         return TC_OK;
     };
@@ -678,14 +684,41 @@ __global__ void blocks_join_pad_kernel(BlockSet bs, BlockSet pk, const double* _
     }
 }
 
+// Blocks of up to this dimension run on the DMMA GEMM (two launches of a few
+// 32 x 32 tiles; six launches on 128 x 128 padding otherwise).
+constexpr int kDmmaBlock = 64;
+
+// interleaved d x d -> FP64 planes of row stride Np
+__global__ void split_block_kernel(const double2* __restrict__ src, int d, int Np, double* __restrict__ re,
+                                   double* __restrict__ im) {
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < d * d; e += gridDim.x * blockDim.x) {
+        const double2 v = src[e];
+        const size_t o = (size_t)(e / d) * Np + e % d;
+        re[o] = v.x;
+        im[o] = v.y;
+    }
+}
+
+// From n = 13 on one left operand serves every block, loaded anew in each
+// step (n = 14: 1.9e9 elements of U_k would take 120 GB of residues; loading
+// them costs about 1 % of a step).
+bool shared_left(int n) { return n >= 13; }
+
 size_t evolve_oz_bytes_blocks(int n) {
     const Layout& L = layout_of(n);
     const size_t PT = padded_total(L);
     const int NpMax = padded(L.N);
     size_t b = tables_bytes(n) + 2 * round256(PT * sizeof(double));
-    for (int k = 0; k <= n; k++) b += oz_mat_bytes(padded(L.dims[k]), true);   // U_k slices
-    b += oz_mat_bytes(NpMax, false) + oz_scratch_bytes(NpMax);            // B operand, scratch of the products
-    b += 2 * round256((size_t)NpMax * NpMax * sizeof(double));            // X planes
+    if (shared_left(n)) b += oz_mat_bytes(NpMax, true);
+    for (int k = 0; k <= n; k++) {
+        const size_t Np = (size_t)padded(L.dims[k]);
+        if (L.dims[k] <= kDmmaBlock)
+            b += 2 * round256(Np * Np * sizeof(double));
+        else if (!shared_left(n))
+            b += oz_mat_bytes((int)Np, true);
+    }
+    b += oz_mat_bytes(NpMax, false) + oz_scratch_bytes(NpMax);   // B operand, scratch of the products
+    b += 2 * round256((size_t)NpMax * NpMax * sizeof(double));   // X planes
     return b + obs_scratch_bytes(L) + 256;
 }
 
@@ -700,7 +733,20 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     double* Rr = ar.take<double>(PT);
     double* Ri = ar.take<double>(PT);
     std::vector<OzMat> Uk(n + 1);
-    for (int k = 0; k <= n; k++) TC_TRY(oz_mat_init(Uk[k], ar, padded(L.dims[k]), true));
+    std::vector<double*> Ur(n + 1, nullptr), Ui(n + 1, nullptr);   // planes of the small blocks
+    OzMat Amax{};
+    if (shared_left(n)) TC_TRY(oz_mat_init(Amax, ar, NpMax, true));
+    for (int k = 0; k <= n; k++) {
+        const int Np = padded(L.dims[k]);
+        if (L.dims[k] <= kDmmaBlock) {
+            Ur[k] = ar.take<double>((size_t)Np * Np);
+            Ui[k] = ar.take<double>((size_t)Np * Np);
+        } else if (shared_left(n)) {
+            TC_TRY(oz_mat_view(Uk[k], Amax, Np));
+        } else {
+            TC_TRY(oz_mat_init(Uk[k], ar, Np, true));
+        }
+    }
     OzMat Bmax{};
     TC_TRY(oz_mat_init(Bmax, ar, NpMax, false));
     double* Xr = ar.take<double>(NN);
@@ -724,6 +770,26 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
             double* rr = Rr + bs.off[k];
             double* ri = Ri + bs.off[k];
             const double d3 = (double)d * d * d;
+            if (d <= kDmmaBlock) {
+                GemmF64 g1{};
+                g1.M = g1.N = g1.K = d;
+                g1.Ar = Ur[k]; g1.Ai = Ui[k]; g1.lda = Np;
+                g1.Br = rr; g1.Bi = ri; g1.ldb = Np;
+                g1.Cr = Xr; g1.Ci = Xi; g1.ldc = Np;
+                g1.alpha = 1.0;
+                g1.cplx = 1;
+                g1.tile = 32;
+                GemmF64 g2 = g1;
+                g2.Ar = Xr; g2.Ai = Xi;
+                g2.Br = Ur[k]; g2.Bi = Ui[k]; g2.conjB = 1;
+                g2.Cr = rr; g2.Ci = ri;
+                g2.herm_lower = 1;
+                TC_TRY(gemm_f64(g1, cs));
+                TC_TRY(gemm_f64(g2, cs));
+                continue;
+            }
+            if (shared_left(n))
+                TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs));
             TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs));
             {
                 ProductTimer pt(8.0 * d3 * oz_products(), cs);   // X_k = U_k rho_k
@@ -748,8 +814,15 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     };
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(launch_layout(L, t, cs));
-        for (int k = 0; k <= n; k++)
-            TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, L.dims[k], (size_t)L.dims[k], cs));
+        for (int k = 0; k <= n; k++) {
+            const int d = L.dims[k], Np = bs.ld[k];
+            if (d <= kDmmaBlock) {   // zero padding: the planes' rows are read up to d only
+                split_block_kernel<<<64, 256, 0, cs>>>(reinterpret_cast<const double2*>(U) + L.off[k], d, Np, Ur[k], Ui[k]);
+                TC_LAUNCH_CHECK();
+            } else if (!shared_left(n)) {
+                TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs));
+            }
+        }
         dim3 g(256, (unsigned)(n + 1));
         blocks_split_pad_kernel<<<g, 256, 0, cs>>>(bs, pk, reinterpret_cast<const double2*>(rho), Rr, Ri);
         TC_LAUNCH_CHECK();
@@ -770,16 +843,24 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
 }
 
+// The least a call needs; TC_FP64 runs on the DMMA in this much.
 size_t evolve_bytes(int n, int precision) {
     if (precision == TC_FP64_OZAKI) return evolve_oz_bytes_blocks(n);
     return precision == TC_FP64 ? evolve_f64_bytes(n) : evolve_lowp_bytes_blocks(n, precision);
 }
 
+// TC_FP64 takes the tensor-core form from n = 7 (below, every block but the
+// last one or two has at most 64 states) to n = 13 (as the closed system, the
+// workspace must leave room for what fitted beside the DMMA form's).
+bool blocks_f64_on_tensor_cores(int n) { return f64_on_tensor_cores(n) && n <= 13; }
+
 }  // namespace
 
 size_t lindblad_bytes(int n, int precision) {
     if (precision < TC_FP64 || precision > TC_FP64_OZAKI) return 0;
-    return std::max(propagators_bytes(n), evolve_bytes(n, precision));
+    size_t b = std::max(propagators_bytes(n), evolve_bytes(n, precision));
+    if (precision == TC_FP64 && blocks_f64_on_tensor_cores(n)) b = std::max(b, evolve_oz_bytes_blocks(n));
+    return b;
 }
 
 }  // namespace tc
@@ -843,9 +924,9 @@ extern "C" TC_API tc_status tc_lindblad_evolve(const tc_params* params, double k
     Arena ar{static_cast<char*>(work), work_bytes, 0};
     const double* Ud = static_cast<const double*>(U);
     double* Rd = static_cast<double*>(rho);
-    if (precision == TC_FP64)
+    if (precision == TC_FP64 && !(blocks_f64_on_tensor_cores(m.n) && work_bytes >= evolve_oz_bytes_blocks(m.n)))
         return evolve_f64(L, m, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
-    if (precision == TC_FP64_OZAKI)
+    if (precision == TC_FP64 || precision == TC_FP64_OZAKI)
         return evolve_oz_blocks(L, m, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
     return evolve_lowp_blocks(L, m, precision, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
 }
