@@ -236,32 +236,75 @@ size_t oz_backward_extra(int n) {
            2 * round256(N * N * sizeof(double)) + 256;
 }
 
-// Q <- U' P U'^dag with U' = U (or conj U for the adjoint step); P Hermitian, Q may be P
-tc_status step_oz(int N, OzBufs& z, bool adjoint, CM P, CM Q, CM X, cudaStream_t s) {
-    const OzMat& A = adjoint ? z.Uc : z.U;
-    TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
-    TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = U' P^H
-    TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s));
-    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, z.scratch}, z.group, s);    // Q = U' X^H
+// Q <- A P A^H from P's planes, loaded into `Bp` already or here; B, X, scratch: the product's own (B may
+// be Bp); Q may be P
+tc_status step_oz(int N, const OzMat& A, OzMat& Bp, bool loaded, OzMat& B, CM P, CM Q, CM X, void* scratch, int group,
+                  cudaStream_t s) {
+    if (!loaded) TC_TRY(oz_mat_load(Bp, P.r, P.i, false, false, N, (size_t)N, s));
+    TC_TRY(oz_product(0, A, Bp, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, scratch}, group, s));   // X = A P^H
+    TC_TRY(oz_mat_load(B, X.r, X.i, false, false, N, (size_t)N, s));
+    return oz_product(1, A, B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, scratch}, group, s);     // Q = A X^H
 }
 
-// out = A R^H (+ out): the left operand as it is, R's planes as they are or conjugated
-tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
+// out = A R^H (+ out): the left operand as it is, R's planes as they are or
+// conjugated, loaded into B already or here
+tc_status mul_oz(int N, OzBufs& z, CM A, OzMat& B, bool loaded, CM R, bool conj_r, CM out, bool add, void* scratch,
+                 cudaStream_t s) {
     if (A.r) TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s));   // else: as loaded last
-    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s));
-    OzOut o{out.r, out.i, z.scratch};
+    if (!loaded) TC_TRY(oz_mat_load(B, R.r, R.i, false, conj_r, N, (size_t)N, s));
+    OzOut o{out.r, out.i, scratch};
     o.conj_b = conj_r;
     if (add && !oz_modular()) {   // the digit form does not accumulate
         o.yr = z.Y.r;
         o.yi = z.Y.i;
-        TC_TRY(oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s));
+        TC_TRY(oz_product(0, z.A2, B, R.r, R.i, N, (size_t)N, o, z.group, s));
         const size_t NN = (size_t)N * N;
         axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, out.r, out.i, 1.0, z.Y.r, z.Y.i, out.r, out.i, NN);
         TC_LAUNCH_CHECK();
         return TC_OK;
     }
     o.accumulate = add;
-    return oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s);
+    return oz_product(0, z.A2, B, R.r, R.i, N, (size_t)N, o, z.group, s);
+}
+tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
+    return mul_oz(N, z, A, z.B, false, R, conj_r, out, add, z.scratch, s);
+}
+
+// Up to n = 11 the reverse pass runs as three chains side by side: the adjoint
+// steps on the call's stream, W += rho_k Lambda_k on a second, and the states
+// of the next segment on a third.  Their launches are a few us each at n <= 9
+// (a gradient at n = 8, 100 steps: 22.6 -> 16.6 ms) and at n = 11 one chain's
+// residues and recombinations run beside another's products.  Each chain has
+// its own operand and scratch; Lambda and its operand alternate between two
+// buffers, the segments between two sets.
+struct Chains {
+    bool on = false;
+    cudaStream_t w = nullptr, f = nullptr;
+    OzMat BL[2], BF;
+    CM L[2], XF;
+    void *scratch_w = nullptr, *scratch_f = nullptr;
+    cudaEvent_t start = nullptr, lambda[2] = {}, used[2] = {}, seg[2] = {}, freed[2] = {};
+    ~Chains() {
+        if (on) {   // the caller's buffers are not in use once the call returns, also after an error
+            cudaStreamSynchronize(w);
+            cudaStreamSynchronize(f);
+        }
+        for (cudaEvent_t e : {start, lambda[0], lambda[1], used[0], used[1], seg[0], seg[1], freed[0], freed[1]})
+            if (e) cudaEventDestroy(e);
+    }
+};
+tc_status make_event(cudaEvent_t* e) {
+    TC_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    return TC_OK;
+}
+
+constexpr int kChainMax = 11;
+size_t chains_extra(int n, int steps, int ckpt_every) {
+    const size_t N = (size_t)1 << n;
+    const int c = ckpt_every < steps ? ckpt_every : steps;
+    const size_t segs = steps > ckpt_every ? (size_t)c * cm_bytes(n) : 0;
+    if (n < 7 || n > kChainMax || segs > ((size_t)4 << 30) || !oz_modular()) return 0;
+    return 3 * oz_mat_bytes((int)N, false) + 2 * oz_scratch_bytes((int)N) + 2 * cm_bytes(n) + segs;
 }
 
 // conjugate transpose of planar R, one 32 x 32 tile per block of 32 x 8 threads (N a multiple of 32)
@@ -328,9 +371,17 @@ size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
 
 }  // namespace
 
+namespace {
+// with the tensor-core products, one chain
+size_t backward_tensor_bytes(int n, int steps, int ckpt_every) {
+    return backward_least_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
+}
+}  // namespace
+
 size_t backward_bytes(int n, int steps, int ckpt_every, int precision) {
-    return backward_least_bytes(n, steps, ckpt_every,
-                                precision == TC_FP64 && backward_f64_on_tensor_cores(n) ? TC_FP64_OZAKI : precision);
+    if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
+    if (precision == TC_FP64 && !backward_f64_on_tensor_cores(n)) return backward_least_bytes(n, steps, ckpt_every, TC_FP64);
+    return backward_tensor_bytes(n, steps, ckpt_every) + chains_extra(n, steps, ckpt_every);
 }
 
 }  // namespace tc
@@ -387,8 +438,10 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     b.small = ar.take<double>(2 * (size_t)N + 64);
     if (!b.small) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
     const bool oz = precision == TC_FP64_OZAKI || (backward_f64_on_tensor_cores(n) &&
-                                                   work_bytes >= backward_bytes(n, steps, ckpt_every, TC_FP64));
+                                                   work_bytes >= backward_tensor_bytes(n, steps, ckpt_every));
     OzBufs z{};
+    Chains ch;
+    std::vector<CM> seg2;
     if (oz) {
         TC_TRY(oz_mat_init(z.U, ar, N, true));
         TC_TRY(oz_mat_init(z.Uc, ar, N, true));
@@ -401,20 +454,47 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));
         TC_TRY(oz_mat_load(z.Uc, static_cast<const double*>(U), nullptr, true, true, N, (size_t)N, s));
     }
-    // Q <- U P U^dag, Q may be P
-    auto fwd_step = [&](CM P, CM Q) -> tc_status {
-        if (oz) return step_oz(N, z, false, P, Q, b.X, s);
+    ch.on = oz && chains_extra(n, steps, ckpt_every) > 0 && work_bytes >= backward_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
+    if (ch.on) {
+        TC_TRY(side_streams(&ch.w, &ch.f));
+        for (OzMat* m2 : {&ch.BL[0], &ch.BL[1], &ch.BF}) TC_TRY(oz_mat_init(*m2, ar, N, false));
+        ch.scratch_w = ar.take<uint8_t>(oz_scratch_bytes(N));
+        ch.scratch_f = ar.take<uint8_t>(oz_scratch_bytes(N));
+        ch.L[0] = b.L;
+        ch.L[1] = take_cm(ar, NN);
+        ch.XF = take_cm(ar, NN);
+        if (b.nck > 1)
+            for (int k = 0; k < b.c; k++) seg2.push_back(take_cm(ar, NN));
+        if (!ch.XF.i || (b.nck > 1 && !seg2.back().i)) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
+        for (cudaEvent_t* e : {&ch.start, &ch.lambda[0], &ch.lambda[1], &ch.used[0], &ch.used[1], &ch.seg[0], &ch.seg[1],
+                               &ch.freed[0], &ch.freed[1]})
+            TC_TRY(make_event(e));
+    } else {   // one chain: every buffer and stream the same
+        ch.w = ch.f = s;
+        ch.BL[0] = ch.BL[1] = ch.BF = z.B;
+        ch.L[0] = ch.L[1] = b.L;
+        ch.XF = b.X;
+        ch.scratch_w = ch.scratch_f = z.scratch;
+    }
+    // Q <- U P U^dag, Q may be P; on the call's stream or the third chain's
+    auto fwd_step = [&](CM P, CM Q, bool third) -> tc_status {
+        if (oz)
+            return third ? step_oz(N, z.U, ch.BF, false, ch.BF, P, Q, ch.XF, ch.scratch_f, z.group, ch.f)
+                         : step_oz(N, z.U, z.B, false, z.B, P, Q, b.X, z.scratch, z.group, s);
         if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, s));
         return step(N, b.U, Q, b.X, 0, s);
     };
 
     // ---------------------------------------------------------------- forward
+    // rho_k goes to its checkpoint, to the last segment's buffers, or to seg0 (the running state; rho_K)
     TC_TRY(launch_split_c128(static_cast<const double*>(U), b.U.r, b.U.i, NN, s));
     TC_TRY(launch_split_c128(static_cast<const double*>(rho0), ck[0].r, ck[0].i, NN, s));
-    TC_TRY(copy_cm(ck[0], b.seg0, NN, s));   // seg0 = running rho
+    const int last0 = (b.nck - 1) * ckpt_every;   // the last segment is last0 .. steps - 1
+    CM cur = ck[0];
     for (int k = 1; k <= steps; k++) {
-        TC_TRY(fwd_step(b.seg0, b.seg0));
-        if (k < steps && k % ckpt_every == 0) TC_TRY(copy_cm(b.seg0, ck[k / ckpt_every], NN, s));
+        const CM dst = k == steps ? b.seg0 : k % ckpt_every == 0 ? ck[k / ckpt_every] : k > last0 ? seg[k - last0] : b.seg0;
+        TC_TRY(fwd_step(cur, dst, false));
+        cur = dst;
     }
     // loss from rho_K (in seg0)
     loss_kernel<<<1, 1024, 0, s>>>(b.seg0.r, O_diag, N, b.small);
@@ -423,27 +503,64 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // ---------------------------------------------------------------- backward
     diag_set_kernel<<<grid_for(NN), 256, 0, s>>>(O_diag, b.L.r, b.L.i, N);   // Lambda_K = O
     TC_LAUNCH_CHECK();
-    bool w_init = false;
+    if (ch.on) {
+        TC_CUDA(cudaEventRecord(ch.start, s));
+        TC_CUDA(cudaStreamWaitEvent(ch.w, ch.start, 0));
+        TC_CUDA(cudaStreamWaitEvent(ch.f, ch.start, 0));
+    }
+    const std::vector<CM>* sets[2] = {&seg, ch.on && b.nck > 1 ? &seg2 : &seg};
+    // rho_{k0 + 1 .. k1 - 1} of segment j from its checkpoint
+    auto recompute = [&](int j, const std::vector<CM>& to) -> tc_status {
+        const int k0 = j * ckpt_every, k1 = k0 + ckpt_every;
+        for (int k = k0 + 1; k < k1; k++) TC_TRY(fwd_step(k == k0 + 1 ? ck[j] : to[k - 1 - k0], to[k - k0], true));
+        return TC_OK;
+    };
+    bool w_init = false, lambda_loaded = false;
+    bool used[2] = {false, false}, freed[2] = {false, false};
+    int a = 0;   // buffer of the current Lambda
     for (int j = b.nck - 1; j >= 0; j--) {
+        const int par = (b.nck - 1 - j) & 1;
         const int k0 = j * ckpt_every;
         const int k1 = (k0 + ckpt_every < steps) ? k0 + ckpt_every : steps;   // segment k0 .. k1-1
-        // recompute rho_{k0..k1-1} into seg[0..]
-        TC_TRY(copy_cm(ck[j], seg[0], NN, s));
-        for (int k = k0 + 1; k < k1; k++) {
-            TC_TRY(fwd_step(seg[k - 1 - k0], seg[k - k0]));
+        if (!ch.on && j < b.nck - 1) {
+            TC_TRY(recompute(j, seg));
+            lambda_loaded = false;   // the one right operand now holds a state
         }
+        if (ch.on && j > 0) {   // the next segment beside this one
+            if (freed[par ^ 1]) TC_CUDA(cudaStreamWaitEvent(ch.f, ch.freed[par ^ 1], 0));
+            TC_TRY(recompute(j - 1, *sets[par ^ 1]));
+            TC_CUDA(cudaEventRecord(ch.seg[par ^ 1], ch.f));
+        }
+        if (ch.on && j < b.nck - 1) TC_CUDA(cudaStreamWaitEvent(ch.w, ch.seg[par], 0));
         for (int k = k1 - 1; k >= k0; k--) {
+            const CM rho_k = k == k0 ? ck[j] : (*sets[par])[k - k0];
             // Lambda_k = U^dag Lambda_{k+1} U  (the step with conj(U)); W += rho_k Lambda_k
             if (oz) {
-                TC_TRY(step_oz(N, z, true, b.L, b.L, b.X, s));
-                TC_TRY(mul_oz(N, z, seg[k - k0], b.L, false, b.W, w_init, s));   // Lambda Hermitian
+                const int nx = a ^ 1;
+                if (ch.on && used[nx]) TC_CUDA(cudaStreamWaitEvent(s, ch.used[nx], 0));
+                TC_TRY(step_oz(N, z.Uc, ch.BL[a], lambda_loaded, z.B, ch.L[a], ch.L[nx], b.X, z.scratch, z.group, s));
+                TC_TRY(oz_mat_load(ch.BL[nx], ch.L[nx].r, ch.L[nx].i, false, false, N, (size_t)N, s));
+                lambda_loaded = true;
+                if (ch.on) {
+                    TC_CUDA(cudaEventRecord(ch.lambda[nx], s));
+                    TC_CUDA(cudaStreamWaitEvent(ch.w, ch.lambda[nx], 0));
+                }
+                // Lambda Hermitian: rho Lambda = rho Lambda^H
+                TC_TRY(mul_oz(N, z, rho_k, ch.BL[nx], true, ch.L[nx], false, b.W, w_init, ch.scratch_w, ch.w));
+                if (ch.on) TC_CUDA(cudaEventRecord(ch.used[nx], ch.w));
+                used[nx] = true;
+                a = nx;
             } else {
                 TC_TRY(step(N, b.U, b.L, b.X, 1, s));
-                TC_TRY(gemm_c(N, seg[k - k0], 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, s));
+                TC_TRY(gemm_c(N, rho_k, 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, s));
             }
             w_init = true;
         }
+        if (ch.on) TC_CUDA(cudaEventRecord(ch.freed[par], ch.w));
+        freed[par] = true;
     }
+    // the chains meet (the third one's work was waited for by the second)
+    if (ch.on) TC_CUDA(cudaStreamWaitEvent(s, ch.used[a], 0));
     // M = W U^dag = W conj(U)  -> into L (free now)
     CM M = b.L;
     if (oz)

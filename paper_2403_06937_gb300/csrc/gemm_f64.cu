@@ -1,8 +1,8 @@
 // gemm_f64.cu -- FP64 complex / real GEMM on the DMMA path (mma.sync .f64).
 //
-// Used for every product of the plain FP64 form: the Taylor polynomial and
-// squarings of e^{-iHdt} (Sec. III.A, Eqs. 7-8 and 10), the two products of
-// one step rho <- U rho U^dag (Eqs. 6 and 12), and the adjoint products.
+// Used for the products of the FP64 form that do not run as residue products on
+// the tensor cores (cgemm_crt.cu): small systems, small workspaces, the
+// squarings of the structured e^{-iHdt}.
 //
 // On GB300 the FP64 pipe delivers about 1 TFLOP/s for the whole chip (a few
 // FP64 FMAs per clock per SM), so this kernel is bound by the FP64 issue rate,
@@ -229,6 +229,70 @@ __global__ void splitk_reduce_kernel(GemmF64 p, int splits) {
     }
 }
 
+// Small products: complex up to 64, real up to 128 a side.  An SM's FP64 pipe
+// finishes about 1.9 multiply-adds a clock, so one 32 x 32 x 64 complex tile of
+// the DMMA kernel takes 70 us; here the work is spread as far as it goes: 8 x 4
+// outputs per block, K in eight slices (a warp each) summed in a fixed order.
+// A step at n = 6: 170 -> 20 us.
+constexpr int kSmallComplex = 64, kSmallReal = 128;
+template <bool CPLX>
+__global__ void __launch_bounds__(256) gemm_small_kernel(GemmF64 p) {
+    constexpr int KM = CPLX ? kSmallComplex : kSmallReal, I = CPLX ? 1 : 0;
+    __shared__ double sa[1 + I][8][KM + 1], sb[1 + I][KM][4], part[1 + I][8][32];
+    const int m0 = (int)blockIdx.y * 8, n0 = (int)blockIdx.x * 4;
+    if (p.herm_lower && n0 > m0 + 7) return;   // above the diagonal: written as mirrors
+    for (int e = threadIdx.x; e < 8 * p.K; e += 256) {
+        const int r = e / p.K, k = e % p.K;
+        const bool ok = m0 + r < p.M;
+        const long o = (long)(m0 + r) * p.lda + k;
+        sa[0][r][k] = ok ? p.Ar[o] : 0.0;
+        if (CPLX) sa[I][r][k] = ok ? (p.conjA ? -p.Ai[o] : p.Ai[o]) : 0.0;
+    }
+    for (int e = threadIdx.x; e < 4 * p.K; e += 256) {
+        const int k = e / 4, c = e % 4;
+        const bool ok = n0 + c < p.N;
+        const long o = (long)k * p.ldb + n0 + c;
+        sb[0][k][c] = ok ? p.Br[o] : 0.0;
+        if (CPLX) sb[I][k][c] = ok ? (p.conjB ? -p.Bi[o] : p.Bi[o]) : 0.0;
+    }
+    __syncthreads();
+    const int out = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const int r = out >> 2, c = out & 3;
+    double xr = 0.0, xi = 0.0;
+    for (int k = slice; k < p.K; k += 8) {
+        const double ar = sa[0][r][k], br = sb[0][k][c];
+        if (CPLX) {
+            const double ai = sa[I][r][k], bi = sb[I][k][c];
+            xr = fma(ar, br, fma(-ai, bi, xr));
+            xi = fma(ar, bi, fma(ai, br, xi));
+        } else {
+            xr = fma(ar, br, xr);
+        }
+    }
+    part[0][slice][out] = xr;
+    if (CPLX) part[I][slice][out] = xi;
+    __syncthreads();
+    const int row = m0 + r, col = n0 + c;
+    if (slice != 0 || row >= p.M || col >= p.N) return;
+    auto sum = [&](const double (&v)[8][32]) {
+        return ((v[0][out] + v[1][out]) + (v[2][out] + v[3][out])) + ((v[4][out] + v[5][out]) + (v[6][out] + v[7][out]));
+    };
+    double vr = p.alpha * sum(part[0]), vi = CPLX ? p.alpha * sum(part[I]) : 0.0;
+    const long o = (long)row * p.ldc + col;
+    if (p.beta != 0.0) {
+        vr += p.beta * p.Cr[o];
+        if (CPLX) vi += p.beta * p.Ci[o];
+    }
+    if (p.herm_lower && row < col) return;
+    p.Cr[o] = vr;
+    if (CPLX) p.Ci[o] = p.herm_lower && row == col ? 0.0 : vi;
+    if (p.herm_lower && row > col) {
+        const long mir = (long)col * p.ldc + row;
+        p.Cr[mir] = vr;
+        if (CPLX) p.Ci[mir] = -vi;
+    }
+}
+
 int sm_count() {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
@@ -292,6 +356,16 @@ tc_status gemm_f64(const GemmF64& g, cudaStream_t s) {
     if (g.M <= 0 || g.N <= 0 || g.K <= 0) return TC_OK;
     if (g.herm_lower && (g.M != g.N || g.beta != 0.0))
         return fail(TC_ERR_INVALID_ARG, "gemm_f64: Hermitian mode needs M == N and beta == 0");
+    const int small = g.cplx ? kSmallComplex : kSmallReal;
+    if (g.M <= small && g.N <= small && g.K <= small) {
+        const dim3 grid((unsigned)((g.N + 3) / 4), (unsigned)((g.M + 7) / 8));
+        if (g.cplx)
+            gemm_small_kernel<true><<<grid, 256, 0, s>>>(g);
+        else
+            gemm_small_kernel<false><<<grid, 256, 0, s>>>(g);
+        TC_LAUNCH_CHECK();
+        return TC_OK;
+    }
     const int tile = g.tile ? g.tile : tuned_f64_tile(g.N > g.M ? g.N : g.M);
     if (tile == 32) return launch_bt<32>(g, s);
     if (tile == 64) return launch_bt<64>(g, s);

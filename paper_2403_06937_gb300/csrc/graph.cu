@@ -10,6 +10,7 @@ struct GraphStream {
     cudaEvent_t before = nullptr, after = nullptr;
     cudaStream_t side = nullptr;                     // SideBranch's stream and events
     cudaEvent_t fork = nullptr, join = nullptr;
+    cudaStream_t more[2] = {};                       // side_streams
 };
 std::mutex g_mu;
 GraphStream g_gs[64];
@@ -27,6 +28,7 @@ tc_status graph_stream(GraphStream** out) {
         TC_CUDA(cudaStreamCreateWithFlags(&g.side, cudaStreamNonBlocking));
         TC_CUDA(cudaEventCreateWithFlags(&g.fork, cudaEventDisableTiming));
         TC_CUDA(cudaEventCreateWithFlags(&g.join, cudaEventDisableTiming));
+        for (cudaStream_t& m : g.more) TC_CUDA(cudaStreamCreateWithFlags(&m, cudaStreamNonBlocking));
     }
     *out = &g;
     return TC_OK;
@@ -77,6 +79,14 @@ tc_status run_captured(cudaStream_t user, const std::function<tc_status(cudaStre
     cudaEventRecord(gs->after, s);
     cudaStreamWaitEvent(user, gs->after, 0);
     return st;
+}
+
+tc_status side_streams(cudaStream_t* a, cudaStream_t* b) {
+    GraphStream* gs = nullptr;
+    TC_TRY(graph_stream(&gs));
+    *a = gs->more[0];
+    *b = gs->more[1];
+    return TC_OK;
 }
 
 SideBranch::SideBranch(cudaStream_t main) : main_(main) {

@@ -38,4 +38,8 @@ class SideBranch {
     bool pending_ = false;
 };
 
+// Two more library streams of the current device, for chains of work that run
+// beside a call's own stream (ordered by the caller with events of its own).
+tc_status side_streams(cudaStream_t* a, cudaStream_t* b);
+
 }  // namespace tc

@@ -684,9 +684,9 @@ __global__ void blocks_join_pad_kernel(BlockSet bs, BlockSet pk, const double* _
     }
 }
 
-// Blocks of up to this dimension run on the DMMA GEMM (two launches of a few
-// 32 x 32 tiles; six launches on 128 x 128 padding otherwise).
-constexpr int kDmmaBlock = 64;
+// Blocks of up to this dimension run on gemm_f64's small-product kernel (two
+// launches instead of six on 128 x 128 padding).
+constexpr int kSmallBlock = 64;
 
 // interleaved d x d -> FP64 planes of row stride Np
 __global__ void split_block_kernel(const double2* __restrict__ src, int d, int Np, double* __restrict__ re,
@@ -712,7 +712,7 @@ size_t evolve_oz_bytes_blocks(int n) {
     if (shared_left(n)) b += oz_mat_bytes(NpMax, true);
     for (int k = 0; k <= n; k++) {
         const size_t Np = (size_t)padded(L.dims[k]);
-        if (L.dims[k] <= kDmmaBlock)
+        if (L.dims[k] <= kSmallBlock)
             b += 2 * round256(Np * Np * sizeof(double));
         else if (!shared_left(n))
             b += oz_mat_bytes((int)Np, true);
@@ -738,7 +738,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     if (shared_left(n)) TC_TRY(oz_mat_init(Amax, ar, NpMax, true));
     for (int k = 0; k <= n; k++) {
         const int Np = padded(L.dims[k]);
-        if (L.dims[k] <= kDmmaBlock) {
+        if (L.dims[k] <= kSmallBlock) {
             Ur[k] = ar.take<double>((size_t)Np * Np);
             Ui[k] = ar.take<double>((size_t)Np * Np);
         } else if (shared_left(n)) {
@@ -770,7 +770,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
             double* rr = Rr + bs.off[k];
             double* ri = Ri + bs.off[k];
             const double d3 = (double)d * d * d;
-            if (d <= kDmmaBlock) {
+            if (d <= kSmallBlock) {
                 GemmF64 g1{};
                 g1.M = g1.N = g1.K = d;
                 g1.Ar = Ur[k]; g1.Ai = Ui[k]; g1.lda = Np;
@@ -778,7 +778,6 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
                 g1.Cr = Xr; g1.Ci = Xi; g1.ldc = Np;
                 g1.alpha = 1.0;
                 g1.cplx = 1;
-                g1.tile = 32;
                 GemmF64 g2 = g1;
                 g2.Ar = Xr; g2.Ai = Xi;
                 g2.Br = Ur[k]; g2.Bi = Ui[k]; g2.conjB = 1;
@@ -816,7 +815,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
         TC_TRY(launch_layout(L, t, cs));
         for (int k = 0; k <= n; k++) {
             const int d = L.dims[k], Np = bs.ld[k];
-            if (d <= kDmmaBlock) {   // zero padding: the planes' rows are read up to d only
+            if (d <= kSmallBlock) {   // zero padding: the planes' rows are read up to d only
                 split_block_kernel<<<64, 256, 0, cs>>>(reinterpret_cast<const double2*>(U) + L.off[k], d, Np, Ur[k], Ui[k]);
                 TC_LAUNCH_CHECK();
             } else if (!shared_left(n)) {

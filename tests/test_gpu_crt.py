@@ -128,16 +128,20 @@ def test_gradient_on_the_tensor_cores_with_squarings(tc, oracle):
     grad, loss = tc.evolve_backward(p, dt, steps, rho0, U, O, ckpt_every=2)
     grad2, loss2 = tc.evolve_backward(p, dt, steps, rho0, U, O, ckpt_every=2, precision="ozaki")
     assert torch.equal(grad, grad2) and loss == loss2   # one route for both from n = 7 on
-    least = tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_BACKWARD, steps, 2) - 65536
-    work = torch.empty(least, dtype=torch.uint8, device="cuda")
-    ref = (ctypes.c_double * (n + 2))()
-    c = p.c()
-    tc._abi.call("tc_evolve_backward", ctypes.byref(c), dt, steps, ctypes.c_void_p(rho0.data_ptr()),
-                 ctypes.c_void_p(U.data_ptr()), 2, tc.TC_FP64, ctypes.c_void_p(O.data_ptr()), ref, None,
-                 ctypes.c_void_p(work.data_ptr()), work.numel(),
-                 ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
-    ref = torch.tensor(list(ref), dtype=torch.float64)
-    assert torch.max(torch.abs(grad - ref)).item() < 1e-11 * torch.max(torch.abs(ref)).item()
+    # one chain instead of three (64 KiB less), and the DMMA form (its planes: 11 + 2 checkpoints + 2 states of
+    # two N x N matrices, one real one, the small buffers)
+    cm = 2 * 8 * N * N
+    for size, tol in ((tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_BACKWARD, steps, 2) - 65536, 0.0),
+                      (15 * cm + cm // 2 + 16384, 1e-11)):
+        work = torch.empty(size, dtype=torch.uint8, device="cuda")
+        ref = (ctypes.c_double * (n + 2))()
+        c = p.c()
+        tc._abi.call("tc_evolve_backward", ctypes.byref(c), dt, steps, ctypes.c_void_p(rho0.data_ptr()),
+                     ctypes.c_void_p(U.data_ptr()), 2, tc.TC_FP64, ctypes.c_void_p(O.data_ptr()), ref, None,
+                     ctypes.c_void_p(work.data_ptr()), work.numel(),
+                     ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+        ref = torch.tensor(list(ref), dtype=torch.float64)
+        assert torch.max(torch.abs(grad - ref)).item() <= tol * torch.max(torch.abs(ref)).item()
 
 
 @pytest.mark.parametrize("n,degree,squarings", [(8, 0, -1), (8, 6, 3), (9, 0, -1), (11, 12, 1)])
