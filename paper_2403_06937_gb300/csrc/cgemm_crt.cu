@@ -648,6 +648,8 @@ struct CrtCombine {
     int accumulate;          // MODE 0: add to Y
     double* yr;
     double* yi;
+    const double2* b_c128;   // B interleaved instead of (br, bi)
+    double2* out_c128;       // MODE 1: Y interleaved (row stride Np) instead of (yr, yi)
 };
 
 // One tile of 32 rows x 8 COLS columns of Y per block of 256 threads, COLS
@@ -686,8 +688,10 @@ __global__ void __launch_bounds__(256, 4) crt_combine_kernel(CrtCombine p) {
         const int b = tb + k;
         const bool in = j0 + ta < p.N && i0 + b < p.N;
         const size_t ob = (size_t)(j0 + ta) * p.ldb + (size_t)(i0 + b);
-        sr[ta][b] = in ? p.br[ob] : 0.0;
-        si[ta][b] = in ? __longlong_as_double(__double_as_longlong(p.bi[ob]) ^ p.bi_flip) : 0.0;
+        double2 v = make_double2(0.0, 0.0);
+        if (in) v = p.b_c128 ? p.b_c128[ob] : make_double2(p.br[ob], p.bi[ob]);
+        sr[ta][b] = v.x;
+        si[ta][b] = __longlong_as_double(__double_as_longlong(v.y) ^ p.bi_flip);
     }
     const int ea = p.ea[i];
     int eb[COLS];
@@ -731,7 +735,12 @@ __global__ void __launch_bounds__(256, 4) crt_combine_kernel(CrtCombine p) {
             vi[k] += yi[k];
         }
     }
-    if (COLS == 4 && (MODE == 0 || j0 + W <= i0)) {
+    if (MODE == 1 && p.out_c128) {
+        double2* y = p.out_c128 + (size_t)i * p.Np + j;
+#pragma unroll
+        for (int k = 0; k < COLS; k++)
+            if (j + k <= i) y[k] = make_double2(vr[k], j + k == i ? 0.0 : vi[k]);
+    } else if (COLS == 4 && (MODE == 0 || j0 + W <= i0)) {
 #pragma unroll
         for (int k = 0; k < COLS; k += 2) {
             *reinterpret_cast<double2*>(yr + k) = make_double2(vr[k], vr[k + 1 < COLS ? k + 1 : k]);
@@ -755,7 +764,12 @@ __global__ void __launch_bounds__(256, 4) crt_combine_kernel(CrtCombine p) {
         __syncthreads();
         double* mr = p.yr + (size_t)(j0 + ta) * p.Np + i0 + tb;
         double* mi = p.yi + (size_t)(j0 + ta) * p.Np + i0 + tb;
-        if (COLS == 4 && j0 + W <= i0) {
+        if (p.out_c128) {
+            double2* m = p.out_c128 + (size_t)(j0 + ta) * p.Np + i0 + tb;
+#pragma unroll
+            for (int k = 0; k < COLS; k++)
+                if (j0 + ta < i0 + tb + k) m[k] = make_double2(sr[ta][tb + k], -si[ta][tb + k]);
+        } else if (COLS == 4 && j0 + W <= i0) {
 #pragma unroll
             for (int k = 0; k < COLS; k += 2) {
                 const int k1 = k + 1 < COLS ? k + 1 : k;
@@ -946,6 +960,8 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
         c.yi = out.yi;
         c.bi_flip = out.conj_b ? LLONG_MIN : 0;
         c.accumulate = out.accumulate ? 1 : 0;
+        c.b_c128 = static_cast<const double2*>(out.b_c128);
+        c.out_c128 = static_cast<double2*>(out.y_c128);
         const int cols = Np <= 512 ? 1 : 4;
         const dim3 grid((unsigned)((mode == 0 ? Np : row0 + band) / (8 * cols)), (unsigned)(band / 32));
         if (cols == 1)

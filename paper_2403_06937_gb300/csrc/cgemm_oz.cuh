@@ -78,7 +78,10 @@ struct OzOut {
     double* yi;
     void* scratch;     // oz_scratch_bytes(Np)
     bool accumulate = false;   // residue form only: add to what yr, yi hold (mode 0)
-    bool conj_b = false;       // B was loaded with conj: its planes (br, bi) hold the conjugate
+    bool conj_b = false;       // B was loaded with conj: (br, bi) are the planes before it
+    // residue form only
+    const void* b_c128 = nullptr;   // B interleaved (complex128, row stride ldb) instead of (br, bi)
+    void* y_c128 = nullptr;         // mode 1: the result interleaved (row stride Np) instead of (yr, yi)
 };
 size_t oz_mat_bytes(int Np, bool left);
 size_t oz_scratch_bytes(int Np);
@@ -105,10 +108,14 @@ struct OzSystem {
     const Model* m = nullptr;
     double* obs = nullptr;
     tc_status carve(int n, Arena& ar);
-    tc_status first(const double* U, const double* rho, const Model* m, double* obs, int renorm_every,
+    // planes: rho into the FP64 planes; else step 1 reads it as it is (step_from)
+    tc_status first(const double* U, const double* rho, const Model* m, double* obs, int renorm_every, bool planes,
                     cudaStream_t cs);
     // the row is read beside the next step's first product when `side` is a branch of cs
-    tc_status step(int k, cudaStream_t cs, SideBranch& side);
+    // from, to (residue form, no padding): rho read interleaved in place of the planes, rho' written interleaved
+    tc_status step(int k, cudaStream_t cs, SideBranch& side, const double* from = nullptr, double* to = nullptr);
+    // true when a step may read and write the caller's interleaved rho itself
+    bool interleaved() const;
     tc_status tail(double* rho, cudaStream_t cs);
 };
 

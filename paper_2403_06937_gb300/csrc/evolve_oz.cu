@@ -105,24 +105,29 @@ tc_status OzSystem::carve(int n_, Arena& ar) {
 }
 
 tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, double* obs_, int renorm_every_,
-                          cudaStream_t cs) {
+                          bool planes, cudaStream_t cs) {
     m = m_;
     obs = obs_;
     renorm_every = renorm_every_;
     const size_t NN = (size_t)Np * Np;
     TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs));
-    const double2* src = reinterpret_cast<const double2*>(rho);
-    split_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(src, N, Np, Rr, Ri);
-    TC_LAUNCH_CHECK();
+    if (planes) {
+        split_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(reinterpret_cast<const double2*>(rho), N, Np, Rr, Ri);
+        TC_LAUNCH_CHECK();
+    }
     if (obs) TC_TRY(launch_observables(kRhoInterleaved, rho, nullptr, m, n, obs, scratch, cs));
     return TC_OK;
 }
 
-tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side) {
+bool OzSystem::interleaved() const { return N == Np && oz_modular(); }
+
+tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double* from, double* to) {
     const size_t NN = (size_t)Np * Np;
     const double N3 = (double)N * N * N;
-    const OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
-    TC_TRY(oz_mat_load(Ps, Rr, Ri, false, false, N, (size_t)Np, cs));
+    OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
+    X.b_c128 = from;
+    R.y_c128 = to;
+    TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs));
     {
         ProductTimer t(8.0 * N3 * oz_products(), cs);   // X = U rho^H
         TC_TRY(oz_product(0, Us, Ps, Rr, Ri, N, (size_t)Np, X, group, cs));
@@ -141,8 +146,8 @@ tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side) {
     }
     if (obs) {
         TC_TRY(side.begin());
-        TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs + (size_t)k * TC_OBS_STRIDE(n), scratch,
-                                  side.stream(), (size_t)Np));
+        TC_TRY(launch_observables(to ? kRhoInterleaved : kRhoPlanarF64, to ? to : Rr, Ri, m, n,
+                                  obs + (size_t)k * TC_OBS_STRIDE(n), scratch, side.stream(), (size_t)Np));
         TC_TRY(side.end());
     }
     return TC_OK;
@@ -173,20 +178,26 @@ tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_e
         if (obs) TC_TRY(launch_observables(kRhoInterleaved, rho, nullptr, m, n, obs, z.scratch, s));
         return TC_OK;
     }
+    // without padding the first step reads the caller's rho and the last one writes it (unless it is
+    // renormalised after that), with no pass to and from the planes
+    const bool direct = z.interleaved();
+    auto to = [&](int k) {
+        return direct && k == steps && !(renorm_every > 0 && k % renorm_every == 0) ? rho : nullptr;
+    };
     auto first = [&](cudaStream_t cs) -> tc_status {
-        TC_TRY(z.first(U, rho, m, obs, renorm_every, cs));
+        TC_TRY(z.first(U, rho, m, obs, renorm_every, !direct, cs));
         SideBranch side(cs);
-        TC_TRY(z.step(1, cs, side));
+        TC_TRY(z.step(1, cs, side, direct ? rho : nullptr, to(1)));
         return side.wait();
     };
     auto rest = [&](cudaStream_t cs) -> tc_status {
         SideBranch side(cs);
         tc_status st = TC_OK;
-        for (int k = 2; k <= steps && st == TC_OK; k++) st = z.step(k, cs, side);
+        for (int k = 2; k <= steps && st == TC_OK; k++) st = z.step(k, cs, side, nullptr, to(k));
         const tc_status joined = side.wait();
         return st == TC_OK ? joined : st;
     };
-    auto tail = [&](cudaStream_t cs) -> tc_status { return z.tail(rho, cs); };
+    auto tail = [&](cudaStream_t cs) -> tc_status { return to(steps) ? TC_OK : z.tail(rho, cs); };
     return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
 }
 
