@@ -25,11 +25,17 @@
 // right, F_k = (F_{k-1} A' + T_{k-1} E) / k, so that only E, once, needs an
 // explicit adjoint.  On the DMMA GEMM the recurrence alone took 1.7 s at
 // n = 11 (real products 16 ms, complex ones 64 ms; 0.5 ms here).
+#include <algorithm>
+#include <array>
 #include <cmath>
+#include <functional>
+#include <map>
 #include <vector>
 
 #include "cgemm_oz.cuh"
+#include "graph.cuh"
 #include "paths.cuh"
+#include "timing.cuh"
 
 namespace tc {
 namespace {
@@ -279,17 +285,18 @@ tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cu
 // buffers, the segments between two sets.
 struct Chains {
     bool on = false;
+    StreamLease set;
     cudaStream_t w = nullptr, f = nullptr;
     OzMat BL[2], BF;
     CM L[2], XF;
     void *scratch_w = nullptr, *scratch_f = nullptr;
-    cudaEvent_t start = nullptr, lambda[2] = {}, used[2] = {}, seg[2] = {}, freed[2] = {};
+    cudaEvent_t lambda[2] = {}, used[2] = {}, seg[2] = {}, freed = nullptr;
     ~Chains() {
         if (on) {   // the caller's buffers are not in use once the call returns, also after an error
             cudaStreamSynchronize(w);
             cudaStreamSynchronize(f);
         }
-        for (cudaEvent_t e : {start, lambda[0], lambda[1], used[0], used[1], seg[0], seg[1], freed[0], freed[1]})
+        for (cudaEvent_t e : {lambda[0], lambda[1], used[0], used[1], seg[0], seg[1], freed})
             if (e) cudaEventDestroy(e);
     }
 };
@@ -299,6 +306,7 @@ tc_status make_event(cudaEvent_t* e) {
 }
 
 constexpr int kChainMax = 11;
+constexpr int kPiece = 16;   // steps a graph
 size_t chains_extra(int n, int steps, int ckpt_every) {
     const size_t N = (size_t)1 << n;
     const int c = ckpt_every < steps ? ckpt_every : steps;
@@ -456,7 +464,9 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     }
     ch.on = oz && chains_extra(n, steps, ckpt_every) > 0 && work_bytes >= backward_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
     if (ch.on) {
-        TC_TRY(side_streams(&ch.w, &ch.f));
+        TC_TRY(ch.set.take());
+        ch.w = ch.set->more[0];
+        ch.f = ch.set->more[1];
         for (OzMat* m2 : {&ch.BL[0], &ch.BL[1], &ch.BF}) TC_TRY(oz_mat_init(*m2, ar, N, false));
         ch.scratch_w = ar.take<uint8_t>(oz_scratch_bytes(N));
         ch.scratch_f = ar.take<uint8_t>(oz_scratch_bytes(N));
@@ -466,8 +476,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         if (b.nck > 1)
             for (int k = 0; k < b.c; k++) seg2.push_back(take_cm(ar, NN));
         if (!ch.XF.i || (b.nck > 1 && !seg2.back().i)) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
-        for (cudaEvent_t* e : {&ch.start, &ch.lambda[0], &ch.lambda[1], &ch.used[0], &ch.used[1], &ch.seg[0], &ch.seg[1],
-                               &ch.freed[0], &ch.freed[1]})
+        for (cudaEvent_t* e : {&ch.lambda[0], &ch.lambda[1], &ch.used[0], &ch.used[1], &ch.seg[0], &ch.seg[1], &ch.freed})
             TC_TRY(make_event(e));
     } else {   // one chain: every buffer and stream the same
         ch.w = ch.f = s;
@@ -476,25 +485,56 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         ch.XF = b.X;
         ch.scratch_w = ch.scratch_f = z.scratch;
     }
-    // Q <- U P U^dag, Q may be P; on the call's stream or the third chain's
-    auto fwd_step = [&](CM P, CM Q, bool third) -> tc_status {
-        if (oz)
-            return third ? step_oz(N, z.U, ch.BF, false, ch.BF, P, Q, ch.XF, ch.scratch_f, z.group, ch.f)
-                         : step_oz(N, z.U, z.B, false, z.B, P, Q, b.X, z.scratch, z.group, s);
-        if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, s));
-        return step(N, b.U, Q, b.X, 0, s);
+    // Q <- U P U^dag with the third chain's buffers, Q may be P
+    auto fwd_step = [&](CM P, CM Q, cudaStream_t cs) -> tc_status {
+        if (oz) return step_oz(N, z.U, ch.BF, false, ch.BF, P, Q, ch.XF, ch.scratch_f, z.group, cs);
+        if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, cs));
+        return step(N, b.U, Q, b.X, 0, cs);
+    };
+    // Runs `body` as a graph, captured at the first use of its key, or (no chains, timing) launch by launch.
+    const bool graphs = ch.on && !timing_enabled();
+    std::map<std::array<int, 4>, StepGraph> graph;
+    auto replay = [&](const std::array<int, 4>& key, cudaStream_t on, const std::function<tc_status(cudaStream_t)>& body) -> tc_status {
+        if (!graphs) return body(on);
+        const auto at = graph.try_emplace(key);
+        if (at.second) TC_TRY(at.first->second.capture(ch.set->s, body));
+        return at.first->second.launch(on);
+    };
+    const std::vector<CM>* sets[2] = {&seg, ch.on && b.nck > 1 ? &seg2 : &seg};
+    // the `len` states of a segment from the first one, in set[p]
+    auto states = [&](int p, int len, cudaStream_t on) -> tc_status {
+        const std::vector<CM>& v = *sets[p];
+        for (int lo = 1; lo < len; lo += kPiece) {
+            const int hi = std::min(len, lo + kPiece);
+            TC_TRY(replay({0, p, lo, hi}, on, [&](cudaStream_t cs) -> tc_status {
+                for (int i = lo; i < hi; i++) TC_TRY(fwd_step(v[i - 1], v[i], cs));
+                return TC_OK;
+            }));
+        }
+        return TC_OK;
     };
 
+    // H's trace and norm, which plan the Frechet series, read back before anything long is enqueued
+    double* Hs = b.B;   // build H into B, then shift and scale in place
+    TC_TRY(launch_build_h(m, Hs, s));
+    double trace = 0.0, norm1 = 0.0;
+    TC_TRY(matrix_trace_and_norm1(N, Hs, true, &trace, &norm1, b.small + 8, s));
+
     // ---------------------------------------------------------------- forward
-    // rho_k goes to its checkpoint, to the last segment's buffers, or to seg0 (the running state; rho_K)
+    // every segment's states in set 0 (the last segment's stay there), from one checkpoint to the next; rho_K to seg0
     TC_TRY(launch_split_c128(static_cast<const double*>(U), b.U.r, b.U.i, NN, s));
     TC_TRY(launch_split_c128(static_cast<const double*>(rho0), ck[0].r, ck[0].i, NN, s));
-    const int last0 = (b.nck - 1) * ckpt_every;   // the last segment is last0 .. steps - 1
-    CM cur = ck[0];
-    for (int k = 1; k <= steps; k++) {
-        const CM dst = k == steps ? b.seg0 : k % ckpt_every == 0 ? ck[k / ckpt_every] : k > last0 ? seg[k - last0] : b.seg0;
-        TC_TRY(fwd_step(cur, dst, false));
-        cur = dst;
+    auto length = [&](int j) { return std::min(ckpt_every, steps - j * ckpt_every); };
+    for (int j = 0; j < b.nck; j++) {
+        const int len = length(j);
+        TC_TRY(copy_cm(ck[j], seg[0], NN, s));
+        if (!oz && j + 1 < b.nck) {   // in place, with no copy a step
+            for (int i = 0; i < len; i++) TC_TRY(fwd_step(seg[0], seg[0], s));
+            TC_TRY(copy_cm(seg[0], ck[j + 1], NN, s));
+            continue;
+        }
+        TC_TRY(states(0, len, s));
+        TC_TRY(fwd_step(seg[len - 1], j + 1 < b.nck ? ck[j + 1] : b.seg0, s));
     }
     // loss from rho_K (in seg0)
     loss_kernel<<<1, 1024, 0, s>>>(b.seg0.r, O_diag, N, b.small);
@@ -503,64 +543,67 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // ---------------------------------------------------------------- backward
     diag_set_kernel<<<grid_for(NN), 256, 0, s>>>(O_diag, b.L.r, b.L.i, N);   // Lambda_K = O
     TC_LAUNCH_CHECK();
-    if (ch.on) {
-        TC_CUDA(cudaEventRecord(ch.start, s));
-        TC_CUDA(cudaStreamWaitEvent(ch.w, ch.start, 0));
-        TC_CUDA(cudaStreamWaitEvent(ch.f, ch.start, 0));
-    }
-    const std::vector<CM>* sets[2] = {&seg, ch.on && b.nck > 1 ? &seg2 : &seg};
-    // rho_{k0 + 1 .. k1 - 1} of segment j from its checkpoint
-    auto recompute = [&](int j, const std::vector<CM>& to) -> tc_status {
-        const int k0 = j * ckpt_every, k1 = k0 + ckpt_every;
-        for (int k = k0 + 1; k < k1; k++) TC_TRY(fwd_step(k == k0 + 1 ? ck[j] : to[k - 1 - k0], to[k - k0], true));
-        return TC_OK;
-    };
     bool w_init = false, lambda_loaded = false;
-    bool used[2] = {false, false}, freed[2] = {false, false};
     int a = 0;   // buffer of the current Lambda
+    if (oz) {   // W accumulates from zero, Lambda_K is loaded
+        TC_CUDA(cudaMemsetAsync(b.W.r, 0, NN * sizeof(double), s));
+        TC_CUDA(cudaMemsetAsync(b.W.i, 0, NN * sizeof(double), s));
+        TC_TRY(oz_mat_load(ch.BL[0], b.L.r, b.L.i, false, false, N, (size_t)N, s));
+        lambda_loaded = w_init = true;
+    }
+    // the reverse steps of rho_k = v[hi - 1] .. v[lo]: Lambda_k = U^dag Lambda_{k+1} U (the step with conj(U)),
+    // W += rho_k Lambda_k
+    auto reverse = [&](const std::vector<CM>& v, int lo, int hi, cudaStream_t cs) -> tc_status {
+        const cudaStream_t w = ch.on ? ch.w : cs;
+        bool used[2] = {false, false};
+        for (int i = hi - 1; i >= lo; i--) {
+            if (!oz) {
+                TC_TRY(step(N, b.U, b.L, b.X, 1, cs));
+                TC_TRY(gemm_c(N, v[i], 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, cs));
+                w_init = true;
+                continue;
+            }
+            const int nx = a ^ 1;
+            if (ch.on && used[nx]) TC_CUDA(cudaStreamWaitEvent(cs, ch.used[nx], 0));
+            TC_TRY(step_oz(N, z.Uc, ch.BL[a], lambda_loaded, z.B, ch.L[a], ch.L[nx], b.X, z.scratch, z.group, cs));
+            TC_TRY(oz_mat_load(ch.BL[nx], ch.L[nx].r, ch.L[nx].i, false, false, N, (size_t)N, cs));
+            lambda_loaded = true;
+            if (ch.on) {
+                TC_CUDA(cudaEventRecord(ch.lambda[nx], cs));
+                TC_CUDA(cudaStreamWaitEvent(w, ch.lambda[nx], 0));
+            }
+            // Lambda Hermitian: rho Lambda = rho Lambda^H
+            TC_TRY(mul_oz(N, z, v[i], ch.BL[nx], true, ch.L[nx], false, b.W, true, ch.scratch_w, w));
+            if (ch.on) TC_CUDA(cudaEventRecord(ch.used[nx], w));
+            used[nx] = true;
+            a = nx;
+        }
+        // the accumulation joins (its products are in sequence, the last one marks the end)
+        return ch.on && used[a] ? (cudaStreamWaitEvent(cs, ch.used[a], 0) == cudaSuccess
+                                       ? TC_OK : fail(TC_ERR_CUDA, "backward: joining the chains")) : TC_OK;
+    };
     for (int j = b.nck - 1; j >= 0; j--) {
-        const int par = (b.nck - 1 - j) & 1;
-        const int k0 = j * ckpt_every;
-        const int k1 = (k0 + ckpt_every < steps) ? k0 + ckpt_every : steps;   // segment k0 .. k1-1
+        const int par = (b.nck - 1 - j) & 1, len = length(j);
         if (!ch.on && j < b.nck - 1) {
-            TC_TRY(recompute(j, seg));
+            TC_TRY(copy_cm(ck[j], seg[0], NN, s));
+            TC_TRY(states(0, len, s));
             lambda_loaded = false;   // the one right operand now holds a state
         }
-        if (ch.on && j > 0) {   // the next segment beside this one
-            if (freed[par ^ 1]) TC_CUDA(cudaStreamWaitEvent(ch.f, ch.freed[par ^ 1], 0));
-            TC_TRY(recompute(j - 1, *sets[par ^ 1]));
+        if (ch.on && j > 0) {   // the next segment beside this one, once the reverse steps of the last are done with its buffers
+            TC_CUDA(cudaEventRecord(ch.freed, s));
+            TC_CUDA(cudaStreamWaitEvent(ch.f, ch.freed, 0));
+            TC_TRY(copy_cm(ck[j - 1], (*sets[par ^ 1])[0], NN, ch.f));
+            TC_TRY(states(par ^ 1, ckpt_every, ch.f));
             TC_CUDA(cudaEventRecord(ch.seg[par ^ 1], ch.f));
         }
-        if (ch.on && j < b.nck - 1) TC_CUDA(cudaStreamWaitEvent(ch.w, ch.seg[par], 0));
-        for (int k = k1 - 1; k >= k0; k--) {
-            const CM rho_k = k == k0 ? ck[j] : (*sets[par])[k - k0];
-            // Lambda_k = U^dag Lambda_{k+1} U  (the step with conj(U)); W += rho_k Lambda_k
-            if (oz) {
-                const int nx = a ^ 1;
-                if (ch.on && used[nx]) TC_CUDA(cudaStreamWaitEvent(s, ch.used[nx], 0));
-                TC_TRY(step_oz(N, z.Uc, ch.BL[a], lambda_loaded, z.B, ch.L[a], ch.L[nx], b.X, z.scratch, z.group, s));
-                TC_TRY(oz_mat_load(ch.BL[nx], ch.L[nx].r, ch.L[nx].i, false, false, N, (size_t)N, s));
-                lambda_loaded = true;
-                if (ch.on) {
-                    TC_CUDA(cudaEventRecord(ch.lambda[nx], s));
-                    TC_CUDA(cudaStreamWaitEvent(ch.w, ch.lambda[nx], 0));
-                }
-                // Lambda Hermitian: rho Lambda = rho Lambda^H
-                TC_TRY(mul_oz(N, z, rho_k, ch.BL[nx], true, ch.L[nx], false, b.W, w_init, ch.scratch_w, ch.w));
-                if (ch.on) TC_CUDA(cudaEventRecord(ch.used[nx], ch.w));
-                used[nx] = true;
-                a = nx;
-            } else {
-                TC_TRY(step(N, b.U, b.L, b.X, 1, s));
-                TC_TRY(gemm_c(N, rho_k, 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, s));
-            }
-            w_init = true;
+        if (ch.on && j < b.nck - 1) TC_CUDA(cudaStreamWaitEvent(s, ch.seg[par], 0));
+        for (int hi = len; hi > 0; hi = (hi - 1) / kPiece * kPiece) {
+            const int lo = (hi - 1) / kPiece * kPiece, from = a;
+            TC_TRY(replay({1 + 2 * from + par, lo, hi, 0}, s,
+                          [&](cudaStream_t cs) { return reverse(*sets[par], lo, hi, cs); }));
+            a = from ^ ((hi - lo) & 1);
         }
-        if (ch.on) TC_CUDA(cudaEventRecord(ch.freed[par], ch.w));
-        freed[par] = true;
     }
-    // the chains meet (the third one's work was waited for by the second)
-    if (ch.on) TC_CUDA(cudaStreamWaitEvent(s, ch.used[a], 0));
     // M = W U^dag = W conj(U)  -> into L (free now)
     CM M = b.L;
     if (oz)
@@ -569,11 +612,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         TC_TRY(gemm_c(N, b.W, 0, b.U, 1, M, 1.0, 0.0, 0, s));
 
     // ---------------------------------------------------------------- Frechet
-    // plan from H's trace and norm (computed on the device, read back)
-    double* Hs = b.B;   // build H into B, then shift and scale in place
-    TC_TRY(launch_build_h(m, Hs, s));
-    double trace = 0.0, norm1 = 0.0;
-    TC_TRY(matrix_trace_and_norm1(N, Hs, true, &trace, &norm1, b.small + 8, s));
+    // plan from H's trace and norm
     const double mu = trace / N;
     double bn = norm1 * dt;
     int sq = 0;

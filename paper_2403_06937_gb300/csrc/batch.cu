@@ -7,7 +7,6 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
-#include <mutex>
 #include <numeric>
 #include <vector>
 
@@ -22,34 +21,8 @@
 namespace tc {
 namespace {
 
-// Streams on which the systems of a batch in the FP64 forms run side by side
-// (one pool per device, created on first use), with a fork event and one join
-// event per lane.
-constexpr int kOzLanes = 8;
-struct OzLanes {
-    cudaStream_t s[kOzLanes] = {};
-    cudaEvent_t join[kOzLanes] = {};
-    cudaEvent_t fork = nullptr;
-};
-std::mutex g_lanes_mu;
-OzLanes g_lanes[64];
-
-tc_status oz_lanes(OzLanes** out) {
-    int dev = 0;
-    TC_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return fail(TC_ERR_UNSUPPORTED_DEVICE, "device index out of range");
-    std::lock_guard<std::mutex> lk(g_lanes_mu);
-    OzLanes& l = g_lanes[dev];
-    if (!l.fork) {
-        for (int i = 0; i < kOzLanes; i++) {
-            TC_CUDA(cudaStreamCreateWithFlags(&l.s[i], cudaStreamNonBlocking));
-            TC_CUDA(cudaEventCreateWithFlags(&l.join[i], cudaEventDisableTiming));
-        }
-        TC_CUDA(cudaEventCreateWithFlags(&l.fork, cudaEventDisableTiming));
-    }
-    *out = &l;
-    return TC_OK;
-}
+// Systems of a batch in the FP64 forms run side by side on this many streams.
+constexpr int kOzLanes = StreamSet::kLanes;
 
 // The systems of a batch spread over at most kOzLanes lanes: largest first to
 // the lane with the least work (N^3 each).
@@ -111,8 +84,6 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
         lane = assign_lanes(count, n);
     }
     const int L = (int)lane.size();
-    OzLanes* ls = nullptr;
-    TC_TRY(oz_lanes(&ls));
     Arena all{static_cast<char*>(work), work_bytes, 0};
     std::vector<char*> base(L);
     std::vector<size_t> bytes(L, 0);
@@ -123,8 +94,16 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
     }
     auto none = [](cudaStream_t) -> tc_status { return TC_OK; };
     auto run = [&](cudaStream_t cs) -> tc_status {
-        TC_CUDA(cudaEventRecord(ls->fork, cs));
-        for (int l = 0; l < L; l++) TC_CUDA(cudaStreamWaitEvent(ls->s[l], ls->fork, 0));
+        StreamLease own;   // outside a capture of this call's: a set for the lanes alone
+        StreamSet* ls = leased_streams();
+        if (!ls || ls->s != cs) {
+            TC_TRY(own.take());
+            ls = own.get();
+            TC_TRY(ls->create_lanes());
+            ls->in_callers_graph = caller_captures(cs);
+        }
+        TC_CUDA(cudaEventRecord(ls->lane_fork, cs));
+        for (int l = 0; l < L; l++) TC_CUDA(cudaStreamWaitEvent(ls->lane[l], ls->lane_fork, 0));
         tc_status st = TC_OK;
         for (int l = 0; l < L && st == TC_OK; l++)
             for (int b : lane[l]) {
@@ -135,18 +114,19 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
                 const double* Ub = static_cast<const double*>(U[b]);
                 double* rb = static_cast<double*>(rho[b]);
                 if (precision == TC_FP64_OZAKI || (!dmma && f64_on_tensor_cores(n[b])))
-                    st = evolve_oz(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->s[l]);
+                    st = evolve_oz(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->lane[l]);
                 else
-                    st = evolve_f64(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->s[l]);
+                    st = evolve_f64(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->lane[l]);
             }
         // every lane joins back, also after a failure (a capture ends only with its streams joined)
         for (int l = 0; l < L; l++) {
-            cudaEventRecord(ls->join[l], ls->s[l]);
-            cudaStreamWaitEvent(cs, ls->join[l], 0);
+            cudaEventRecord(ls->lane_join[l], ls->lane[l]);
+            cudaStreamWaitEvent(cs, ls->lane_join[l], 0);
         }
         return st;
     };
-    return run_captured(us, none, run, none, steps >= 1 && !timing_enabled());
+    auto first = [](cudaStream_t) -> tc_status { return leased_streams() ? leased_streams()->create_lanes() : TC_OK; };
+    return run_captured(us, first, run, none, steps >= 1 && !timing_enabled());
 }
 
 }  // namespace

@@ -113,7 +113,8 @@ struct OzSystem {
                     cudaStream_t cs);
     // the row is read beside the next step's first product when `side` is a branch of cs
     // from, to (residue form, no padding): rho read interleaved in place of the planes, rho' written interleaved
-    tc_status step(int k, cudaStream_t cs, SideBranch& side, const double* from = nullptr, double* to = nullptr);
+    tc_status step(int k, cudaStream_t cs, SideBranch& side, const double* from = nullptr, double* to = nullptr,
+                   unsigned* row = nullptr);
     // true when a step may read and write the caller's interleaved rho itself
     bool interleaved() const;
     tc_status tail(double* rho, cudaStream_t cs);

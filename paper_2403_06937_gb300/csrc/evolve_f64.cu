@@ -46,7 +46,7 @@ tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_
     g2.Cr = Rr; g2.Ci = Ri;
     g2.herm_lower = 1;
 
-    auto one_step = [&](int k, cudaStream_t cs) -> tc_status {
+    auto one_step = [&](int k, cudaStream_t cs, SideBranch&, unsigned* row) -> tc_status {
         {
             ProductTimer t(8.0 * (double)N * N * N, cs);   // X = U rho: 8 N^3
             TC_TRY(gemm_f64(g1, cs));
@@ -57,22 +57,19 @@ tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_
         }
         if (renorm_every > 0 && k % renorm_every == 0)
             TC_TRY(launch_renormalise(kRhoPlanarF64, Rr, Ri, n, scratch, cs));
-        if (obs) TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs + (size_t)k * stride, scratch, cs));
+        if (obs)
+            TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs + (size_t)(row ? 1 : k) * stride, scratch, cs, 0,
+                                      row));
         return TC_OK;
     };
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(launch_split_c128(U, Ur, Ui, NN, cs));
         TC_TRY(launch_split_c128(rho, Rr, Ri, NN, cs));
         if (obs) TC_TRY(launch_observables(kRhoPlanarF64, Rr, Ri, m, n, obs, scratch, cs));
-        if (steps >= 1) TC_TRY(one_step(1, cs));
-        return TC_OK;
-    };
-    auto rest = [&](cudaStream_t cs) -> tc_status {
-        for (int k = 2; k <= steps; k++) TC_TRY(one_step(k, cs));
         return TC_OK;
     };
     auto tail = [&](cudaStream_t cs) -> tc_status { return launch_join_c128(Rr, Ri, rho, NN, cs); };
-    return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
+    return run_steps(s, steps, renorm_every, false, observables_row(scratch, n), first, one_step, tail, steps > 2 && !timing_enabled());
 }
 
 }  // namespace tc

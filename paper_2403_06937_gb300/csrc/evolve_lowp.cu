@@ -457,7 +457,7 @@ tc_status evolve_lowp(const double* U, double* rho, int n, int steps, int precis
     const double prod = (double)cgemm_products(precision);
 
     // the observable row is read beside the next step's first product when `side` is a branch of cs
-    auto one_step = [&](int k, cudaStream_t cs, SideBranch& side) -> tc_status {
+    auto one_step = [&](int k, cudaStream_t cs, SideBranch& side, unsigned* row) -> tc_status {
         {
             ProductTimer t(8.0 * N3 * prod, cs);
             TC_TRY(cgemm_tc(precision, 0, tmU, tmR, e1, cs, tune.tc_stages, &sp.wU, &sp.wR, &sp.nR));
@@ -470,8 +470,8 @@ tc_status evolve_lowp(const double* U, double* rho, int n, int steps, int precis
         if (renorm_every > 0 && k % renorm_every == 0) TC_TRY(lowp_renorm(precision, b, cs));
         if (obs) {
             TC_TRY(side.begin());
-            TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs + (size_t)k * stride, b.scratch,
-                                      side.stream(), (size_t)b.Np));
+            TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs + (size_t)(row ? 1 : k) * stride, b.scratch,
+                                      side.stream(), (size_t)b.Np, row));
             TC_TRY(side.end());
         }
         return TC_OK;
@@ -479,19 +479,10 @@ tc_status evolve_lowp(const double* U, double* rho, int n, int steps, int precis
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(lowp_prep(precision, U, rho, b, cs));
         if (obs) TC_TRY(launch_observables(kRhoPlanarF32, b.Rr, b.Ri, m, n, obs, b.scratch, cs, (size_t)b.Np));
-        SideBranch side(cs);
-        if (steps >= 1) TC_TRY(one_step(1, cs, side));
-        return side.wait();
-    };
-    auto rest = [&](cudaStream_t cs) -> tc_status {
-        SideBranch side(cs);
-        tc_status st = TC_OK;
-        for (int k = 2; k <= steps && st == TC_OK; k++) st = one_step(k, cs, side);
-        const tc_status joined = side.wait();
-        return st == TC_OK ? joined : st;
+        return TC_OK;
     };
     auto tail = [&](cudaStream_t cs) -> tc_status { return lowp_finish(b, rho, cs); };
-    return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
+    return run_steps(s, steps, renorm_every, false, observables_row(b.scratch, n), first, one_step, tail, steps > 2 && !timing_enabled());
 }
 
 int lowp_host_chunks(int n, int precision) {

@@ -121,7 +121,7 @@ tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, d
 
 bool OzSystem::interleaved() const { return N == Np && oz_modular(); }
 
-tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double* from, double* to) {
+tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double* from, double* to, unsigned* row) {
     const size_t NN = (size_t)Np * Np;
     const double N3 = (double)N * N * N;
     OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
@@ -147,7 +147,7 @@ tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double*
     if (obs) {
         TC_TRY(side.begin());
         TC_TRY(launch_observables(to ? kRhoInterleaved : kRhoPlanarF64, to ? to : Rr, Ri, m, n,
-                                  obs + (size_t)k * TC_OBS_STRIDE(n), scratch, side.stream(), (size_t)Np));
+                                  obs + (size_t)(row ? 1 : k) * TC_OBS_STRIDE(n), scratch, side.stream(), (size_t)Np, row));
         TC_TRY(side.end());
     }
     return TC_OK;
@@ -185,20 +185,14 @@ tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_e
         return direct && k == steps && !(renorm_every > 0 && k % renorm_every == 0) ? rho : nullptr;
     };
     auto first = [&](cudaStream_t cs) -> tc_status {
-        TC_TRY(z.first(U, rho, m, obs, renorm_every, !direct, cs));
-        SideBranch side(cs);
-        TC_TRY(z.step(1, cs, side, direct ? rho : nullptr, to(1)));
-        return side.wait();
+        return z.first(U, rho, m, obs, renorm_every, !direct, cs);
     };
-    auto rest = [&](cudaStream_t cs) -> tc_status {
-        SideBranch side(cs);
-        tc_status st = TC_OK;
-        for (int k = 2; k <= steps && st == TC_OK; k++) st = z.step(k, cs, side, nullptr, to(k));
-        const tc_status joined = side.wait();
-        return st == TC_OK ? joined : st;
+    auto one_step = [&](int k, cudaStream_t cs, SideBranch& side, unsigned* row) -> tc_status {
+        return z.step(k, cs, side, direct && k == 1 ? rho : nullptr, to(k), row);
     };
     auto tail = [&](cudaStream_t cs) -> tc_status { return to(steps) ? TC_OK : z.tail(rho, cs); };
-    return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
+    return run_steps(s, steps, renorm_every, to(steps) != nullptr, observables_row(z.scratch, n), first, one_step, tail,
+                     steps > 2 && !timing_enabled());
 }
 
 }  // namespace tc

@@ -140,7 +140,13 @@ __global__ void obs_partial_kernel(Rho<L> rho, Model m, int has_model, int n, do
 // One warp per column of the partials: lanes stride the blocks, then a tree
 // in a fixed order.  (One thread per column, adding the blocks one after
 // another, waited for up to 1024 dependent loads: 57 us at n = 12.)
-__global__ void __launch_bounds__(1024) obs_final_kernel(const double* partials, int blocks, int stride, double* out) {
+__global__ void __launch_bounds__(1024) obs_final_kernel(const double* partials, int blocks, int stride, double* out,
+                                                         unsigned* row) {
+    if (row) {   // the next row of a run; the counter moves on once every warp has read it
+        out += (size_t)*row * stride;
+        __syncthreads();
+        if (threadIdx.x == 0) *row += 1;
+    }
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int j = warp; j < stride; j += 32) {
         double s = 0.0;
@@ -196,12 +202,14 @@ __global__ void expectation_diag_kernel(const double* rho, const double* O, unsi
 
 }  // namespace
 
-size_t observables_scratch_bytes(int n) {
-    return round256((size_t)obs_grid(n) * (2 * n + 5) * sizeof(double)) + 256;
+static size_t partials_bytes(int n) { return round256((size_t)obs_grid(n) * (2 * n + 5) * sizeof(double)); }
+size_t observables_scratch_bytes(int n) { return partials_bytes(n) + 256; }
+unsigned* observables_row(double* scratch, int n) {
+    return reinterpret_cast<unsigned*>(reinterpret_cast<char*>(scratch) + partials_bytes(n));
 }
 
 tc_status launch_observables(int layout, const void* a, const void* b, const Model* m, int n,
-                             double* out, double* scratch, cudaStream_t s, size_t ld) {
+                             double* out, double* scratch, cudaStream_t s, size_t ld, unsigned* row) {
     if (ld == 0) ld = (size_t)1 << n;
     unsigned grid = obs_grid(n);
     Model mm{};
@@ -225,7 +233,7 @@ tc_status launch_observables(int layout, const void* a, const void* b, const Mod
             return fail(TC_ERR_INVALID_ARG, "observables: unknown layout");
     }
     TC_LAUNCH_CHECK();
-    obs_final_kernel<<<1, 1024, 0, s>>>(scratch, (int)grid, 2 * n + 5, out);
+    obs_final_kernel<<<1, 1024, 0, s>>>(scratch, (int)grid, 2 * n + 5, out, row);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
