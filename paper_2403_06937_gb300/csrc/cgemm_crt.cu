@@ -68,10 +68,18 @@ constexpr int kRB = 128;                     // bytes of K per operand row in a 
 constexpr int kTile = 128 * kRB;             // one 128-row operand tile
 constexpr int kKPer = kRB / 2;               // BF16 K values per stage
 constexpr int kSteps = kRB / 32;             // MMA K steps per stage
-constexpr int kRing = 192 * 1024;
-constexpr int kStage = 2 * kTile;            // own 128 rows of A and of B
-constexpr int kStages = kRing / kStage;      // 6
-constexpr int kSmem = kRing + 1024 /*align*/ + 512 /*barriers*/;
+// Column tiles of NT: 256, or half the matrix up to Np = 256 (Ring<64>, Ring<128>).  Shared memory is
+// asked for as if the ring were full in each: one CTA an SM, whatever else runs beside it.  Two pairs on one
+// pair of SMs could each wait in tcgen05.alloc for the other (each CTA allocates for both).
+template <int NT>
+struct Ring {
+    static constexpr int kBRows = NT / 2;                     // of B, a CTA
+    static constexpr int kStage = kTile + kBRows * kRB;       // own 128 rows of A and half of B's
+    static constexpr int kStages = NT == 256 ? 6 : 4;
+    static constexpr int kBytes = kStages * kStage;
+    static constexpr int kSmem = 192 * 1024 + 1024 /*align*/ + 512 /*barriers*/;
+    static_assert(kBytes <= 192 * 1024, "ring");
+};
 constexpr int kChunkStages = crt::kChunk / kKPer;
 constexpr int kGroup = 8;                    // 256-row tiles per raster group (a wave: ~8 x 9 tiles)
 constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN
@@ -89,8 +97,14 @@ struct CrtLaunch {
 };
 
 // unit -> (plane, row tile, column tile), in tiles of 256
-template <int MODE>
+template <int MODE, int NT>
 __device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int& z, int& P, int& J) {
+    if (NT < 256) {   // one row of two tiles a plane
+        z = u >> 1;
+        P = 0;
+        J = u & 1;
+        return;
+    }
     z = u / L.units_per;
     const int t = u - z * L.units_per, side = (L.tiles + 1) / 2;
     if (MODE == 1) {
@@ -209,13 +223,47 @@ __device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_t
     }
 }
 
-template <int MODE>
+// A chunk that is all of K, straight to bytes: columns c .. c + NT / 2 - 1 of a thread's row.  `done` as above.
+template <int COLS, typename Done>
+__device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, uint4 (&y)[COLS / 16], Done done) {
+    const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
+    const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic);
+    const uint64_t b2 = pack2(kMagic + 128.0f, kMagic + 128.0f);
+    auto four = [&](const float* x) -> uint32_t {   // |residue| <= p / 2 + 1 < 128: any representative will do
+        uint32_t v[4];
+#pragma unroll
+        for (int q = 0; q < 4; q += 2) {
+            const uint64_t x2 = pack2(x[q], x[q + 1]);
+            const uint64_t q2 = add2(fma2(x2, inv2, m2), m2n);
+            unpack2(add2(fma2(q2, p2n, x2), b2), v[q], v[q + 1]);
+        }
+        return __byte_perm(__byte_perm(v[0], v[1], 0x0040), __byte_perm(v[2], v[3], 0x0040), 0x5410);
+    };
+    float a[2][8], b[2][8];
+    tmem_ld8(tl, a[0]);
+    tmem_ld8(tl + 8, b[0]);
+#pragma unroll
+    for (int c = 0; c < COLS; c += 16) {
+        const int k = (c >> 4) & 1;
+        tmem_wait8(a[k], b[k]);
+        if (c + 16 < COLS) {
+            tmem_ld8(tl + c + 16, a[k ^ 1]);
+            tmem_ld8(tl + c + 24, b[k ^ 1]);
+        } else {
+            done();
+        }
+        y[c / 16] = make_uint4(four(a[k]), four(a[k] + 4), four(b[k]), four(b[k] + 4));
+    }
+}
+
+template <int MODE, int NT>
 __global__ void __launch_bounds__(kThreads, 1)
     cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
-    constexpr uint32_t kIdesc = make_idesc(1u, 256u, 256u);
+    constexpr uint32_t kIdesc = make_idesc(1u, 256u, (uint32_t)NT);
+    constexpr int kStages = Ring<NT>::kStages, kStage = Ring<NT>::kStage;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + Ring<NT>::kBytes);
     uint64_t* empty = full + kStages;
     uint64_t* accum = empty + kStages;   // [2] MMA -> epilogue, one per buffer
     uint64_t* tmem_empty = accum + 2;        // [2] both epilogues -> MMA (even CTA, count 2)
@@ -242,7 +290,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc_pair(saddr(tmem_slot), 512);
+        tmem_alloc_pair(saddr(tmem_slot), 2 * NT);
         tmem_relinquish_pair();
     }
     if (warp == 8 && lane == 0) {
@@ -264,8 +312,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             for (int u = worker; u < L.units && ok; u += workers) {
                 int z, P, J;
-                unit_at<MODE>(L, u, z, P, J);
-                const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * 128;
+                unit_at<MODE, NT>(L, u, z, P, J);
+                const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * Ring<NT>::kBRows;
                 for (int kb = 0; kb < L.kb_total; kb++, it++) {
                     const int b = it % kStages;
                     const uint32_t ph = (it / kStages) & 1u;
@@ -333,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint64_t bd = desc_kmajor<kRB>(saddr(st + kTile));
 #pragma unroll
                         for (int ks = 0; ks < kSteps; ks++)   // 32 bytes of K further in each row
-                            umma_pair(tmem + 256u * buf, ad + 2u * (uint64_t)ks, bd + 2u * (uint64_t)ks, kIdesc,
+                            umma_pair(tmem + (uint32_t)NT * buf, ad + 2u * (uint64_t)ks, bd + 2u * (uint64_t)ks, kIdesc,
                                       (kb > kb0 || ks > 0) ? 1u : 0u);
                         umma_commit_pair(saddr(&empty[b]));
                         umma_commit_pair(peer_empty + 8u * (uint32_t)b);
@@ -353,13 +401,30 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lead_tmem_empty = cluster_addr(saddr(&tmem_empty[0]), 0u);
         const int half = warp >> 2;
         const int row = (warp & 3) * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * (uint32_t)half;
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(NT / 2) * (uint32_t)half;
         uint32_t pass = 0;
         bool stop = false;
         for (int u = worker; u < L.units && !stop; u += workers) {
             int z, P, J;
-            unit_at<MODE>(L, u, z, P, J);
+            unit_at<MODE, NT>(L, u, z, P, J);
             const float p = (float)kC.p[z % kModuli], inv_p = 1.0f / p;
+            if constexpr (NT < 256) {   // one chunk
+                const uint32_t buf = pass & 1u;
+                if (!chunk_ready(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
+                    stop = true;
+                    break;
+                }
+                uint4 w[NT / 32];
+                chunk_bytes<NT / 2>(tl + (uint32_t)NT * buf, p, inv_p, w,
+                                    [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
+                pass++;
+                if ((int)rank * 128 >= (int)L.Np) continue;   // Np = 128: the odd CTA's rows lie outside
+                uint4* y = reinterpret_cast<uint4*>(L.bytes + ((size_t)z * L.band + (size_t)((int)rank * 128 + row)) * L.Np +
+                                                    (size_t)(J * NT + NT / 2 * half));
+#pragma unroll
+                for (int c = 0; c < NT / 32; c++) y[c] = w[c];
+                continue;
+            }
             // rows and columns past the end (an odd number of 128-tiles) are not written
             const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
             uint32_t acc[64];
@@ -406,7 +471,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster_sync();   // neither CTA frees TMEM or leaves while the other may still use it
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem, 512);
+        tmem_dealloc_pair(tmem, 2 * NT);
     }
 }
 
@@ -828,9 +893,10 @@ int sm_count() {
     return sms;
 }
 
-template <int MODE>
+template <int MODE, int NT>
 tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
-    auto k = cgemm_crt_kernel<MODE>;
+    constexpr int kSmem = Ring<NT>::kSmem;
+    auto k = cgemm_crt_kernel<MODE, NT>;
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -862,6 +928,16 @@ int band_rows(int Np) { return Np <= 16384 ? Np : 4096; }
 
 size_t plane_bytes(int Np, int planes) { return round256((size_t)planes * Np * Np * 2); }
 
+// Half the columns a unit up to Np = 256, where one 256-column tile a plane leaves 88 of 152 SMs idle and
+// the epilogue's 128 columns a warp are a third of the launch (n = 8: 9.8 us).
+bool narrow_tiles(int Np) { return Np <= 256; }
+
+tc_status maps(CrtMat& m) {
+    TC_TRY(make_part_map_rows(&m.map, m.planes, m.Np, m.count, TC_BF16X3, kRB));
+    return !m.left && narrow_tiles(m.Np)
+               ? make_part_map_rows(&m.narrow, m.planes, m.Np, m.count, TC_BF16X3, kRB, m.Np / 4) : TC_OK;
+}
+
 tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
     m.Np = Np;
     m.left = left;
@@ -870,7 +946,7 @@ tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
     m.ex = ar.take<int>((size_t)Np);
     m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
     if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
-    return make_part_map_rows(&m.map, m.planes, Np, planes, TC_BF16X3, kRB);
+    return maps(m);
 }
 
 // The residue products of one band of rows (all of them: lo = 0, hi = side).
@@ -887,7 +963,11 @@ tc_status gemm(int mode, const CrtMat& A, const CrtMat& B, int lo, int hi, void*
     L.status = device_status_word();
     L.units_per = mode == 0 ? side * (hi - lo) : hi * (hi + 1) / 2 - lo * (lo + 1) / 2;
     L.units = L.units_per * A.count;
-    return mode == 0 ? launch<0>(A.map, B.map, L, s) : launch<1>(A.map, B.map, L, s);
+    if (narrow_tiles(A.Np)) {   // the whole matrix in either mode
+        L.units = 2 * A.count;
+        return A.Np == 128 ? launch<0, 64>(A.map, B.narrow, L, s) : launch<0, 128>(A.map, B.narrow, L, s);
+    }
+    return mode == 0 ? launch<0, 256>(A.map, B.map, L, s) : launch<1, 256>(A.map, B.map, L, s);
 }
 
 }  // namespace
@@ -905,7 +985,7 @@ tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
     if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
     view = base;
     view.Np = Np;
-    return make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
+    return maps(view);
 }
 
 tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
