@@ -223,9 +223,9 @@ __device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_t
     }
 }
 
-// A chunk that is all of K, straight to bytes: columns c .. c + NT / 2 - 1 of a thread's row.  `done` as above.
+// A chunk that is all of K, straight to bytes: COLS columns of a thread's row, to y if `own`.  `done` as above.
 template <int COLS, typename Done>
-__device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, uint4 (&y)[COLS / 16], Done done) {
+__device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, uint4* y, bool own, Done done) {
     const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
     const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic);
     const uint64_t b2 = pack2(kMagic + 128.0f, kMagic + 128.0f);
@@ -252,7 +252,8 @@ __device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, u
         } else {
             done();
         }
-        y[c / 16] = make_uint4(four(a[k]), four(a[k] + 4), four(b[k]), four(b[k] + 4));
+        const uint4 w = make_uint4(four(a[k]), four(a[k] + 4), four(b[k]), four(b[k] + 4));
+        if (own) y[c / 16] = w;
     }
 }
 
@@ -408,25 +409,21 @@ __global__ void __launch_bounds__(kThreads, 1)
             int z, P, J;
             unit_at<MODE, NT>(L, u, z, P, J);
             const float p = (float)kC.p[z % kModuli], inv_p = 1.0f / p;
-            if constexpr (NT < 256) {   // one chunk
+            // rows and columns past the end (an odd number of 128-tiles) are not written
+            const bool own = 2 * P + (int)rank < L.tiles && (NT < 256 || 2 * J + half < L.tiles);
+            uint8_t* y = L.bytes + ((size_t)z * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
+                         (size_t)(J * NT + NT / 2 * half);
+            if (NT < 256 || chunks == 1) {
                 const uint32_t buf = pass & 1u;
                 if (!chunk_ready(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
                     stop = true;
                     break;
                 }
-                uint4 w[NT / 32];
-                chunk_bytes<NT / 2>(tl + (uint32_t)NT * buf, p, inv_p, w,
+                chunk_bytes<NT / 2>(tl + (uint32_t)NT * buf, p, inv_p, reinterpret_cast<uint4*>(y), own,
                                     [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
                 pass++;
-                if ((int)rank * 128 >= (int)L.Np) continue;   // Np = 128: the odd CTA's rows lie outside
-                uint4* y = reinterpret_cast<uint4*>(L.bytes + ((size_t)z * L.band + (size_t)((int)rank * 128 + row)) * L.Np +
-                                                    (size_t)(J * NT + NT / 2 * half));
-#pragma unroll
-                for (int c = 0; c < NT / 32; c++) y[c] = w[c];
                 continue;
             }
-            // rows and columns past the end (an odd number of 128-tiles) are not written
-            const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
             uint32_t acc[64];
 #pragma unroll
             for (int c = 0; c < 64; c++) acc[c] = 0u;
@@ -440,8 +437,6 @@ __global__ void __launch_bounds__(kThreads, 1)
                                [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
             }
             if (stop || !own) continue;
-            uint8_t* y = L.bytes + ((size_t)z * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
-                         (size_t)J * 256 + 128 * half;
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
                 uint32_t wl[4], wh[4];
