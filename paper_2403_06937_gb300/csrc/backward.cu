@@ -242,78 +242,37 @@ size_t oz_backward_extra(int n) {
            2 * round256(N * N * sizeof(double)) + 256;
 }
 
-// Q <- A P A^H from P's planes, loaded into `Bp` already or here; B, X, scratch: the product's own (B may
-// be Bp); Q may be P
-tc_status step_oz(int N, const OzMat& A, OzMat& Bp, bool loaded, OzMat& B, CM P, CM Q, CM X, void* scratch, int group,
-                  cudaStream_t s) {
-    if (!loaded) TC_TRY(oz_mat_load(Bp, P.r, P.i, false, false, N, (size_t)N, s));
-    TC_TRY(oz_product(0, A, Bp, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, scratch}, group, s));   // X = A P^H
-    TC_TRY(oz_mat_load(B, X.r, X.i, false, false, N, (size_t)N, s));
-    return oz_product(1, A, B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, scratch}, group, s);     // Q = A X^H
+// Q <- A P A^H from P's planes, in z.B already or loaded here; Q may be P
+tc_status step_oz(int N, OzBufs& z, const OzMat& A, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
+    if (!loaded) TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
+    TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = A P^H
+    TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s));
+    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, z.scratch}, z.group, s);     // Q = A X^H
 }
 
-// out = A R^H (+ out): the left operand as it is, R's planes as they are or
-// conjugated, loaded into B already or here
-tc_status mul_oz(int N, OzBufs& z, CM A, OzMat& B, bool loaded, CM R, bool conj_r, CM out, bool add, void* scratch,
-                 cudaStream_t s) {
+// out = A R^H (+ out): the left operand as it is, R's planes as they are or conjugated
+tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
     if (A.r) TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s));   // else: as loaded last
-    if (!loaded) TC_TRY(oz_mat_load(B, R.r, R.i, false, conj_r, N, (size_t)N, s));
-    OzOut o{out.r, out.i, scratch};
+    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s));
+    OzOut o{out.r, out.i, z.scratch};
     o.conj_b = conj_r;
     if (add && !oz_modular()) {   // the digit form does not accumulate
         o.yr = z.Y.r;
         o.yi = z.Y.i;
-        TC_TRY(oz_product(0, z.A2, B, R.r, R.i, N, (size_t)N, o, z.group, s));
+        TC_TRY(oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s));
         const size_t NN = (size_t)N * N;
         axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, out.r, out.i, 1.0, z.Y.r, z.Y.i, out.r, out.i, NN);
         TC_LAUNCH_CHECK();
         return TC_OK;
     }
     o.accumulate = add;
-    return oz_product(0, z.A2, B, R.r, R.i, N, (size_t)N, o, z.group, s);
-}
-tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
-    return mul_oz(N, z, A, z.B, false, R, conj_r, out, add, z.scratch, s);
+    return oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s);
 }
 
-// Up to n = 11 the reverse pass runs as three chains side by side: the adjoint
-// steps on the call's stream, W += rho_k Lambda_k on a second, and the states
-// of the next segment on a third.  Their launches are a few us each at n <= 9
-// (a gradient at n = 8, 100 steps: 22.6 -> 16.6 ms) and at n = 11 one chain's
-// residues and recombinations run beside another's products.  Each chain has
-// its own operand and scratch; Lambda and its operand alternate between two
-// buffers, the segments between two sets.
-struct Chains {
-    bool on = false;
-    StreamLease set;
-    cudaStream_t w = nullptr, f = nullptr;
-    OzMat BL[2], BF;
-    CM L[2], XF;
-    void *scratch_w = nullptr, *scratch_f = nullptr;
-    cudaEvent_t lambda[2] = {}, used[2] = {}, seg[2] = {}, freed = nullptr;
-    ~Chains() {
-        if (on) {   // the caller's buffers are not in use once the call returns, also after an error
-            cudaStreamSynchronize(w);
-            cudaStreamSynchronize(f);
-        }
-        for (cudaEvent_t e : {lambda[0], lambda[1], used[0], used[1], seg[0], seg[1], freed})
-            if (e) cudaEventDestroy(e);
-    }
-};
-tc_status make_event(cudaEvent_t* e) {
-    TC_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
-    return TC_OK;
-}
-
-constexpr int kChainMax = 11;
-constexpr int kPiece = 16;   // steps a graph
-size_t chains_extra(int n, int steps, int ckpt_every) {
-    const size_t N = (size_t)1 << n;
-    const int c = ckpt_every < steps ? ckpt_every : steps;
-    const size_t segs = steps > ckpt_every ? (size_t)c * cm_bytes(n) : 0;
-    if (n < 7 || n > kChainMax || segs > ((size_t)4 << 30) || !oz_modular()) return 0;
-    return 3 * oz_mat_bytes((int)N, false) + 2 * oz_scratch_bytes((int)N) + 2 * cm_bytes(n) + segs;
-}
+// Steps of the forward and the reverse pass go out as graphs of at most this many, captured once and launched
+// again for every segment of the same length: beside the launches that saves the host, a dependent launch
+// starts sooner in a graph (n = 8: a step of six launches 45 us one by one, 33 us in a graph).
+constexpr int kPiece = 16;
 
 // conjugate transpose of planar R, one 32 x 32 tile per block of 32 x 8 threads (N a multiple of 32)
 __global__ void __launch_bounds__(256)
@@ -380,7 +339,7 @@ size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
 }  // namespace
 
 namespace {
-// with the tensor-core products, one chain
+// with the tensor-core products
 size_t backward_tensor_bytes(int n, int steps, int ckpt_every) {
     return backward_least_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
 }
@@ -389,7 +348,7 @@ size_t backward_tensor_bytes(int n, int steps, int ckpt_every) {
 size_t backward_bytes(int n, int steps, int ckpt_every, int precision) {
     if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
     if (precision == TC_FP64 && !backward_f64_on_tensor_cores(n)) return backward_least_bytes(n, steps, ckpt_every, TC_FP64);
-    return backward_tensor_bytes(n, steps, ckpt_every) + chains_extra(n, steps, ckpt_every);
+    return backward_tensor_bytes(n, steps, ckpt_every);
 }
 
 }  // namespace tc
@@ -448,8 +407,6 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     const bool oz = precision == TC_FP64_OZAKI || (backward_f64_on_tensor_cores(n) &&
                                                    work_bytes >= backward_tensor_bytes(n, steps, ckpt_every));
     OzBufs z{};
-    Chains ch;
-    std::vector<CM> seg2;
     if (oz) {
         TC_TRY(oz_mat_init(z.U, ar, N, true));
         TC_TRY(oz_mat_init(z.Uc, ar, N, true));
@@ -462,52 +419,30 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));
         TC_TRY(oz_mat_load(z.Uc, static_cast<const double*>(U), nullptr, true, true, N, (size_t)N, s));
     }
-    ch.on = oz && chains_extra(n, steps, ckpt_every) > 0 && work_bytes >= backward_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
-    if (ch.on) {
-        TC_TRY(ch.set.take());
-        ch.w = ch.set->more[0];
-        ch.f = ch.set->more[1];
-        for (OzMat* m2 : {&ch.BL[0], &ch.BL[1], &ch.BF}) TC_TRY(oz_mat_init(*m2, ar, N, false));
-        ch.scratch_w = ar.take<uint8_t>(oz_scratch_bytes(N));
-        ch.scratch_f = ar.take<uint8_t>(oz_scratch_bytes(N));
-        ch.L[0] = b.L;
-        ch.L[1] = take_cm(ar, NN);
-        ch.XF = take_cm(ar, NN);
-        if (b.nck > 1)
-            for (int k = 0; k < b.c; k++) seg2.push_back(take_cm(ar, NN));
-        if (!ch.XF.i || (b.nck > 1 && !seg2.back().i)) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
-        for (cudaEvent_t* e : {&ch.lambda[0], &ch.lambda[1], &ch.used[0], &ch.used[1], &ch.seg[0], &ch.seg[1], &ch.freed})
-            TC_TRY(make_event(e));
-    } else {   // one chain: every buffer and stream the same
-        ch.w = ch.f = s;
-        ch.BL[0] = ch.BL[1] = ch.BF = z.B;
-        ch.L[0] = ch.L[1] = b.L;
-        ch.XF = b.X;
-        ch.scratch_w = ch.scratch_f = z.scratch;
-    }
-    // Q <- U P U^dag with the third chain's buffers, Q may be P
+    // Q <- U P U^dag, Q may be P
     auto fwd_step = [&](CM P, CM Q, cudaStream_t cs) -> tc_status {
-        if (oz) return step_oz(N, z.U, ch.BF, false, ch.BF, P, Q, ch.XF, ch.scratch_f, z.group, cs);
+        if (oz) return step_oz(N, z, z.U, false, P, Q, b.X, cs);
         if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, cs));
         return step(N, b.U, Q, b.X, 0, cs);
     };
-    // Runs `body` as a graph, captured at the first use of its key, or (no chains, timing) launch by launch.
-    const bool graphs = ch.on && !timing_enabled();
-    std::map<std::array<int, 4>, StepGraph> graph;
-    auto replay = [&](const std::array<int, 4>& key, cudaStream_t on, const std::function<tc_status(cudaStream_t)>& body) -> tc_status {
-        if (!graphs) return body(on);
-        const auto at = graph.try_emplace(key);
-        if (at.second) TC_TRY(at.first->second.capture(ch.set->s, body));
-        return at.first->second.launch(on);
+    // Runs `body` on s as a graph, captured at the first use of its key (forward or reverse steps lo .. hi - 1 of a
+    // segment), or, while products are timed, launch by launch.
+    StreamLease set;
+    TC_TRY(set.take());
+    const bool graphs = !timing_enabled() && !caller_captures(s);
+    std::map<std::array<int, 3>, StepGraph> graph;
+    auto replay = [&](bool reverse, int lo, int hi, const std::function<tc_status(cudaStream_t)>& body) -> tc_status {
+        if (!graphs) return body(s);
+        const auto at = graph.try_emplace({reverse ? 1 : 0, lo, hi});
+        if (at.second) TC_TRY(at.first->second.capture(set->s, body));
+        return at.first->second.launch(s);
     };
-    const std::vector<CM>* sets[2] = {&seg, ch.on && b.nck > 1 ? &seg2 : &seg};
-    // the `len` states of a segment from the first one, in set[p]
-    auto states = [&](int p, int len, cudaStream_t on) -> tc_status {
-        const std::vector<CM>& v = *sets[p];
+    // the `len` states of a segment, from the first one
+    auto states = [&](int len) -> tc_status {
         for (int lo = 1; lo < len; lo += kPiece) {
             const int hi = std::min(len, lo + kPiece);
-            TC_TRY(replay({0, p, lo, hi}, on, [&](cudaStream_t cs) -> tc_status {
-                for (int i = lo; i < hi; i++) TC_TRY(fwd_step(v[i - 1], v[i], cs));
+            TC_TRY(replay(false, lo, hi, [&](cudaStream_t cs) -> tc_status {
+                for (int i = lo; i < hi; i++) TC_TRY(fwd_step(seg[i - 1], seg[i], cs));
                 return TC_OK;
             }));
         }
@@ -521,7 +456,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     TC_TRY(matrix_trace_and_norm1(N, Hs, true, &trace, &norm1, b.small + 8, s));
 
     // ---------------------------------------------------------------- forward
-    // every segment's states in set 0 (the last segment's stay there), from one checkpoint to the next; rho_K to seg0
+    // every segment's states (the last one's stay), from one checkpoint to the next; rho_K to seg0
     TC_TRY(launch_split_c128(static_cast<const double*>(U), b.U.r, b.U.i, NN, s));
     TC_TRY(launch_split_c128(static_cast<const double*>(rho0), ck[0].r, ck[0].i, NN, s));
     auto length = [&](int j) { return std::min(ckpt_every, steps - j * ckpt_every); };
@@ -533,7 +468,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
             TC_TRY(copy_cm(seg[0], ck[j + 1], NN, s));
             continue;
         }
-        TC_TRY(states(0, len, s));
+        TC_TRY(states(len));
         TC_TRY(fwd_step(seg[len - 1], j + 1 < b.nck ? ck[j + 1] : b.seg0, s));
     }
     // loss from rho_K (in seg0)
@@ -543,65 +478,32 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // ---------------------------------------------------------------- backward
     diag_set_kernel<<<grid_for(NN), 256, 0, s>>>(O_diag, b.L.r, b.L.i, N);   // Lambda_K = O
     TC_LAUNCH_CHECK();
-    bool w_init = false, lambda_loaded = false;
-    int a = 0;   // buffer of the current Lambda
-    if (oz) {   // W accumulates from zero, Lambda_K is loaded
-        TC_CUDA(cudaMemsetAsync(b.W.r, 0, NN * sizeof(double), s));
-        TC_CUDA(cudaMemsetAsync(b.W.i, 0, NN * sizeof(double), s));
-        TC_TRY(oz_mat_load(ch.BL[0], b.L.r, b.L.i, false, false, N, (size_t)N, s));
-        lambda_loaded = w_init = true;
-    }
-    // the reverse steps of rho_k = v[hi - 1] .. v[lo]: Lambda_k = U^dag Lambda_{k+1} U (the step with conj(U)),
-    // W += rho_k Lambda_k
-    auto reverse = [&](const std::vector<CM>& v, int lo, int hi, cudaStream_t cs) -> tc_status {
-        const cudaStream_t w = ch.on ? ch.w : cs;
-        bool used[2] = {false, false};
+    TC_CUDA(cudaMemsetAsync(b.W.r, 0, NN * sizeof(double), s));   // W = 0
+    TC_CUDA(cudaMemsetAsync(b.W.i, 0, NN * sizeof(double), s));
+    // from k = hi - 1 to lo: Lambda_k = U^dag Lambda_{k+1} U (the step with conj(U)), W += rho_k Lambda_k
+    auto reverse = [&](int lo, int hi, cudaStream_t cs) -> tc_status {
         for (int i = hi - 1; i >= lo; i--) {
             if (!oz) {
                 TC_TRY(step(N, b.U, b.L, b.X, 1, cs));
-                TC_TRY(gemm_c(N, v[i], 0, b.L, 0, b.W, 1.0, w_init ? 1.0 : 0.0, 0, cs));
-                w_init = true;
+                TC_TRY(gemm_c(N, seg[i], 0, b.L, 0, b.W, 1.0, 1.0, 0, cs));
                 continue;
             }
-            const int nx = a ^ 1;
-            if (ch.on && used[nx]) TC_CUDA(cudaStreamWaitEvent(cs, ch.used[nx], 0));
-            TC_TRY(step_oz(N, z.Uc, ch.BL[a], lambda_loaded, z.B, ch.L[a], ch.L[nx], b.X, z.scratch, z.group, cs));
-            TC_TRY(oz_mat_load(ch.BL[nx], ch.L[nx].r, ch.L[nx].i, false, false, N, (size_t)N, cs));
-            lambda_loaded = true;
-            if (ch.on) {
-                TC_CUDA(cudaEventRecord(ch.lambda[nx], cs));
-                TC_CUDA(cudaStreamWaitEvent(w, ch.lambda[nx], 0));
-            }
+            // the right operand holds Lambda from the product before, at first a state
+            TC_TRY(step_oz(N, z, z.Uc, i < hi - 1, b.L, b.L, b.X, cs));
             // Lambda Hermitian: rho Lambda = rho Lambda^H
-            TC_TRY(mul_oz(N, z, v[i], ch.BL[nx], true, ch.L[nx], false, b.W, true, ch.scratch_w, w));
-            if (ch.on) TC_CUDA(cudaEventRecord(ch.used[nx], w));
-            used[nx] = true;
-            a = nx;
+            TC_TRY(mul_oz(N, z, seg[i], b.L, false, b.W, true, cs));
         }
-        // the accumulation joins (its products are in sequence, the last one marks the end)
-        return ch.on && used[a] ? (cudaStreamWaitEvent(cs, ch.used[a], 0) == cudaSuccess
-                                       ? TC_OK : fail(TC_ERR_CUDA, "backward: joining the chains")) : TC_OK;
+        return TC_OK;
     };
     for (int j = b.nck - 1; j >= 0; j--) {
-        const int par = (b.nck - 1 - j) & 1, len = length(j);
-        if (!ch.on && j < b.nck - 1) {
+        const int len = length(j);
+        if (j < b.nck - 1) {
             TC_TRY(copy_cm(ck[j], seg[0], NN, s));
-            TC_TRY(states(0, len, s));
-            lambda_loaded = false;   // the one right operand now holds a state
+            TC_TRY(states(len));
         }
-        if (ch.on && j > 0) {   // the next segment beside this one, once the reverse steps of the last are done with its buffers
-            TC_CUDA(cudaEventRecord(ch.freed, s));
-            TC_CUDA(cudaStreamWaitEvent(ch.f, ch.freed, 0));
-            TC_TRY(copy_cm(ck[j - 1], (*sets[par ^ 1])[0], NN, ch.f));
-            TC_TRY(states(par ^ 1, ckpt_every, ch.f));
-            TC_CUDA(cudaEventRecord(ch.seg[par ^ 1], ch.f));
-        }
-        if (ch.on && j < b.nck - 1) TC_CUDA(cudaStreamWaitEvent(s, ch.seg[par], 0));
         for (int hi = len; hi > 0; hi = (hi - 1) / kPiece * kPiece) {
-            const int lo = (hi - 1) / kPiece * kPiece, from = a;
-            TC_TRY(replay({1 + 2 * from + par, lo, hi, 0}, s,
-                          [&](cudaStream_t cs) { return reverse(*sets[par], lo, hi, cs); }));
-            a = from ^ ((hi - lo) & 1);
+            const int lo = (hi - 1) / kPiece * kPiece;
+            TC_TRY(replay(true, lo, hi, [&](cudaStream_t cs) { return reverse(lo, hi, cs); }));
         }
     }
     // M = W U^dag = W conj(U)  -> into L (free now)

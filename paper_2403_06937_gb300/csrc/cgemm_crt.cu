@@ -68,18 +68,10 @@ constexpr int kRB = 128;                     // bytes of K per operand row in a 
 constexpr int kTile = 128 * kRB;             // one 128-row operand tile
 constexpr int kKPer = kRB / 2;               // BF16 K values per stage
 constexpr int kSteps = kRB / 32;             // MMA K steps per stage
-// Column tiles of NT: 256, or half the matrix up to Np = 256 (Ring<64>, Ring<128>).  Shared memory is
-// asked for as if the ring were full in each: one CTA an SM, whatever else runs beside it.  Two pairs on one
-// pair of SMs could each wait in tcgen05.alloc for the other (each CTA allocates for both).
-template <int NT>
-struct Ring {
-    static constexpr int kBRows = NT / 2;                     // of B, a CTA
-    static constexpr int kStage = kTile + kBRows * kRB;       // own 128 rows of A and half of B's
-    static constexpr int kStages = NT == 256 ? 6 : 4;
-    static constexpr int kBytes = kStages * kStage;
-    static constexpr int kSmem = 192 * 1024 + 1024 /*align*/ + 512 /*barriers*/;
-    static_assert(kBytes <= 192 * 1024, "ring");
-};
+constexpr int kRing = 192 * 1024;
+constexpr int kStage = 2 * kTile;            // own 128 rows of A and of B
+constexpr int kStages = kRing / kStage;      // 6
+constexpr int kSmem = kRing + 1024 /*align*/ + 512 /*barriers*/;
 constexpr int kChunkStages = crt::kChunk / kKPer;
 constexpr int kGroup = 8;                    // 256-row tiles per raster group (a wave: ~8 x 9 tiles)
 constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN
@@ -97,14 +89,8 @@ struct CrtLaunch {
 };
 
 // unit -> (plane, row tile, column tile), in tiles of 256
-template <int MODE, int NT>
+template <int MODE>
 __device__ __forceinline__ void unit_at(const CrtLaunch& L, int u, int& z, int& P, int& J) {
-    if (NT < 256) {   // one row of two tiles a plane
-        z = u >> 1;
-        P = 0;
-        J = u & 1;
-        return;
-    }
     z = u / L.units_per;
     const int t = u - z * L.units_per, side = (L.tiles + 1) / 2;
     if (MODE == 1) {
@@ -223,8 +209,9 @@ __device__ __forceinline__ void chunk_read(uint64_t* tmem_empty, uint32_t lead_t
     }
 }
 
-// A chunk that is all of K, straight to bytes: COLS columns of a thread's row, to y if `own`.  `done` as above.
-template <int COLS, typename Done>
+// A chunk that is all of K (N <= 1024), straight to bytes: 128 columns of a thread's row, to y if `own`; n = 9:
+// 15.8 -> 13.2 us a launch.  `done` as above.
+template <typename Done>
 __device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, uint4* y, bool own, Done done) {
     const uint64_t p2n = pack2(-p, -p), inv2 = pack2(inv_p, inv_p);
     const uint64_t m2 = pack2(kMagic, kMagic), m2n = pack2(-kMagic, -kMagic);
@@ -243,10 +230,10 @@ __device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, u
     tmem_ld8(tl, a[0]);
     tmem_ld8(tl + 8, b[0]);
 #pragma unroll
-    for (int c = 0; c < COLS; c += 16) {
+    for (int c = 0; c < 128; c += 16) {
         const int k = (c >> 4) & 1;
         tmem_wait8(a[k], b[k]);
-        if (c + 16 < COLS) {
+        if (c + 16 < 128) {
             tmem_ld8(tl + c + 16, a[k ^ 1]);
             tmem_ld8(tl + c + 24, b[k ^ 1]);
         } else {
@@ -257,14 +244,13 @@ __device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, u
     }
 }
 
-template <int MODE, int NT>
+template <int MODE>
 __global__ void __launch_bounds__(kThreads, 1)
     cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
-    constexpr uint32_t kIdesc = make_idesc(1u, 256u, (uint32_t)NT);
-    constexpr int kStages = Ring<NT>::kStages, kStage = Ring<NT>::kStage;
+    constexpr uint32_t kIdesc = make_idesc(1u, 256u, 256u);
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t* full = reinterpret_cast<uint64_t*>(smem + Ring<NT>::kBytes);
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + kRing);
     uint64_t* empty = full + kStages;
     uint64_t* accum = empty + kStages;   // [2] MMA -> epilogue, one per buffer
     uint64_t* tmem_empty = accum + 2;        // [2] both epilogues -> MMA (even CTA, count 2)
@@ -291,7 +277,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         fence_mbar_init();
     }
     if (warp == 0) {
-        tmem_alloc_pair(saddr(tmem_slot), 2 * NT);
+        tmem_alloc_pair(saddr(tmem_slot), 512);
         tmem_relinquish_pair();
     }
     if (warp == 8 && lane == 0) {
@@ -313,8 +299,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             bool ok = true;
             for (int u = worker; u < L.units && ok; u += workers) {
                 int z, P, J;
-                unit_at<MODE, NT>(L, u, z, P, J);
-                const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * Ring<NT>::kBRows;
+                unit_at<MODE>(L, u, z, P, J);
+                const int ra = (2 * P + (int)rank) * 128, rb = (2 * J + (int)rank) * 128;
                 for (int kb = 0; kb < L.kb_total; kb++, it++) {
                     const int b = it % kStages;
                     const uint32_t ph = (it / kStages) & 1u;
@@ -382,7 +368,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                         const uint64_t bd = desc_kmajor<kRB>(saddr(st + kTile));
 #pragma unroll
                         for (int ks = 0; ks < kSteps; ks++)   // 32 bytes of K further in each row
-                            umma_pair(tmem + (uint32_t)NT * buf, ad + 2u * (uint64_t)ks, bd + 2u * (uint64_t)ks, kIdesc,
+                            umma_pair(tmem + 256u * buf, ad + 2u * (uint64_t)ks, bd + 2u * (uint64_t)ks, kIdesc,
                                       (kb > kb0 || ks > 0) ? 1u : 0u);
                         umma_commit_pair(saddr(&empty[b]));
                         umma_commit_pair(peer_empty + 8u * (uint32_t)b);
@@ -402,24 +388,24 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t lead_tmem_empty = cluster_addr(saddr(&tmem_empty[0]), 0u);
         const int half = warp >> 2;
         const int row = (warp & 3) * 32 + lane;
-        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(NT / 2) * (uint32_t)half;
+        const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16) + 128u * (uint32_t)half;
         uint32_t pass = 0;
         bool stop = false;
         for (int u = worker; u < L.units && !stop; u += workers) {
             int z, P, J;
-            unit_at<MODE, NT>(L, u, z, P, J);
+            unit_at<MODE>(L, u, z, P, J);
             const float p = (float)kC.p[z % kModuli], inv_p = 1.0f / p;
             // rows and columns past the end (an odd number of 128-tiles) are not written
-            const bool own = 2 * P + (int)rank < L.tiles && (NT < 256 || 2 * J + half < L.tiles);
+            const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
             uint8_t* y = L.bytes + ((size_t)z * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
-                         (size_t)(J * NT + NT / 2 * half);
-            if (NT < 256 || chunks == 1) {
+                         (size_t)(256 * J + 128 * half);
+            if (chunks == 1) {
                 const uint32_t buf = pass & 1u;
                 if (!chunk_ready(&accum[buf], (pass >> 1) & 1u, abort, lim, peer_abort)) {
                     stop = true;
                     break;
                 }
-                chunk_bytes<NT / 2>(tl + (uint32_t)NT * buf, p, inv_p, reinterpret_cast<uint4*>(y), own,
+                chunk_bytes(tl + 256u * buf, p, inv_p, reinterpret_cast<uint4*>(y), own,
                                     [&]() { chunk_read(&tmem_empty[buf], lead_tmem_empty + 8u * buf, rank, lane); });
                 pass++;
                 continue;
@@ -466,7 +452,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     cluster_sync();   // neither CTA frees TMEM or leaves while the other may still use it
     if (warp == 0) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem, 2 * NT);
+        tmem_dealloc_pair(tmem, 512);
     }
 }
 
@@ -888,10 +874,9 @@ int sm_count() {
     return sms;
 }
 
-template <int MODE, int NT>
+template <int MODE>
 tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
-    constexpr int kSmem = Ring<NT>::kSmem;
-    auto k = cgemm_crt_kernel<MODE, NT>;
+    auto k = cgemm_crt_kernel<MODE>;
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -923,16 +908,6 @@ int band_rows(int Np) { return Np <= 16384 ? Np : 4096; }
 
 size_t plane_bytes(int Np, int planes) { return round256((size_t)planes * Np * Np * 2); }
 
-// Half the columns a unit up to Np = 256, where one 256-column tile a plane leaves 88 of 152 SMs idle and
-// the epilogue's 128 columns a warp are a third of the launch (n = 8: 9.8 us).
-bool narrow_tiles(int Np) { return Np <= 256; }
-
-tc_status maps(CrtMat& m) {
-    TC_TRY(make_part_map_rows(&m.map, m.planes, m.Np, m.count, TC_BF16X3, kRB));
-    return !m.left && narrow_tiles(m.Np)
-               ? make_part_map_rows(&m.narrow, m.planes, m.Np, m.count, TC_BF16X3, kRB, m.Np / 4) : TC_OK;
-}
-
 tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
     m.Np = Np;
     m.left = left;
@@ -941,7 +916,7 @@ tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
     m.ex = ar.take<int>((size_t)Np);
     m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
     if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
-    return maps(m);
+    return make_part_map_rows(&m.map, m.planes, Np, planes, TC_BF16X3, kRB);
 }
 
 // The residue products of one band of rows (all of them: lo = 0, hi = side).
@@ -958,11 +933,7 @@ tc_status gemm(int mode, const CrtMat& A, const CrtMat& B, int lo, int hi, void*
     L.status = device_status_word();
     L.units_per = mode == 0 ? side * (hi - lo) : hi * (hi + 1) / 2 - lo * (lo + 1) / 2;
     L.units = L.units_per * A.count;
-    if (narrow_tiles(A.Np)) {   // the whole matrix in either mode
-        L.units = 2 * A.count;
-        return A.Np == 128 ? launch<0, 64>(A.map, B.narrow, L, s) : launch<0, 128>(A.map, B.narrow, L, s);
-    }
-    return mode == 0 ? launch<0, 256>(A.map, B.map, L, s) : launch<1, 256>(A.map, B.map, L, s);
+    return mode == 0 ? launch<0>(A.map, B.map, L, s) : launch<1>(A.map, B.map, L, s);
 }
 
 }  // namespace
@@ -980,7 +951,7 @@ tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
     if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
     view = base;
     view.Np = Np;
-    return maps(view);
+    return make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
 }
 
 tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,

@@ -17,7 +17,6 @@ struct CrtMat {
     int* ex;          // row r holds round(x 2^ex[r])
     double* diag;     // left operands: [2][Np], the diagonal kept in FP64 (planes hold zero there)
     CUtensorMap map;
-    CUtensorMap narrow;   // Np <= 256: the same in boxes of Np / 4 rows
     int Np;
     int count;        // planes
     bool left;

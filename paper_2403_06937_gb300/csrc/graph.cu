@@ -22,7 +22,7 @@ tc_status current_device(int* dev) {
 
 tc_status StreamSet::create(int device) {
     dev = device;
-    for (cudaStream_t* p : {&s, &side, &more[0], &more[1]}) TC_CUDA(cudaStreamCreateWithFlags(p, cudaStreamNonBlocking));
+    for (cudaStream_t* p : {&s, &side}) TC_CUDA(cudaStreamCreateWithFlags(p, cudaStreamNonBlocking));
     for (cudaEvent_t* e : {&before, &after, &fork, &join}) TC_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
     return TC_OK;
 }
@@ -42,7 +42,7 @@ StreamSet::~StreamSet() {
         if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : lane_join)
         if (e) cudaEventDestroy(e);
-    for (cudaStream_t x : {s, side, more[0], more[1]})
+    for (cudaStream_t x : {s, side})
         if (x) cudaStreamDestroy(x);
     for (cudaStream_t x : lane)
         if (x) cudaStreamDestroy(x);

@@ -18,7 +18,6 @@ struct StreamSet {
     int dev = 0;
     cudaStream_t s = nullptr;                        // the captured stream
     cudaStream_t side = nullptr;                     // SideBranch's
-    cudaStream_t more[2] = {};                       // chains beside the call's own stream
     cudaStream_t lane[kLanes] = {};                  // systems of a batch (created with the first batch)
     cudaEvent_t before = nullptr, after = nullptr, fork = nullptr, join = nullptr;
     cudaEvent_t lane_fork = nullptr, lane_join[kLanes] = {};

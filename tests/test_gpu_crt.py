@@ -128,11 +128,9 @@ def test_gradient_on_the_tensor_cores_with_squarings(tc, oracle):
     grad, loss = tc.evolve_backward(p, dt, steps, rho0, U, O, ckpt_every=2)
     grad2, loss2 = tc.evolve_backward(p, dt, steps, rho0, U, O, ckpt_every=2, precision="ozaki")
     assert torch.equal(grad, grad2) and loss == loss2   # one route for both from n = 7 on
-    # one chain instead of three (64 KiB less), and the DMMA form (its planes: 11 + 2 checkpoints + 2 states of
-    # two N x N matrices, one real one, the small buffers)
+    # the DMMA form (its planes: 11 + 2 checkpoints + 2 states of two N x N matrices, one real one, the small buffers)
     cm = 2 * 8 * N * N
-    for size, tol in ((tc.workspace_size(n, tc.TC_FP64, tc.TC_OP_BACKWARD, steps, 2) - 65536, 0.0),
-                      (15 * cm + cm // 2 + 16384, 1e-11)):
+    for size, tol in ((15 * cm + cm // 2 + 16384, 1e-11),):
         work = torch.empty(size, dtype=torch.uint8, device="cuda")
         ref = (ctypes.c_double * (n + 2))()
         c = p.c()
