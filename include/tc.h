@@ -9,7 +9,7 @@
  *          or from the model with H applied as a stencil (no dense H);
  *   rho <- U rho U^dag step after step (Eqs. 6 and 12), on FP64 DMMA, on
  *          tcgen05 tensor cores in split-BF16 / TF32 arithmetic, or at FP64
- *          accuracy from exact integer digit slices on the BF16 tensor cores;
+ *          accuracy from exact integer residues on the BF16 tensor cores;
  *   observables read from rho by reduction (populations, the photon-number
  *          probabilities of Eq. 13, trace, purity, energy);
  *   the gradient of a diagonal observable at the final time with respect to
@@ -338,10 +338,12 @@ TC_API tc_status tc_lindblad_propagators(const tc_params* params, double dt, voi
  * with D_tau the exact damping over tau (the bosonic pure-loss channel,
  * mixing block k+m into block k) and U from tc_lindblad_propagators with the
  * same dt.  Second order in dt; kappa = 0 is the closed evolution of Eq. 6.
- * The block products run on the DMMA GEMM (TC_FP64) or on the tcgen05
- * tensor cores (split forms, as tc_evolve: one persistent launch over the
- * tiles of every block per product, CTA pairs by default, rho stored FP32
- * between steps; FP64 emulated: the blocks one after another on CTA pairs).
+ * The block products run on the tcgen05 tensor cores: in the split forms as
+ * tc_evolve, one persistent launch over the tiles of every block per product
+ * (CTA pairs by default, rho stored FP32 between steps); in the FP64 forms
+ * (TC_FP64 for 7 <= n <= 13, given the workspace that tc_workspace_size
+ * states) block after block as FP64-accurate products, blocks of at most 64
+ * rows on the FP64 DMMA.  TC_FP64 otherwise: the DMMA GEMM.
  *  U, rho      : device packed complex128; rho in/out (Hermitian blocks).
  *  precision   : TC_FP64, TC_BF16X3, TC_TF32, TC_TF32X3, TC_FP64_OZAKI.
  *  renorm_every: 0 = never; else after every renorm_every-th step all
@@ -413,7 +415,8 @@ TC_API tc_status tc_evolve_host(const void* U, void* rho_host, int n, int steps,
  * atoms at `precision` on synthetic operands in `work` and keep the fastest
  * for later calls in this process (tc_evolve, tc_evolve_host, tc_expm,
  * tc_evolve_backward, tc_batch_evolve, tc_lindblad_evolve):
- *   FP64: the DMMA GEMM tile, 32 x 32 or 64 x 64 (timed on a K slice);
+ *   FP64: the DMMA GEMM tile, 32 x 32 or 64 x 64 (timed on a K slice; used
+ *   where TC_FP64 and tc_expm run on the DMMA);
  *   tensor cores: the tile shape (1: one CTA per 128 x 128 complex tile;
  *   2: CTA pairs on the 2-SM MMA, a 256 x 128 tile per pair, 32 bytes of K
  *   per operand row a stage; 3: CTA pairs with 64-byte rows, 128 for TF32),

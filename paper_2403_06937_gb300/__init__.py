@@ -259,8 +259,8 @@ class EvolveFn(torch.autograd.Function):
     (tc_evolve) and L (tc_expectation_diag); nothing of the reverse pass runs.
     backward (only when a gradient is asked for): tc_evolve_backward, the
     reverse mode with checkpoints every `ckpt_every` steps.
-    precision: "fp64" (DMMA products) or "ozaki" (the products emulated at FP64
-    accuracy on the BF16 tensor cores; n >= 7), for both passes.
+    precision: "fp64" or "ozaki" (n >= 7), for both passes; from n = 7 on both are
+    FP64-accurate products on the BF16 tensor cores.
     Inputs g (n,), omega_a (), omega_c () are float64 tensors; rho0 and O_diag
     are CUDA tensors.  Returns a 0-d float64 tensor on rho0's device.
     """

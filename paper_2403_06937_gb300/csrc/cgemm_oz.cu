@@ -1,10 +1,13 @@
 // cgemm_oz.cu -- FP64-accurate complex GEMM Y = U P^H on the BF16 tensor
-// cores by exact integer slices (the Ozaki splitting), for the step
-// rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12) at FP64 accuracy.
+// cores, for the step rho <- U rho U^dag (Sec. III.A, Eqs. 6, 12) at FP64
+// accuracy: the operands and products of the residue form (OzMat, oz_product,
+// which pass on to cgemm_crt.cu), and the digit form below (exact integer
+// slices, the Ozaki splitting), taken with TC_OZ_BITS=6 only: an independent
+// check, half the accuracy in bits and about four times the products.
 //
 // Slicing.  Every row r of an operand (both planes together) gets an
 // exponent e_r with max |x| < 2^(e_r - 1); with S digits of b bits
-// (oz_digits: b = 6, 7 or 8 as K allows, bS = 54 or 56), x 2^(bS - e_r) is
+// (kOzDigits: nine of 6), x 2^(bS - e_r) is
 // rounded to an integer below 2^(bS - 1) and written in balanced base-2^b
 // digits,
 //     x = 2^e_r sum_{t=0..S-1} d_t 2^(-b(t+1)),   d_t integers, |d_t| <= 2^(b-1),
@@ -18,8 +21,7 @@
 // the row and column scales) accumulates that pair in TMEM; the epilogue
 // accumulates the exact integer results in int64 with the level weights as
 // shifts and the last pass writes Y = sum 2^(e_i + f_j - b(t + u + 2))
-// (integer) in FP64.  With 6-bit digits, K above 16384 is cut into chunks of
-// 16384, one pass each.
+// (integer) in FP64.  K above 16384 is cut into chunks of 16384, one pass each.
 //
 // Tile and roles as the split-BF16 kernel (cgemm_tc.cu): one CTA per 128 x 128
 // complex tile, A = slice t of U_r and U_i (M = 128), B = slice u of

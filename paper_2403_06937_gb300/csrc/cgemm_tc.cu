@@ -32,8 +32,9 @@
 // 32-byte slice of K sit in one pipeline stage, and all part products of the
 // stage are issued from it, so each operand byte crosses L2 -> SMEM once.
 //
-// Roles (192 threads): warp 4 lane 0 issues TMA loads into a ring of STAGES
-// stages; warp 5 lane 0 issues tcgen05.mma and commits each stage back to the
+// Roles of the single-CTA kernel (192 threads; the pair kernels have eight
+// epilogue warps, 320 threads): warp 4 lane 0 issues TMA loads into a ring of
+// STAGES stages; warp 5 lane 0 issues tcgen05.mma and commits each stage back to the
 // producer; warps 0-3 (one TMEM lane quarter each) run the epilogue.  Every
 // wait is bounded: on timeout the CTA records kStatusTimeout, stops issuing,
 // waits (bounded) for its own copies and MMAs, frees TMEM and returns.

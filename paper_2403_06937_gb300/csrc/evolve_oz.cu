@@ -161,12 +161,12 @@ tc_status OzSystem::tail(double* rho, cudaStream_t cs) {
 
 // TC_FP64 takes the products of this file from n = 7 on: below, the padding to
 // 128 costs more than the DMMA product (n = 6: 64^3).  At n = 15 its operands
-// take 206 GB of workspace, which would not leave room for what a caller could
+// take 176 GB of workspace, which would not leave room for what a caller could
 // hold beside the DMMA form's 52 GB (n = 14: 52 GB, DMMA 26 GB).  Its error against 64
 // bits is no larger than the DMMA sums' (rows held to at least 51 bits of
 // their largest entry in a common scale, sums exact; the DMMA form rounds
-// each of N additions); a step takes 53 us at n = 8 (DMMA 251), 0.22 ms at n = 10
-// (13.1), 5.7 ms at n = 12 (768).  TC_OZ_BITS=6 (the less accurate digit form) keeps
+// each of N additions); a step takes 33 us at n = 8 (DMMA 251), 0.18 ms at n = 10
+// (13.1), 5.2 ms at n = 12 (768).  TC_OZ_BITS=6 (the less accurate digit form) keeps
 // TC_FP64 on the DMMA.
 bool f64_on_tensor_cores(int n) { return n >= 7 && n <= 14 && oz_modular(); }
 
