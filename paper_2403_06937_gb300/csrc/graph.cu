@@ -1,5 +1,6 @@
 // graph.cu -- see graph.cuh.
 #include <algorithm>
+#include <array>
 #include <memory>
 #include <mutex>
 #include <vector>
@@ -10,7 +11,8 @@ namespace tc {
 namespace {
 constexpr size_t kIdleSets = 4;   // a device
 std::mutex g_mu;
-std::vector<std::unique_ptr<StreamSet>> g_idle[64];
+// never destroyed: the runtime may be gone when static objects are
+auto& g_idle = *new std::array<std::vector<std::unique_ptr<StreamSet>>, 64>;
 thread_local StreamSet* t_leased = nullptr;
 
 tc_status current_device(int* dev) {
