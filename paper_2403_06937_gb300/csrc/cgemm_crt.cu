@@ -72,6 +72,7 @@ constexpr int kRing = 192 * 1024;
 constexpr int kStage = 2 * kTile;            // own 128 rows of A and of B
 constexpr int kStages = kRing / kStage;      // 6
 constexpr int kSmem = kRing + 1024 /*align*/ + 512 /*barriers*/;
+static_assert(alone_on_sm(kSmem), "a pair that waits for TMEM must be the only one on its SM");
 constexpr int kChunkStages = crt::kChunk / kKPer;
 constexpr int kGroup = 8;                    // 256-row tiles per raster group (a wave: ~8 x 9 tiles)
 constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN

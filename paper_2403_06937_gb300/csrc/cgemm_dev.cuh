@@ -37,7 +37,10 @@ constexpr int split_pair_stages() {
 }
 template <int S, int RB, int NC = 128>
 constexpr int split_pair_smem() {
-    return split_pair_stages<S, RB, NC>() * split_pair_stage_bytes<S, RB, NC>() + 1024 /*align*/ + 512 /*barriers*/;
+    constexpr int bytes =
+        split_pair_stages<S, RB, NC>() * split_pair_stage_bytes<S, RB, NC>() + 1024 /*align*/ + 512 /*barriers*/;
+    static_assert(sm100::alone_on_sm(bytes), "a pair that waits for TMEM must be the only one on its SM");
+    return bytes;
 }
 
 template <int S>

@@ -573,6 +573,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 constexpr int kPairSmem = kPairRing + 1024 /*align*/ + 512 /*barriers*/;
+static_assert(alone_on_sm(kPairSmem), "a pair that waits for TMEM must be the only one on its SM");
 
 // One warp per row r < Np: the row exponent over both planes, then the S
 // balanced base-2^b digits of every entry (zero beyond the valid N x N block).

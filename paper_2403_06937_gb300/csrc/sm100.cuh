@@ -188,6 +188,17 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 }
 // The same for a CTA pair (cta_group::2): one warp of each of the two CTAs
 // executes these together; each CTA gets `ncols` columns at the same address.
+//
+// An allocation waits, with no limit of its own, until the columns are free.
+// Two pairs on the same two SMs could each hold one SM's columns and wait for
+// the other's, so a kernel that allocates for a pair must leave no room on its
+// SM for another CTA that does: its shared memory is more than half of the
+// SM's (alone_on_sm, asserted beside every such kernel's size).  Streams may
+// then run pair kernels of several calls side by side: on any SM a pair waits
+// only for CTAs that end by themselves (single CTAs, or a pair that has its
+// columns already).
+constexpr int kSmemOfSm = 228 * 1024, kSmemOfCta = 1024;   // shared memory of an SM; kept by the system in each CTA
+constexpr bool alone_on_sm(int dynamic_smem) { return 2 * (dynamic_smem + kSmemOfCta) > kSmemOfSm; }
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t slot_smem, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot_smem), "r"(ncols)
                  : "memory");
