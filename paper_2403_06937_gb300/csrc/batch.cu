@@ -114,7 +114,7 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
                 const double* Ub = static_cast<const double*>(U[b]);
                 double* rb = static_cast<double*>(rho[b]);
                 if (precision == TC_FP64_OZAKI || (!dmma && f64_on_tensor_cores(n[b])))
-                    st = evolve_oz(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->lane[l]);
+                    st = evolve_oz(Ub, rb, n[b], steps, precision, renorm_every, mp, ob, ar, ls->lane[l]);
                 else
                     st = evolve_f64(Ub, rb, n[b], steps, renorm_every, mp, ob, ar, ls->lane[l]);
             }

@@ -475,11 +475,11 @@ TC_API tc_status tc_evolve(const void* U, void* rho, int n, int steps, int preci
     cudaStream_t s = as_stream(stream);
     Arena ar{static_cast<char*>(work), work_bytes, 0};
     if (precision == TC_FP64_OZAKI)
-        return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, renorm_every, mp, obs,
-                         ar, s);
+        return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision, renorm_every, mp,
+                         obs, ar, s);
     if (precision == TC_FP64 && f64_on_tensor_cores(n) && ar.size >= evolve_oz_bytes(n))
-        return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, renorm_every, mp, obs,
-                         ar, s);
+        return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision, renorm_every, mp,
+                         obs, ar, s);
     if (precision != TC_FP64)
         return evolve_lowp(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision,
                            renorm_every, mp, obs, ar, s);
@@ -527,7 +527,7 @@ TC_API tc_status tc_evolve_host(const void* U, void* rho_host, int n, int steps,
         else
             TC_CUDA(cudaMemcpyAsync(rho_dev, rho_host, 16 * N * N, cudaMemcpyHostToDevice, s));
         if (precision == TC_FP64_OZAKI || (f64_on_tensor_cores(n) && ar.size - ar.used >= evolve_oz_bytes(n)))
-            TC_TRY(evolve_oz(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));
+            TC_TRY(evolve_oz(Ud, rho_dev, n, steps, precision, renorm_every, mp, od, ar, s));
         else
             TC_TRY(evolve_f64(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));
         if (mapped)

@@ -16,6 +16,18 @@
 // close to the identity, and Y = diag(U) B^H + V B^H with the first term in
 // FP64 leaves the integers the small part V only.
 //
+// Column scales (TC_FP64).  One scale a row keeps nothing of an entry below
+// 2^-59 of its row's norm, and both U (an entry falls by a factor g dt for each
+// atom that differs) and a state after a few steps have such entries, on which
+// small populations rest.  There K gets a power of two of its own as well: the
+// products are those of A D and B D^-1, D_kk = 2^floor(log2(rho_kk) / 2)
+// (crt_columns_kernel).  For a positive rho, |rho_jk| <= sqrt(rho_jj rho_kk) and
+// |X_jk| <= sqrt(rho'_jj rho_kk): no entry of a row of B D^-1 is far above what
+// its row's population allows, and with a_i^2 = sum_k |U_ik|^2 rho_kk the error
+// of X_ij stays below K 2^-55 a_i sqrt(rho_jj), that of rho'_ij below
+// K 2^-55 a_i sqrt(rho'_jj).  At i = j those are the sums of magnitudes (of a
+// pure state, or less) that the DMMA form rounds K times at 2^-53.
+//
 // Products.  Modulo p_s a complex number is the pair a_r + iota a_i,
 // a_r - iota a_i (iota^2 = -1), and the pairs multiply componentwise, so each
 // modulus takes two real BF16 products: plane 0 of A with plane 0 of B, plane
@@ -466,8 +478,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 // entry; the second read of the row comes from L2); no FP64 instruction, since
 // one FP64 conversion per entry alone would take as long as a third of the
 // writes on this GPU.
+constexpr int kShiftBias = 4096;     // added to shifted exponents, so that 0 still means an empty row
+constexpr int kNotFinite = 1 << 16;
+constexpr int kEmptyColumn = INT32_MIN;   // column scale of a zero column
 struct RowStat {
-    int e;       // largest biased exponent (0: all zero, 0x7FF: not finite)
+    int e;       // largest biased exponent (0: all zero, kNotFinite: an infinity or a NaN)
     float ss;    // sum of squares over 2^(2 (e - 1022))
 };
 __device__ __forceinline__ RowStat stat_join(RowStat a, RowStat b) {
@@ -477,10 +492,11 @@ __device__ __forceinline__ RowStat stat_join(RowStat a, RowStat b) {
     r.ss = a.ss * __uint_as_float((uint32_t)(127 + 2 * da) << 23) + b.ss * __uint_as_float((uint32_t)(127 + 2 * db) << 23);
     return r;
 }
-__device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits) {
+__device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits, int shift) {   // of x 2^shift
     const uint32_t hi = (uint32_t)(bits >> 32) & 0x7FFFFFFFu;
     if ((bits << 1) == 0) return;
-    const int e = max((int)(hi >> 20), 1);   // a subnormal counts as the normal number of the same significand bits
+    // a subnormal counts as the normal number of the same significand bits
+    const int e = (hi >> 20) == 0x7FFu ? kNotFinite : max((int)(hi >> 20), 1) + shift;
     if (e > a.e) {   // rescale to the new exponent
         const int d = max(a.e - e, -63);
         a.ss *= __uint_as_float((uint32_t)(127 + 2 * d) << 23);
@@ -526,11 +542,12 @@ __device__ __forceinline__ uint32_t bf16_pair(uint64_t v) {
     return __byte_perm(a, b, 0x7632);
 }
 
-template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false>
+// SCALED: column k carries 2^col[k] (a left operand; a right one 2^-col[k]).
+template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false, bool SCALED = false>
 __global__ void __launch_bounds__(128)
     crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
-                       int tpr, uint64_t im_flip, __nv_bfloat16* __restrict__ planes, int* __restrict__ ex,
-                       double* __restrict__ diag) {
+                       int tpr, uint64_t im_flip, const int* __restrict__ col, __nv_bfloat16* __restrict__ planes,
+                       int* __restrict__ ex, double* __restrict__ diag) {
     const int sub = threadIdx.x % tpr;                       // thread within the row
     const int r = blockIdx.x * (128 / tpr) + threadIdx.x / tpr;
     // CPT consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
@@ -577,6 +594,21 @@ __global__ void __launch_bounds__(128)
                 }
         }
     };
+    // exponents of the columns' powers of two; what meets an empty column is left out (an infinity or a NaN stays)
+    auto shifts = [&](int c0, uint64_t (&xr)[CPT], uint64_t (&xi)[CPT], int (&sc)[CPT]) {
+#pragma unroll
+        for (int q = 0; q < CPT; q++) {
+            sc[q] = 0;
+            if (!SCALED) continue;
+            const int v = col[c0 + q];
+            if (v != kEmptyColumn) {
+                sc[q] = LEFT ? v : -v;
+            } else {
+                if ((xr[q] << 1) < 0xFFE0000000000000ull) xr[q] = 0;
+                if ((xi[q] << 1) < 0xFFE0000000000000ull) xi[q] = 0;
+            }
+        }
+    };
     auto put = [](__nv_bfloat16* d, const uint32_t (&w)[CPT / 2]) {
         if constexpr (CPT == 4)
             *reinterpret_cast<uint2*>(d) = make_uint2(w[0], w[1]);
@@ -586,11 +618,13 @@ __global__ void __launch_bounds__(128)
     RowStat st{0, 0.0f};
     for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
         uint64_t xr[CPT], xi[CPT];
+        int sc[CPT];
         load(c0, xr, xi);
+        shifts(c0, xr, xi, sc);
 #pragma unroll
         for (int q = 0; q < CPT; q++) {
-            stat_add(st, xr[q]);
-            if (!REAL) stat_add(st, xi[q]);
+            stat_add(st, xr[q], (SCALED ? kShiftBias : 0) + sc[q]);
+            if (!REAL) stat_add(st, xi[q], (SCALED ? kShiftBias : 0) + sc[q]);
         }
     }
     for (int o = min(tpr, 32) / 2; o > 0; o >>= 1) {
@@ -609,8 +643,10 @@ __global__ void __launch_bounds__(128)
         for (int k = 1; k < tpr / 32; k++) st = stat_join(st, part[w0 + k]);
     }
     // ex = the largest shift with 2-norm * 2^ex <= 2^58.32 (any for a row of zeros)
-    const bool finite = st.e < 0x7FF;
-    const int sh = st.e == 0 ? 0 : (int)floorf(crt::kNormBits - 0.5f * log2f(st.ss * 1.0001f)) - (st.e - 1022);
+    const bool finite = st.e < kNotFinite;
+    const int sh = st.e == 0 ? 0
+                             : (int)floorf(crt::kNormBits - 0.5f * log2f(st.ss * 1.0001f)) -
+                                   (st.e - (SCALED ? kShiftBias : 0) - 1022);
     if (r < Np && sub == 0) {
         ex[r] = finite ? sh : kNoScale;
         if (LEFT) {
@@ -627,15 +663,17 @@ __global__ void __launch_bounds__(128)
     const size_t plane = (size_t)Np * Np;
     for (int c0 = CPT * sub; c0 < Np; c0 += CPT * tpr) {
         uint64_t xr[CPT], xi[CPT];
+        int sc[CPT];
         load(c0, xr, xi);
+        shifts(c0, xr, xi, sc);
         Pieces2 pr[CPT / 2], pi[CPT / 2];
-        auto pieces = [&](uint64_t b) {
-            return crt::split_pieces(finite ? crt::to_magnitude(b, sh) : 0, (b >> 63) != 0);
+        auto pieces = [&](uint64_t b, int q) {
+            return crt::split_pieces(finite ? crt::to_magnitude(b, sh + sc[q]) : 0, (b >> 63) != 0);
         };
 #pragma unroll
         for (int h = 0; h < CPT / 2; h++) {
-            pr[h] = pieces2(pieces(xr[2 * h]), pieces(xr[2 * h + 1]));
-            if (!REAL) pi[h] = pieces2(pieces(xi[2 * h] ^ im_flip), pieces(xi[2 * h + 1] ^ im_flip));
+            pr[h] = pieces2(pieces(xr[2 * h], 2 * h), pieces(xr[2 * h + 1], 2 * h + 1));
+            if (!REAL) pi[h] = pieces2(pieces(xi[2 * h] ^ im_flip, 2 * h), pieces(xi[2 * h + 1] ^ im_flip, 2 * h + 1));
         }
         __nv_bfloat16* dst = planes + (size_t)r * Np + c0;
 #pragma unroll
@@ -656,6 +694,77 @@ __global__ void __launch_bounds__(128)
             if (!REAL) put(dst + (size_t)(LEFT ? kModuli + s : s) * plane, w1);
         }
     }
+}
+
+// Column scales of a state: col[k] = floor(log2(m_k) / 2) with m_k = |rho_kk|
+// up to a factor of 2, or, where an off-diagonal entry is larger than a
+// positive rho allows, the square of the largest entry of row and column k over
+// the matrix's largest (so that a matrix which is no state keeps its accuracy
+// relative to its norm: an entry of B D^-1 stays below 2 sqrt(max |rho|), one of
+// A D below |A_ik| 2 sqrt(max |rho|)).  One pass over rho, exponents only; a
+// block takes 32 rows x 128 columns, and the last one to finish turns the
+// maxima into scales and clears them.  n = 12: 16 N^2 bytes at HBM rate beside
+// a step of 5 ms.
+__device__ __forceinline__ unsigned exponent_of(uint64_t bits) {   // 0: zero or not finite
+    const unsigned e = (unsigned)(bits >> 52) & 0x7FFu;
+    return e == 0x7FFu || (bits << 1) == 0 ? 0u : max(e, 1u);
+}
+template <bool INTERLEAVED>
+__global__ void __launch_bounds__(256)
+    crt_columns_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
+                       unsigned* __restrict__ top, int* __restrict__ col) {
+    __shared__ unsigned cmax[128], warp_max[8];
+    __shared__ bool last;
+    unsigned* ticket = top + Np;
+    auto bits = [&](int r, int c, int part) -> uint64_t {
+        const size_t o = (size_t)r * ld + c;
+        if (INTERLEAVED) return (uint64_t)__double_as_longlong(re[2 * o + part]);
+        return (uint64_t)__double_as_longlong(part ? im[o] : re[o]);
+    };
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int i0 = 32 * (int)blockIdx.y + warp, j0 = 128 * (int)blockIdx.x + lane;
+    if (threadIdx.x < 128) cmax[threadIdx.x] = 0;
+    __syncthreads();
+    unsigned c[4] = {};
+#pragma unroll
+    for (int r = 0; r < 32; r += 8) {
+        unsigned row = 0;
+        if (i0 + r < N) {
+#pragma unroll
+            for (int q = 0; q < 4; q++) {
+                if (j0 + 32 * q >= N) continue;
+                const unsigned e = max(exponent_of(bits(i0 + r, j0 + 32 * q, 0)), exponent_of(bits(i0 + r, j0 + 32 * q, 1)));
+                c[q] = max(c[q], e);
+                row = max(row, e);
+            }
+        }
+        row = __reduce_max_sync(0xffffffffu, row);
+        if (lane == 0 && row) atomicMax(&top[i0 + r], row);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; q++)
+        if (c[q]) atomicMax(&cmax[lane + 32 * q], c[q]);
+    __syncthreads();
+    if (threadIdx.x < 128 && cmax[threadIdx.x]) atomicMax(&top[128 * (int)blockIdx.x + threadIdx.x], cmax[threadIdx.x]);
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x * gridDim.y - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    unsigned m = 0;
+    for (int k = threadIdx.x; k < Np; k += 256) m = max(m, __ldcg(&top[k]));
+    m = __reduce_max_sync(0xffffffffu, m);
+    if (lane == 0) warp_max[warp] = m;
+    __syncthreads();
+    for (int w = 0; w < 8; w++) m = max(m, warp_max[w]);
+    for (int k = threadIdx.x; k < Np; k += 256) {
+        const int e = (int)__ldcg(&top[k]);
+        const int d = k < N ? (int)exponent_of(bits(k, k, 0)) : 0;
+        col[k] = e == 0 ? kEmptyColumn : (max(d, 2 * e - (int)m) - 1023) >> 1;
+        top[k] = 0;
+    }
+    if (threadIdx.x == 0) *ticket = 0;
 }
 
 // ---------------------------------------------------------------- recombination
@@ -955,8 +1064,35 @@ tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
     return make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
 }
 
+size_t crt_columns_bytes(int Np) { return round256((size_t)(Np + 1) * sizeof(unsigned)) + round256((size_t)Np * sizeof(int)); }
+
+tc_status crt_columns_init(CrtColumns& c, Arena& ar, int Np) {
+    c.Np = Np;
+    c.top = ar.take<unsigned>((size_t)Np + 1);
+    c.col = ar.take<int>((size_t)Np);
+    if (!c.top || !c.col) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
+    return TC_OK;
+}
+
+tc_status crt_columns_clear(const CrtColumns& c, cudaStream_t s) {
+    TC_CUDA(cudaMemsetAsync(c.top, 0, ((size_t)c.Np + 1) * sizeof(unsigned), s));
+    return TC_OK;
+}
+
+tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, bool interleaved, int N, size_t ld,
+                      cudaStream_t s) {
+    if (N > c.Np || c.Np % 128 != 0) return fail(TC_ERR_INVALID_ARG, "column scales: size");
+    const dim3 grid((unsigned)((N + 127) / 128), (unsigned)((N + 31) / 32));
+    if (interleaved)
+        crt_columns_kernel<true><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+    else
+        crt_columns_kernel<false><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+    TC_LAUNCH_CHECK();
+    return TC_OK;
+}
+
 tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
-                       size_t ld, cudaStream_t s) {
+                       size_t ld, cudaStream_t s, const int* col) {
     if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
         (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
@@ -966,8 +1102,10 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
     const unsigned grid = (unsigned)((m.Np + 128 / tpr - 1) / (128 / tpr));
     const uint64_t flip = conj ? 1ull << 63 : 0;
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
-#define TC_RES(I_, L_, C_) \
-    crt_residue_kernel<I_, L_, C_><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, out, m.ex, m.diag)
+#define TC_RES(I_, L_, C_)                                                                                          \
+    col ? crt_residue_kernel<I_, L_, C_, false, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, col, out, \
+                                                                           m.ex, m.diag)                            \
+        : crt_residue_kernel<I_, L_, C_><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, nullptr, out, m.ex, m.diag)
     if (interleaved && m.left) {
         if (cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
     } else if (interleaved) {
@@ -1035,9 +1173,9 @@ tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
     const unsigned grid = (unsigned)(N / (128 / tpr));
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
     if (m.left)
-        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, m.diag);
+        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, out, m.ex, m.diag);
     else
-        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, out, m.ex, nullptr);
+        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, out, m.ex, nullptr);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }

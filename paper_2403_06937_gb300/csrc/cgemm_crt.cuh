@@ -27,9 +27,23 @@ tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left);
 // `view`: the buffers of `base` seen as an operand of the smaller padded size Np
 tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np);
 // Residues of the N x N matrix (row stride ld; zero-padded to Np).  interleaved:
-// re points to complex128; conj negates the imaginary part.
+// re points to complex128; conj negates the imaginary part.  col: column scales
+// of the pair of operands, the same for both (crt_columns), or none.
 tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
-                       size_t ld, cudaStream_t s);
+                       size_t ld, cudaStream_t s, const int* col = nullptr);
+
+// Powers of two along K, taken from a state: see cgemm_crt.cu.  `top` is zero
+// between calls (crt_columns_clear, once).
+struct CrtColumns {
+    unsigned* top;
+    int* col;
+    int Np;
+};
+size_t crt_columns_bytes(int Np);
+tc_status crt_columns_init(CrtColumns& c, Arena& ar, int Np);
+tc_status crt_columns_clear(const CrtColumns& c, cudaStream_t s);
+tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, bool interleaved, int N, size_t ld,
+                      cudaStream_t s);
 // Bytes of scratch of a product: one byte per residue of the result (of a band
 // of rows above Np = 16384).
 size_t crt_scratch_bytes(int Np);

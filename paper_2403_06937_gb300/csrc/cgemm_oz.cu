@@ -833,8 +833,8 @@ tc_status oz_mat_view(OzMat& view, const OzMat& base, int Np) {
 }
 
 tc_status oz_mat_load(OzMat& m, const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld,
-                      cudaStream_t s) {
-    if (oz_modular()) return crt_mat_load(m.crt, re, im, interleaved, conj, N, ld, s);
+                      cudaStream_t s, const int* col) {
+    if (oz_modular()) return crt_mat_load(m.crt, re, im, interleaved, conj, N, ld, s, col);
     return oz_slice(re, im, interleaved, conj, N, ld, m.Np, kOzDigits, m.slices, m.ex, s);
 }
 

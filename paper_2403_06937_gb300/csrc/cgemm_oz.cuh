@@ -88,8 +88,9 @@ size_t oz_scratch_bytes(int Np);
 tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left);
 // `view` = `base`'s buffers seen as an operand of the smaller padded size Np
 tc_status oz_mat_view(OzMat& view, const OzMat& base, int Np);
+// col: column scales (residue form only)
 tc_status oz_mat_load(OzMat& m, const double* re, const double* im, bool interleaved, bool conj, int N, size_t ld,
-                      cudaStream_t s);
+                      cudaStream_t s, const int* col = nullptr);
 // Y = A B^H at FP64 accuracy; mode 1 (Hermitian result): block-lower tiles and
 // the mirror.  (br, bi): the FP64 planes B was loaded from (N valid rows and
 // columns, row stride ldb), distinct from the result's.
@@ -102,12 +103,15 @@ tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br,
 // (observable row k when obs is given), tail() writes rho back interleaved.
 struct OzSystem {
     int n = 0, N = 0, Np = 0, group = 8, renorm_every = 0;
+    bool scaled = false;   // TC_FP64: column scales from rho in every step
+    CrtColumns cols{};
+    const double* U = nullptr;
     OzMat Us{}, Ps{};
     double *Rr = nullptr, *Ri = nullptr, *Xr = nullptr, *Xi = nullptr, *scratch = nullptr;
     void* prod = nullptr;   // scratch of the products
     const Model* m = nullptr;
     double* obs = nullptr;
-    tc_status carve(int n, Arena& ar);
+    tc_status carve(int n, bool scaled, Arena& ar);
     // planes: rho into the FP64 planes; else step 1 reads it as it is (step_from)
     tc_status first(const double* U, const double* rho, const Model* m, double* obs, int renorm_every, bool planes,
                     cudaStream_t cs);

@@ -6,7 +6,9 @@
 //
 // Per step: the operand form of rho, X = U rho^H (all tiles), that of X,
 // rho' = U X^H = U rho U^H (block-lower tiles, the upper half mirrored),
-// observables from the FP64 planes; U's is made once per call.
+// observables from the FP64 planes.  U's operand form is made once per call for
+// TC_FP64_OZAKI, and once per step with the column scales of that step's rho for
+// TC_FP64 (small populations, see cgemm_crt.cu).
 #include "cgemm_oz.cuh"
 #include "cgemm_tc.cuh"
 #include "graph.cuh"
@@ -83,11 +85,12 @@ int padded_dim(int n) { return (1 << n) < 128 ? 128 : (1 << n); }
 size_t evolve_oz_bytes(int n) {
     const size_t Np = (size_t)padded_dim(n);
     return oz_mat_bytes((int)Np, true) + oz_mat_bytes((int)Np, false) + oz_scratch_bytes((int)Np) +
-           4 * round256(Np * Np * sizeof(double)) + observables_scratch_bytes(n) + 512;
+           4 * round256(Np * Np * sizeof(double)) + observables_scratch_bytes(n) + crt_columns_bytes((int)Np) + 512;
 }
 
-tc_status OzSystem::carve(int n_, Arena& ar) {
+tc_status OzSystem::carve(int n_, bool scaled_, Arena& ar) {
     n = n_;
+    scaled = scaled_;
     N = 1 << n;
     Np = padded_dim(n);
     const size_t NN = (size_t)Np * Np;
@@ -98,19 +101,24 @@ tc_status OzSystem::carve(int n_, Arena& ar) {
     Xr = ar.take<double>(NN);
     Xi = ar.take<double>(NN);
     prod = ar.take<uint8_t>(oz_scratch_bytes(Np));
+    TC_TRY(crt_columns_init(cols, ar, Np));
     scratch = ar.take<double>(observables_scratch_bytes(n) / sizeof(double));
     if (!scratch) return fail(TC_ERR_WORKSPACE, "evolve: workspace too small");
     group = tune_lookup(n, TC_BF16X3).tc_group;
     return TC_OK;
 }
 
-tc_status OzSystem::first(const double* U, const double* rho, const Model* m_, double* obs_, int renorm_every_,
+tc_status OzSystem::first(const double* U_, const double* rho, const Model* m_, double* obs_, int renorm_every_,
                           bool planes, cudaStream_t cs) {
+    U = U_;
     m = m_;
     obs = obs_;
     renorm_every = renorm_every_;
     const size_t NN = (size_t)Np * Np;
-    TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs));
+    if (scaled)
+        TC_TRY(crt_columns_clear(cols, cs));
+    else
+        TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs));
     if (planes) {
         split_pad_kernel<<<grid_for(NN), 256, 0, cs>>>(reinterpret_cast<const double2*>(rho), N, Np, Rr, Ri);
         TC_LAUNCH_CHECK();
@@ -127,12 +135,17 @@ tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double*
     OzOut X{Xr, Xi, prod}, R{Rr, Ri, prod};
     X.b_c128 = from;
     R.y_c128 = to;
-    TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs));
+    const int* col = scaled ? cols.col : nullptr;
+    if (scaled) {
+        TC_TRY(crt_columns(cols, from ? from : Rr, Ri, from != nullptr, N, (size_t)Np, cs));
+        TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs, col));
+    }
+    TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs, col));
     {
         ProductTimer t(8.0 * N3 * oz_products(), cs);   // X = U rho^H
         TC_TRY(oz_product(0, Us, Ps, Rr, Ri, N, (size_t)Np, X, group, cs));
     }
-    TC_TRY(oz_mat_load(Ps, Xr, Xi, false, false, N, (size_t)Np, cs));
+    TC_TRY(oz_mat_load(Ps, Xr, Xi, false, false, N, (size_t)Np, cs, col));
     TC_TRY(side.wait());   // rho is overwritten from here on
     {
         ProductTimer t(4.0 * N3 * oz_products(), cs);   // rho' = U X^H, Hermitian half + mirror
@@ -170,10 +183,10 @@ tc_status OzSystem::tail(double* rho, cudaStream_t cs) {
 // TC_FP64 on the DMMA.
 bool f64_on_tensor_cores(int n) { return n >= 7 && n <= 14 && oz_modular(); }
 
-tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m, double* obs,
-                    Arena& ar, cudaStream_t s) {
+tc_status evolve_oz(const double* U, double* rho, int n, int steps, int precision, int renorm_every, const Model* m,
+                    double* obs, Arena& ar, cudaStream_t s) {
     OzSystem z;
-    TC_TRY(z.carve(n, ar));
+    TC_TRY(z.carve(n, precision == TC_FP64, ar));
     if (steps == 0) {   // rho stays as it is
         if (obs) TC_TRY(launch_observables(kRhoInterleaved, rho, nullptr, m, n, obs, z.scratch, s));
         return TC_OK;

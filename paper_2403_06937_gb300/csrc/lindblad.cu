@@ -719,12 +719,15 @@ size_t evolve_oz_bytes_blocks(int n) {
     }
     b += oz_mat_bytes(NpMax, false) + oz_scratch_bytes(NpMax);   // B operand, scratch of the products
     b += 2 * round256((size_t)NpMax * NpMax * sizeof(double));   // X planes
+    b += crt_columns_bytes(NpMax);
     return b + obs_scratch_bytes(L) + 256;
 }
 
-tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double dt, const double* U, double* rho,
-                           int steps, int renorm_every, double* obs, Arena& ar, cudaStream_t s) {
+tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, double kappa, double dt, const double* U,
+                           double* rho, int steps, int renorm_every, double* obs, Arena& ar, cudaStream_t s) {
     const int n = L.n;
+    // TC_FP64: column scales from every block's rho, so U_k is loaded anew in each step (as in evolve_oz.cu)
+    const bool scaled = precision == TC_FP64, load_once = !scaled && !shared_left(n);
     const size_t PT = padded_total(L);
     const int NpMax = padded(L.N);
     const size_t NN = (size_t)NpMax * NpMax;
@@ -752,6 +755,9 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     double* Xr = ar.take<double>(NN);
     double* Xi = ar.take<double>(NN);
     void* prod = ar.take<uint8_t>(oz_scratch_bytes(NpMax));
+    CrtColumns cols{};
+    TC_TRY(crt_columns_init(cols, ar, NpMax));
+    const int* col = scaled ? cols.col : nullptr;
     double* scratch = ar.take<double>(obs_scratch_bytes(L) / sizeof(double));
     if (!scratch) return fail(TC_ERR_WORKSPACE, "lindblad evolve: workspace too small");
     // the B operand slices seen at each block's padded size (one map per block)
@@ -787,14 +793,15 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
                 TC_TRY(gemm_f64(g2, cs));
                 continue;
             }
-            if (shared_left(n))
-                TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs));
-            TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs));
+            if (scaled) TC_TRY(crt_columns(cols, rr, ri, false, d, (size_t)Np, cs));
+            if (!load_once)
+                TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs, col));
+            TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs, col));
             {
                 ProductTimer pt(8.0 * d3 * oz_products(), cs);   // X_k = U_k rho_k
                 TC_TRY(oz_product(0, Uk[k], Bk[k], rr, ri, d, (size_t)Np, OzOut{Xr, Xi, prod}, group, cs));
             }
-            TC_TRY(oz_mat_load(Bk[k], Xr, Xi, false, false, d, (size_t)Np, cs));
+            TC_TRY(oz_mat_load(Bk[k], Xr, Xi, false, false, d, (size_t)Np, cs, col));
             {
                 ProductTimer pt(4.0 * d3 * oz_products(), cs);   // rho_k = U_k X_k^H, Hermitian
                 TC_TRY(oz_product(1, Uk[k], Bk[k], Xr, Xi, d, (size_t)Np, OzOut{rr, ri, prod}, group, cs));
@@ -813,12 +820,13 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, double kappa, double
     };
     auto first = [&](cudaStream_t cs) -> tc_status {
         TC_TRY(launch_layout(L, t, cs));
+        if (scaled) TC_TRY(crt_columns_clear(cols, cs));
         for (int k = 0; k <= n; k++) {
             const int d = L.dims[k], Np = bs.ld[k];
             if (d <= kSmallBlock) {   // zero padding: the planes' rows are read up to d only
                 split_block_kernel<<<64, 256, 0, cs>>>(reinterpret_cast<const double2*>(U) + L.off[k], d, Np, Ur[k], Ui[k]);
                 TC_LAUNCH_CHECK();
-            } else if (!shared_left(n)) {
+            } else if (load_once) {
                 TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs));
             }
         }
@@ -926,6 +934,6 @@ extern "C" TC_API tc_status tc_lindblad_evolve(const tc_params* params, double k
     if (precision == TC_FP64 && !(blocks_f64_on_tensor_cores(m.n) && work_bytes >= evolve_oz_bytes_blocks(m.n)))
         return evolve_f64(L, m, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
     if (precision == TC_FP64 || precision == TC_FP64_OZAKI)
-        return evolve_oz_blocks(L, m, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
+        return evolve_oz_blocks(L, m, precision, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
     return evolve_lowp_blocks(L, m, precision, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
 }

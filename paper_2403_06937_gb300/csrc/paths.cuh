@@ -36,8 +36,8 @@ tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_
 
 // FP64-accurate step loop on the BF16 tensor cores (exact integer products).
 size_t evolve_oz_bytes(int n);
-tc_status evolve_oz(const double* U, double* rho, int n, int steps, int renorm_every, const Model* m, double* obs,
-                    Arena& ar, cudaStream_t s);
+tc_status evolve_oz(const double* U, double* rho, int n, int steps, int precision, int renorm_every, const Model* m,
+                    double* obs, Arena& ar, cudaStream_t s);
 // True when TC_FP64 runs on those products for n atoms, given a workspace of their size.
 bool f64_on_tensor_cores(int n);
 
