@@ -504,6 +504,12 @@ TC_API tc_status tc_batch_autotune_set(int count, const int* n, int precision, c
  * takes the tc_autotune choice for its largest n. */
 TC_API tc_status tc_batch_autotune_lookup(int count, const int* n, int precision, int* choice, int* found);
 
+/* Give back the streams and events that the library keeps for later calls (at
+ * most two sets a device, each of two streams, or ten after a batch in the
+ * FP64 forms).  Work that still runs on them completes.  Returns the number of
+ * sets. */
+TC_API int tc_release_idle(void);
+
 /* ----------------------------------------------------------- measurement */
 
 /* Number of kernels this library has launched in this process. */

@@ -402,6 +402,11 @@ def batch_autotune_lookup(ns, precision="bf16x3"):
     return {"tc_group": out[0], "tc_shape": out[1]} if found.value else None
 
 
+def release_idle() -> int:
+    """tc_release_idle: give back the streams kept for later calls; returns the number of sets."""
+    return int(_abi.load().tc_release_idle())
+
+
 def launch_count() -> int:
     """Kernels launched by libtc in this process."""
     return int(_abi.load().tc_launch_count())
@@ -443,7 +448,7 @@ __all__ = ["Params", "TCError", "build_hamiltonian", "expm", "expm_model", "evol
            "lindblad_layout", "lindblad_propagators", "lindblad_evolve", "evolve_host", "observables",
            "expectation_diag",
            "evolve_backward", "EvolveFn", "batch_evolve", "autotune", "autotune_lookup", "autotune_set", "batch_autotune", "batch_autotune_set", "batch_autotune_lookup",
-           "workspace_size", "launch_count", "timing_enable", "timing_read", "phases_enable", "phases_read",
+           "workspace_size", "release_idle", "launch_count", "timing_enable", "timing_read", "phases_enable", "phases_read",
            "device_check", "sync_status", "obs_stride", "PRECISIONS", "TC_FP64", "TC_BF16X3", "TC_TF32",
            "TC_TF32X3", "TC_COUPLING_BOSONIC", "TC_COUPLING_QUBIT_PHOTON", "TC_OP_EXPM", "TC_OP_EVOLVE",
            "TC_OP_OBSERVABLES", "TC_OP_BACKWARD"]

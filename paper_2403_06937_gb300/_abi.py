@@ -73,6 +73,7 @@ SIGNATURES = {
     "tc_batch_workspace_size": (SZ, [I, ctypes.POINTER(I), I]),
     "tc_batch_evolve": (I, [I, ctypes.POINTER(I), ctypes.POINTER(VP), ctypes.POINTER(VP), I, I, I,
                             ctypes.POINTER(tc_params), ctypes.POINTER(VP), VP, SZ, VP]),
+    "tc_release_idle": (I, []),
     "tc_launch_count": (ctypes.c_longlong, []),
     "tc_timing_enable": (I, [I]),
     "tc_timing_read": (I, [ctypes.POINTER(ctypes.c_longlong), DP, DP]),

@@ -9,6 +9,7 @@
 #include "kernels.cuh"
 #include "cgemm_oz.cuh"
 #include "cgemm_tc.cuh"
+#include "graph.cuh"
 #include "paths.cuh"
 
 namespace tc {
@@ -392,6 +393,8 @@ extern "C" {
 TC_API const char* tc_version(void) { return "libtc 0.1 (sm_103a)"; }
 
 TC_API const char* tc_last_error(void) { return g_last_error.c_str(); }
+
+TC_API int tc_release_idle(void) { return StreamSet::release_idle(); }
 
 TC_API tc_status tc_device_check(void) { return check_device(); }
 

@@ -1,18 +1,14 @@
 // graph.cu -- see graph.cuh.
 #include <algorithm>
-#include <array>
-#include <memory>
 #include <mutex>
-#include <vector>
+#include <new>
 
 #include "graph.cuh"
 
 namespace tc {
 namespace {
-constexpr size_t kIdleSets = 4;   // a device
 std::mutex g_mu;
-// never destroyed: the runtime may be gone when static objects are
-auto& g_idle = *new std::array<std::vector<std::unique_ptr<StreamSet>>, 64>;
+StreamSet* g_idle[64] = {};   // lists; not destroyed with the process: the runtime may be gone by then
 thread_local StreamSet* t_leased = nullptr;
 
 tc_status current_device(int* dev) {
@@ -39,6 +35,53 @@ tc_status StreamSet::create_lanes() {
     return TC_OK;
 }
 
+// Takes out of the device's list all idle sets but the first `keep`, and returns them as a list.  A set whose lanes
+// were forked from a stream that its caller still captures counts as idle once that capture has ended.
+StreamSet* StreamSet::surplus(int device, int keep) {
+    StreamSet* out = nullptr;
+    for (StreamSet** at = &g_idle[device]; *at;) {
+        StreamSet* x = *at;
+        if (x->in_callers_graph && !caller_captures(x->lane[0])) x->in_callers_graph = false;
+        if (x->in_callers_graph || keep-- > 0) {
+            at = &x->next;
+            continue;
+        }
+        *at = x->next;
+        x->next = out;
+        out = x;
+    }
+    return out;
+}
+
+void StreamSet::destroy(StreamSet* list) {
+    while (list) {
+        StreamSet* x = list;
+        list = x->next;
+        delete x;
+    }
+}
+
+int StreamSet::release_idle() {
+    StreamSet* list = nullptr;
+    for (int d = 0; d < 64; d++) {
+        StreamSet* got;
+        {
+            std::lock_guard<std::mutex> lk(g_mu);
+            got = surplus(d, 0);
+        }
+        while (got) {
+            StreamSet* x = got;
+            got = x->next;
+            x->next = list;
+            list = x;
+        }
+    }
+    int n = 0;
+    for (StreamSet* x = list; x; x = x->next) n++;
+    destroy(list);
+    return n;
+}
+
 StreamSet::~StreamSet() {
     for (cudaEvent_t e : {before, after, fork, join, lane_fork})
         if (e) cudaEventDestroy(e);
@@ -53,24 +96,30 @@ StreamSet::~StreamSet() {
 tc_status StreamLease::take() {
     int dev = 0;
     TC_TRY(current_device(&dev));
-    std::unique_ptr<StreamSet> got;
+    StreamSet* got = nullptr;
     {
         std::lock_guard<std::mutex> lk(g_mu);
-        auto& idle = g_idle[dev];
-        for (size_t i = idle.size(); i-- > 0 && !got;) {
-            if (idle[i]->in_callers_graph) {   // free again once the caller's capture has ended
-                if (caller_captures(idle[i]->lane[0])) continue;
-                idle[i]->in_callers_graph = false;
+        for (StreamSet** at = &g_idle[dev]; *at; at = &(*at)->next) {
+            if ((*at)->in_callers_graph) {   // free again once the caller's capture has ended
+                if (caller_captures((*at)->lane[0])) continue;
+                (*at)->in_callers_graph = false;
             }
-            got = std::move(idle[i]);
-            idle.erase(idle.begin() + (long)i);
+            got = *at;
+            *at = got->next;
+            break;
         }
     }
     if (!got) {
-        got = std::make_unique<StreamSet>();
-        TC_TRY(got->create(dev));
+        got = new (std::nothrow) StreamSet;
+        if (!got) return fail(TC_ERR_CUDA, "out of host memory");
+        const tc_status st = got->create(dev);
+        if (st != TC_OK) {
+            delete got;
+            return st;
+        }
     }
-    set_ = got.release();
+    got->next = nullptr;
+    set_ = got;
     outer_ = t_leased;
     t_leased = set_;
     return TC_OK;
@@ -79,11 +128,14 @@ tc_status StreamLease::take() {
 StreamLease::~StreamLease() {
     if (!set_) return;
     t_leased = outer_;
-    std::unique_ptr<StreamSet> back(set_);
-    std::lock_guard<std::mutex> lk(g_mu);
-    auto& idle = g_idle[back->dev];
-    // one whose streams the caller still captures is kept in any case: it cannot be destroyed yet
-    if (idle.size() < kIdleSets || back->in_callers_graph) idle.push_back(std::move(back));
+    StreamSet* out;
+    {
+        std::lock_guard<std::mutex> lk(g_mu);
+        set_->next = g_idle[set_->dev];
+        g_idle[set_->dev] = set_;
+        out = StreamSet::surplus(set_->dev, kIdleSets);
+    }
+    StreamSet::destroy(out);   // work still running on them completes
 }
 
 StreamSet* leased_streams() { return t_leased; }

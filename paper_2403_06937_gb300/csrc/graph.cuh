@@ -11,8 +11,9 @@ namespace tc {
 // The streams and events that one call uses beside its caller's stream.  A
 // call leases a set and gives it back when it returns (its work may still be
 // running: the next call on the set is ordered after it by the streams), so
-// calls on several threads never share one.  Idle sets are kept, at most
-// kIdleSets a device.
+// calls on several threads never share one.  Idle sets are kept for the next
+// call, at most kIdleSets a device; tc_release_idle gives them back.
+constexpr int kIdleSets = 2;
 struct StreamSet {
     static constexpr int kLanes = 8;
     int dev = 0;
@@ -22,9 +23,13 @@ struct StreamSet {
     cudaEvent_t before = nullptr, after = nullptr, fork = nullptr, join = nullptr;
     cudaEvent_t lane_fork = nullptr, lane_join[kLanes] = {};
     bool in_callers_graph = false;                   // its lanes were forked from a stream the caller captures
+    StreamSet* next = nullptr;                       // in the list of idle sets
     tc_status create(int device);
     tc_status create_lanes();
     ~StreamSet();
+    static StreamSet* surplus(int device, int keep);
+    static void destroy(StreamSet* list);
+    static int release_idle();                       // every device's; how many there were
 };
 
 class StreamLease {
