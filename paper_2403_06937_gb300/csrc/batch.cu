@@ -24,13 +24,19 @@ namespace {
 // Systems of a batch in the FP64 forms run side by side on this many streams.
 constexpr int kOzLanes = StreamSet::kLanes;
 
-// The systems of a batch spread over at most kOzLanes lanes: largest first to
+// Lanes beyond the first few of large systems hold memory and little else: one
+// product at n = 10 already has seven units for each CTA pair of the GPU.  The
+// stated workspace has the most lanes that stay within this (n = 12: eight,
+// n = 13: two, n = 14: one), an eighth of the memory.
+constexpr size_t kLanesBytes = (size_t)32 << 30;
+
+// The systems of a batch spread over at most `lanes` lanes: largest first to
 // the lane with the least work (N^3 each).
-std::vector<std::vector<int>> assign_lanes(int count, const int* n) {
+std::vector<std::vector<int>> assign_lanes(int count, const int* n, int lanes) {
     std::vector<int> order(count);
     std::iota(order.begin(), order.end(), 0);
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return n[a] > n[b]; });
-    std::vector<std::vector<int>> lane(count < kOzLanes ? count : kOzLanes);
+    std::vector<std::vector<int>> lane(std::min(count, lanes));
     std::vector<double> load(lane.size(), 0.0);
     for (int b : order) {
         const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
@@ -47,48 +53,67 @@ size_t lane_system_bytes(int n, int precision, bool dmma) {
     return round256(tensor ? evolve_oz_bytes(n) : evolve_f64_bytes(n));
 }
 
-// A lane runs its systems one after another, each from its first kernel to its
-// last, so it needs the buffers of its largest one only.
-size_t lanes_bytes(int count, const int* n, int precision) {
-    size_t total = 256;
-    for (const auto& lane : assign_lanes(count, n)) {
+// A batch in the FP64 forms: its lanes and their buffers.  A lane runs its
+// systems one after another, each from its first kernel to its last, so it
+// needs the buffer of its largest one only.
+struct Lanes {
+    std::vector<std::vector<int>> lane;
+    std::vector<size_t> bytes;
+    size_t total = 0;
+    bool dmma = false;
+};
+Lanes make_lanes(int count, const int* n, int precision, int lanes, bool dmma) {
+    Lanes p;
+    p.dmma = dmma;
+    p.lane = assign_lanes(count, n, lanes);
+    p.total = 256;
+    for (const auto& lane : p.lane) {
         size_t most = 0;
-        for (int b : lane) most = std::max(most, lane_system_bytes(n[b], precision, false));
-        total += most;
+        for (int b : lane) most = std::max(most, lane_system_bytes(n[b], precision, dmma));
+        p.bytes.push_back(most);
+        p.total += most;
     }
-    return total;
+    return p;
 }
-
-// What TC_FP64 needs at least: one lane, every system on the DMMA.
-size_t one_lane_bytes(int count, const int* n) {
-    size_t most = 0;
-    for (int b = 0; b < count; b++) most = std::max(most, lane_system_bytes(n[b], TC_FP64, true));
-    return most + 256;
+// The most lanes that fit: every system on the tensor cores if that can be had
+// with one lane, else (TC_FP64) on the DMMA.  total > have when nothing fits.
+Lanes fit_lanes(int count, const int* n, int precision, size_t have) {
+    for (const bool dmma : {false, true}) {
+        if (dmma && precision != TC_FP64) break;
+        for (int l = std::min(count, kOzLanes); l >= 1; l--) {
+            Lanes p = make_lanes(count, n, precision, l, dmma);
+            if (p.total <= have) return p;
+        }
+    }
+    return make_lanes(count, n, precision, 1, precision == TC_FP64);
+}
+size_t lanes_bytes(int count, const int* n, int precision) {
+    for (int l = std::min(count, kOzLanes); l > 1; l--) {
+        const size_t b = make_lanes(count, n, precision, l, false).total;
+        if (b <= kLanesBytes) return b;
+    }
+    return make_lanes(count, n, precision, 1, false).total;
+}
+size_t least_lanes_bytes(int count, const int* n, int precision) {
+    return make_lanes(count, n, precision, 1, precision == TC_FP64).total;
 }
 
 // The FP64 forms: every system's run is one sequence on one of up to kOzLanes
 // concurrent lanes, captured into one graph (fork from the capture stream, join
 // back before its end), so the small systems' launches fill the SMs the large
 // products leave idle.  Each system's launches are those of tc_evolve on it
-// alone, so its results are bitwise the same.  TC_FP64 with less workspace
-// than the lanes want runs on one lane, every system on the DMMA.
+// alone, so its results are bitwise the same, on any number of lanes.
 tc_status batch_lanes(int count, const int* n, const void* const* U, void* const* rho, int steps, int precision,
                       int renorm_every, const Model* models, double* const* obs, void* work, size_t work_bytes,
                       cudaStream_t us) {
-    const bool dmma = precision == TC_FP64 && work_bytes < lanes_bytes(count, n, precision);
-    std::vector<std::vector<int>> lane;
-    if (dmma) {
-        lane.resize(1);
-        for (int b = 0; b < count; b++) lane[0].push_back(b);
-    } else {
-        lane = assign_lanes(count, n);
-    }
+    const Lanes plan = fit_lanes(count, n, precision, work_bytes);
+    const auto& lane = plan.lane;
+    const auto& bytes = plan.bytes;
+    const bool dmma = plan.dmma;
     const int L = (int)lane.size();
     Arena all{static_cast<char*>(work), work_bytes, 0};
     std::vector<char*> base(L);
-    std::vector<size_t> bytes(L, 0);
     for (int l = 0; l < L; l++) {
-        for (int b : lane[l]) bytes[l] = std::max(bytes[l], lane_system_bytes(n[b], precision, dmma));
         base[l] = all.take<char>(bytes[l]);
         if (!base[l]) return fail(TC_ERR_WORKSPACE, "batch: workspace too small");
     }
@@ -170,7 +195,8 @@ TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, 
             if (models[b].n != n[b]) return fail(TC_ERR_INVALID_ARG, "system %d: params.n != n", b);
         }
     }
-    const size_t need = precision == TC_FP64 ? one_lane_bytes(count, n) : batch_bytes(count, n, precision);
+    const size_t need = precision == TC_FP64 || precision == TC_FP64_OZAKI ? least_lanes_bytes(count, n, precision)
+                                                                             : batch_bytes(count, n, precision);
     if (!work) return fail(TC_ERR_WORKSPACE, "work is NULL (need %zu bytes)", need);
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(TC_ERR_WORKSPACE, "work is not 256-byte aligned");
     if (work_bytes < need) return fail(TC_ERR_WORKSPACE, "work has %zu bytes, need %zu", work_bytes, need);
