@@ -70,11 +70,29 @@ typedef enum tc_status {
 
 /* Arithmetic of the rho <- U rho U^dag products (the tensor-core path).
  *  TC_FP64   : products at FP64 accuracy, rho stored in FP64.  For
- *              7 <= n <= 14 (gradient: 13) and a workspace of the size that
- *              tc_workspace_size states they run as TC_FP64_OZAKI's residue
- *              products; at other sizes, in a smaller workspace (down to the
- *              six N x N FP64 planes of the DMMA form and its scratch) or
- *              under TC_OZ_BITS=6, on the FP64 DMMA (mma.sync .f64).
+ *              7 <= n <= 14 (gradient and open system: 13) and a workspace of
+ *              the size that tc_workspace_size states they run as
+ *              TC_FP64_OZAKI's residue products; at other sizes, in a smaller
+ *              workspace (down to tc_workspace_least) or under TC_OZ_BITS=6, on
+ *              the FP64 DMMA.
+ *              Accuracy of the residue products: the DMMA form rounds sums of
+ *              products of 53-bit entries, so every entry of a result is
+ *              accurate relative to its own sum of magnitudes.  The residue
+ *              form holds an operand as integers in one scale a row.  In the
+ *              step loops (tc_evolve, tc_evolve_host, tc_batch_evolve,
+ *              tc_lindblad_evolve) the columns are scaled by the state's
+ *              populations too, which keeps every population of a positive
+ *              rho as accurate as the DMMA form does, and a coherence rho_ij
+ *              relative to sqrt(rho_ii rho_jj).  In tc_expm and
+ *              tc_evolve_backward there is no such scale: errors are relative
+ *              to the norms of rows (2^-59 of a row's norm an entry), so an
+ *              entry of U far below its row's norm, or a gradient of a loss far
+ *              below 1, has fewer right digits than from the DMMA form.  Ask
+ *              for TC_FP64_DMMA (tc_expm: a workspace of tc_workspace_least
+ *              bytes; tc_expm_model does not use these products) where such
+ *              numbers matter.
+ *  TC_FP64_DMMA : TC_FP64 on the FP64 DMMA (mma.sync .f64) at every size, as
+ *              accurate entry by entry as FP64 sums are, at about 1 TFLOP/s.
  *  TC_BF16X3 : each FP32 operand split in three BF16 parts, six BF16 products
  *              accumulated in FP32 in tensor memory (tcgen05 kind::f16).
  *  TC_TF32   : one TF32 product, FP32 accumulate (tcgen05 kind::tf32).
@@ -100,7 +118,8 @@ typedef enum tc_precision {
     TC_BF16X3 = 1,
     TC_TF32 = 2,
     TC_TF32X3 = 3,
-    TC_FP64_OZAKI = 4
+    TC_FP64_OZAKI = 4,
+    TC_FP64_DMMA = 5
 } tc_precision;
 
 /* Coupling matrix element between s_e (atom i excited, p photons) and s_g
@@ -167,10 +186,17 @@ TC_API const char* tc_last_error(void);
 /* TC_OK if the current CUDA device is an sm_103 GPU the kernels were built for. */
 TC_API tc_status tc_device_check(void);
 
-/* Bytes of `work` needed by the operations in `ops` (TC_OP_*) for n atoms at
- * the given precision.  For TC_OP_BACKWARD, `steps` and `ckpt_every` size the
- * checkpoint store; elsewhere they are ignored.  Returns 0 for invalid n. */
+/* Bytes of `work` for the operations in `ops` (TC_OP_*) with n atoms at the
+ * given precision.  For TC_OP_BACKWARD, `steps` and `ckpt_every` size the
+ * checkpoint store, for TC_OP_EVOLVE_HOST* `steps` the observable rows;
+ * elsewhere they are ignored.  Returns 0 for invalid n.
+ * tc_workspace_size: for the fastest form.  tc_workspace_least: the least that
+ * the calls accept; with less than the stated size TC_FP64 and tc_expm run on
+ * the FP64 DMMA (much slower), and TC_FP64_OZAKI makes its operands' residues
+ * four moduli at a time (the same bits; some percent slower at large n).  The
+ * two differ in the FP64 forms only. */
 TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ckpt_every);
+TC_API size_t tc_workspace_least(int n, int precision, int ops, int steps, int ckpt_every);
 
 /* ------------------------------------------------------------- the path */
 
@@ -368,8 +394,8 @@ TC_API tc_status tc_lindblad_evolve(const tc_params* params, double kappa, doubl
  * checkpoints stored every `ckpt_every` steps.
  *  rho0   : device, N*N c128 (Hermitian, read only).
  *  U      : device, N*N c128, e^{-iH dt} of the same params and dt.
- *  precision: TC_FP64, or TC_FP64_OZAKI (n >= 7).  The products run on the
- *           tensor cores (see tc_precision) or on the DMMA.
+ *  precision: TC_FP64, TC_FP64_DMMA or TC_FP64_OZAKI (n >= 7).  The products run
+ *           on the tensor cores or on the DMMA (see tc_precision).
  *  O_diag : device, N doubles.
  *  grad   : host, n + 2 doubles, written when the call returns (this call
  *           synchronises `stream`).
@@ -451,27 +477,34 @@ TC_API tc_status tc_autotune_set(int n, int precision, const int* choice);
 
 /* ------------------------------------------------------------- batching */
 
-/* Bytes of `work` for tc_batch_evolve of `count` systems with n[b] atoms. */
+/* Bytes of `work` for tc_batch_evolve of `count` systems with n[b] atoms, and
+ * the least that it accepts.  In the FP64 forms the stated size holds as many
+ * concurrent systems (at most eight) as stay within 32 GiB, and a call uses as
+ * many as its workspace holds; with less than one system on the tensor cores
+ * needs, they run as in tc_workspace_least. */
 TC_API size_t tc_batch_workspace_size(int count, const int* n, int precision);
+TC_API size_t tc_batch_workspace_least(int count, const int* n, int precision);
 
 /* tc_batch_evolve -- `count` independent systems of uneven size (n[b] atoms
  * each, own U and rho), each stepped `steps` times by rho <- U rho U^dag
  * (Eq. 6) as in tc_evolve.  The tensor-core forms run each product of a step
  * as ONE persistent launch over the tiles of all systems (systems in
  * decreasing size, static round-robin over the SMs; single CTAs or CTA
- * pairs, see tc_batch_autotune); TC_FP64 and TC_FP64_OZAKI run each system's
- * step loop on one of eight concurrent branches of the graph (library-owned
- * streams, one such call at a time per device).  The step loop is captured
- * into one CUDA graph on a library-owned stream and launched once; the call
- * returns after the batch has finished.  Every system's result (rho, observables) is
- * bitwise the result of tc_evolve on that system alone with the same
- * precision.
+ * pairs, see tc_batch_autotune); the FP64 forms run each system's step loop on
+ * one of up to eight concurrent branches of the graph.  The step loop is
+ * captured into one CUDA graph on a library-owned stream and launched once, in
+ * the order of `stream`; the call does not wait for it (in the tensor-core
+ * forms it synchronises `stream` once at its start), and calls on several
+ * threads may run at the same time, each on streams of its own.  Every
+ * system's result (rho, observables) is bitwise the result of tc_evolve on that
+ * system alone with the same precision in the same form (residue products or
+ * DMMA).
  *  n, U, rho, params, obs : host arrays of `count` entries.  U[b] and rho[b]
  *             are device pointers (N_b x N_b c128, 16-byte aligned; rho in/out);
  *             params may be NULL (energy column 0) or give each system's
  *             parameters; obs may be NULL or hold device pointers (entries
  *             may be NULL) of (steps + 1) * TC_OBS_STRIDE(n[b]) doubles.
- *  work     : device, >= tc_batch_workspace_size(count, n, precision).
+ *  work     : device, >= tc_batch_workspace_least(count, n, precision).
  *  Errors: as tc_evolve, for any system. */
 TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, void* const* rho, int steps,
                                  int precision, int renorm_every, const tc_params* params,

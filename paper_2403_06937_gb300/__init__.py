@@ -23,7 +23,7 @@ from ._abi import (TC_BF16X3, TC_COUPLING_BOSONIC, TC_COUPLING_QUBIT_PHOTON, TC_
                    TC_OP_EVOLVE, TC_OP_EXPM, TC_OP_OBSERVABLES, TC_TF32, TC_TF32X3, TCError)
 
 PRECISIONS = {"fp64": TC_FP64, "bf16x3": TC_BF16X3, "tf32": TC_TF32, "tf32x3": TC_TF32X3,
-              "ozaki": _abi.TC_FP64_OZAKI}
+              "ozaki": _abi.TC_FP64_OZAKI, "fp64_dmma": _abi.TC_FP64_DMMA}
 
 
 @dataclass
@@ -57,9 +57,33 @@ def _work(nbytes: int, device) -> torch.Tensor:
     return torch.empty(max(int(nbytes), 256), dtype=torch.uint8, device=device)
 
 
+def _workspace(work: Optional[torch.Tensor], wanted: int, least: int, device, halving: bool = False) -> torch.Tensor:
+    """The caller's buffer if the call can run in it (`least` bytes), else one of `wanted` bytes, or of what fits
+    (halving: half of it and so on, for calls that use what they get) down to `least`."""
+    if work is not None and work.numel() >= least:
+        return work
+    while True:
+        try:
+            return _work(wanted, device)
+        except torch.cuda.OutOfMemoryError:
+            if wanted <= least:
+                raise
+            wanted = max(least, wanted // 2) if halving else least
+
+
 def workspace_size(n: int, precision: int = TC_FP64, ops: int = TC_OP_EVOLVE, steps: int = 0,
                    ckpt_every: int = 0) -> int:
     return int(_abi.load().tc_workspace_size(n, precision, ops, steps, ckpt_every))
+
+
+def workspace_least(n: int, precision: int = TC_FP64, ops: int = TC_OP_EVOLVE, steps: int = 0,
+                    ckpt_every: int = 0) -> int:
+    return int(_abi.load().tc_workspace_least(n, precision, ops, steps, ckpt_every))
+
+
+def _sized(work, device, n, precision, ops, steps=0, ckpt_every=0):
+    return _workspace(work, workspace_size(n, precision, ops, steps, ckpt_every),
+                      workspace_least(n, precision, ops, steps, ckpt_every), device)
 
 
 def device_check() -> None:
@@ -76,16 +100,19 @@ def build_hamiltonian(params: Params, device="cuda", stream=None) -> torch.Tenso
 
 
 def expm(H: torch.Tensor, n: int, dt: float, taylor_degree: int = 0, squarings: int = -1, shift: bool = True,
-         stream=None, work: Optional[torch.Tensor] = None) -> torch.Tensor:
-    """tc_expm: U = e^{-iH dt} (N x N complex128); {10, 0, False} is the paper's Eq. 10."""
+         stream=None, work: Optional[torch.Tensor] = None, precision="fp64") -> torch.Tensor:
+    """tc_expm: U = e^{-iH dt} (N x N complex128); {10, 0, False} is the paper's Eq. 10.
+
+    precision: "fp64", or "fp64_dmma" for entries of U far below the norms of their rows (tc_precision in tc.h)."""
     N = 1 << n
     assert H.dtype == torch.float64 and H.is_contiguous() and H.shape == (N, N)
     U = torch.empty((N, N), dtype=torch.complex128, device=H.device)
-    need = workspace_size(n, TC_FP64, TC_OP_EXPM)
-    if work is None or work.numel() < need:
-        work = _work(need, H.device)
+    prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
+    work = _sized(work, H.device, n, prec, TC_OP_EXPM)
+    # the size says which form: tc_expm has no precision argument
+    nbytes = workspace_least(n, prec, TC_OP_EXPM) if prec == _abi.TC_FP64_DMMA else work.numel()
     opts = _abi.tc_expm_opts(int(taylor_degree), int(squarings), int(bool(shift)))
-    _abi.call("tc_expm", _ptr(H), n, float(dt), ctypes.byref(opts), _ptr(U), _ptr(work), work.numel(),
+    _abi.call("tc_expm", _ptr(H), n, float(dt), ctypes.byref(opts), _ptr(U), _ptr(work), nbytes,
               ctypes.c_void_p(_stream(stream)))
     return U
 
@@ -116,9 +143,7 @@ def evolve(U: torch.Tensor, rho: torch.Tensor, n: int, steps: int, precision="fp
     assert rho.dtype == torch.complex128 and rho.is_contiguous() and rho.shape == (N, N)
     out = rho if inplace else rho.clone()
     obs = torch.empty((steps + 1, obs_stride(n)), dtype=torch.float64, device=rho.device) if observe else None
-    need = workspace_size(n, prec, TC_OP_EVOLVE)
-    if work is None or work.numel() < need:
-        work = _work(need, rho.device)
+    work = _sized(work, rho.device, n, prec, TC_OP_EVOLVE)
     p = params.c() if params is not None else None
     _abi.call("tc_evolve", _ptr(U), _ptr(out), n, int(steps), prec, int(renorm_every),
               ctypes.byref(p) if p is not None else None, _ptr(obs), _ptr(work), work.numel(),
@@ -158,7 +183,7 @@ def lindblad_propagators(params: Params, dt: float, device="cuda", stream=None,
     """tc_lindblad_propagators: packed U_k = e^{-i H_k dt} for every excitation block."""
     lay = lindblad_layout(params.n)
     U = torch.empty(lay.total, dtype=torch.complex128, device=device)
-    need = workspace_size(params.n, TC_FP64, _abi.TC_OP_LINDBLAD)
+    need = workspace_size(params.n, _abi.TC_FP64_DMMA, _abi.TC_OP_LINDBLAD)
     if work is None or work.numel() < need:
         work = _work(need, device)
     p = params.c()
@@ -178,9 +203,7 @@ def lindblad_evolve(params: Params, kappa: float, dt: float, U: torch.Tensor, rh
         assert t.dtype == torch.complex128 and t.is_contiguous() and t.numel() == lay.total
     out = rho if inplace else rho.clone()
     obs = torch.empty((steps + 1, obs_stride(n)), dtype=torch.float64, device=rho.device) if observe else None
-    need = workspace_size(n, prec, _abi.TC_OP_LINDBLAD)
-    if work is None or work.numel() < need:
-        work = _work(need, rho.device)
+    work = _sized(work, rho.device, n, prec, _abi.TC_OP_LINDBLAD)
     p = params.c()
     _abi.call("tc_lindblad_evolve", ctypes.byref(p), float(kappa), float(dt), _ptr(U), _ptr(out), int(steps), prec,
               int(renorm_every), _ptr(obs), _ptr(work), work.numel(), ctypes.c_void_p(_stream(stream)))
@@ -218,9 +241,7 @@ def evolve_host(U: torch.Tensor, rho_host: torch.Tensor, n: int, steps: int, pre
     assert rho_host.device.type == "cpu" and rho_host.dtype == torch.complex128 and rho_host.shape == (N, N)
     # a page-locked buffer lets the pipelined tensor-core forms skip the device copy of rho
     op = _abi.TC_OP_EVOLVE_HOST_PINNED if rho_host.is_pinned() else _abi.TC_OP_EVOLVE_HOST
-    need = workspace_size(n, prec, op, steps)
-    if work is None or work.numel() < need:
-        work = _work(need, U.device)
+    work = _sized(work, U.device, n, prec, op, steps)
     p = params.c() if params is not None else None
     _abi.call("tc_evolve_host", _ptr(U), _ptr(rho_host), n, int(steps), prec, int(renorm_every),
               ctypes.byref(p) if p is not None else None, _ptr(obs_host), _ptr(work), work.numel(),
@@ -240,9 +261,7 @@ def evolve_backward(params: Params, dt: float, steps: int, rho0: torch.Tensor, U
     assert U.dtype == torch.complex128 and U.is_contiguous() and U.shape == (N, N)
     assert O_diag.dtype == torch.float64 and O_diag.is_cuda and O_diag.numel() == N
     prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
-    need = workspace_size(n, prec, TC_OP_BACKWARD, steps, ckpt_every)
-    if work is None or work.numel() < need:
-        work = _work(need, rho0.device)
+    work = _sized(work, rho0.device, n, prec, TC_OP_BACKWARD, steps, ckpt_every)
     grad = (ctypes.c_double * (n + 2))()
     loss = ctypes.c_double()
     p = params.c()
@@ -259,8 +278,10 @@ class EvolveFn(torch.autograd.Function):
     (tc_evolve) and L (tc_expectation_diag); nothing of the reverse pass runs.
     backward (only when a gradient is asked for): tc_evolve_backward, the
     reverse mode with checkpoints every `ckpt_every` steps.
-    precision: "fp64" or "ozaki" (n >= 7), for both passes; from n = 7 on both are
-    FP64-accurate products on the BF16 tensor cores.
+    precision: "fp64" or "ozaki" (n >= 7), for both passes: from n = 7 on
+    FP64-accurate products on the BF16 tensor cores, whose errors are relative to
+    the norms of rows in H's exponential and in the reverse pass; "fp64_dmma", all
+    of it on the FP64 DMMA, for losses far below 1.
     Inputs g (n,), omega_a (), omega_c () are float64 tensors; rho0 and O_diag
     are CUDA tensors.  Returns a 0-d float64 tensor on rho0's device.
     """
@@ -268,11 +289,12 @@ class EvolveFn(torch.autograd.Function):
     @staticmethod
     def forward(ctx, g, omega_a, omega_c, rho0, O_diag, dt, steps, ckpt_every=20, coupling=TC_COUPLING_BOSONIC,
                 precision="fp64"):
-        if precision not in ("fp64", "ozaki"):
-            raise ValueError("EvolveFn: precision must be 'fp64' or 'ozaki'")
+        if precision not in ("fp64", "ozaki", "fp64_dmma"):
+            raise ValueError("EvolveFn: precision must be 'fp64', 'ozaki' or 'fp64_dmma'")
         n = int(g.numel())
         params = Params(n, [float(x) for x in g.detach().cpu()], float(omega_a), float(omega_c), coupling)
-        U = expm(build_hamiltonian(params, device=rho0.device), n, dt)
+        U = expm(build_hamiltonian(params, device=rho0.device), n, dt,
+                 precision="fp64_dmma" if precision == "fp64_dmma" else "fp64")
         rho, _ = evolve(U, rho0, n, steps, precision, params=params, observe=False)
         O = O_diag.contiguous()
         loss = expectation_diag(rho, n, O)
@@ -315,9 +337,8 @@ def batch_evolve(Us, rhos, steps: int, precision="bf16x3", renorm_every: int = 0
     obs = [torch.empty((steps + 1, obs_stride(n)), dtype=torch.float64, device=r.device) for n, r in zip(ns, rhos)] \
         if observe else None
     n_arr = (ctypes.c_int * count)(*ns)
-    need = int(_abi.load().tc_batch_workspace_size(count, n_arr, prec))
-    if work is None or work.numel() < need:
-        work = _work(need, rhos[0].device)
+    work = _workspace(work, int(_abi.load().tc_batch_workspace_size(count, n_arr, prec)),
+                      int(_abi.load().tc_batch_workspace_least(count, n_arr, prec)), rhos[0].device, halving=True)
     U_arr = (ctypes.c_void_p * count)(*[U.data_ptr() for U in Us])
     R_arr = (ctypes.c_void_p * count)(*[r.data_ptr() for r in outs])
     O_arr = (ctypes.c_void_p * count)(*[o.data_ptr() for o in obs]) if observe else None
@@ -336,7 +357,7 @@ def batch_evolve(Us, rhos, steps: int, precision="bf16x3", renorm_every: int = 0
 def autotune(n: int, precision="bf16x3", stream=None, work: Optional[torch.Tensor] = None):
     """tc_autotune: time the built kernel configurations for (n, precision); returns the choice."""
     prec = PRECISIONS[precision] if isinstance(precision, str) else int(precision)
-    need = workspace_size(n, prec, TC_OP_EVOLVE)
+    need = workspace_least(n, prec, TC_OP_EVOLVE)
     if work is None or work.numel() < need:
         work = _work(need, "cuda")
     out = (ctypes.c_int * 4)()
@@ -448,7 +469,7 @@ __all__ = ["Params", "TCError", "build_hamiltonian", "expm", "expm_model", "evol
            "lindblad_layout", "lindblad_propagators", "lindblad_evolve", "evolve_host", "observables",
            "expectation_diag",
            "evolve_backward", "EvolveFn", "batch_evolve", "autotune", "autotune_lookup", "autotune_set", "batch_autotune", "batch_autotune_set", "batch_autotune_lookup",
-           "workspace_size", "release_idle", "launch_count", "timing_enable", "timing_read", "phases_enable", "phases_read",
+           "workspace_size", "workspace_least", "release_idle", "launch_count", "timing_enable", "timing_read", "phases_enable", "phases_read",
            "device_check", "sync_status", "obs_stride", "PRECISIONS", "TC_FP64", "TC_BF16X3", "TC_TF32",
            "TC_TF32X3", "TC_COUPLING_BOSONIC", "TC_COUPLING_QUBIT_PHOTON", "TC_OP_EXPM", "TC_OP_EVOLVE",
            "TC_OP_OBSERVABLES", "TC_OP_BACKWARD"]

@@ -18,7 +18,7 @@ TC_OK = 0
 STATUS_NAMES = {0: "TC_OK", 1: "TC_ERR_INVALID_ARG", 2: "TC_ERR_UNSUPPORTED_DEVICE", 3: "TC_ERR_WORKSPACE",
                 4: "TC_ERR_CUDA", 5: "TC_ERR_TIMEOUT", 6: "TC_ERR_NUMERIC"}
 
-TC_FP64, TC_BF16X3, TC_TF32, TC_TF32X3, TC_FP64_OZAKI = 0, 1, 2, 3, 4
+TC_FP64, TC_BF16X3, TC_TF32, TC_TF32X3, TC_FP64_OZAKI, TC_FP64_DMMA = 0, 1, 2, 3, 4, 5
 TC_COUPLING_BOSONIC, TC_COUPLING_QUBIT_PHOTON = 0, 1
 TC_OP_EXPM, TC_OP_EVOLVE, TC_OP_OBSERVABLES, TC_OP_BACKWARD, TC_OP_EVOLVE_HOST, TC_OP_EXPM_MODEL = 1, 2, 4, 8, 16, 32
 TC_OP_LINDBLAD = 64
@@ -52,6 +52,7 @@ SIGNATURES = {
     "tc_last_error": (ctypes.c_char_p, []),
     "tc_device_check": (I, []),
     "tc_workspace_size": (SZ, [I, I, I, I, I]),
+    "tc_workspace_least": (SZ, [I, I, I, I, I]),
     "tc_build_hamiltonian": (I, [ctypes.POINTER(tc_params), VP, VP]),
     "tc_expm": (I, [VP, I, D, ctypes.POINTER(tc_expm_opts), VP, VP, SZ, VP]),
     "tc_expm_model": (I, [ctypes.POINTER(tc_params), D, ctypes.POINTER(tc_expm_opts), VP, VP, SZ, VP]),
@@ -71,6 +72,7 @@ SIGNATURES = {
     "tc_batch_autotune_set": (I, [I, ctypes.POINTER(I), I, ctypes.POINTER(I)]),
     "tc_batch_autotune_lookup": (I, [I, ctypes.POINTER(I), I, ctypes.POINTER(I), ctypes.POINTER(I)]),
     "tc_batch_workspace_size": (SZ, [I, ctypes.POINTER(I), I]),
+    "tc_batch_workspace_least": (SZ, [I, ctypes.POINTER(I), I]),
     "tc_batch_evolve": (I, [I, ctypes.POINTER(I), ctypes.POINTER(VP), ctypes.POINTER(VP), I, I, I,
                             ctypes.POINTER(tc_params), ctypes.POINTER(VP), VP, SZ, VP]),
     "tc_release_idle": (I, []),

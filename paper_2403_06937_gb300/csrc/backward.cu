@@ -236,9 +236,9 @@ struct OzBufs {
     int group;
 };
 
-size_t oz_backward_extra(int n) {
+size_t oz_backward_extra(int n, bool lazy) {
     const size_t N = (size_t)1 << n;
-    return 3 * oz_mat_bytes((int)N, true) + oz_mat_bytes((int)N, false) + oz_scratch_bytes((int)N) +
+    return 3 * oz_mat_bytes((int)N, true, lazy) + oz_mat_bytes((int)N, false, lazy) + oz_scratch_bytes((int)N, lazy) +
            2 * round256(N * N * sizeof(double)) + 256;
 }
 
@@ -326,6 +326,7 @@ __global__ void term_kernel(double inv, CM Fn, CM Tn, CM F, CM T, CM D, CM X, si
 // operands' 77 GB would come on top of 220 GB of checkpoints).
 bool backward_f64_on_tensor_cores(int n) { return f64_on_tensor_cores(n) && n <= 13; }
 
+// TC_FP64 on the DMMA, TC_FP64_OZAKI with lazy operands.
 size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
     if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
     const int nck = (steps + ckpt_every - 1) / ckpt_every;
@@ -333,7 +334,7 @@ size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
     // U, Lambda, X, W, seg0 + checkpoints + segment + Frechet (T, F, Tn, Fn, P, Q) + B + small
     const size_t b = (size_t)(5 + nck + c + 6) * cm_bytes(n) + real_bytes(n) +
                      round256((2 * ((size_t)1 << n) + 64) * 8) + 1024;
-    return precision == TC_FP64_OZAKI ? b + oz_backward_extra(n) : b;
+    return precision == TC_FP64_OZAKI ? b + oz_backward_extra(n, true) : b;
 }
 
 }  // namespace
@@ -341,13 +342,16 @@ size_t backward_least_bytes(int n, int steps, int ckpt_every, int precision) {
 namespace {
 // with the tensor-core products
 size_t backward_tensor_bytes(int n, int steps, int ckpt_every) {
-    return backward_least_bytes(n, steps, ckpt_every, TC_FP64_OZAKI);
+    const size_t b = backward_least_bytes(n, steps, ckpt_every, TC_FP64);
+    return b ? b + oz_backward_extra(n, false) : 0;
 }
 }  // namespace
 
-size_t backward_bytes(int n, int steps, int ckpt_every, int precision) {
+size_t backward_bytes(int n, int steps, int ckpt_every, int precision, bool least) {
     if (n < 1 || n > kMaxAtoms || steps < 1 || ckpt_every < 1) return 0;
-    if (precision == TC_FP64 && !backward_f64_on_tensor_cores(n)) return backward_least_bytes(n, steps, ckpt_every, TC_FP64);
+    if (least) return backward_least_bytes(n, steps, ckpt_every, precision);
+    if (precision != TC_FP64_OZAKI && !(precision == TC_FP64 && backward_f64_on_tensor_cores(n)))
+        return backward_least_bytes(n, steps, ckpt_every, TC_FP64);
     return backward_tensor_bytes(n, steps, ckpt_every);
 }
 
@@ -365,8 +369,10 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     if (!(dt > 0.0) || !std::isfinite(dt)) return fail(TC_ERR_INVALID_ARG, "dt must be finite and > 0");
     if (steps < 1) return fail(TC_ERR_INVALID_ARG, "steps must be >= 1");
     if (ckpt_every < 1) return fail(TC_ERR_INVALID_ARG, "ckpt_every must be >= 1");
+    const bool dmma = precision == TC_FP64_DMMA;   // TC_FP64 without the residue products
+    if (dmma) precision = TC_FP64;
     if (precision != TC_FP64 && precision != TC_FP64_OZAKI)
-        return fail(TC_ERR_INVALID_ARG, "backward: precision must be TC_FP64 or TC_FP64_OZAKI");
+        return fail(TC_ERR_INVALID_ARG, "backward: precision must be TC_FP64, TC_FP64_DMMA or TC_FP64_OZAKI");
     if (precision == TC_FP64_OZAKI && n < 7)
         return fail(TC_ERR_INVALID_ARG, "backward: the emulated form needs n >= 7 (dimension a multiple of 128)");
     if (!rho0 || !U || !O_diag || !grad) return fail(TC_ERR_INVALID_ARG, "null pointer");
@@ -404,16 +410,17 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     b.B = ar.take<double>(NN);
     b.small = ar.take<double>(2 * (size_t)N + 64);
     if (!b.small) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
-    const bool oz = precision == TC_FP64_OZAKI || (backward_f64_on_tensor_cores(n) &&
+    const bool oz = precision == TC_FP64_OZAKI || (!dmma && backward_f64_on_tensor_cores(n) &&
                                                    work_bytes >= backward_tensor_bytes(n, steps, ckpt_every));
     OzBufs z{};
     if (oz) {
-        TC_TRY(oz_mat_init(z.U, ar, N, true));
-        TC_TRY(oz_mat_init(z.Uc, ar, N, true));
-        TC_TRY(oz_mat_init(z.B, ar, N, false));
-        TC_TRY(oz_mat_init(z.A2, ar, N, true));
+        const bool lazy = work_bytes < backward_tensor_bytes(n, steps, ckpt_every);
+        TC_TRY(oz_mat_init(z.U, ar, N, true, lazy));
+        TC_TRY(oz_mat_init(z.Uc, ar, N, true, lazy));
+        TC_TRY(oz_mat_init(z.B, ar, N, false, lazy));
+        TC_TRY(oz_mat_init(z.A2, ar, N, true, lazy));
         z.Y = take_cm(ar, NN);
-        z.scratch = ar.take<uint8_t>(oz_scratch_bytes(N));
+        z.scratch = ar.take<uint8_t>(oz_scratch_bytes(N, lazy));
         if (!z.scratch) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
         z.group = tune_lookup(n, TC_BF16X3).tc_group;
         TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));

@@ -47,10 +47,10 @@ std::vector<std::vector<int>> assign_lanes(int count, const int* n, int lanes) {
 }
 
 // Workspace of one system's whole run in the FP64 forms: on the tensor cores, or
-// (dmma) TC_FP64 on the DMMA GEMM.
-size_t lane_system_bytes(int n, int precision, bool dmma) {
-    const bool tensor = precision == TC_FP64_OZAKI || (!dmma && f64_on_tensor_cores(n));
-    return round256(tensor ? evolve_oz_bytes(n) : evolve_f64_bytes(n));
+// (least) TC_FP64 on the DMMA GEMM, TC_FP64_OZAKI with lazy operands.
+size_t lane_system_bytes(int n, int precision, bool least) {
+    if (precision == TC_FP64_OZAKI) return round256(evolve_oz_bytes(n, least));
+    return round256(precision == TC_FP64 && !least && f64_on_tensor_cores(n) ? evolve_oz_bytes(n) : evolve_f64_bytes(n));
 }
 
 // A batch in the FP64 forms: its lanes and their buffers.  A lane runs its
@@ -60,32 +60,30 @@ struct Lanes {
     std::vector<std::vector<int>> lane;
     std::vector<size_t> bytes;
     size_t total = 0;
-    bool dmma = false;
+    bool least = false;
 };
-Lanes make_lanes(int count, const int* n, int precision, int lanes, bool dmma) {
+Lanes make_lanes(int count, const int* n, int precision, int lanes, bool least) {
     Lanes p;
-    p.dmma = dmma;
+    p.least = least;
     p.lane = assign_lanes(count, n, lanes);
     p.total = 256;
     for (const auto& lane : p.lane) {
         size_t most = 0;
-        for (int b : lane) most = std::max(most, lane_system_bytes(n[b], precision, dmma));
+        for (int b : lane) most = std::max(most, lane_system_bytes(n[b], precision, least));
         p.bytes.push_back(most);
         p.total += most;
     }
     return p;
 }
-// The most lanes that fit: every system on the tensor cores if that can be had
-// with one lane, else (TC_FP64) on the DMMA.  total > have when nothing fits.
+// The most lanes that fit: of the usual form if one lane of it fits, else of the
+// one that needs least.  total > have when nothing fits.
 Lanes fit_lanes(int count, const int* n, int precision, size_t have) {
-    for (const bool dmma : {false, true}) {
-        if (dmma && precision != TC_FP64) break;
+    for (const bool least : {false, true})
         for (int l = std::min(count, kOzLanes); l >= 1; l--) {
-            Lanes p = make_lanes(count, n, precision, l, dmma);
+            Lanes p = make_lanes(count, n, precision, l, least);
             if (p.total <= have) return p;
         }
-    }
-    return make_lanes(count, n, precision, 1, precision == TC_FP64);
+    return make_lanes(count, n, precision, 1, true);
 }
 size_t lanes_bytes(int count, const int* n, int precision) {
     for (int l = std::min(count, kOzLanes); l > 1; l--) {
@@ -95,7 +93,7 @@ size_t lanes_bytes(int count, const int* n, int precision) {
     return make_lanes(count, n, precision, 1, false).total;
 }
 size_t least_lanes_bytes(int count, const int* n, int precision) {
-    return make_lanes(count, n, precision, 1, precision == TC_FP64).total;
+    return make_lanes(count, n, precision, 1, true).total;
 }
 
 // The FP64 forms: every system's run is one sequence on one of up to kOzLanes
@@ -109,7 +107,7 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
     const Lanes plan = fit_lanes(count, n, precision, work_bytes);
     const auto& lane = plan.lane;
     const auto& bytes = plan.bytes;
-    const bool dmma = plan.dmma;
+    const bool dmma = precision == TC_FP64_DMMA || (precision == TC_FP64 && plan.least);
     const int L = (int)lane.size();
     Arena all{static_cast<char*>(work), work_bytes, 0};
     std::vector<char*> base(L);
@@ -154,12 +152,16 @@ tc_status batch_lanes(int count, const int* n, const void* const* U, void* const
     return run_captured(us, first, run, none, steps >= 1 && !timing_enabled());
 }
 
+bool lanes_form(int precision) {
+    return precision == TC_FP64 || precision == TC_FP64_OZAKI || precision == TC_FP64_DMMA;
+}
+
 }  // namespace
 
 size_t batch_bytes(int count, const int* n, int precision) {
     for (int b = 0; b < count; b++)
         if (n[b] < 1 || n[b] > kMaxAtoms) return 0;
-    if (precision == TC_FP64_OZAKI || precision == TC_FP64) return lanes_bytes(count, n, precision);
+    if (lanes_form(precision)) return lanes_bytes(count, n, precision);
     size_t total = 256 + round256(sizeof(BatchSys) * (size_t)count) + 64;
     for (int b = 0; b < count; b++) total += lowp_system_bytes(n[b], precision) + 512;
     return total;
@@ -169,12 +171,24 @@ size_t batch_bytes(int count, const int* n, int precision) {
 
 using namespace tc;
 
+static size_t least_bytes(int count, const int* n, int precision) {
+    for (int b = 0; b < count; b++)
+        if (n[b] < 1 || n[b] > kMaxAtoms) return 0;
+    return lanes_form(precision) ? least_lanes_bytes(count, n, precision) : batch_bytes(count, n, precision);
+}
+
 extern "C" {
 
 TC_API size_t tc_batch_workspace_size(int count, const int* n, int precision) {
     if (count < 1 || !n) return 0;
-    if (precision < TC_FP64 || precision > TC_FP64_OZAKI) return 0;
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA) return 0;
     return batch_bytes(count, n, precision);
+}
+
+TC_API size_t tc_batch_workspace_least(int count, const int* n, int precision) {
+    if (count < 1 || !n) return 0;
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA) return 0;
+    return least_bytes(count, n, precision);
 }
 
 TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, void* const* rho, int steps,
@@ -182,7 +196,7 @@ TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, 
                                  void* work, size_t work_bytes, void* stream) {
     if (count < 1 || !n || !U || !rho) return fail(TC_ERR_INVALID_ARG, "count, n, U or rho missing");
     if (steps < 0 || renorm_every < 0) return fail(TC_ERR_INVALID_ARG, "steps / renorm_every < 0");
-    if (precision < TC_FP64 || precision > TC_FP64_OZAKI)
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA)
         return fail(TC_ERR_INVALID_ARG, "unknown precision %d", precision);
     std::vector<Model> models(count);
     for (int b = 0; b < count; b++) {
@@ -195,14 +209,13 @@ TC_API tc_status tc_batch_evolve(int count, const int* n, const void* const* U, 
             if (models[b].n != n[b]) return fail(TC_ERR_INVALID_ARG, "system %d: params.n != n", b);
         }
     }
-    const size_t need = precision == TC_FP64 || precision == TC_FP64_OZAKI ? least_lanes_bytes(count, n, precision)
-                                                                             : batch_bytes(count, n, precision);
+    const size_t need = least_bytes(count, n, precision);
     if (!work) return fail(TC_ERR_WORKSPACE, "work is NULL (need %zu bytes)", need);
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(TC_ERR_WORKSPACE, "work is not 256-byte aligned");
     if (work_bytes < need) return fail(TC_ERR_WORKSPACE, "work has %zu bytes, need %zu", work_bytes, need);
     TC_TRY(check_device());
     cudaStream_t us = as_stream(stream);
-    if (precision == TC_FP64_OZAKI || precision == TC_FP64)
+    if (lanes_form(precision))
         return batch_lanes(count, n, U, rho, steps, precision, renorm_every, params ? models.data() : nullptr, obs,
                            work, work_bytes, us);
 

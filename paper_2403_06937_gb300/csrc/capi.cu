@@ -105,14 +105,16 @@ size_t expm_tensor_bytes(int n) {
 size_t wanted_expm_bytes(int n) { return expm_bytes(n) + (expm_on_tensor_cores(n) ? expm_tensor_bytes(n) : 0); }
 
 // The least a call needs.  TC_FP64 runs its DMMA form in this much and the
-// tensor-core form in what tc_workspace_size states (wanted_evolve_bytes).
+// tensor-core form in what tc_workspace_size states (wanted_evolve_bytes);
+// TC_FP64_OZAKI makes its operands' planes a few moduli at a time.
 size_t evolve_bytes(int n, int precision) {
-    if (precision == TC_FP64_OZAKI) return evolve_oz_bytes(n);
+    if (precision == TC_FP64_OZAKI) return evolve_oz_bytes(n, true);
     return precision == TC_FP64 ? evolve_f64_bytes(n) : evolve_lowp_bytes(n, precision);
 }
 
 size_t wanted_evolve_bytes(int n, int precision) {
     const size_t least = evolve_bytes(n, precision);
+    if (precision == TC_FP64_OZAKI) return evolve_oz_bytes(n);
     if (precision != TC_FP64 || !f64_on_tensor_cores(n)) return least;
     return least > evolve_oz_bytes(n) ? least : evolve_oz_bytes(n);
 }
@@ -398,19 +400,32 @@ TC_API int tc_release_idle(void) { return StreamSet::release_idle(); }
 
 TC_API tc_status tc_device_check(void) { return check_device(); }
 
-TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ckpt_every) {
+static size_t workspace_bytes(int n, int precision, int ops, int steps, int ckpt_every, bool least) {
     if (n < 1 || n > kMaxAtoms) return 0;
+    if (precision == TC_FP64_DMMA) {
+        precision = TC_FP64;
+        least = true;
+    }
     size_t need = 0;
     auto upd = [&](size_t b) { if (b > need) need = b; };
-    if (ops & TC_OP_EXPM) upd(wanted_expm_bytes(n));
-    if (ops & TC_OP_EVOLVE) upd(wanted_evolve_bytes(n, precision));
+    auto evolve = [&]() { return least ? evolve_bytes(n, precision) : wanted_evolve_bytes(n, precision); };
+    if (ops & TC_OP_EXPM) upd(least ? expm_bytes(n) : wanted_expm_bytes(n));
+    if (ops & TC_OP_EVOLVE) upd(evolve());
     if (ops & TC_OP_OBSERVABLES) upd(observables_scratch_bytes(n));
     if (ops & TC_OP_EXPM_MODEL) upd(expm_model_bytes(n));
-    if (ops & TC_OP_LINDBLAD) upd(lindblad_bytes(n, precision));
-    if (ops & TC_OP_EVOLVE_HOST) upd(wanted_evolve_bytes(n, precision) + evolve_host_extra(n, steps));
-    if (ops & TC_OP_EVOLVE_HOST_PINNED) upd(wanted_evolve_bytes(n, precision) + evolve_host_pinned_extra(n, steps, precision));
-    if (ops & TC_OP_BACKWARD) upd(backward_bytes(n, steps, ckpt_every, precision));
+    if (ops & TC_OP_LINDBLAD) upd(lindblad_bytes(n, precision, least));
+    if (ops & TC_OP_EVOLVE_HOST) upd(evolve() + evolve_host_extra(n, steps));
+    if (ops & TC_OP_EVOLVE_HOST_PINNED) upd(evolve() + evolve_host_pinned_extra(n, steps, precision));
+    if (ops & TC_OP_BACKWARD) upd(backward_bytes(n, steps, ckpt_every, precision, least));
     return need;
+}
+
+TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ckpt_every) {
+    return workspace_bytes(n, precision, ops, steps, ckpt_every, false);
+}
+
+TC_API size_t tc_workspace_least(int n, int precision, int ops, int steps, int ckpt_every) {
+    return workspace_bytes(n, precision, ops, steps, ckpt_every, true);
 }
 
 TC_API tc_status tc_build_hamiltonian(const tc_params* params, double* H, void* stream) {
@@ -464,8 +479,10 @@ TC_API tc_status tc_evolve(const void* U, void* rho, int n, int steps, int preci
     if (obs && (reinterpret_cast<uintptr_t>(obs) & 7u)) return fail(TC_ERR_INVALID_ARG, "obs must be 8-byte aligned");
     if (steps < 0) return fail(TC_ERR_INVALID_ARG, "steps < 0");
     if (renorm_every < 0) return fail(TC_ERR_INVALID_ARG, "renorm_every < 0");
-    if (precision < TC_FP64 || precision > TC_FP64_OZAKI)
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA)
         return fail(TC_ERR_INVALID_ARG, "unknown precision %d", precision);
+    const bool dmma = precision == TC_FP64_DMMA;   // TC_FP64 without the residue products
+    if (dmma) precision = TC_FP64;
     Model m;
     const Model* mp = nullptr;
     if (params) {
@@ -480,7 +497,7 @@ TC_API tc_status tc_evolve(const void* U, void* rho, int n, int steps, int preci
     if (precision == TC_FP64_OZAKI)
         return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision, renorm_every, mp,
                          obs, ar, s);
-    if (precision == TC_FP64 && f64_on_tensor_cores(n) && ar.size >= evolve_oz_bytes(n))
+    if (precision == TC_FP64 && !dmma && f64_on_tensor_cores(n) && ar.size >= evolve_oz_bytes(n))
         return evolve_oz(static_cast<const double*>(U), static_cast<double*>(rho), n, steps, precision, renorm_every, mp,
                          obs, ar, s);
     if (precision != TC_FP64)
@@ -497,8 +514,10 @@ TC_API tc_status tc_evolve_host(const void* U, void* rho_host, int n, int steps,
     if (!U || !rho_host) return fail(TC_ERR_INVALID_ARG, "U or rho_host is NULL");
     if (reinterpret_cast<uintptr_t>(U) & 15u) return fail(TC_ERR_INVALID_ARG, "U must be 16-byte aligned");
     if (steps < 0 || renorm_every < 0) return fail(TC_ERR_INVALID_ARG, "steps / renorm_every < 0");
-    if (precision < TC_FP64 || precision > TC_FP64_OZAKI)
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA)
         return fail(TC_ERR_INVALID_ARG, "unknown precision %d", precision);
+    const bool dmma = precision == TC_FP64_DMMA;   // TC_FP64 without the residue products
+    if (dmma) precision = TC_FP64;
     Model m;
     const Model* mp = nullptr;
     if (params) {
@@ -529,7 +548,7 @@ TC_API tc_status tc_evolve_host(const void* U, void* rho_host, int n, int steps,
             TC_TRY(copy_by_sms(rho_dev, mapped, 16 * N * N, s));
         else
             TC_CUDA(cudaMemcpyAsync(rho_dev, rho_host, 16 * N * N, cudaMemcpyHostToDevice, s));
-        if (precision == TC_FP64_OZAKI || (f64_on_tensor_cores(n) && ar.size - ar.used >= evolve_oz_bytes(n)))
+        if (precision == TC_FP64_OZAKI || (!dmma && f64_on_tensor_cores(n) && ar.size - ar.used >= evolve_oz_bytes(n)))
             TC_TRY(evolve_oz(Ud, rho_dev, n, steps, precision, renorm_every, mp, od, ar, s));
         else
             TC_TRY(evolve_f64(Ud, rho_dev, n, steps, renorm_every, mp, od, ar, s));

@@ -53,6 +53,12 @@
 // columns 128 (w / 4) .. + 127 of the tile), warp 8 TMA, warp 9 MMA.  Barriers
 // and bounded waits of the CTA pairs as cgemm_oz_pair_kernel (cgemm_oz.cu).
 //
+// A workspace too small for whole operands: an operand then keeps its source
+// instead of planes (lazy), and a product makes the planes of four moduli at a
+// time, multiplies those, and goes on to the next four; the same bits, 96 N^2
+// bytes of workspace a run instead of 192 (n = 14: 26 GB instead of 52), eight
+// residue passes a product instead of one.
+//
 // crt_combine_kernel turns the bytes of an entry into FP64 (integer work up to
 // the diagonal term's multiply-adds).
 #include <cuda_bf16.h>
@@ -95,6 +101,7 @@ struct CrtLaunch {
     int lo, hi;          // rows of 256-tiles: the band [lo, hi)
     int units_per;       // units per plane
     int units;           // units_per * planes
+    int first, moduli;   // the operands' planes are those of the moduli [first, first + moduli), each pair's in turn
     size_t Np;           // row stride of the byte planes
     size_t band;         // rows of a byte plane
     uint8_t* bytes;      // [planes][band][Np], rows from 256 lo on
@@ -407,10 +414,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = worker; u < L.units && !stop; u += workers) {
             int z, P, J;
             unit_at<MODE>(L, u, z, P, J);
-            const float p = (float)kC.p[z % kModuli], inv_p = 1.0f / p;
+            const int s = L.first + z % L.moduli;
+            const float p = (float)kC.p[s], inv_p = 1.0f / p;
             // rows and columns past the end (an odd number of 128-tiles) are not written
             const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
-            uint8_t* y = L.bytes + ((size_t)z * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
+            uint8_t* y = L.bytes + ((size_t)(z / L.moduli * kModuli + s) * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
                          (size_t)(256 * J + 128 * half);
             if (chunks == 1) {
                 const uint32_t buf = pass & 1u;
@@ -478,6 +486,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 // entry; the second read of the row comes from L2); no FP64 instruction, since
 // one FP64 conversion per entry alone would take as long as a third of the
 // writes on this GPU.
+constexpr int kGroupModuli = 4;      // moduli at a time of an operand without planes of its own
 constexpr int kShiftBias = 4096;     // added to shifted exponents, so that 0 still means an empty row
 constexpr int kNotFinite = 1 << 16;
 constexpr int kEmptyColumn = INT32_MIN;   // column scale of a zero column
@@ -543,11 +552,12 @@ __device__ __forceinline__ uint32_t bf16_pair(uint64_t v) {
 }
 
 // SCALED: column k carries 2^col[k] (a left operand; a right one 2^-col[k]).
-template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false, bool SCALED = false>
+// GROUP: the planes of kGroupModuli moduli from `first` on only.
+template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false, bool SCALED = false, bool GROUP = false>
 __global__ void __launch_bounds__(128)
     crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
-                       int tpr, uint64_t im_flip, const int* __restrict__ col, __nv_bfloat16* __restrict__ planes,
-                       int* __restrict__ ex, double* __restrict__ diag) {
+                       int tpr, uint64_t im_flip, const int* __restrict__ col, int first,
+                       __nv_bfloat16* __restrict__ planes, int* __restrict__ ex, double* __restrict__ diag) {
     const int sub = threadIdx.x % tpr;                       // thread within the row
     const int r = blockIdx.x * (128 / tpr) + threadIdx.x / tpr;
     // CPT consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
@@ -678,6 +688,7 @@ __global__ void __launch_bounds__(128)
         __nv_bfloat16* dst = planes + (size_t)r * Np + c0;
 #pragma unroll
         for (int s = 0; s < kModuli; s++) {
+            if (GROUP && (s < first || s >= first + kGroupModuli)) continue;
             uint32_t w0[CPT / 2], w1[CPT / 2];
 #pragma unroll
             for (int h = 0; h < CPT / 2; h++) {
@@ -690,8 +701,9 @@ __global__ void __launch_bounds__(128)
                 w1[h] = bf16_pair(v);
             }
             // plane s: re + iota im of a left operand, its conjugate re - iota im of a right one
-            put(dst + (size_t)(REAL || LEFT ? s : kModuli + s) * plane, w0);
-            if (!REAL) put(dst + (size_t)(LEFT ? kModuli + s : s) * plane, w1);
+            const int at = GROUP ? s - first : s, second = GROUP ? kGroupModuli : kModuli;
+            put(dst + (size_t)(REAL || LEFT ? at : second + at) * plane, w0);
+            if (!REAL) put(dst + (size_t)(LEFT ? second + at : at) * plane, w1);
         }
     }
 }
@@ -1018,50 +1030,97 @@ int band_rows(int Np) { return Np <= 16384 ? Np : 4096; }
 
 size_t plane_bytes(int Np, int planes) { return round256((size_t)planes * Np * Np * 2); }
 
-tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes) {
+tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes, bool lazy = false) {
+    m = CrtMat{};
     m.Np = Np;
     m.left = left;
+    m.lazy = lazy;
     m.count = planes;
-    m.planes = ar.take<uint8_t>((size_t)planes * Np * Np * 2);
+    if (!lazy) m.planes = ar.take<uint8_t>((size_t)planes * Np * Np * 2);
     m.ex = ar.take<int>((size_t)Np);
     m.diag = left ? ar.take<double>((size_t)2 * Np) : nullptr;
-    if (!m.planes || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
-    return make_part_map_rows(&m.map, m.planes, Np, planes, TC_BF16X3, kRB);
+    if ((!lazy && !m.planes) || !m.ex || (left && !m.diag)) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");
+    return lazy ? TC_OK : make_part_map_rows(&m.map, m.planes, Np, planes, TC_BF16X3, kRB);
 }
 
-// The residue products of one band of rows (all of them: lo = 0, hi = side).
-tc_status gemm(int mode, const CrtMat& A, const CrtMat& B, int lo, int hi, void* scratch, cudaStream_t s) {
+// The residue products of one band of rows (all of them: lo = 0, hi = side);
+// `planes` planes of each operand, of the moduli from `first` on.
+tc_status gemm(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, int Np, int planes, int first, int moduli,
+               int lo, int hi, void* scratch, cudaStream_t s) {
     CrtLaunch L{};
-    L.tiles = A.Np / 128;
+    L.tiles = Np / 128;
     const int side = (L.tiles + 1) / 2;
-    L.kb_total = A.Np / kKPer;
+    L.kb_total = Np / kKPer;
+    L.first = first;
+    L.moduli = moduli;
     L.lo = lo;
     L.hi = hi;
-    L.Np = (size_t)A.Np;
-    L.band = hi == side ? (size_t)A.Np - 256 * (size_t)lo : 256 * (size_t)(hi - lo);
+    L.Np = (size_t)Np;
+    L.band = hi == side ? (size_t)Np - 256 * (size_t)lo : 256 * (size_t)(hi - lo);
     L.bytes = static_cast<uint8_t*>(scratch);
     L.status = device_status_word();
     L.units_per = mode == 0 ? side * (hi - lo) : hi * (hi + 1) / 2 - lo * (lo + 1) / 2;
-    L.units = L.units_per * A.count;
-    return mode == 0 ? launch<0>(A.map, B.map, L, s) : launch<1>(A.map, B.map, L, s);
+    L.units = L.units_per * planes;
+    return mode == 0 ? launch<0>(tmA, tmB, L, s) : launch<1>(tmA, tmB, L, s);
+}
+
+// Threads of the residue kernel: `cpt` columns a thread and step, `tpr` threads a
+// row (a power of two, at most 128 and Np / cpt).
+struct RowSplit {
+    int cpt, tpr;
+    unsigned grid;
+};
+RowSplit row_split(int Np) {
+    RowSplit w{Np <= 512 ? 2 : 4, 16, 0};
+    while (2 * w.tpr <= std::min(128, Np / w.cpt)) w.tpr *= 2;
+    w.grid = (unsigned)((Np + 128 / w.tpr - 1) / (128 / w.tpr));
+    return w;
+}
+
+size_t group_bytes(int Np) { return plane_bytes(Np, 2 * kGroupModuli); }
+
+// The planes of one group of moduli of an operand that has none of its own.
+tc_status load_group(const CrtMat& m, int first, void* planes, cudaStream_t s) {
+    const RowSplit w = row_split(m.Np);
+    const uint64_t flip = m.src.conj ? 1ull << 63 : 0;
+    auto* out = static_cast<__nv_bfloat16*>(planes);
+    const CrtSource& o = m.src;
+#define TC_RES(I_, L_, C_)                                                                                       \
+    crt_residue_kernel<I_, L_, C_, false, false, true><<<w.grid, 128, 0, s>>>(o.re, o.im, o.N, o.ld, m.Np, w.tpr, \
+                                                                              flip, nullptr, first, out, m.ex, m.diag)
+    if (o.interleaved && m.left) {
+        if (w.cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
+    } else if (o.interleaved) {
+        if (w.cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 4);
+    } else if (m.left) {
+        if (w.cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 4);
+    } else {
+        if (w.cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 4);
+    }
+#undef TC_RES
+    TC_LAUNCH_CHECK();
+    return TC_OK;
 }
 
 }  // namespace
 
-size_t crt_mat_bytes(int Np, bool left) {
-    return plane_bytes(Np, 2 * kModuli) + round256((size_t)Np * sizeof(int)) +
+size_t crt_mat_bytes(int Np, bool left, bool lazy) {
+    return (lazy ? 0 : plane_bytes(Np, 2 * kModuli)) + round256((size_t)Np * sizeof(int)) +
            (left ? round256((size_t)2 * Np * sizeof(double)) : 0);
 }
 
-size_t crt_scratch_bytes(int Np) { return round256((size_t)2 * kModuli * band_rows(Np) * Np); }
+static size_t bytes_scratch(int Np) { return round256((size_t)2 * kModuli * band_rows(Np) * Np); }
+size_t crt_scratch_bytes(int Np, bool lazy) { return bytes_scratch(Np) + (lazy ? 2 * group_bytes(Np) : 0); }
 
-tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left) { return mat_init(m, ar, Np, left, 2 * kModuli); }
+tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left, bool lazy) {
+    return mat_init(m, ar, Np, left, 2 * kModuli, lazy);
+}
 
 tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np) {
     if (Np > base.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand view larger than its buffers");
     view = base;
     view.Np = Np;
-    return make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
+    return base.lazy ? TC_OK : make_part_map_rows(&view.map, base.planes, Np, base.count, TC_BF16X3, kRB);
 }
 
 size_t crt_columns_bytes(int Np) { return round256((size_t)(Np + 1) * sizeof(unsigned)) + round256((size_t)Np * sizeof(int)); }
@@ -1091,29 +1150,31 @@ tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, b
     return TC_OK;
 }
 
-tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
+tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
                        size_t ld, cudaStream_t s, const int* col) {
     if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
         (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
-    const int cpt = m.Np <= 512 ? 2 : 4;
-    int tpr = 16;   // threads a row: a power of two, at most 128 and Np / cpt
-    while (2 * tpr <= std::min(128, m.Np / cpt)) tpr *= 2;
-    const unsigned grid = (unsigned)((m.Np + 128 / tpr - 1) / (128 / tpr));
+    if (m.lazy) {
+        if (col) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: column scales need an operand's own planes");
+        m.src = CrtSource{re, im, interleaved, conj, N, ld};
+        return TC_OK;
+    }
+    const RowSplit w = row_split(m.Np);
     const uint64_t flip = conj ? 1ull << 63 : 0;
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
 #define TC_RES(I_, L_, C_)                                                                                          \
-    col ? crt_residue_kernel<I_, L_, C_, false, true><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, col, out, \
-                                                                           m.ex, m.diag)                            \
-        : crt_residue_kernel<I_, L_, C_><<<grid, 128, 0, s>>>(re, im, N, ld, m.Np, tpr, flip, nullptr, out, m.ex, m.diag)
+    col ? crt_residue_kernel<I_, L_, C_, false, true><<<w.grid, 128, 0, s>>>(re, im, N, ld, m.Np, w.tpr, flip, col, 0,   \
+                                                                           out, m.ex, m.diag)                       \
+        : crt_residue_kernel<I_, L_, C_><<<w.grid, 128, 0, s>>>(re, im, N, ld, m.Np, w.tpr, flip, nullptr, 0, out, m.ex, m.diag)
     if (interleaved && m.left) {
-        if (cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
+        if (w.cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
     } else if (interleaved) {
-        if (cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 4);
+        if (w.cpt == 2) TC_RES(true, false, 2); else TC_RES(true, false, 4);
     } else if (m.left) {
-        if (cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 4);
+        if (w.cpt == 2) TC_RES(false, true, 2); else TC_RES(false, true, 4);
     } else {
-        if (cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 4);
+        if (w.cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 4);
     }
 #undef TC_RES
     TC_LAUNCH_CHECK();
@@ -1123,12 +1184,27 @@ tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
                       size_t ldb, const CrtOut& out, cudaStream_t s) {
     const int Np = A.Np;
-    if (B.Np != Np || !A.left || B.left || Np < 128 || Np % 128 != 0 || Np > 65536)
+    if (B.Np != Np || !A.left || B.left || Np < 128 || Np % 128 != 0 || Np > 65536 || A.lazy != B.lazy)
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes or roles");
     if (mode != 0 && mode != 1) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: mode");
     const int band = band_rows(Np);   // Np itself, or a divisor that is a multiple of 256 kGroup
+    CUtensorMap tmA = A.map, tmB = B.map;
+    uint8_t* const ga = static_cast<uint8_t*>(out.scratch) + bytes_scratch(Np);   // planes of a group (lazy)
+    uint8_t* const gb = ga + group_bytes(Np);
+    if (A.lazy) {
+        TC_TRY(make_part_map_rows(&tmA, ga, Np, 2 * kGroupModuli, TC_BF16X3, kRB));
+        TC_TRY(make_part_map_rows(&tmB, gb, Np, 2 * kGroupModuli, TC_BF16X3, kRB));
+    }
+    const int moduli = A.lazy ? kGroupModuli : kModuli;
     for (int row0 = 0; row0 < Np; row0 += band) {
-        TC_TRY(gemm(mode, A, B, row0 / 256, (row0 + band + 255) / 256, out.scratch, s));
+        for (int first = 0; first < kModuli; first += moduli) {
+            if (A.lazy) {
+                TC_TRY(load_group(A, first, ga, s));
+                TC_TRY(load_group(B, first, gb, s));
+            }
+            TC_TRY(gemm(mode, tmA, tmB, Np, 2 * moduli, first, moduli, row0 / 256, (row0 + band + 255) / 256,
+                        out.scratch, s));
+        }
         CrtCombine c{};
         c.bytes = static_cast<const uint8_t*>(out.scratch);
         c.Np = (size_t)Np;
@@ -1173,9 +1249,9 @@ tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
     const unsigned grid = (unsigned)(N / (128 / tpr));
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
     if (m.left)
-        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, out, m.ex, m.diag);
+        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, 0, out, m.ex, m.diag);
     else
-        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, out, m.ex, nullptr);
+        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, 0, out, m.ex, nullptr);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -1184,7 +1260,7 @@ tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, do
     const int N = A.Np;
     if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0 || N > 16384)
         return fail(TC_ERR_INVALID_ARG, "real products: operands of different sizes or roles");
-    TC_TRY(gemm(0, A, B, 0, N / 256, scratch, s));
+    TC_TRY(gemm(0, A.map, B.map, N, kModuli, 0, kModuli, 0, N / 256, scratch, s));
     CrtCombine p{};
     p.bytes = static_cast<const uint8_t*>(scratch);
     p.Np = (size_t)N;

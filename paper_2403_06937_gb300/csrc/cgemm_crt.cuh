@@ -11,7 +11,14 @@ namespace tc {
 // One operand: residue planes [Np][Np] in BF16 (2 x 16: re + iota im and
 // re - iota im, in that order for a left operand, the other way round for a
 // right one; a real operand has 16), the power-of-two scale of each row, and,
-// for a left operand, its diagonal.
+// for a left operand, its diagonal.  A lazy operand has no planes: products
+// read its source, which must stay as it is until they have run.
+struct CrtSource {
+    const double *re, *im;
+    bool interleaved, conj;
+    int N;
+    size_t ld;
+};
 struct CrtMat {
     void* planes;
     int* ex;          // row r holds round(x 2^ex[r])
@@ -20,16 +27,18 @@ struct CrtMat {
     int Np;
     int count;        // planes
     bool left;
+    bool lazy;
+    CrtSource src;    // lazy
 };
 
-size_t crt_mat_bytes(int Np, bool left);
-tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left);
+size_t crt_mat_bytes(int Np, bool left, bool lazy = false);
+tc_status crt_mat_init(CrtMat& m, Arena& ar, int Np, bool left, bool lazy = false);
 // `view`: the buffers of `base` seen as an operand of the smaller padded size Np
 tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np);
 // Residues of the N x N matrix (row stride ld; zero-padded to Np).  interleaved:
 // re points to complex128; conj negates the imaginary part.  col: column scales
 // of the pair of operands, the same for both (crt_columns), or none.
-tc_status crt_mat_load(const CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
+tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
                        size_t ld, cudaStream_t s, const int* col = nullptr);
 
 // Powers of two along K, taken from a state: see cgemm_crt.cu.  `top` is zero
@@ -45,8 +54,8 @@ tc_status crt_columns_clear(const CrtColumns& c, cudaStream_t s);
 tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, bool interleaved, int N, size_t ld,
                       cudaStream_t s);
 // Bytes of scratch of a product: one byte per residue of the result (of a band
-// of rows above Np = 16384).
-size_t crt_scratch_bytes(int Np);
+// of rows above Np = 16384); with lazy operands two groups of planes too.
+size_t crt_scratch_bytes(int Np, bool lazy = false);
 // Y = A B^H, FP64 planes of row stride Np.  mode 1: Y Hermitian, the
 // block-lower half computed and mirrored.  (br, bi): B's FP64 planes of row
 // stride ldb, valid for N rows and columns, for the diagonal term of A.

@@ -803,19 +803,19 @@ size_t oz_slice_bytes(int Np) {
     return round256((size_t)2 * kOzDigits.slices * Np * Np * sizeof(__nv_bfloat16));
 }
 
-size_t oz_mat_bytes(int Np, bool left) {
-    return oz_modular() ? crt_mat_bytes(Np, left) : oz_slice_bytes(Np) + round256((size_t)Np * sizeof(int));
+size_t oz_mat_bytes(int Np, bool left, bool lazy) {
+    return oz_modular() ? crt_mat_bytes(Np, left, lazy) : oz_slice_bytes(Np) + round256((size_t)Np * sizeof(int));
 }
 
 // residue form: the result's residue bytes; digit form: two int64 planes of the low levels
-size_t oz_scratch_bytes(int Np) {
-    return oz_modular() ? crt_scratch_bytes(Np) : 2 * round256((size_t)Np * Np * sizeof(long long));
+size_t oz_scratch_bytes(int Np, bool lazy) {
+    return oz_modular() ? crt_scratch_bytes(Np, lazy) : 2 * round256((size_t)Np * Np * sizeof(long long));
 }
 
-tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left) {
+tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left, bool lazy) {
     m.Np = Np;
     m.left = left;
-    if (oz_modular()) return crt_mat_init(m.crt, ar, Np, left);
+    if (oz_modular()) return crt_mat_init(m.crt, ar, Np, left, lazy);
     m.slices = ar.take<uint8_t>(oz_slice_bytes(Np));
     m.ex = ar.take<int>((size_t)Np);
     if (!m.ex) return fail(TC_ERR_WORKSPACE, "FP64 emulation: workspace too small");

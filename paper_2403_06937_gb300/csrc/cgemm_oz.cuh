@@ -83,9 +83,10 @@ struct OzOut {
     const void* b_c128 = nullptr;   // B interleaved (complex128, row stride ldb) instead of (br, bi)
     void* y_c128 = nullptr;         // mode 1: the result interleaved (row stride Np) instead of (yr, yi)
 };
-size_t oz_mat_bytes(int Np, bool left);
-size_t oz_scratch_bytes(int Np);
-tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left);
+// lazy: without planes of its own (residue form; see CrtMat), both operands of a product alike
+size_t oz_mat_bytes(int Np, bool left, bool lazy = false);
+size_t oz_scratch_bytes(int Np, bool lazy = false);
+tc_status oz_mat_init(OzMat& m, Arena& ar, int Np, bool left, bool lazy = false);
 // `view` = `base`'s buffers seen as an operand of the smaller padded size Np
 tc_status oz_mat_view(OzMat& view, const OzMat& base, int Np);
 // col: column scales (residue form only)

@@ -82,9 +82,9 @@ int padded_dim(int n) { return (1 << n) < 128 ? 128 : (1 << n); }
 
 }  // namespace
 
-size_t evolve_oz_bytes(int n) {
+size_t evolve_oz_bytes(int n, bool lazy) {
     const size_t Np = (size_t)padded_dim(n);
-    return oz_mat_bytes((int)Np, true) + oz_mat_bytes((int)Np, false) + oz_scratch_bytes((int)Np) +
+    return oz_mat_bytes((int)Np, true, lazy) + oz_mat_bytes((int)Np, false, lazy) + oz_scratch_bytes((int)Np, lazy) +
            4 * round256(Np * Np * sizeof(double)) + observables_scratch_bytes(n) + crt_columns_bytes((int)Np) + 512;
 }
 
@@ -94,13 +94,14 @@ tc_status OzSystem::carve(int n_, bool scaled_, Arena& ar) {
     N = 1 << n;
     Np = padded_dim(n);
     const size_t NN = (size_t)Np * Np;
-    TC_TRY(oz_mat_init(Us, ar, Np, true));
-    TC_TRY(oz_mat_init(Ps, ar, Np, false));
+    const bool lazy = !scaled && ar.size - ar.used < evolve_oz_bytes(n);
+    TC_TRY(oz_mat_init(Us, ar, Np, true, lazy));
+    TC_TRY(oz_mat_init(Ps, ar, Np, false, lazy));
     Rr = ar.take<double>(NN);
     Ri = ar.take<double>(NN);
     Xr = ar.take<double>(NN);
     Xi = ar.take<double>(NN);
-    prod = ar.take<uint8_t>(oz_scratch_bytes(Np));
+    prod = ar.take<uint8_t>(oz_scratch_bytes(Np, lazy));
     TC_TRY(crt_columns_init(cols, ar, Np));
     scratch = ar.take<double>(observables_scratch_bytes(n) / sizeof(double));
     if (!scratch) return fail(TC_ERR_WORKSPACE, "evolve: workspace too small");

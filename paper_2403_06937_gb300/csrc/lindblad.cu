@@ -704,20 +704,20 @@ __global__ void split_block_kernel(const double2* __restrict__ src, int d, int N
 // them costs about 1 % of a step).
 bool shared_left(int n) { return n >= 13; }
 
-size_t evolve_oz_bytes_blocks(int n) {
+size_t evolve_oz_bytes_blocks(int n, bool lazy = false) {
     const Layout& L = layout_of(n);
     const size_t PT = padded_total(L);
     const int NpMax = padded(L.N);
     size_t b = tables_bytes(n) + 2 * round256(PT * sizeof(double));
-    if (shared_left(n)) b += oz_mat_bytes(NpMax, true);
+    if (shared_left(n)) b += oz_mat_bytes(NpMax, true, lazy);
     for (int k = 0; k <= n; k++) {
         const size_t Np = (size_t)padded(L.dims[k]);
         if (L.dims[k] <= kSmallBlock)
             b += 2 * round256(Np * Np * sizeof(double));
         else if (!shared_left(n))
-            b += oz_mat_bytes((int)Np, true);
+            b += oz_mat_bytes((int)Np, true, lazy);
     }
-    b += oz_mat_bytes(NpMax, false) + oz_scratch_bytes(NpMax);   // B operand, scratch of the products
+    b += oz_mat_bytes(NpMax, false, lazy) + oz_scratch_bytes(NpMax, lazy);   // B operand, scratch of the products
     b += 2 * round256((size_t)NpMax * NpMax * sizeof(double));   // X planes
     b += crt_columns_bytes(NpMax);
     return b + obs_scratch_bytes(L) + 256;
@@ -731,6 +731,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
     const size_t PT = padded_total(L);
     const int NpMax = padded(L.N);
     const size_t NN = (size_t)NpMax * NpMax;
+    const bool lazy = !scaled && ar.size - ar.used < evolve_oz_bytes_blocks(n);
     Tables t{};
     TC_TRY(take_tables(L, ar, &t));
     double* Rr = ar.take<double>(PT);
@@ -738,7 +739,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
     std::vector<OzMat> Uk(n + 1);
     std::vector<double*> Ur(n + 1, nullptr), Ui(n + 1, nullptr);   // planes of the small blocks
     OzMat Amax{};
-    if (shared_left(n)) TC_TRY(oz_mat_init(Amax, ar, NpMax, true));
+    if (shared_left(n)) TC_TRY(oz_mat_init(Amax, ar, NpMax, true, lazy));
     for (int k = 0; k <= n; k++) {
         const int Np = padded(L.dims[k]);
         if (L.dims[k] <= kSmallBlock) {
@@ -747,14 +748,14 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
         } else if (shared_left(n)) {
             TC_TRY(oz_mat_view(Uk[k], Amax, Np));
         } else {
-            TC_TRY(oz_mat_init(Uk[k], ar, Np, true));
+            TC_TRY(oz_mat_init(Uk[k], ar, Np, true, lazy));
         }
     }
     OzMat Bmax{};
-    TC_TRY(oz_mat_init(Bmax, ar, NpMax, false));
+    TC_TRY(oz_mat_init(Bmax, ar, NpMax, false, lazy));
     double* Xr = ar.take<double>(NN);
     double* Xi = ar.take<double>(NN);
-    void* prod = ar.take<uint8_t>(oz_scratch_bytes(NpMax));
+    void* prod = ar.take<uint8_t>(oz_scratch_bytes(NpMax, lazy));
     CrtColumns cols{};
     TC_TRY(crt_columns_init(cols, ar, NpMax));
     const int* col = scaled ? cols.col : nullptr;
@@ -850,9 +851,9 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
     return run_captured(s, first, rest, tail, steps > 2 && !timing_enabled());
 }
 
-// The least a call needs; TC_FP64 runs on the DMMA in this much.
+// The least a call needs; TC_FP64 runs on the DMMA in this much, TC_FP64_OZAKI with lazy operands.
 size_t evolve_bytes(int n, int precision) {
-    if (precision == TC_FP64_OZAKI) return evolve_oz_bytes_blocks(n);
+    if (precision == TC_FP64_OZAKI) return evolve_oz_bytes_blocks(n, true);
     return precision == TC_FP64 ? evolve_f64_bytes(n) : evolve_lowp_bytes_blocks(n, precision);
 }
 
@@ -863,10 +864,11 @@ bool blocks_f64_on_tensor_cores(int n) { return f64_on_tensor_cores(n) && n <= 1
 
 }  // namespace
 
-size_t lindblad_bytes(int n, int precision) {
+size_t lindblad_bytes(int n, int precision, bool least) {
     if (precision < TC_FP64 || precision > TC_FP64_OZAKI) return 0;
     size_t b = std::max(propagators_bytes(n), evolve_bytes(n, precision));
-    if (precision == TC_FP64 && blocks_f64_on_tensor_cores(n)) b = std::max(b, evolve_oz_bytes_blocks(n));
+    if (least) return b;
+    if (precision == TC_FP64_OZAKI || (precision == TC_FP64 && blocks_f64_on_tensor_cores(n))) b = std::max(b, evolve_oz_bytes_blocks(n));
     return b;
 }
 
@@ -923,15 +925,17 @@ extern "C" TC_API tc_status tc_lindblad_evolve(const tc_params* params, double k
     if (!(kappa >= 0.0) || !std::isfinite(kappa)) return fail(TC_ERR_INVALID_ARG, "kappa must be finite and >= 0");
     if (!(dt > 0.0) || !std::isfinite(dt)) return fail(TC_ERR_INVALID_ARG, "dt must be finite and > 0");
     if (steps < 0 || renorm_every < 0) return fail(TC_ERR_INVALID_ARG, "steps / renorm_every < 0");
-    if (precision < TC_FP64 || precision > TC_FP64_OZAKI)
+    if (precision < TC_FP64 || precision > TC_FP64_DMMA)
         return fail(TC_ERR_INVALID_ARG, "unknown precision %d", precision);
+    const bool dmma = precision == TC_FP64_DMMA;   // TC_FP64 without the residue products
+    if (dmma) precision = TC_FP64;
     TC_TRY(check_work(work, work_bytes, evolve_bytes(m.n, precision)));
     TC_TRY(check_device());
     const Layout& L = layout_of(m.n);
     Arena ar{static_cast<char*>(work), work_bytes, 0};
     const double* Ud = static_cast<const double*>(U);
     double* Rd = static_cast<double*>(rho);
-    if (precision == TC_FP64 && !(blocks_f64_on_tensor_cores(m.n) && work_bytes >= evolve_oz_bytes_blocks(m.n)))
+    if (precision == TC_FP64 && (dmma || !(blocks_f64_on_tensor_cores(m.n) && work_bytes >= evolve_oz_bytes_blocks(m.n))))
         return evolve_f64(L, m, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));
     if (precision == TC_FP64 || precision == TC_FP64_OZAKI)
         return evolve_oz_blocks(L, m, precision, kappa, dt, Ud, Rd, steps, renorm_every, obs, ar, as_stream(stream));

@@ -35,7 +35,7 @@ tc_status evolve_f64(const double* U, double* rho, int n, int steps, int renorm_
                      double* obs, Arena& ar, cudaStream_t s);
 
 // FP64-accurate step loop on the BF16 tensor cores (exact integer products).
-size_t evolve_oz_bytes(int n);
+size_t evolve_oz_bytes(int n, bool lazy = false);   // lazy: TC_FP64_OZAKI in the least workspace (CrtMat)
 tc_status evolve_oz(const double* U, double* rho, int n, int steps, int precision, int renorm_every, const Model* m,
                     double* obs, Arena& ar, cudaStream_t s);
 // True when TC_FP64 runs on those products for n atoms, given a workspace of their size.
@@ -57,9 +57,9 @@ int lowp_host_chunks(int n, int precision);   // row blocks in (4, 2 or 1)
 int lowp_host_bands(int n, int precision);    // row bands out (8, 4, 2 or 1)
 
 // Open-system form (packed excitation blocks).
-size_t lindblad_bytes(int n, int precision);
+size_t lindblad_bytes(int n, int precision, bool least = false);
 
 // Reverse-mode gradient.
-size_t backward_bytes(int n, int steps, int ckpt_every, int precision);
+size_t backward_bytes(int n, int steps, int ckpt_every, int precision, bool least = false);
 
 }  // namespace tc

@@ -328,7 +328,7 @@ TC_API tc_status tc_autotune_set(int n, int precision, const int* choice) {
 TC_API tc_status tc_autotune(int n, int precision, void* work, size_t work_bytes, void* stream, int* choice) {
     if (n < 1 || n > kMaxAtoms) return fail(TC_ERR_INVALID_ARG, "n = %d outside 1..16", n);
     if (precision < TC_FP64 || precision > TC_TF32X3) return fail(TC_ERR_INVALID_ARG, "unknown precision");
-    const size_t need = tc_workspace_size(n, precision, TC_OP_EVOLVE, 0, 0);
+    const size_t need = tc_workspace_least(n, precision, TC_OP_EVOLVE, 0, 0);   // (FP64: the DMMA form is what is tuned)
     if (!work) return fail(TC_ERR_WORKSPACE, "work is NULL (need %zu bytes)", need);
     if (reinterpret_cast<uintptr_t>(work) & 255u) return fail(TC_ERR_WORKSPACE, "work is not 256-byte aligned");
     if (work_bytes < need) return fail(TC_ERR_WORKSPACE, "work has %zu bytes, need %zu", work_bytes, need);
