@@ -218,7 +218,7 @@ tc_status gemm_real(RealMul& rm, int N, const double* A, const double* B, double
         if (rm.loaded != A) TC_TRY(crt_real_load(rm.left, A, s));
         rm.loaded = A;
         TC_TRY(crt_real_load(rm.right, B, s));
-        return crt_real_product(rm.left, rm.right, B, C, rm.scratch, s);
+        return crt_real_product(rm.left, rm.right, A, B, C, rm.scratch, s);
     }
     GemmF64 g{};
     g.M = g.N = g.K = N;

@@ -810,6 +810,7 @@ struct CrtCombine {
     const int* ea;
     const int* eb;
     const double* diag;      // [2][Np]
+    const double* diag_b;    // real products
     const double* br;
     const double* bi;
     long long bi_flip;       // the sign bit when B was loaded conjugated
@@ -955,10 +956,11 @@ __global__ void __launch_bounds__(256, 4) crt_combine_kernel(CrtCombine p) {
     }
 }
 
-// The same for a real product: 32 x 32 tiles, C[i][j] += A_ii B_ji on top.
+// The same for a real product: 32 x 32 tiles, the terms of both diagonals on top: A_ii B_ji and, off the
+// diagonal, A_ij B_jj.
 __global__ void __launch_bounds__(256) crt_combine_real_kernel(CrtCombine p) {
     __shared__ double sr[32][33];   // [column of the tile][row of the tile]
-    const int i0 = 32 * (int)blockIdx.y, j0 = 32 * (int)blockIdx.x;
+    const int i0 = 32 * (int)blockIdx.y, j0 = 32 * (int)blockIdx.x;   // (a: A's FP64 values in p.bi)
     const int ti = threadIdx.x >> 3, tj = (threadIdx.x & 7) * 4;
     const int i = i0 + ti, j = j0 + tj;
     uint32_t w[kModuli];
@@ -983,7 +985,10 @@ __global__ void __launch_bounds__(256) crt_combine_real_kernel(CrtCombine p) {
     }
     __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 4; k++) v[k] = fma(d, sr[tj + k][ti], v[k]);
+    for (int k = 0; k < 4; k++) {
+        v[k] = fma(d, sr[tj + k][ti], v[k]);
+        if (i != j + k) v[k] = fma(p.bi[(size_t)i * p.ldb + j + k], p.diag_b[j + k], v[k]);
+    }
     double2* y = reinterpret_cast<double2*>(p.yr + (size_t)i * p.Np + j);
     y[0] = make_double2(v[0], v[1]);
     y[1] = make_double2(v[2], v[3]);
@@ -1235,28 +1240,30 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
 }
 
 size_t crt_real_mat_bytes(int N, bool left) {
-    return plane_bytes(N, kModuli) + round256((size_t)N * sizeof(int)) +
-           (left ? round256((size_t)2 * N * sizeof(double)) : 0);
+    (void)left;   // both keep their diagonal
+    return plane_bytes(N, kModuli) + round256((size_t)N * sizeof(int)) + round256((size_t)2 * N * sizeof(double));
 }
 
 size_t crt_real_scratch_bytes(int N) { return round256((size_t)kModuli * N * N); }
 
-tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) { return mat_init(m, ar, N, left, kModuli); }
+tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left) {
+    TC_TRY(mat_init(m, ar, N, true, kModuli));
+    m.left = left;
+    return TC_OK;
+}
 
 tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s) {
     if (reinterpret_cast<uintptr_t>(a) & 15u) return fail(TC_ERR_INVALID_ARG, "real products: operand misaligned");
     const int N = m.Np, tpr = std::min(128, N / 4);   // N a power of two
     const unsigned grid = (unsigned)(N / (128 / tpr));
     auto* out = static_cast<__nv_bfloat16*>(m.planes);
-    if (m.left)
-        crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, 0, out, m.ex, m.diag);
-    else
-        crt_residue_kernel<false, false, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, 0, out, m.ex, nullptr);
+    crt_residue_kernel<false, true, 4, true><<<grid, 128, 0, s>>>(a, nullptr, N, (size_t)N, N, tpr, 0, nullptr, 0, out, m.ex, m.diag);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
 
-tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, double* c, void* scratch, cudaStream_t s) {
+tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* a, const double* b, double* c, void* scratch,
+                           cudaStream_t s) {
     const int N = A.Np;
     if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0 || N > 16384)
         return fail(TC_ERR_INVALID_ARG, "real products: operands of different sizes or roles");
@@ -1268,7 +1275,9 @@ tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, do
     p.ea = A.ex;
     p.eb = B.ex;
     p.diag = A.diag;
+    p.diag_b = B.diag;
     p.br = b;
+    p.bi = a;
     p.yr = c;
     crt_combine_real_kernel<<<dim3((unsigned)(N / 32), (unsigned)(N / 32)), 256, 0, s>>>(p);
     TC_LAUNCH_CHECK();

@@ -72,11 +72,15 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
                       size_t ldb, const CrtOut& out, cudaStream_t s);
 
 // Real operands (N x N, row stride N, N a power of two >= 256): sixteen planes
-// each; c = A B^T.  b: B's FP64 values (c must not overlap a or b).
+// each, without their diagonals (the matrices of a Taylor polynomial are close
+// to multiples of the identity, beside which a row's scale would keep little of
+// its other entries); c = A B^T.  a, b: the FP64 values of A and B (c must not
+// overlap them).
 size_t crt_real_mat_bytes(int N, bool left);
 size_t crt_real_scratch_bytes(int N);
 tc_status crt_real_mat_init(CrtMat& m, Arena& ar, int N, bool left);
 tc_status crt_real_load(const CrtMat& m, const double* a, cudaStream_t s);
-tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* b, double* c, void* scratch, cudaStream_t s);
+tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* a, const double* b, double* c, void* scratch,
+                           cudaStream_t s);
 
 }  // namespace tc

@@ -139,3 +139,16 @@ def test_small_populations_of_the_open_system(tc):
         x, y = x.diagonal().real, y.diagonal().real
         big = y > 1e-280
         assert ((x - y).abs()[big] / y[big]).max().item() < 4 * np.sqrt(1 << n) * _tol(1 << n, steps) if big.any() else True, k
+
+
+@pytest.mark.parametrize("n", [8, 10, 11])
+def test_small_entries_of_the_exponential(tc, n):
+    """tc_expm on the tensor cores against the DMMA, the same polynomial: with both diagonals apart a product's error
+    is relative to the off-diagonal parts of its rows, beta for B = (H - mu) dt, beta^2 and more for every matrix of
+    the polynomial, so below beta^4 in all; the DMMA sums' N roundings of sums like the entry itself."""
+    N, dt = 1 << n, 0.05
+    p = tc.Params(n, list(map(float, W.draw_couplings(n, 3))), 1.002, 1.0)
+    H = tc.build_hamiltonian(p)
+    a, b = tc.expm(H, n, dt), tc.expm(H, n, dt, precision="fp64_dmma")
+    beta = (torch.linalg.vector_norm(H - torch.diag(H.diagonal()), dim=1).max() * dt).item()
+    assert ((a - b).abs() <= N * 2.0 ** -52 * (b.abs() + beta ** 4)).all()
