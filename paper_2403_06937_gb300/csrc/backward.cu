@@ -23,7 +23,12 @@
 // one of cgemm_crt.cu, Y = A B^H.  With B' = conj(S) for a symmetric S
 // (U, A', the T_k) that is A S; the Frechet recurrence is taken from the
 // right, F_k = (F_{k-1} A' + T_{k-1} E) / k, so that only E, once, needs an
-// explicit adjoint.  On the DMMA GEMM the recurrence alone took 1.7 s at
+// explicit adjoint.  Every product's operands carry powers of two along K
+// (cgemm_crt.cu, "Column scales"): the steps' and W's those of the state or of
+// Lambda, the others those of the operand whose columns differ most.  A loss far
+// below 1 rests on entries that far below their rows' norms: n = 8, two steps
+// from the all-excited state, L = P(6 photons) = 3e-33: dL/dg was off by 1.5e-2
+// with one scale a row alone.  On the DMMA GEMM the recurrence alone took 1.7 s at
 // n = 11 (real products 16 ms, complex ones 64 ms; 0.5 ms here).
 #include <algorithm>
 #include <array>
@@ -227,33 +232,52 @@ tc_status minus_i_times(int N, const double* Bs, CM X, CM Y, CM Q, cudaStream_t 
     return TC_OK;
 }
 
-// FP64-accurate products on the tensor cores: U and conj(U) as left operands,
-// one more left and one more right operand for whatever a product needs.
+// FP64-accurate products on the tensor cores: one left and one right operand
+// for whatever a product needs, loaded for it (the digit form keeps U and
+// conj(U) in two more left ones).
 struct OzBufs {
     OzMat U, Uc, B, A2;
-    CM Y;            // adjoint of a right operand that is not symmetric
+    CrtColumns cols, cols2;
+    const double* Uin;   // the caller's U
+    CM Y;                // adjoint of a right operand that is not symmetric
     void* scratch;
     int group;
 };
 
 size_t oz_backward_extra(int n, bool lazy) {
     const size_t N = (size_t)1 << n;
-    return 3 * oz_mat_bytes((int)N, true, lazy) + oz_mat_bytes((int)N, false, lazy) + oz_scratch_bytes((int)N, lazy) +
+    return (oz_modular() ? 1 : 3) * oz_mat_bytes((int)N, true, lazy) + oz_mat_bytes((int)N, false, lazy) +
+           oz_scratch_bytes((int)N, lazy) + 2 * crt_columns_bytes((int)N < 128 ? 128 : (int)N) +
            2 * round256(N * N * sizeof(double)) + 256;
 }
 
-// Q <- A P A^H from P's planes, in z.B already or loaded here; Q may be P
-tc_status step_oz(int N, OzBufs& z, const OzMat& A, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
-    if (!loaded) TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
+// Column scales of the next product from R (none in the digit form).
+tc_status columns(int N, const CrtColumns& c, CrtColumnsOf of, CM R, const int** col, cudaStream_t s) {
+    *col = nullptr;
+    if (!oz_modular()) return TC_OK;
+    *col = c.col;
+    return crt_columns(c, of, R.r, R.i, false, N, (size_t)N, s);
+}
+
+// Q <- A P A^H with A = U or (adjoint) conj(U).  P's planes are loaded here, or already in z.B with the scales of
+// P in z.cols.  Q may be P.
+tc_status step_oz(int N, OzBufs& z, bool adjoint, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
+    const int* col = oz_modular() ? z.cols.col : nullptr;
+    if (!loaded) {
+        TC_TRY(columns(N, z.cols, kColsOfState, P, &col, s));
+        TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s, col));
+    }
+    if (col) TC_TRY(oz_mat_load(z.A2, z.Uin, nullptr, true, adjoint, N, (size_t)N, s, col));
+    const OzMat& A = col ? z.A2 : (adjoint ? z.Uc : z.U);
     TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = A P^H
-    TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s));
+    TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s, col));
     return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, z.scratch}, z.group, s);     // Q = A X^H
 }
 
-// out = A R^H (+ out): the left operand as it is, R's planes as they are or conjugated
-tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
-    if (A.r) TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s));   // else: as loaded last
-    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s));
+// out = A R^H (+ out), R's planes as they are or conjugated, with the column scales `col`
+tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, const int* col, cudaStream_t s) {
+    TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s, col));
+    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s, col));
     OzOut o{out.r, out.i, z.scratch};
     o.conj_b = conj_r;
     if (add && !oz_modular()) {   // the digit form does not accumulate
@@ -267,6 +291,12 @@ tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, cu
     }
     o.accumulate = add;
     return oz_product(0, z.A2, z.B, R.r, R.i, N, (size_t)N, o, z.group, s);
+}
+// the same with scales made here from A's or R's own columns
+tc_status mul_oz_scaled(int N, OzBufs& z, CrtColumnsOf of, CM A, CM R, bool conj_r, CM out, bool add, cudaStream_t s) {
+    const int* col;
+    TC_TRY(columns(N, z.cols, of, of == kColsOfRight ? R : A, &col, s));
+    return mul_oz(N, z, A, R, conj_r, out, add, col, s);
 }
 
 // Steps of the forward and the reverse pass go out as graphs of at most this many, captured once and launched
@@ -415,20 +445,30 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     OzBufs z{};
     if (oz) {
         const bool lazy = work_bytes < backward_tensor_bytes(n, steps, ckpt_every);
-        TC_TRY(oz_mat_init(z.U, ar, N, true, lazy));
-        TC_TRY(oz_mat_init(z.Uc, ar, N, true, lazy));
+        if (!oz_modular()) {
+            TC_TRY(oz_mat_init(z.U, ar, N, true));
+            TC_TRY(oz_mat_init(z.Uc, ar, N, true));
+        }
+        TC_TRY(crt_columns_init(z.cols, ar, N));
+        TC_TRY(crt_columns_init(z.cols2, ar, N));
         TC_TRY(oz_mat_init(z.B, ar, N, false, lazy));
         TC_TRY(oz_mat_init(z.A2, ar, N, true, lazy));
         z.Y = take_cm(ar, NN);
         z.scratch = ar.take<uint8_t>(oz_scratch_bytes(N, lazy));
         if (!z.scratch) return fail(TC_ERR_WORKSPACE, "backward: workspace too small");
         z.group = tune_lookup(n, TC_BF16X3).tc_group;
-        TC_TRY(oz_mat_load(z.U, static_cast<const double*>(U), nullptr, true, false, N, (size_t)N, s));
-        TC_TRY(oz_mat_load(z.Uc, static_cast<const double*>(U), nullptr, true, true, N, (size_t)N, s));
+        z.Uin = static_cast<const double*>(U);
+        if (oz_modular()) {
+            TC_TRY(crt_columns_clear(z.cols, s));
+            TC_TRY(crt_columns_clear(z.cols2, s));
+        } else {
+            TC_TRY(oz_mat_load(z.U, z.Uin, nullptr, true, false, N, (size_t)N, s));
+            TC_TRY(oz_mat_load(z.Uc, z.Uin, nullptr, true, true, N, (size_t)N, s));
+        }
     }
     // Q <- U P U^dag, Q may be P
     auto fwd_step = [&](CM P, CM Q, cudaStream_t cs) -> tc_status {
-        if (oz) return step_oz(N, z, z.U, false, P, Q, b.X, cs);
+        if (oz) return step_oz(N, z, false, false, P, Q, b.X, cs);
         if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, cs));
         return step(N, b.U, Q, b.X, 0, cs);
     };
@@ -495,10 +535,12 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
                 TC_TRY(gemm_c(N, seg[i], 0, b.L, 0, b.W, 1.0, 1.0, 0, cs));
                 continue;
             }
-            // the right operand holds Lambda from the product before, at first a state
-            TC_TRY(step_oz(N, z, z.Uc, i < hi - 1, b.L, b.L, b.X, cs));
+            // the right operand holds Lambda and its scales from the product before, at first a state
+            TC_TRY(step_oz(N, z, true, i < hi - 1, b.L, b.L, b.X, cs));
             // Lambda Hermitian: rho Lambda = rho Lambda^H
-            TC_TRY(mul_oz(N, z, seg[i], b.L, false, b.W, true, cs));
+            const int* col;
+            TC_TRY(columns(N, z.cols, kColsOfState, b.L, &col, cs));
+            TC_TRY(mul_oz(N, z, seg[i], b.L, false, b.W, true, col, cs));
         }
         return TC_OK;
     };
@@ -516,7 +558,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // M = W U^dag = W conj(U)  -> into L (free now)
     CM M = b.L;
     if (oz)
-        TC_TRY(mul_oz(N, z, b.W, b.U, false, M, false, s));   // W U^H, U symmetric
+        TC_TRY(mul_oz_scaled(N, z, kColsOfLeft, b.W, b.U, false, M, false, s));   // W U^H, U symmetric
     else
         TC_TRY(gemm_c(N, b.W, 0, b.U, 1, M, 1.0, 0.0, 0, s));
 
@@ -559,18 +601,18 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         axpby_kernel<<<grid_for(NN), 256, 0, s>>>(1.0, Xs.r, Xs.i, 1.0, b.T.r, b.T.i, Xs.r, Xs.i, NN);
         TC_LAUNCH_CHECK();
     }
-    const CM again{nullptr, nullptr};   // the left operand loaded last
     const bool oz_frechet = oz && oz_modular();
     if (oz_frechet) {
         // Q = conj(A') (A' symmetric) and Y = E^H, the right operands of the recurrence
         times_i_kernel<<<grid_for(NN), 256, 0, s>>>(b.B, b.Q.r, b.Q.i, NN);
         TC_LAUNCH_CHECK();
         TC_TRY(adjoint(N, b.P, z.Y, s));
+        TC_TRY(crt_columns(z.cols2, kColsOfRight, z.Y.r, z.Y.i, false, N, (size_t)N, s));   // E's rows
         for (int k = 2; k <= mt; k++) {
             // F_k = (F_{k-1} A' + T_{k-1} E) / k ;  T_k = T_{k-1} A' / k
-            TC_TRY(mul_oz(N, z, b.F, b.Q, false, b.Fn, false, s));
-            TC_TRY(mul_oz(N, z, b.T, b.Q, false, b.Tn, false, s));
-            TC_TRY(mul_oz(N, z, again, z.Y, false, b.Fn, true, s));
+            TC_TRY(mul_oz_scaled(N, z, kColsOfLeft, b.F, b.Q, false, b.Fn, false, s));
+            TC_TRY(mul_oz(N, z, b.T, b.Q, false, b.Tn, false, nullptr, s));
+            TC_TRY(mul_oz(N, z, b.T, z.Y, false, b.Fn, true, z.cols2.col, s));
             term_kernel<<<grid_for(NN), 256, 0, s>>>(1.0 / k, b.Fn, b.Tn, b.F, b.T, D, Xs, NN);
             TC_LAUNCH_CHECK();
         }
@@ -593,10 +635,10 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
     // squarings: D <- X D + D X ; X <- X X
     for (int q = 0; q < sq; q++) {
         if (oz_frechet) {
-            TC_TRY(mul_oz(N, z, D, Xs, true, b.Fn, false, s));       // D X (X symmetric: X = conj(X)^H)
-            TC_TRY(mul_oz(N, z, Xs, Xs, true, b.Tn, false, s));      // X X
+            TC_TRY(mul_oz_scaled(N, z, kColsOfLeft, D, Xs, true, b.Fn, false, s));       // D X (X symmetric: X = conj(X)^H)
+            TC_TRY(mul_oz(N, z, Xs, Xs, true, b.Tn, false, nullptr, s));                 // X X
             TC_TRY(adjoint(N, D, z.Y, s));
-            TC_TRY(mul_oz(N, z, again, z.Y, false, b.Fn, true, s));  // + X D
+            TC_TRY(mul_oz_scaled(N, z, kColsOfRight, Xs, z.Y, false, b.Fn, true, s));    // + X D
             TC_TRY(copy_cm(b.Fn, D, NN, s));
             TC_TRY(copy_cm(b.Tn, Xs, NN, s));
             continue;

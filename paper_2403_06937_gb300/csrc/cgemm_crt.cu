@@ -717,11 +717,16 @@ __global__ void __launch_bounds__(128)
 // block takes 32 rows x 128 columns, and the last one to finish turns the
 // maxima into scales and clears them.  n = 12: 16 N^2 bytes at HBM rate beside
 // a step of 5 ms.
+//
+// MODE kColsOfRight, kColsOfLeft: for operands that are no states, the powers of
+// two that make the columns of the given operand alike (in its sign: the other
+// operand takes the inverse).  A matrix r_i f_ij c_j with f of one size, as the
+// gradient's are, then has flat rows, and the other operand carries c.
 __device__ __forceinline__ unsigned exponent_of(uint64_t bits) {   // 0: zero or not finite
     const unsigned e = (unsigned)(bits >> 52) & 0x7FFu;
     return e == 0x7FFu || (bits << 1) == 0 ? 0u : max(e, 1u);
 }
-template <bool INTERLEAVED>
+template <int MODE, bool INTERLEAVED>
 __global__ void __launch_bounds__(256)
     crt_columns_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
                        unsigned* __restrict__ top, int* __restrict__ col) {
@@ -750,6 +755,7 @@ __global__ void __launch_bounds__(256)
                 row = max(row, e);
             }
         }
+        if (MODE != kColsOfState) continue;
         row = __reduce_max_sync(0xffffffffu, row);
         if (lane == 0 && row) atomicMax(&top[i0 + r], row);
     }
@@ -772,8 +778,11 @@ __global__ void __launch_bounds__(256)
     for (int w = 0; w < 8; w++) m = max(m, warp_max[w]);
     for (int k = threadIdx.x; k < Np; k += 256) {
         const int e = (int)__ldcg(&top[k]);
-        const int d = k < N ? (int)exponent_of(bits(k, k, 0)) : 0;
-        col[k] = e == 0 ? kEmptyColumn : (max(d, 2 * e - (int)m) - 1023) >> 1;
+        const int d = MODE == kColsOfState && k < N ? (int)exponent_of(bits(k, k, 0)) : 0;
+        const int v = MODE == kColsOfState   ? (max(d, 2 * e - (int)m) - 1023) >> 1
+                      : MODE == kColsOfRight ? e - 1023
+                                             : 1023 - e;
+        col[k] = e == 0 ? kEmptyColumn : v;
         top[k] = 0;
     }
     if (threadIdx.x == 0) *ticket = 0;
@@ -1090,9 +1099,11 @@ tc_status load_group(const CrtMat& m, int first, void* planes, cudaStream_t s) {
     const uint64_t flip = m.src.conj ? 1ull << 63 : 0;
     auto* out = static_cast<__nv_bfloat16*>(planes);
     const CrtSource& o = m.src;
-#define TC_RES(I_, L_, C_)                                                                                       \
-    crt_residue_kernel<I_, L_, C_, false, false, true><<<w.grid, 128, 0, s>>>(o.re, o.im, o.N, o.ld, m.Np, w.tpr, \
-                                                                              flip, nullptr, first, out, m.ex, m.diag)
+#define TC_RES(I_, L_, C_)                                                                                         \
+    o.col ? crt_residue_kernel<I_, L_, C_, false, true, true><<<w.grid, 128, 0, s>>>(                               \
+                o.re, o.im, o.N, o.ld, m.Np, w.tpr, flip, o.col, first, out, m.ex, m.diag)                          \
+          : crt_residue_kernel<I_, L_, C_, false, false, true><<<w.grid, 128, 0, s>>>(                              \
+                o.re, o.im, o.N, o.ld, m.Np, w.tpr, flip, nullptr, first, out, m.ex, m.diag)
     if (o.interleaved && m.left) {
         if (w.cpt == 2) TC_RES(true, true, 2); else TC_RES(true, true, 4);
     } else if (o.interleaved) {
@@ -1143,14 +1154,19 @@ tc_status crt_columns_clear(const CrtColumns& c, cudaStream_t s) {
     return TC_OK;
 }
 
-tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, bool interleaved, int N, size_t ld,
-                      cudaStream_t s) {
+tc_status crt_columns(const CrtColumns& c, CrtColumnsOf mode, const double* re, const double* im, bool interleaved, int N,
+                      size_t ld, cudaStream_t s) {
     if (N > c.Np || c.Np % 128 != 0) return fail(TC_ERR_INVALID_ARG, "column scales: size");
+    if (interleaved && mode != kColsOfState) return fail(TC_ERR_INVALID_ARG, "column scales: mode");
     const dim3 grid((unsigned)((N + 127) / 128), (unsigned)((N + 31) / 32));
     if (interleaved)
-        crt_columns_kernel<true><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+        crt_columns_kernel<kColsOfState, true><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+    else if (mode == kColsOfState)
+        crt_columns_kernel<kColsOfState, false><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+    else if (mode == kColsOfRight)
+        crt_columns_kernel<kColsOfRight, false><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
     else
-        crt_columns_kernel<false><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
+        crt_columns_kernel<kColsOfLeft, false><<<grid, 256, 0, s>>>(re, im, N, ld, c.Np, c.top, c.col);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -1161,8 +1177,7 @@ tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool inter
         (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
     if (m.lazy) {
-        if (col) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: column scales need an operand's own planes");
-        m.src = CrtSource{re, im, interleaved, conj, N, ld};
+        m.src = CrtSource{re, im, col, interleaved, conj, N, ld};
         return TC_OK;
     }
     const RowSplit w = row_split(m.Np);

@@ -15,6 +15,7 @@ namespace tc {
 // read its source, which must stay as it is until they have run.
 struct CrtSource {
     const double *re, *im;
+    const int* col;
     bool interleaved, conj;
     int N;
     size_t ld;
@@ -51,8 +52,11 @@ struct CrtColumns {
 size_t crt_columns_bytes(int Np);
 tc_status crt_columns_init(CrtColumns& c, Arena& ar, int Np);
 tc_status crt_columns_clear(const CrtColumns& c, cudaStream_t s);
-tc_status crt_columns(const CrtColumns& c, const double* re, const double* im, bool interleaved, int N, size_t ld,
-                      cudaStream_t s);
+// kColsOfState: re, im is a density matrix, the right operand; kColsOfRight,
+// kColsOfLeft: from the right or the left operand's own columns (planes only)
+enum CrtColumnsOf { kColsOfState, kColsOfRight, kColsOfLeft };
+tc_status crt_columns(const CrtColumns& c, CrtColumnsOf mode, const double* re, const double* im, bool interleaved, int N,
+                      size_t ld, cudaStream_t s);
 // Bytes of scratch of a product: one byte per residue of the result (of a band
 // of rows above Np = 16384); with lazy operands two groups of planes too.
 size_t crt_scratch_bytes(int Np, bool lazy = false);

@@ -138,7 +138,7 @@ tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double*
     R.y_c128 = to;
     const int* col = scaled ? cols.col : nullptr;
     if (scaled) {
-        TC_TRY(crt_columns(cols, from ? from : Rr, Ri, from != nullptr, N, (size_t)Np, cs));
+        TC_TRY(crt_columns(cols, kColsOfState, from ? from : Rr, Ri, from != nullptr, N, (size_t)Np, cs));
         TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs, col));
     }
     TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs, col));

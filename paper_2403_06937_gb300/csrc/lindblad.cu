@@ -794,7 +794,7 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
                 TC_TRY(gemm_f64(g2, cs));
                 continue;
             }
-            if (scaled) TC_TRY(crt_columns(cols, rr, ri, false, d, (size_t)Np, cs));
+            if (scaled) TC_TRY(crt_columns(cols, kColsOfState, rr, ri, false, d, (size_t)Np, cs));
             if (!load_once)
                 TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs, col));
             TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs, col));

@@ -152,3 +152,20 @@ def test_small_entries_of_the_exponential(tc, n):
     a, b = tc.expm(H, n, dt), tc.expm(H, n, dt, precision="fp64_dmma")
     beta = (torch.linalg.vector_norm(H - torch.diag(H.diagonal()), dim=1).max() * dt).item()
     assert ((a - b).abs() <= N * 2.0 ** -52 * (b.abs() + beta ** 4)).all()
+
+
+@pytest.mark.parametrize("n,steps,ckpt", [(8, 2, 2), (8, 20, 6), (7, 3, 1)])
+def test_gradient_of_a_small_loss(tc, n, steps, ckpt):
+    """L = P(m photons) from the all-excited state, down to 1e-33, against the DMMA form of the same series: 4 products
+    a step, three a Taylor term (at most 20), each within K 2^-52 of its sum of magnitudes."""
+    N, dt = 1 << n, 0.05
+    p, U = _setup(tc, n, dt)
+    rho = torch.from_numpy(W.all_excited_rho(n)).cuda()
+    pop = np.array([bin(s).count("1") for s in range(N)])
+    for m in (1, 2, 4, 6):
+        O = torch.from_numpy((pop == n - m).astype(np.float64)).cuda()
+        a, la = tc.evolve_backward(p, dt, steps, rho, U, O, ckpt_every=ckpt)
+        b, lb = tc.evolve_backward(p, dt, steps, rho, U, O, ckpt_every=ckpt, precision="fp64_dmma")
+        tol = (4 * steps + 60) * N * 2.0 ** -52
+        assert abs(la - lb) <= tol * lb, m
+        assert (a - b).abs().max().item() <= tol * b.abs().max().item(), m
