@@ -76,23 +76,26 @@ typedef enum tc_status {
  *              workspace (down to tc_workspace_least) or under TC_OZ_BITS=6, on
  *              the FP64 DMMA.
  *              Accuracy of the residue products: the DMMA form rounds sums of
- *              products of 53-bit entries, so every entry of a result is
- *              accurate relative to its own sum of magnitudes.  The residue
- *              form holds an operand as integers in one scale a row.  In the
- *              step loops (tc_evolve, tc_evolve_host, tc_batch_evolve,
- *              tc_lindblad_evolve) the columns are scaled by the state's
- *              populations too, which keeps every population of a positive
- *              rho as accurate as the DMMA form does, and a coherence rho_ij
- *              relative to sqrt(rho_ii rho_jj).  In tc_expm and
- *              tc_evolve_backward there is no such scale: errors are relative
- *              to the norms of rows (2^-59 of a row's norm an entry), so an
- *              entry of U far below its row's norm, or a gradient of a loss far
- *              below 1, has fewer right digits than from the DMMA form.  Ask
- *              for TC_FP64_DMMA (tc_expm: a workspace of tc_workspace_least
- *              bytes; tc_expm_model does not use these products) where such
- *              numbers matter.
- *  TC_FP64_DMMA : TC_FP64 on the FP64 DMMA (mma.sync .f64) at every size, as
- *              accurate entry by entry as FP64 sums are, at about 1 TFLOP/s.
+ *              products of 53-bit entries, so an entry of a result is accurate
+ *              relative to its own sum of magnitudes.  The residue form holds
+ *              an operand as integers in one scale a row, which keeps nothing
+ *              of an entry below 2^-59 of its row's norm; so that small numbers
+ *              stay right, powers of two are taken out along K as well.
+ *              - Steps (tc_evolve, tc_evolve_host, tc_batch_evolve,
+ *                tc_lindblad_evolve): from the populations.  For a positive rho
+ *                every population is as accurate as in the DMMA form, a
+ *                coherence rho_ij relative to sqrt(rho_ii rho_jj).
+ *              - tc_evolve_backward: from the state, from Lambda or from the
+ *                operand whose columns differ most; gradients of small losses
+ *                agree with the DMMA form's to FP64.
+ *              - tc_expm: both factors' diagonals stay in FP64; errors are
+ *                relative to the off-diagonal parts of rows.
+ *              Entries smaller than that allows (a coherence far below the
+ *              populations' geometric mean, say) have fewer right digits than
+ *              from the DMMA form: ask for TC_FP64_DMMA (tc_expm: a workspace
+ *              of tc_workspace_least bytes) where they matter.
+ *  TC_FP64_DMMA : TC_FP64 on the FP64 DMMA (mma.sync .f64) at every size, at
+ *              about 1 TFLOP/s.
  *  TC_BF16X3 : each FP32 operand split in three BF16 parts, six BF16 products
  *              accumulated in FP32 in tensor memory (tcgen05 kind::f16).
  *  TC_TF32   : one TF32 product, FP32 accumulate (tcgen05 kind::tf32).
@@ -104,7 +107,8 @@ typedef enum tc_status {
  *              complex product is two real BF16 products per modulus, exact
  *              in FP32 over K chunks of 1024; the remainder theorem gives the
  *              exact integer product.  The left operand's diagonal is kept
- *              in FP64.  Within sqrt(2 K) 2^-56.3 of the product of the two
+ *              in FP64.  Without TC_FP64's scales along K (but for the
+ *              gradient): within sqrt(2 K) 2^-56.3 of the product of the two
  *              rows' 2-norms, plus the rounding of the result; a row with an
  *              infinity or a NaN gives NaN in its row or column.  rho stored
  *              in FP64.  TC_OZ_BITS=6 in the environment takes 45 products of

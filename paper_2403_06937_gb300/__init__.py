@@ -103,7 +103,7 @@ def expm(H: torch.Tensor, n: int, dt: float, taylor_degree: int = 0, squarings: 
          stream=None, work: Optional[torch.Tensor] = None, precision="fp64") -> torch.Tensor:
     """tc_expm: U = e^{-iH dt} (N x N complex128); {10, 0, False} is the paper's Eq. 10.
 
-    precision: "fp64", or "fp64_dmma" for entries of U far below the norms of their rows (tc_precision in tc.h)."""
+    precision: "fp64", or "fp64_dmma" for the FP64 DMMA at every size (tc_precision in tc.h)."""
     N = 1 << n
     assert H.dtype == torch.float64 and H.is_contiguous() and H.shape == (N, N)
     U = torch.empty((N, N), dtype=torch.complex128, device=H.device)
@@ -279,9 +279,8 @@ class EvolveFn(torch.autograd.Function):
     backward (only when a gradient is asked for): tc_evolve_backward, the
     reverse mode with checkpoints every `ckpt_every` steps.
     precision: "fp64" or "ozaki" (n >= 7), for both passes: from n = 7 on
-    FP64-accurate products on the BF16 tensor cores, whose errors are relative to
-    the norms of rows in H's exponential and in the reverse pass; "fp64_dmma", all
-    of it on the FP64 DMMA, for losses far below 1.
+    FP64-accurate products on the BF16 tensor cores; "fp64_dmma": all of it on the
+    FP64 DMMA.
     Inputs g (n,), omega_a (), omega_c () are float64 tensors; rho0 and O_diag
     are CUDA tensors.  Returns a 0-d float64 tensor on rho0's device.
     """

@@ -28,7 +28,7 @@
 // Lambda, the others those of the operand whose columns differ most.  A loss far
 // below 1 rests on entries that far below their rows' norms: n = 8, two steps
 // from the all-excited state, L = P(6 photons) = 3e-33: dL/dg was off by 1.5e-2
-// with one scale a row alone.  On the DMMA GEMM the recurrence alone took 1.7 s at
+// with one scale a row alone (and the gradient of 100 steps took 10.8 ms, not 14.4).  On the DMMA GEMM the recurrence alone took 1.7 s at
 // n = 11 (real products 16 ms, complex ones 64 ms; 0.5 ms here).
 #include <algorithm>
 #include <array>
@@ -263,11 +263,14 @@ tc_status columns(int N, const CrtColumns& c, CrtColumnsOf of, CM R, const int**
 // P in z.cols.  Q may be P.
 tc_status step_oz(int N, OzBufs& z, bool adjoint, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
     const int* col = oz_modular() ? z.cols.col : nullptr;
-    if (!loaded) {
-        TC_TRY(columns(N, z.cols, kColsOfState, P, &col, s));
-        TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s, col));
-    }
-    if (col) TC_TRY(oz_mat_load(z.A2, z.Uin, nullptr, true, adjoint, N, (size_t)N, s, col));
+    const CrtSource u{z.Uin, nullptr, col, true, adjoint, N, (size_t)N};
+    if (!loaded) TC_TRY(columns(N, z.cols, kColsOfState, P, &col, s));
+    if (!loaded && col)
+        TC_TRY(crt_mat_load_both(z.A2.crt, u, z.B.crt, CrtSource{P.r, P.i, col, false, false, N, (size_t)N}, s));
+    else if (!loaded)
+        TC_TRY(oz_mat_load(z.B, P.r, P.i, false, false, N, (size_t)N, s));
+    else if (col)
+        TC_TRY(oz_mat_load(z.A2, u.re, nullptr, true, adjoint, N, (size_t)N, s, col));
     const OzMat& A = col ? z.A2 : (adjoint ? z.Uc : z.U);
     TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = A P^H
     TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s, col));
@@ -276,8 +279,13 @@ tc_status step_oz(int N, OzBufs& z, bool adjoint, bool loaded, CM P, CM Q, CM X,
 
 // out = A R^H (+ out), R's planes as they are or conjugated, with the column scales `col`
 tc_status mul_oz(int N, OzBufs& z, CM A, CM R, bool conj_r, CM out, bool add, const int* col, cudaStream_t s) {
-    TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s, col));
-    TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s, col));
+    if (col) {
+        TC_TRY(crt_mat_load_both(z.A2.crt, CrtSource{A.r, A.i, col, false, false, N, (size_t)N}, z.B.crt,
+                                 CrtSource{R.r, R.i, col, false, conj_r, N, (size_t)N}, s));
+    } else {
+        TC_TRY(oz_mat_load(z.A2, A.r, A.i, false, false, N, (size_t)N, s));
+        TC_TRY(oz_mat_load(z.B, R.r, R.i, false, conj_r, N, (size_t)N, s));
+    }
     OzOut o{out.r, out.i, z.scratch};
     o.conj_b = conj_r;
     if (add && !oz_modular()) {   // the digit form does not accumulate

@@ -94,6 +94,7 @@ static_assert(alone_on_sm(kSmem), "a pair that waits for TMEM must be the only o
 constexpr int kChunkStages = crt::kChunk / kKPer;
 constexpr int kGroup = 8;                    // 256-row tiles per raster group (a wave: ~8 x 9 tiles)
 constexpr int kNoScale = INT32_MIN;          // ex of a row with an infinity or a NaN
+constexpr int kGroupModuli = 4;              // moduli at a time of an operand without planes of its own
 
 struct CrtLaunch {
     int tiles;           // Np / 128
@@ -101,7 +102,7 @@ struct CrtLaunch {
     int lo, hi;          // rows of 256-tiles: the band [lo, hi)
     int units_per;       // units per plane
     int units;           // units_per * planes
-    int first, moduli;   // the operands' planes are those of the moduli [first, first + moduli), each pair's in turn
+    int first;           // GROUP: the operands' planes are those of kGroupModuli moduli from here on, twice
     size_t Np;           // row stride of the byte planes
     size_t band;         // rows of a byte plane
     uint8_t* bytes;      // [planes][band][Np], rows from 256 lo on
@@ -264,7 +265,8 @@ __device__ __forceinline__ void chunk_bytes(uint32_t tl, float p, float inv_p, u
     }
 }
 
-template <int MODE>
+// GROUP: operands of some of the moduli only (CrtLaunch::first)
+template <int MODE, bool GROUP>
 __global__ void __launch_bounds__(kThreads, 1)
     cgemm_crt_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, CrtLaunch L) {
     constexpr uint32_t kIdesc = make_idesc(1u, 256u, 256u);
@@ -414,11 +416,11 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int u = worker; u < L.units && !stop; u += workers) {
             int z, P, J;
             unit_at<MODE>(L, u, z, P, J);
-            const int s = L.first + z % L.moduli;
+            const int s = GROUP ? L.first + z % kGroupModuli : z % kModuli;
             const float p = (float)kC.p[s], inv_p = 1.0f / p;
             // rows and columns past the end (an odd number of 128-tiles) are not written
             const bool own = 2 * P + (int)rank < L.tiles && 2 * J + half < L.tiles;
-            uint8_t* y = L.bytes + ((size_t)(z / L.moduli * kModuli + s) * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
+            uint8_t* y = L.bytes + ((size_t)(GROUP ? z / kGroupModuli * kModuli + s : z) * L.band + (size_t)(2 * (P - L.lo) + (int)rank) * 128 + row) * L.Np +
                          (size_t)(256 * J + 128 * half);
             if (chunks == 1) {
                 const uint32_t buf = pass & 1u;
@@ -480,18 +482,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 // ---------------------------------------------------------------- residues
 // Row scale and residue planes of one operand.  A row is handled by TPR
 // consecutive threads of a 128-thread block (CPT columns a thread and step; 2
-// up to N = 512, where the threads would be too few to fill the SMs, else 8):
+// up to N = 512, where the threads would be too few to fill the SMs, else 4):
 // first the scale from the row's largest exponent and its 2-norm, then the
-// residues.  Bound by HBM for large matrices (16 B read, 60 B written per
+// residues.  Bound by HBM for large matrices (16 B read, 64 B written per
 // entry; the second read of the row comes from L2); no FP64 instruction, since
 // one FP64 conversion per entry alone would take as long as a third of the
 // writes on this GPU.
-constexpr int kGroupModuli = 4;      // moduli at a time of an operand without planes of its own
 constexpr int kShiftBias = 4096;     // added to shifted exponents, so that 0 still means an empty row
-constexpr int kNotFinite = 1 << 16;
+template <bool SCALED>
+constexpr int kNotFinite = SCALED ? 1 << 16 : 0x7FF;
 constexpr int kEmptyColumn = INT32_MIN;   // column scale of a zero column
 struct RowStat {
-    int e;       // largest biased exponent (0: all zero, kNotFinite: an infinity or a NaN)
+    int e;       // largest biased exponent (0: all zero, kNotFinite<>: an infinity or a NaN)
     float ss;    // sum of squares over 2^(2 (e - 1022))
 };
 __device__ __forceinline__ RowStat stat_join(RowStat a, RowStat b) {
@@ -501,11 +503,13 @@ __device__ __forceinline__ RowStat stat_join(RowStat a, RowStat b) {
     r.ss = a.ss * __uint_as_float((uint32_t)(127 + 2 * da) << 23) + b.ss * __uint_as_float((uint32_t)(127 + 2 * db) << 23);
     return r;
 }
-__device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits, int shift) {   // of x 2^shift
+template <bool SCALED>
+__device__ __forceinline__ void stat_add(RowStat& a, uint64_t bits, int shift) {   // of x 2^shift (SCALED)
     const uint32_t hi = (uint32_t)(bits >> 32) & 0x7FFFFFFFu;
     if ((bits << 1) == 0) return;
     // a subnormal counts as the normal number of the same significand bits
-    const int e = (hi >> 20) == 0x7FFu ? kNotFinite : max((int)(hi >> 20), 1) + shift;
+    int e = max((int)(hi >> 20), 1);
+    if (SCALED) e = e == 0x7FF ? kNotFinite<true> : e + kShiftBias + shift;
     if (e > a.e) {   // rescale to the new exponent
         const int d = max(a.e - e, -63);
         a.ss *= __uint_as_float((uint32_t)(127 + 2 * d) << 23);
@@ -553,11 +557,11 @@ __device__ __forceinline__ uint32_t bf16_pair(uint64_t v) {
 
 // SCALED: column k carries 2^col[k] (a left operand; a right one 2^-col[k]).
 // GROUP: the planes of kGroupModuli moduli from `first` on only.
-template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false, bool SCALED = false, bool GROUP = false>
-__global__ void __launch_bounds__(128)
-    crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
-                       int tpr, uint64_t im_flip, const int* __restrict__ col, int first,
-                       __nv_bfloat16* __restrict__ planes, int* __restrict__ ex, double* __restrict__ diag) {
+template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL, bool SCALED, bool GROUP>
+__device__ __forceinline__ void residue_rows(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld,
+                                             int Np, int tpr, uint64_t im_flip, const int* __restrict__ col, int first,
+                                             __nv_bfloat16* __restrict__ planes, int* __restrict__ ex,
+                                             double* __restrict__ diag) {
     const int sub = threadIdx.x % tpr;                       // thread within the row
     const int r = blockIdx.x * (128 / tpr) + threadIdx.x / tpr;
     // CPT consecutive columns from c0 as bit patterns (zero outside N x N and, for a left operand, on the diagonal)
@@ -633,8 +637,8 @@ __global__ void __launch_bounds__(128)
         shifts(c0, xr, xi, sc);
 #pragma unroll
         for (int q = 0; q < CPT; q++) {
-            stat_add(st, xr[q], (SCALED ? kShiftBias : 0) + sc[q]);
-            if (!REAL) stat_add(st, xi[q], (SCALED ? kShiftBias : 0) + sc[q]);
+            stat_add<SCALED>(st, xr[q], sc[q]);
+            if (!REAL) stat_add<SCALED>(st, xi[q], sc[q]);
         }
     }
     for (int o = min(tpr, 32) / 2; o > 0; o >>= 1) {
@@ -653,7 +657,7 @@ __global__ void __launch_bounds__(128)
         for (int k = 1; k < tpr / 32; k++) st = stat_join(st, part[w0 + k]);
     }
     // ex = the largest shift with 2-norm * 2^ex <= 2^58.32 (any for a row of zeros)
-    const bool finite = st.e < kNotFinite;
+    const bool finite = st.e < kNotFinite<SCALED>;
     const int sh = st.e == 0 ? 0
                              : (int)floorf(crt::kNormBits - 0.5f * log2f(st.ss * 1.0001f)) -
                                    (st.e - (SCALED ? kShiftBias : 0) - 1022);
@@ -706,6 +710,34 @@ __global__ void __launch_bounds__(128)
             if (!REAL) put(dst + (size_t)(LEFT ? second + at : at) * plane, w1);
         }
     }
+}
+
+template <bool INTERLEAVED, bool LEFT, int CPT, bool REAL = false, bool SCALED = false, bool GROUP = false>
+__global__ void __launch_bounds__(128)
+    crt_residue_kernel(const double* __restrict__ re, const double* __restrict__ im, int N, size_t ld, int Np,
+                       int tpr, uint64_t im_flip, const int* __restrict__ col, int first,
+                       __nv_bfloat16* __restrict__ planes, int* __restrict__ ex, double* __restrict__ diag) {
+    residue_rows<INTERLEAVED, LEFT, CPT, REAL, SCALED, GROUP>(re, im, N, ld, Np, tpr, im_flip, col, first, planes, ex, diag);
+}
+
+// Both operands of a product in one launch (blockIdx.y: left, right), with the
+// same column scales.  For N <= 512, where a launch is mostly latency: n = 8
+// 47.5 -> 43.8 us a step.
+struct ResidueArgs {
+    const double *re, *im;
+    size_t ld;
+    uint64_t im_flip;
+    __nv_bfloat16* planes;
+    int* ex;
+    double* diag;
+};
+template <bool INTER_A, bool INTER_B>
+__global__ void __launch_bounds__(128)
+    crt_residue_both_kernel(ResidueArgs a, ResidueArgs b, int N, int Np, int tpr, const int* __restrict__ col) {
+    if (blockIdx.y == 0)
+        residue_rows<INTER_A, true, 2, false, true, false>(a.re, a.im, N, a.ld, Np, tpr, a.im_flip, col, 0, a.planes, a.ex, a.diag);
+    else
+        residue_rows<INTER_B, false, 2, false, true, false>(b.re, b.im, N, b.ld, Np, tpr, b.im_flip, col, 0, b.planes, b.ex, b.diag);
 }
 
 // Column scales of a state: col[k] = floor(log2(m_k) / 2) with m_k = |rho_kk|
@@ -1010,9 +1042,9 @@ int sm_count() {
     return sms;
 }
 
-template <int MODE>
+template <int MODE, bool GROUP>
 tc_status launch(const CUtensorMap& tmA, const CUtensorMap& tmB, const CrtLaunch& L, cudaStream_t s) {
-    auto k = cgemm_crt_kernel<MODE>;
+    auto k = cgemm_crt_kernel<MODE, GROUP>;
     static bool attr_set[64] = {};
     int dev = 0;
     TC_CUDA(cudaGetDevice(&dev));
@@ -1058,15 +1090,14 @@ tc_status mat_init(CrtMat& m, Arena& ar, int Np, bool left, int planes, bool laz
 }
 
 // The residue products of one band of rows (all of them: lo = 0, hi = side);
-// `planes` planes of each operand, of the moduli from `first` on.
-tc_status gemm(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, int Np, int planes, int first, int moduli,
+// `planes` planes of each operand (group: of the moduli from `first` on).
+tc_status gemm(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, int Np, int planes, bool group, int first,
                int lo, int hi, void* scratch, cudaStream_t s) {
     CrtLaunch L{};
     L.tiles = Np / 128;
     const int side = (L.tiles + 1) / 2;
     L.kb_total = Np / kKPer;
     L.first = first;
-    L.moduli = moduli;
     L.lo = lo;
     L.hi = hi;
     L.Np = (size_t)Np;
@@ -1075,7 +1106,8 @@ tc_status gemm(int mode, const CUtensorMap& tmA, const CUtensorMap& tmB, int Np,
     L.status = device_status_word();
     L.units_per = mode == 0 ? side * (hi - lo) : hi * (hi + 1) / 2 - lo * (lo + 1) / 2;
     L.units = L.units_per * planes;
-    return mode == 0 ? launch<0>(tmA, tmB, L, s) : launch<1>(tmA, tmB, L, s);
+    if (group) return mode == 0 ? launch<0, true>(tmA, tmB, L, s) : launch<1, true>(tmA, tmB, L, s);
+    return mode == 0 ? launch<0, false>(tmA, tmB, L, s) : launch<1, false>(tmA, tmB, L, s);
 }
 
 // Threads of the residue kernel: `cpt` columns a thread and step, `tpr` threads a
@@ -1171,13 +1203,19 @@ tc_status crt_columns(const CrtColumns& c, CrtColumnsOf mode, const double* re, 
     return TC_OK;
 }
 
+static tc_status check_source(const CrtSource& o) {
+    if ((reinterpret_cast<uintptr_t>(o.re) & 15u) ||
+        (!o.interleaved && ((reinterpret_cast<uintptr_t>(o.im) & 15u) || (o.ld & 1u))))
+        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
+    return TC_OK;
+}
+
 tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
                        size_t ld, cudaStream_t s, const int* col) {
-    if ((reinterpret_cast<uintptr_t>(re) & 15u) ||
-        (!interleaved && ((reinterpret_cast<uintptr_t>(im) & 15u) || (ld & 1u))))
-        return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operand planes must be 16-byte aligned with an even stride");
+    const CrtSource source{re, im, col, interleaved, conj, N, ld};
+    TC_TRY(check_source(source));
     if (m.lazy) {
-        m.src = CrtSource{re, im, col, interleaved, conj, N, ld};
+        m.src = source;
         return TC_OK;
     }
     const RowSplit w = row_split(m.Np);
@@ -1197,6 +1235,28 @@ tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool inter
         if (w.cpt == 2) TC_RES(false, false, 2); else TC_RES(false, false, 4);
     }
 #undef TC_RES
+    TC_LAUNCH_CHECK();
+    return TC_OK;
+}
+
+tc_status crt_mat_load_both(CrtMat& A, const CrtSource& a, CrtMat& B, const CrtSource& b, cudaStream_t s) {
+    if (A.Np != B.Np || a.N != b.N || a.col != b.col) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
+    if (A.Np > 512 || A.lazy || !a.col || (!a.interleaved && b.interleaved)) {
+        TC_TRY(crt_mat_load(A, a.re, a.im, a.interleaved, a.conj, a.N, a.ld, s, a.col));
+        return crt_mat_load(B, b.re, b.im, b.interleaved, b.conj, b.N, b.ld, s, b.col);
+    }
+    for (const CrtSource* o : {&a, &b}) TC_TRY(check_source(*o));
+    const RowSplit w = row_split(A.Np);
+    const dim3 grid(w.grid, 2);
+    auto args = [](const CrtMat& m, const CrtSource& o) {
+        return ResidueArgs{o.re, o.im, o.ld, o.conj ? 1ull << 63 : 0, static_cast<__nv_bfloat16*>(m.planes), m.ex, m.diag};
+    };
+    if (a.interleaved && b.interleaved)
+        crt_residue_both_kernel<true, true><<<grid, 128, 0, s>>>(args(A, a), args(B, b), a.N, A.Np, w.tpr, a.col);
+    else if (a.interleaved)
+        crt_residue_both_kernel<true, false><<<grid, 128, 0, s>>>(args(A, a), args(B, b), a.N, A.Np, w.tpr, a.col);
+    else
+        crt_residue_both_kernel<false, false><<<grid, 128, 0, s>>>(args(A, a), args(B, b), a.N, A.Np, w.tpr, a.col);
     TC_LAUNCH_CHECK();
     return TC_OK;
 }
@@ -1222,7 +1282,7 @@ tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* 
                 TC_TRY(load_group(A, first, ga, s));
                 TC_TRY(load_group(B, first, gb, s));
             }
-            TC_TRY(gemm(mode, tmA, tmB, Np, 2 * moduli, first, moduli, row0 / 256, (row0 + band + 255) / 256,
+            TC_TRY(gemm(mode, tmA, tmB, Np, 2 * moduli, A.lazy, first, row0 / 256, (row0 + band + 255) / 256,
                         out.scratch, s));
         }
         CrtCombine c{};
@@ -1282,7 +1342,7 @@ tc_status crt_real_product(const CrtMat& A, const CrtMat& B, const double* a, co
     const int N = A.Np;
     if (B.Np != N || !A.left || B.left || N < 256 || N % 256 != 0 || N > 16384)
         return fail(TC_ERR_INVALID_ARG, "real products: operands of different sizes or roles");
-    TC_TRY(gemm(0, A.map, B.map, N, kModuli, 0, kModuli, 0, N / 256, scratch, s));
+    TC_TRY(gemm(0, A.map, B.map, N, kModuli, false, 0, 0, N / 256, scratch, s));
     CrtCombine p{};
     p.bytes = static_cast<const uint8_t*>(scratch);
     p.Np = (size_t)N;

@@ -13,7 +13,7 @@ namespace tc {
 // right one; a real operand has 16), the power-of-two scale of each row, and,
 // for a left operand, its diagonal.  A lazy operand has no planes: products
 // read its source, which must stay as it is until they have run.
-struct CrtSource {
+struct CrtSource {   // the arguments of crt_mat_load
     const double *re, *im;
     const int* col;
     bool interleaved, conj;
@@ -41,6 +41,9 @@ tc_status crt_mat_view(CrtMat& view, const CrtMat& base, int Np);
 // of the pair of operands, the same for both (crt_columns), or none.
 tc_status crt_mat_load(CrtMat& m, const double* re, const double* im, bool interleaved, bool conj, int N,
                        size_t ld, cudaStream_t s, const int* col = nullptr);
+
+// The same for both operands of a product, with the same column scales.
+tc_status crt_mat_load_both(CrtMat& A, const CrtSource& a, CrtMat& B, const CrtSource& b, cudaStream_t s);
 
 // Powers of two along K, taken from a state: see cgemm_crt.cu.  `top` is zero
 // between calls (crt_columns_clear, once).

@@ -3,7 +3,8 @@
 // accuracy: the operands and products of the residue form (OzMat, oz_product,
 // which pass on to cgemm_crt.cu), and the digit form below (exact integer
 // slices, the Ozaki splitting), taken with TC_OZ_BITS=6 only: an independent
-// check, half the accuracy in bits and about four times the products.
+// check: 54 bits of a row's largest entry, the digit products below level 9 left
+// out, 180 real products where the residue form takes 32.
 //
 // Slicing.  Every row r of an operand (both planes together) gets an
 // exponent e_r with max |x| < 2^(e_r - 1); with S digits of b bits

@@ -139,9 +139,11 @@ tc_status OzSystem::step(int k, cudaStream_t cs, SideBranch& side, const double*
     const int* col = scaled ? cols.col : nullptr;
     if (scaled) {
         TC_TRY(crt_columns(cols, kColsOfState, from ? from : Rr, Ri, from != nullptr, N, (size_t)Np, cs));
-        TC_TRY(oz_mat_load(Us, U, nullptr, true, false, N, (size_t)N, cs, col));
+        TC_TRY(crt_mat_load_both(Us.crt, CrtSource{U, nullptr, col, true, false, N, (size_t)N}, Ps.crt,
+                                 CrtSource{from ? from : Rr, Ri, col, from != nullptr, false, N, (size_t)Np}, cs));
+    } else {
+        TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs));
     }
-    TC_TRY(oz_mat_load(Ps, from ? from : Rr, Ri, from != nullptr, false, N, (size_t)Np, cs, col));
     {
         ProductTimer t(8.0 * N3 * oz_products(), cs);   // X = U rho^H
         TC_TRY(oz_product(0, Us, Ps, Rr, Ri, N, (size_t)Np, X, group, cs));
@@ -176,12 +178,13 @@ tc_status OzSystem::tail(double* rho, cudaStream_t cs) {
 // TC_FP64 takes the products of this file from n = 7 on: below, the padding to
 // 128 costs more than the DMMA product (n = 6: 64^3).  At n = 15 its operands
 // take 176 GB of workspace, which would not leave room for what a caller could
-// hold beside the DMMA form's 52 GB (n = 14: 52 GB, DMMA 26 GB).  Its error against 64
-// bits is no larger than the DMMA sums' (rows held to at least 51 bits of
-// their largest entry in a common scale, sums exact; the DMMA form rounds
-// each of N additions); a step takes 33 us at n = 8 (DMMA 251), 0.18 ms at n = 10
-// (13.1), 5.2 ms at n = 12 (768).  TC_OZ_BITS=6 (the less accurate digit form) keeps
-// TC_FP64 on the DMMA.
+// hold beside the DMMA form's 52 GB (n = 14: 52 GB, DMMA 13 GB).  Its error against 64
+// bits is no larger than the DMMA sums', norm by norm (rows held to at least 51 bits of
+// their largest entry, sums exact; the DMMA form rounds each of N additions)
+// and, with the column scales, population by population.  A step takes 44 us at n = 8
+// (DMMA 251; 33 without the scales, which is TC_FP64_OZAKI), 0.21 ms at n = 10 (13.1;
+// 0.18), 5.3 ms at n = 12 (768; 5.2).  TC_OZ_BITS=6 (the less accurate digit form)
+// keeps TC_FP64 on the DMMA.
 bool f64_on_tensor_cores(int n) { return n >= 7 && n <= 14 && oz_modular(); }
 
 tc_status evolve_oz(const double* U, double* rho, int n, int steps, int precision, int renorm_every, const Model* m,

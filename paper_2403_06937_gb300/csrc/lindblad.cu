@@ -794,10 +794,15 @@ tc_status evolve_oz_blocks(const Layout& L, const Model& m, int precision, doubl
                 TC_TRY(gemm_f64(g2, cs));
                 continue;
             }
-            if (scaled) TC_TRY(crt_columns(cols, kColsOfState, rr, ri, false, d, (size_t)Np, cs));
-            if (!load_once)
-                TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs, col));
-            TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs, col));
+            if (scaled) {
+                TC_TRY(crt_columns(cols, kColsOfState, rr, ri, false, d, (size_t)Np, cs));
+                TC_TRY(crt_mat_load_both(Uk[k].crt, CrtSource{U + 2 * L.off[k], nullptr, col, true, false, d, (size_t)d},
+                                         Bk[k].crt, CrtSource{rr, ri, col, false, false, d, (size_t)Np}, cs));
+            } else {
+                if (!load_once)
+                    TC_TRY(oz_mat_load(Uk[k], U + 2 * L.off[k], nullptr, true, false, d, (size_t)d, cs));
+                TC_TRY(oz_mat_load(Bk[k], rr, ri, false, false, d, (size_t)Np, cs));
+            }
             {
                 ProductTimer pt(8.0 * d3 * oz_products(), cs);   // X_k = U_k rho_k
                 TC_TRY(oz_product(0, Uk[k], Bk[k], rr, ri, d, (size_t)Np, OzOut{Xr, Xi, prod}, group, cs));
