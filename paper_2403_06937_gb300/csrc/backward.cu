@@ -28,7 +28,7 @@
 // Lambda, the others those of the operand whose columns differ most.  A loss far
 // below 1 rests on entries that far below their rows' norms: n = 8, two steps
 // from the all-excited state, L = P(6 photons) = 3e-33: dL/dg was off by 1.5e-2
-// with one scale a row alone (and the gradient of 100 steps took 10.8 ms, not 14.4).  On the DMMA GEMM the recurrence alone took 1.7 s at
+// with one scale a row alone (and the gradient of 100 steps took 10.8 ms, not 12.3).  On the DMMA GEMM the recurrence alone took 1.7 s at
 // n = 11 (real products 16 ms, complex ones 64 ms; 0.5 ms here).
 #include <algorithm>
 #include <array>
@@ -259,12 +259,12 @@ tc_status columns(int N, const CrtColumns& c, CrtColumnsOf of, CM R, const int**
     return crt_columns(c, of, R.r, R.i, false, N, (size_t)N, s);
 }
 
-// Q <- A P A^H with A = U or (adjoint) conj(U).  P's planes are loaded here, or already in z.B with the scales of
-// P in z.cols.  Q may be P.
-tc_status step_oz(int N, OzBufs& z, bool adjoint, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
+// Q <- A P A^H with A = U or (adjoint) conj(U); z.cols is left with the scales of Q.  fresh: those of P are made here,
+// else they are in z.cols; loaded: P's planes are in z.B with them.  Q may be P.
+tc_status step_oz(int N, OzBufs& z, bool adjoint, bool fresh, bool loaded, CM P, CM Q, CM X, cudaStream_t s) {
     const int* col = oz_modular() ? z.cols.col : nullptr;
     const CrtSource u{z.Uin, nullptr, col, true, adjoint, N, (size_t)N};
-    if (!loaded) TC_TRY(columns(N, z.cols, kColsOfState, P, &col, s));
+    if (fresh) TC_TRY(columns(N, z.cols, kColsOfState, P, &col, s));
     if (!loaded && col)
         TC_TRY(crt_mat_load_both(z.A2.crt, u, z.B.crt, CrtSource{P.r, P.i, col, false, false, N, (size_t)N}, s));
     else if (!loaded)
@@ -274,7 +274,10 @@ tc_status step_oz(int N, OzBufs& z, bool adjoint, bool loaded, CM P, CM Q, CM X,
     const OzMat& A = col ? z.A2 : (adjoint ? z.Uc : z.U);
     TC_TRY(oz_product(0, A, z.B, P.r, P.i, N, (size_t)N, OzOut{X.r, X.i, z.scratch}, z.group, s));   // X = A P^H
     TC_TRY(oz_mat_load(z.B, X.r, X.i, false, false, N, (size_t)N, s, col));
-    return oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, OzOut{Q.r, Q.i, z.scratch}, z.group, s);     // Q = A X^H
+    OzOut out{Q.r, Q.i, z.scratch};
+    if (col && N <= 16384) out.next = &z.cols;
+    TC_TRY(oz_product(1, A, z.B, X.r, X.i, N, (size_t)N, out, z.group, s));   // Q = A X^H
+    return col && !out.next ? columns(N, z.cols, kColsOfState, Q, &col, s) : TC_OK;
 }
 
 // out = A R^H (+ out), R's planes as they are or conjugated, with the column scales `col`
@@ -474,9 +477,9 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
             TC_TRY(oz_mat_load(z.Uc, z.Uin, nullptr, true, true, N, (size_t)N, s));
         }
     }
-    // Q <- U P U^dag, Q may be P
-    auto fwd_step = [&](CM P, CM Q, cudaStream_t cs) -> tc_status {
-        if (oz) return step_oz(N, z, false, false, P, Q, b.X, cs);
+    // Q <- U P U^dag, Q may be P; fresh: P is not the result of the step before
+    auto fwd_step = [&](CM P, CM Q, bool fresh, cudaStream_t cs) -> tc_status {
+        if (oz) return step_oz(N, z, false, fresh, false, P, Q, b.X, cs);
         if (P.r != Q.r) TC_TRY(copy_cm(P, Q, NN, cs));
         return step(N, b.U, Q, b.X, 0, cs);
     };
@@ -497,7 +500,7 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         for (int lo = 1; lo < len; lo += kPiece) {
             const int hi = std::min(len, lo + kPiece);
             TC_TRY(replay(false, lo, hi, [&](cudaStream_t cs) -> tc_status {
-                for (int i = lo; i < hi; i++) TC_TRY(fwd_step(seg[i - 1], seg[i], cs));
+                for (int i = lo; i < hi; i++) TC_TRY(fwd_step(seg[i - 1], seg[i], i == 1, cs));
                 return TC_OK;
             }));
         }
@@ -519,12 +522,12 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
         const int len = length(j);
         TC_TRY(copy_cm(ck[j], seg[0], NN, s));
         if (!oz && j + 1 < b.nck) {   // in place, with no copy a step
-            for (int i = 0; i < len; i++) TC_TRY(fwd_step(seg[0], seg[0], s));
+            for (int i = 0; i < len; i++) TC_TRY(fwd_step(seg[0], seg[0], true, s));
             TC_TRY(copy_cm(seg[0], ck[j + 1], NN, s));
             continue;
         }
         TC_TRY(states(len));
-        TC_TRY(fwd_step(seg[len - 1], j + 1 < b.nck ? ck[j + 1] : b.seg0, s));
+        TC_TRY(fwd_step(seg[len - 1], j + 1 < b.nck ? ck[j + 1] : b.seg0, len == 1, s));
     }
     // loss from rho_K (in seg0)
     loss_kernel<<<1, 1024, 0, s>>>(b.seg0.r, O_diag, N, b.small);
@@ -543,12 +546,10 @@ extern "C" TC_API tc_status tc_evolve_backward(const tc_params* params, double d
                 TC_TRY(gemm_c(N, seg[i], 0, b.L, 0, b.W, 1.0, 1.0, 0, cs));
                 continue;
             }
-            // the right operand holds Lambda and its scales from the product before, at first a state
-            TC_TRY(step_oz(N, z, true, i < hi - 1, b.L, b.L, b.X, cs));
+            // the right operand holds Lambda with its scales from the product before, at first a state
+            TC_TRY(step_oz(N, z, true, i == hi - 1, i < hi - 1, b.L, b.L, b.X, cs));
             // Lambda Hermitian: rho Lambda = rho Lambda^H
-            const int* col;
-            TC_TRY(columns(N, z.cols, kColsOfState, b.L, &col, cs));
-            TC_TRY(mul_oz(N, z, seg[i], b.L, false, b.W, true, col, cs));
+            TC_TRY(mul_oz(N, z, seg[i], b.L, false, b.W, true, oz_modular() ? z.cols.col : nullptr, cs));
         }
         return TC_OK;
     };

@@ -74,6 +74,7 @@ struct CrtOut {
     bool conj_b;       // B was loaded with conj: (br, bi) are the planes before it
     const void* b_c128;   // B interleaved (complex128, row stride ldb) instead of (br, bi)
     void* y_c128;         // mode 1: Y interleaved (row stride Np) instead of (yr, yi)
+    const CrtColumns* next = nullptr;   // mode 1, planes, N = Np <= 16384: the kColsOfState scales of Y too
 };
 tc_status crt_product(int mode, const CrtMat& A, const CrtMat& B, const double* br, const double* bi, int N,
                       size_t ldb, const CrtOut& out, cudaStream_t s);

@@ -843,7 +843,7 @@ tc_status oz_product(int mode, const OzMat& A, const OzMat& B, const double* br,
                      const OzOut& out, int group, cudaStream_t s) {
     if (A.Np != B.Np) return fail(TC_ERR_INVALID_ARG, "FP64 emulation: operands of different sizes");
     if (oz_modular())
-        return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch, out.accumulate, out.conj_b, out.b_c128, out.y_c128},
+        return crt_product(mode, A.crt, B.crt, br, bi, N, ldb, CrtOut{out.yr, out.yi, out.scratch, out.accumulate, out.conj_b, out.b_c128, out.y_c128, out.next},
                            s);
     if (out.accumulate || out.b_c128 || out.y_c128)
         return fail(TC_ERR_INVALID_ARG, "FP64 emulation: not an output of the digit form");

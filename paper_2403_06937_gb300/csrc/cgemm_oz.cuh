@@ -82,6 +82,7 @@ struct OzOut {
     // residue form only
     const void* b_c128 = nullptr;   // B interleaved (complex128, row stride ldb) instead of (br, bi)
     void* y_c128 = nullptr;         // mode 1: the result interleaved (row stride Np) instead of (yr, yi)
+    const CrtColumns* next = nullptr;   // mode 1: the column scales of the result, a state, too
 };
 // lazy: without planes of its own (residue form; see CrtMat), both operands of a product alike
 size_t oz_mat_bytes(int Np, bool left, bool lazy = false);
