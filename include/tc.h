@@ -197,8 +197,8 @@ TC_API tc_status tc_device_check(void);
  * tc_workspace_size: for the fastest form.  tc_workspace_least: the least that
  * the calls accept; with less than the stated size TC_FP64 and tc_expm run on
  * the FP64 DMMA (much slower), and TC_FP64_OZAKI makes its operands' residues
- * four moduli at a time (the same bits; some percent slower at large n).  The
- * two differ in the FP64 forms only. */
+ * four moduli at a time (the same bits; a step at n = 13 35 -> 43 ms, n = 14
+ * 296 -> 308 ms, n = 15 2.3 -> 3.4 s).  The two differ in the FP64 forms only. */
 TC_API size_t tc_workspace_size(int n, int precision, int ops, int steps, int ckpt_every);
 TC_API size_t tc_workspace_least(int n, int precision, int ops, int steps, int ckpt_every);
 

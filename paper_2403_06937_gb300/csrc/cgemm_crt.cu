@@ -16,7 +16,7 @@
 // close to the identity, and Y = diag(U) B^H + V B^H with the first term in
 // FP64 leaves the integers the small part V only.
 //
-// Column scales (TC_FP64).  One scale a row keeps nothing of an entry below
+// Column scales (TC_FP64's steps, the gradient).  One scale a row keeps nothing of an entry below
 // 2^-59 of its row's norm, and both U (an entry falls by a factor g dt for each
 // atom that differs) and a state after a few steps have such entries, on which
 // small populations rest.  There K gets a power of two of its own as well: the
@@ -57,7 +57,8 @@
 // instead of planes (lazy), and a product makes the planes of four moduli at a
 // time, multiplies those, and goes on to the next four; the same bits, 96 N^2
 // bytes of workspace a run instead of 192 (n = 14: 26 GB instead of 52), eight
-// residue passes a product instead of one.
+// residue passes a product instead of one (eight times that in the bands above
+// Np = 16384): a step at n = 13 35 -> 43 ms, n = 14 296 -> 308 ms, n = 15 2.3 -> 3.4 s.
 //
 // crt_combine_kernel turns the bytes of an entry into FP64 (integer work up to
 // the diagonal term's multiply-adds).
